@@ -103,19 +103,29 @@ int fs_profile_stop(fs_ctx *ctx, char *out, int64_t cap);
  * FS_ERR_UNSUPPORTED. */
 int fs_set_rotation_path(fs_ctx *ctx, int path);
 
-/* Arithmetic engine of the complex64 Givens sweeps (§3.2.3).
- *   FS_SWEEP_AUTO:      the CUDA cores (measured faster on GB300 at the
- *                       benchmarked sectors, see FS_SWEEP_TENSOR);
- *   FS_SWEEP_CUDA_CORE: every Givens rotation as FP32 FMAs on CUDA cores;
- *   FS_SWEEP_TENSOR:    each window step of 6 adjacent orbitals as one
- *                       dense product with the compound matrices of the
- *                       step (det V[S', S], §2.3) on the tcgen05 tensor
- *                       cores, both operands split exactly into three
- *                       BF16 pieces and six products kept (FP32
+/* Arithmetic engine of the Givens sweeps (§3.2.3).
+ *   FS_SWEEP_AUTO:      complex64 on the CUDA cores (measured faster on GB300
+ *                       at the benchmarked sectors, see FS_SWEEP_TENSOR);
+ *                       complex128 on the tcgen05 tensor cores as exact
+ *                       fixed-point digits (62 fraction bits relative to
+ *                       each vector's 2-norm, so at least as accurate as
+ *                       FP64 arithmetic) where the sector and the program
+ *                       allow it, else in FP64 on the CUDA cores.  There, a
+ *                       vector that holds a non-finite amplitude comes out
+ *                       not a number throughout;
+ *   FS_SWEEP_CUDA_CORE: every Givens rotation as FP32 / FP64 FMAs on CUDA
+ *                       cores;
+ *   FS_SWEEP_TENSOR:    complex64 too: each window step of 6 adjacent
+ *                       orbitals as one dense product with the compound
+ *                       matrices of the step (det V[S', S], §2.3) on the
+ *                       tcgen05 tensor cores, both operands split exactly
+ *                       into three BF16 pieces and six products kept (FP32
  *                       accuracy); falls back to the CUDA cores where the
- *                       tensor path does not apply (complex128, fewer than
- *                       6 orbitals, vectors spanning more than 2 CTAs).
- * Results agree to FP32 rounding.  FS_ERR_ARG for another value. */
+ *                       tensor path does not apply (fewer than 6 orbitals,
+ *                       vectors spanning more than 2 CTAs).  complex128 as
+ *                       under FS_SWEEP_AUTO.
+ * Results agree to the rounding of the dtype.  FS_ERR_ARG for another
+ * value. */
 enum { FS_SWEEP_AUTO = 0, FS_SWEEP_CUDA_CORE = 1, FS_SWEEP_TENSOR = 2 };
 int fs_set_sweep_engine(fs_ctx *ctx, int engine);
 

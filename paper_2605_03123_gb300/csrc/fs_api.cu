@@ -120,24 +120,29 @@ static void rotate(Ctx* ctx, Space* sa, Space* sb, void* v0, void* v1, int nst, 
   void* ea_a = scratch(ctx, "ea_a", sa->dim * csz);
   void* ea_b = scratch(ctx, "ea_b", sb->dim * csz);
   void* ea_o = scratch(ctx, "ea_o", sa->dim * csz);
-  launch_string_phase(sa, ea_a, dtype, phase_of(&pa, nullptr, 0, nullptr, n), st);
+  const bool fa = fx_supported(ctx, sa, sb, dtype, pa), fb = fx_supported(ctx, sb, sa, dtype, pb);
   PhaseDev ph;
-  ph.ea_a = ea_a;
-  launch_sweep(ctx, sa, sb, 0, v0, v1, nst, dtype, pa, ph, st);
+  if (!fa) {
+    launch_string_phase(sa, ea_a, dtype, phase_of(&pa, nullptr, 0, nullptr, n), st);
+    ph.ea_a = ea_a;
+  }
+  launch_sweep(ctx, sa, sb, 0, v0, v1, nst, dtype, pa, ph, st, nullptr, fa);
   PhaseDev phb;
+  const RotProgram* db = fb ? nullptr : &pb;
   if (dc) {
     launch_string_phase(sb, ea_b, dtype,
-                        phase_of(&pb, dc->J_bb ? dc->J_bb : dc->J_aa, dc->t, nullptr, n), st);
+                        phase_of(db, dc->J_bb ? dc->J_bb : dc->J_aa, dc->t, nullptr, n), st);
+    phb.ea_b = ea_b;
     launch_string_phase(sa, ea_o, dtype, phase_of(nullptr, dc->J_aa, dc->t, nullptr, n), st);
     phb.ea_a = ea_o;
     phb.has_x = 1;
     // mixed terms (p in I_a, q in I_b) and (p in I_b, q in I_a), J_ba = J_ab^T
     phb.X = real_mat(dc->J_ab, n, -dc->t);
-  } else {
+  } else if (!fb) {
     launch_string_phase(sb, ea_b, dtype, phase_of(&pb, nullptr, 0, nullptr, n), st);
+    phb.ea_b = ea_b;
   }
-  phb.ea_b = ea_b;
-  launch_sweep(ctx, sa, sb, 1, v0, v1, nst, dtype, pb, phb, st);
+  launch_sweep(ctx, sa, sb, 1, v0, v1, nst, dtype, pb, phb, st, nullptr, fb);
 }
 
 // The same rotation (and fused diagonal-Coulomb evolution) with every sweep a
@@ -157,45 +162,53 @@ static void rotate_alternating(Ctx* ctx, Space* sa, Space* sb, void* vec, void* 
   void* eo_a = scratch(ctx, "alt_eo_a", sa->dim * csz);
   void* eo_b = scratch(ctx, "alt_eo_b", sb->dim * csz);
   const double* Jbb = dc ? (dc->J_bb ? dc->J_bb : dc->J_aa) : nullptr;
+  const bool fa = fx_supported(ctx, sa, sb, dtype, pa), fb = fx_supported(ctx, sb, sa, dtype, pb);
+  const RotProgram *da = fa ? nullptr : &pa, *db = fb ? nullptr : &pb;
   if (!trans) {
-    launch_string_phase(sb, ea_b, dtype, phase_of(&pb, nullptr, 0, nullptr, n), st);
     PhaseDev p1;
-    p1.ea_b = ea_b;
-    launch_sweep(ctx, sa, sb, 1, vec, nullptr, 1, dtype, pb, p1, st);
+    if (!fb) {
+      launch_string_phase(sb, ea_b, dtype, phase_of(&pb, nullptr, 0, nullptr, n), st);
+      p1.ea_b = ea_b;
+    }
+    launch_sweep(ctx, sa, sb, 1, vec, nullptr, 1, dtype, pb, p1, st, nullptr, fb);
     launch_transpose(vec, tv, sa->dim, sb->dim, dtype, st);
     // alpha on rows of tv: spaces swapped, this spin (alpha) in the b slot
     PhaseDev p2;
     if (dc) {
-      launch_string_phase(sa, ea_a, dtype, phase_of(&pa, dc->J_aa, dc->t, nullptr, n), st);
+      launch_string_phase(sa, ea_a, dtype, phase_of(da, dc->J_aa, dc->t, nullptr, n), st);
+      p2.ea_b = ea_a;
       launch_string_phase(sb, eo_b, dtype, phase_of(nullptr, Jbb, dc->t, nullptr, n), st);
       p2.ea_a = eo_b;
       p2.has_x = 1;
       for (int p = 0; p < n; ++p)
         for (int q = 0; q < n; ++q) p2.X.v[q * n + p] = -dc->t * dc->J_ab[p * n + q];
-    } else {
+    } else if (!fa) {
       launch_string_phase(sa, ea_a, dtype, phase_of(&pa, nullptr, 0, nullptr, n), st);
+      p2.ea_b = ea_a;
     }
-    p2.ea_b = ea_a;
-    launch_sweep(ctx, sb, sa, 1, tv, nullptr, 1, dtype, pa, p2, st);
+    launch_sweep(ctx, sb, sa, 1, tv, nullptr, 1, dtype, pa, p2, st, nullptr, fa);
     trans = true;
   } else {
-    launch_string_phase(sa, ea_a, dtype, phase_of(&pa, nullptr, 0, nullptr, n), st);
     PhaseDev p1;
-    p1.ea_b = ea_a;
-    launch_sweep(ctx, sb, sa, 1, tv, nullptr, 1, dtype, pa, p1, st);
+    if (!fa) {
+      launch_string_phase(sa, ea_a, dtype, phase_of(&pa, nullptr, 0, nullptr, n), st);
+      p1.ea_b = ea_a;
+    }
+    launch_sweep(ctx, sb, sa, 1, tv, nullptr, 1, dtype, pa, p1, st, nullptr, fa);
     launch_transpose(tv, vec, sb->dim, sa->dim, dtype, st);
     PhaseDev p2;
     if (dc) {
-      launch_string_phase(sb, ea_b, dtype, phase_of(&pb, Jbb, dc->t, nullptr, n), st);
+      launch_string_phase(sb, ea_b, dtype, phase_of(db, Jbb, dc->t, nullptr, n), st);
+      p2.ea_b = ea_b;
       launch_string_phase(sa, eo_a, dtype, phase_of(nullptr, dc->J_aa, dc->t, nullptr, n), st);
       p2.ea_a = eo_a;
       p2.has_x = 1;
       p2.X = real_mat(dc->J_ab, n, -dc->t);
-    } else {
+    } else if (!fb) {
       launch_string_phase(sb, ea_b, dtype, phase_of(&pb, nullptr, 0, nullptr, n), st);
+      p2.ea_b = ea_b;
     }
-    p2.ea_b = ea_b;
-    launch_sweep(ctx, sa, sb, 1, vec, nullptr, 1, dtype, pb, p2, st);
+    launch_sweep(ctx, sa, sb, 1, vec, nullptr, 1, dtype, pb, p2, st, nullptr, fb);
     trans = false;
   }
 }
@@ -1181,20 +1194,22 @@ static void lucj_vjp_impl(Ctx* ctx, const fs_lucj* op, void* vec, void* cot, int
       launch_string_phase(sa, e2_a, dtype, phase_of(nullptr, Ja, -1.0, nullptr, n), st);
       launch_string_phase(sb, e2_b, dtype, phase_of(nullptr, Ja, -1.0, nullptr, n), st);
     }
-    launch_string_phase(sb, ea_b, dtype, phase_of(&inv, nullptr, 0, nullptr, n), st);
-    launch_string_phase(sa, ea_a, dtype, phase_of(&inv, nullptr, 0, nullptr, n), st);
+    const bool fa = fx_supported(ctx, sa, sb, dtype, inv);
+    const bool fb = fx_supported(ctx, sb, sa, dtype, inv);
+    if (!fb) launch_string_phase(sb, ea_b, dtype, phase_of(&inv, nullptr, 0, nullptr, n), st);
+    if (!fa) launch_string_phase(sa, ea_a, dtype, phase_of(&inv, nullptr, 0, nullptr, n), st);
     if (alpha_t && trans) {
       // alpha: undo on rows of the copies, T^alpha
       PhaseDev q1;
-      q1.ea_b = ea_a;
+      q1.ea_b = fa ? nullptr : ea_a;
       RevArgs t1;
       t1.T = Tm;
-      launch_sweep(ctx, sb, sa, 1, tpsi, tg, 2, dtype, inv, q1, st, &t1);
+      launch_sweep(ctx, sb, sa, 1, tpsi, tg, 2, dtype, inv, q1, st, &t1, fa);
       launch_transpose(tpsi, vec, sb->dim, sa->dim, dtype, st);
       launch_transpose(tg, cot, sb->dim, sa->dim, dtype, st);
       // beta: undo, T^beta, W and D_{m-1}^dag
       PhaseDev p2;
-      p2.ea_b = ea_b;
+      p2.ea_b = fb ? nullptr : ea_b;
       RevArgs r2;
       r2.T = Tm;
       if (m >= 1) {
@@ -1204,7 +1219,7 @@ static void lucj_vjp_impl(Ctx* ctx, const fs_lucj* op, void* vec, void* cot, int
         p2.has_x = 1;
         p2.X = real_mat(Jab, n, 1.0);
       }
-      launch_sweep(ctx, sa, sb, 1, vec, cot, 2, dtype, inv, p2, st, &r2);
+      launch_sweep(ctx, sa, sb, 1, vec, cot, 2, dtype, inv, p2, st, &r2, fb);
       if (m >= 1)
         launch_dc_grad(ctx, sa, sb, Wb, dtype, dJaa_d + (size_t)(m - 1) * nn,
                        dJab_d + (size_t)(m - 1) * nn, st);
@@ -1213,10 +1228,10 @@ static void lucj_vjp_impl(Ctx* ctx, const fs_lucj* op, void* vec, void* cot, int
     }
     // beta: undo, T^beta
     PhaseDev p1;
-    p1.ea_b = ea_b;
+    p1.ea_b = fb ? nullptr : ea_b;
     RevArgs r1;
     r1.T = Tm;
-    launch_sweep(ctx, sa, sb, 1, vec, cot, 2, dtype, inv, p1, st, &r1);
+    launch_sweep(ctx, sa, sb, 1, vec, cot, 2, dtype, inv, p1, st, &r1, fb);
     // alpha: undo, T^alpha, W and D_{m-1}^dag
     if (alpha_t) {
       // the same sweep as a row sweep of the transposed states: this spin
@@ -1224,7 +1239,7 @@ static void lucj_vjp_impl(Ctx* ctx, const fs_lucj* op, void* vec, void* cot, int
       launch_transpose(vec, tpsi, sa->dim, sb->dim, dtype, st);
       launch_transpose(cot, tg, sa->dim, sb->dim, dtype, st);
       PhaseDev q2;
-      q2.ea_b = ea_a;
+      q2.ea_b = fa ? nullptr : ea_a;
       RevArgs t2;
       t2.T = Tm;
       if (m >= 1) {
@@ -1235,14 +1250,14 @@ static void lucj_vjp_impl(Ctx* ctx, const fs_lucj* op, void* vec, void* cot, int
         for (int p = 0; p < n; ++p)
           for (int q = 0; q < n; ++q) q2.X.v[q * n + p] = Jab[p * n + q];
       }
-      launch_sweep(ctx, sb, sa, 1, tpsi, tg, 2, dtype, inv, q2, st, &t2);
+      launch_sweep(ctx, sb, sa, 1, tpsi, tg, 2, dtype, inv, q2, st, &t2, fa);
       if (m >= 1)
         launch_dc_grad(ctx, sb, sa, Wb, dtype, dJaa_d + (size_t)(m - 1) * nn,
                        dJabT_d + (size_t)(m - 1) * nn, st);
       trans = true;
     } else {
       PhaseDev p2;
-      p2.ea_a = ea_a;
+      p2.ea_a = fa ? nullptr : ea_a;
       RevArgs r2;
       r2.T = Tm;
       if (m >= 1) {
@@ -1252,7 +1267,7 @@ static void lucj_vjp_impl(Ctx* ctx, const fs_lucj* op, void* vec, void* cot, int
         p2.has_x = 1;
         p2.X = real_mat(Jab, n, 1.0);
       }
-      launch_sweep(ctx, sa, sb, 0, vec, cot, 2, dtype, inv, p2, st, &r2);
+      launch_sweep(ctx, sa, sb, 0, vec, cot, 2, dtype, inv, p2, st, &r2, fa);
       if (m >= 1)
         launch_dc_grad(ctx, sa, sb, Wb, dtype, dJaa_d + (size_t)(m - 1) * nn,
                        dJab_d + (size_t)(m - 1) * nn, st);

@@ -126,6 +126,23 @@ void tpass_groups_host(const std::vector<TPass>& passes, const std::vector<TReco
                        const std::vector<uint8_t>& rkey, int b, std::vector<TRecord>& grec,
                        std::vector<int>& goff);
 
+// Gather addresses of one window position of the fixed-point sweeps: start
+// (in uint16 units) and orbits of the classes m = 3, 2, 4, 1, 5, 6.
+namespace fx {
+struct Seg {
+  int start[6], cnt[6];
+};
+constexpr int kMaxSteps = 48;  // steps of one program
+// Sizes and programs the fixed-point sweep takes.  It needs a kernel more
+// (the step images, about 10 us) than the FP64 sweep: 400 amplitudes (6 (3,3))
+// ran 62 against 66 us for both spins, 49 (7 (1,6)) 66 against 52 us.  A step
+// costs as much as the FP64 sweep spends on 2.5 rotations (N = 14: 3.3 clocks
+// per amplitude and SM against 1.4 a rotation), so a program with few
+// rotations a step (a single Givens gate) keeps the FP64 sweep.
+constexpr int64_t kMinAmps = 400;
+constexpr int kMinGivensPerStep = 3;
+}  // namespace fx
+
 // ------------------------------------------------------ device tables
 // Per-sector-spin tables: strings of `nocc` electrons in `norb` orbitals.
 struct Space {
@@ -162,6 +179,10 @@ struct Space {
     std::vector<int> off_h;
     std::vector<uint8_t> okey_h;
   } win[8];
+  // gather addresses of the fixed-point sweeps, per window position
+  fx::Seg* fx_seg = nullptr;
+  uint16_t* fx_idx = nullptr;
+  std::vector<fx::Seg> fx_seg_h;
   // transition-reduction passes (reverse mode), built on first use, and the
   // records regrouped for clusters of 2^b CTAs
   struct TPassDev* tpass = nullptr;
@@ -487,7 +508,15 @@ struct RevArgs {
 void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir,
                   void* st0, void* st1, int nst, int dtype,
                   const RotProgram& prog, const PhaseDev& ph, cudaStream_t st,
-                  const RevArgs* rev = nullptr);
+                  const RevArgs* rev = nullptr, bool fx = false);
+// Whether the complex128 fixed-point sweep (fs_sweep_fx.cu) takes a program:
+// launch_sweep with fx = true then applies the program's diagonal layer too,
+// so `ph` must not hold it.
+bool fx_supported(const Ctx* ctx, const Space* sthis, const Space* sother, int dtype,
+                  const RotProgram& rp);
+// That sweep, on st0 and (unless null) st1, with the phase `ph` behind it.
+void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0, void* st1,
+                     const RotProgram& rp, const PhaseDev& ph, cudaStream_t st);
 
 // dJ from W = Im(conj(g) psi) of one diagonal-Coulomb gate (t = 1):
 //   dJ_ab[p][q] += sum_{ij} W_ij occ_a(i)_p occ_b(j)_q

@@ -485,7 +485,20 @@ static void set_cluster_layout(SweepGeom& g, const Space* sp, int CS, Fits&& fit
 
 void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0,
                   void* st1, int nst, int dtype, const RotProgram& rp,
-                  const PhaseDev& ph, cudaStream_t st, const RevArgs* rev) {
+                  const PhaseDev& ph, cudaStream_t st, const RevArgs* rev, bool fx) {
+  if (fx) {
+    if (nst == 1) {
+      launch_sweep_fx(ctx, sa, sb, dir, st0, nullptr, rp, ph, st);
+      return;
+    }
+    // reverse: both states rotated, then the reductions and the second phase
+    // as a sweep without rotations
+    launch_sweep_fx(ctx, sa, sb, dir, st0, st1, rp, PhaseDev{}, st);
+    RotProgram none;
+    none.phase.assign(sa->norb, zd(1.0));
+    launch_sweep(ctx, sa, sb, dir, st0, st1, nst, dtype, none, ph, st, rev, false);
+    return;
+  }
   FS_REQUIRE((nst == 2) == (rev != nullptr), FS_ERR_ARG, "reverse mode needs two states");
   const Space* sthis = dir == 0 ? sa : sb;
   const Space* sother = dir == 0 ? sb : sa;

@@ -1,0 +1,893 @@
+// Complex128 orbital-rotation sweeps on the tensor cores, in exact
+// fixed-point digits (fs_fx.cuh).
+//
+// The work is that of the window sweeps (fs_sweep.cu): a slab of KV vectors
+// of the rotated spin is staged in shared memory, the program's window steps
+// of W = 6 adjacent orbitals are applied to it in order, and it is written
+// back once with the configuration phases.  A step acts on the C(6, m)
+// strings of an orbit as the compound matrix C_m(V) of its 6 x 6 unitary V
+// (§2.3), so per class m it is a product X' = X C_m(V)^T over all orbits of
+// all vectors of the slab; the diagonal layer of the decomposition is
+// multiplied into the last step that covers each orbital, which makes class
+// m = 6 (one string, factor det V) part of such steps.
+//
+// Each vector is held as 64-bit integers scaled by its own 2-norm, which the
+// rotations keep, from the first step to the last.  A tile is 128 rows
+// (orbit, vector): the sixteen warps gather the rows' amplitudes (the four
+// warps of one TMEM lane quarter share a row's strings), cut them into seven
+// digits and store those to TMEM as the A operand; 28 digit products against
+// the step's images in shared memory accumulate in seven TMEM accumulators;
+// the warps read those back, join them and scatter the new amplitudes.
+//
+// Measured (one GB300, one spin, complex128): N = 14 (7,7) 1.64 ms against
+// 6.74 ms of the FP64 sweep, which runs at 0.8 of the FP64 rate (2 FMA per
+// clock and SM); N = 12 (6,6) 0.105 against 0.80 ms; N = 8 (4,4) 32 + 18
+// (images) against 45 us.  Bound by the integer and FP32 instructions of the
+// digit cutting and joining (about half of the issue slots used, two thirds
+// of the tile rows filled at N = 14) and, behind them, by the products (2250
+// of some 5000 clocks of a class 3 tile).
+#include <algorithm>
+#include <array>
+#include <cmath>
+#include <type_traits>
+#include <vector>
+
+#include "fs_fx.cuh"
+#include "fs_common.cuh"
+#include "fs_internal.h"
+
+namespace fs {
+namespace fx {
+
+constexpr int kThreads = 512;            // the sixteen warps that move data
+constexpr int kWarps = kThreads / 32;
+constexpr int kCta = kThreads + 32;      // and the one that issues the products
+constexpr int kMaxVec = 32;  // vectors per slab
+constexpr size_t kStaticBytes = 10 * 1024;  // bound on the kernel's static shared memory
+// bytes of one digit's image of class m, and of the classes' seven digits in
+// the order 3, 2, 4, 1, 5, then det V as two fixed-point words
+__host__ __device__ constexpr int cls(int i) {
+  return i == 0 ? 3 : i == 1 ? 2 : i == 2 ? 4 : i == 3 ? 1 : 5;
+}
+__host__ __device__ constexpr int img_offset(int m) {
+  int o = 0;
+  for (int i = 0; i < 5; ++i) {
+    if (cls(i) == m) return o;
+    o += kDig * tc::piece_bytes(cls(i));
+  }
+  return o;
+}
+constexpr int kImgBytes = img_offset(6);           // staged in shared memory
+constexpr int kImgFirst = img_offset(2);           // class 3: the first copy
+constexpr int kStepBytes = kImgBytes + 128;        // with det V
+static_assert(kImgBytes % 128 == 0, "images must stay 128-byte aligned");
+// TMEM: the A digits at columns 0 .., the accumulators behind them
+constexpr int kColD = kDig * 24;
+static_assert(kColD + kSum * 48 <= 512, "class 3 tile must fit the TMEM");
+// kind::f16, D f32, A and B f16, K-major both, n columns
+__host__ __device__ constexpr uint32_t idesc(int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(tc::kRows >> 4) << 24);
+}
+
+// --------------------------------------------------------- step images
+struct StepMats {
+  long long v[kMaxSteps][72];  // V of each step, row-major 6 x 6 complex, fixed point
+};
+
+__device__ __forceinline__ longlong2 cmul_fx(longlong2 x, longlong2 y) {
+  return make_longlong2(mul(x.x, y.x) - mul(x.y, y.y), mul(x.x, y.y) + mul(x.y, y.x));
+}
+
+// Per step, the compound matrices C_m(V)[S', S] = det V[S', S] by Laplace
+// expansion along the first row of S', in fixed point (integer multiplies:
+// the FP64 units are the slower ones, and the entries keep 62 bits), then
+// the digits of their real forms [[Re, -Im], [Im, Re]] (rows = output reals,
+// columns = input reals, re/im interleaved, zero padding), K-major core
+// matrices (tc::b_offset).  Two blocks per step: class 3, and the others.
+__global__ void __launch_bounds__(512) k_fx_images(const __grid_constant__ StepMats sm,
+                                                   unsigned char* out) {
+  __shared__ longlong2 M[7][400];  // [m]: ns x ns
+  __shared__ uint8_t list[7][20], index[64];
+  const int tid = threadIdx.x, part = blockIdx.y;
+  unsigned char* img = out + (size_t)blockIdx.x * kStepBytes;
+  if (tid < 64) {
+    const int m = __popc(tid);
+    int k = 0;
+    for (int x = 0; x < tid; ++x) k += __popc(x) == m;
+    list[m][k] = (uint8_t)tid;
+    index[tid] = (uint8_t)k;
+  }
+  if (tid < 36)
+    M[1][tid] = make_longlong2(sm.v[blockIdx.x][2 * tid], sm.v[blockIdx.x][2 * tid + 1]);
+  __syncthreads();
+  for (int m = 2; m <= (part == 0 ? 3 : 6); ++m) {
+    const int ns = tc::binom6(m), n1 = tc::binom6(m - 1);
+    for (int e = tid; e < ns * ns; e += blockDim.x) {
+      const int R = list[m][e / ns], S = list[m][e % ns];
+      const int r0 = __ffs(R) - 1, R1 = index[R & (R - 1)];
+      longlong2 a = make_longlong2(0, 0);
+      bool neg = false;
+      for (int c = S; c; c &= c - 1, neg = !neg) {
+        const int j = __ffs(c) - 1;
+        const longlong2 z = cmul_fx(M[1][r0 * 6 + j], M[m - 1][R1 * n1 + index[S ^ (1 << j)]]);
+        a.x += neg ? -z.x : z.x;
+        a.y += neg ? -z.y : z.y;
+      }
+      M[m][e] = a;
+    }
+    __syncthreads();
+  }
+  for (int ci = part; ci < (part == 0 ? 1 : 5); ++ci) {
+    const int m = cls(ci), ns = tc::binom6(m), kpad = tc::kp(m), nh = tc::np(m) / 2;
+    unsigned char* o = img + img_offset(m);
+    for (int e = tid; e < nh * nh; e += blockDim.x) {
+      const int r = e / nh, c = e - r * nh;
+      longlong2 z = make_longlong2(0, 0);
+      if (r < ns && c < ns) z = M[m][r * ns + c];
+      uint32_t w0[kDig], w1[kDig];
+      digits2(z.x, -z.y, w0);  // row 2r:     columns 2c, 2c + 1
+      digits2(z.y, z.x, w1);   // row 2r + 1
+      const int o0 = tc::b_offset(2 * r, 2 * c, kpad), o1 = tc::b_offset(2 * r + 1, 2 * c, kpad);
+      for (int j = 0; j < kDig; ++j) {
+        *reinterpret_cast<uint32_t*>(o + j * tc::piece_bytes(m) + o0) = w0[j];
+        *reinterpret_cast<uint32_t*>(o + j * tc::piece_bytes(m) + o1) = w1[j];
+      }
+    }
+  }
+  if (part == 1 && tid == 0) *reinterpret_cast<longlong2*>(img + kImgBytes) = M[6][0];
+}
+
+// ------------------------------------------------------------ the sweep
+__device__ __forceinline__ void timeout(int* status) {
+  if (status) atomicCAS(status, 0, (int)FS_ERR_TIMEOUT);
+}
+
+// The strings of class m that column group g of a tile handles (20: 4g ..
+// 4g + 3 and 16 + g; 15: 4g .. 4g + 3; 6: 2g, 2g + 1) and the entries of its
+// row of gather addresses (padded to a power of two).
+__host__ __device__ constexpr int grp_pad(int m) { return m == 3 ? 8 : (m == 2 || m == 4) ? 4 : 2; }
+__host__ __device__ constexpr int grp_string(int m, int g, int j) {
+  if (m == 3) return j < 4 ? 4 * g + j : j == 4 ? 16 + g : -1;
+  const int k = (m == 2 || m == 4) ? 4 * g + j : 2 * g + j;
+  return k < tc::binom6(m) ? k : -1;
+}
+
+// Per-thread state of the tile pipeline.
+struct Thread {
+  uint32_t lane0;  // TMEM base with this warp's lane offset
+  int wg, row;     // column group; row within a tile
+};
+// The strings of one tile row that a thread owns (offset in the slab, -1:
+// none), their digits, and the raw accumulators of their products.
+struct Item {
+  uint32_t p[3];  // 16-bit slab cells (a slab has fewer than 2^14), 0xFFFF: none
+  __device__ __forceinline__ uint32_t off(int j) const { return (p[j >> 1] >> (16 * (j & 1))) & 0xFFFFu; }
+};
+
+// Gather and digits of one tile row of class shape M (3, 2 for 2 and 4, 1
+// for 1 and 5): rows = count x vectors, row = vector * count + orbit.  Rows
+// past the end and strings past the class's last carry zeros.
+template <int M>
+__device__ __forceinline__ void gather(const Thread& t, const longlong2* slab, int d,
+                                       const uint16_t* ix, int count, int rows, int row0,
+                                       Item& it, uint32_t (&w)[5][kDig]) {
+  constexpr int P = grp_pad(M), G = M == 3 ? 5 : P;
+  const int row = row0 + t.row;
+  uint32_t q[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
+  if (row < rows) {
+    const int kv = (int)(((float)row + 0.5f) * (1.f / (float)count)), o = row - kv * count;
+    const uint16_t* src = ix + (t.wg * count + o) * P;
+    if constexpr (P == 8) {
+      const uint4 u = *reinterpret_cast<const uint4*>(src);
+      q[0] = u.x;
+      q[1] = u.y;
+      q[2] = u.z;
+    } else if constexpr (P == 4) {
+      const uint2 u = *reinterpret_cast<const uint2*>(src);
+      q[0] = u.x;
+      q[1] = u.y;
+    } else {
+      q[0] = *reinterpret_cast<const uint32_t*>(src);
+    }
+    // the vector's first cell added to both halves (no carry between them:
+    // cells stay below 2^14), except where there is no string
+    const uint32_t b = (uint32_t)(kv * d), bb = b | (b << 16);
+    if (P == 4 && t.wg == 3) {
+      q[0] += bb;
+      q[1] = ((q[1] + b) & 0xFFFFu) | 0xFFFF0000u;
+    } else {
+#pragma unroll
+      for (int k = 0; k < (G + 1) / 2; ++k) q[k] += bb;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) it.p[k] = q[k];
+#pragma unroll
+  for (int j = 0; j < G; ++j) {
+    longlong2 x = make_longlong2(0, 0);
+    if (it.off(j) != 0xFFFFu) x = slab[it.off(j)];
+    digits2(x.x, x.y, w[j]);
+  }
+}
+template <int M>
+__device__ __forceinline__ void put_digits(const Thread& t, const uint32_t (&w)[5][kDig]) {
+  constexpr int AC = tc::a_cols(M);
+#pragma unroll
+  for (int i = 0; i < kDig; ++i) {
+    if constexpr (M == 1) {
+      if (t.wg < 3) tc::tmem_st2(t.lane0 + i * AC + 2 * t.wg, w[0][i], w[1][i]);
+    } else {
+      const uint32_t q[4] = {w[0][i], w[1][i], w[2][i], w[3][i]};
+      tc::tmem_st4(t.lane0 + i * AC + 4 * t.wg, q);
+      if constexpr (M == 3) tc::tmem_st1(t.lane0 + i * AC + 16 + t.wg, w[4][i]);
+    }
+  }
+}
+// Digit i of A meets digits 1 .. 8 - i of B, which lie one after another as
+// further rows, as their accumulators do: one product of up to 256 columns.
+// (A product of 16 .. 48 columns takes 51 clocks: one per digit pair made a
+// class 3 tile wait 4300 clocks for its products, this form 2250, near the
+// 4096 multiply-adds per clock and SM.)
+template <int M>
+__device__ __forceinline__ void issue(uint32_t tbase, uint32_t b0, uint32_t bar) {
+  constexpr int KP = tc::kp(M), AC = tc::a_cols(M), NP = tc::np(M), MAXJ = 256 / NP;
+#pragma unroll
+  for (int ks = 0; ks < KP / 16; ++ks)
+#pragma unroll
+    for (int i = 1; i <= kDig; ++i)
+#pragma unroll
+      for (int j = 1; j <= 8 - i; j += MAXJ) {
+        const int nj = 8 - i - j + 1 < MAXJ ? 8 - i - j + 1 : MAXJ;
+        const uint64_t bd =
+            tc::sdesc(b0 + (j - 1) * tc::piece_bytes(M) + ks * 256, 128, (KP / 8) * 128);
+        tc::mma_bf16(tbase + kColD + (i + j - 2) * NP, tbase + (i - 1) * AC + 8 * ks, bd,
+                     idesc(nj * NP), ks == 0 && i == 1 ? 0u : 1u);
+      }
+  tc::mma_commit(bar);
+}
+// The raw accumulators of a thread's strings h and h + 1 (of the first four).
+template <int M>
+__device__ __forceinline__ void take(const Thread& t, int h, uint32_t (&f)[kSum][4]) {
+  constexpr int NP = tc::np(M);
+  const uint32_t dl = t.lane0 + kColD + (M == 1 ? 4 : 8) * t.wg + 2 * h;
+#pragma unroll
+  for (int s = 0; s < kSum; ++s) tc::tmem_ld4(dl + s * NP, f[s]);
+  tc::wait_ld();
+}
+// The fifth string of a class 3 row, from its accumulators to the slab.
+__device__ __forceinline__ void finish_fifth(const Thread& t, longlong2* slab, const Item& it) {
+  const uint32_t dl = t.lane0 + kColD + 32 + 2 * t.wg;
+  uint32_t h[kSum][2];
+#pragma unroll
+  for (int s = 0; s < kSum; ++s) tc::tmem_ld2(dl + s * tc::np(3), h[s]);
+  tc::wait_ld();
+  float re[kSum], im[kSum];
+#pragma unroll
+  for (int s = 0; s < kSum; ++s) {
+    re[s] = __uint_as_float(h[s][0]);
+    im[s] = __uint_as_float(h[s][1]);
+  }
+  if (it.off(4) != 0xFFFFu) slab[it.off(4)] = make_longlong2(join(re), join(im));
+}
+__device__ __forceinline__ void scatter(longlong2* slab, const Item& it, int h,
+                                        const uint32_t (&f)[kSum][4]) {
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    float re[kSum], im[kSum];
+#pragma unroll
+    for (int s = 0; s < kSum; ++s) {
+      re[s] = __uint_as_float(f[s][2 * j]);
+      im[s] = __uint_as_float(f[s][2 * j + 1]);
+    }
+    const uint32_t o = it.off(h + j);
+    if (o != 0xFFFFu) slab[o] = make_longlong2(join(re), join(im));
+  }
+}
+
+struct Args {
+  double2* st[2];  // blockIdx.y chooses: psi and the cotangent share a program
+  int64_t d_b;
+  int dir, d, nvec, KV, nsteps, norb, nchunk, has_x;
+  const Seg* seg;        // per window position
+  const uint16_t* idx;
+  int cap_first, cap_rest;  // bytes of the staged addresses: class 3; the others
+  const unsigned char* img;
+  const uint32_t *masks_this, *masks_other;
+  const double2 *ea_this, *ea_other;
+  int* status;
+  uint8_t a[kMaxSteps];     // window position of each step
+  uint8_t full[kMaxSteps];  // class 6 moves in this step (det V != 1)
+};
+
+// A barrier of the sixteen data warps.
+__device__ __forceinline__ void sync_data() {
+  asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
+}
+
+// Walks the tiles of a step: class cls(ci), rows row0 ..; ci = 5 past the
+// last.  on_rest runs when the walk leaves class 3.
+struct Walk {
+  int ci = 0, row0 = 0;
+  template <typename F>
+  __device__ __forceinline__ void settle(const Seg& sg, int nv, F&& on_rest) {
+    while (ci < 5 && row0 >= sg.cnt[ci] * nv) {
+      if (ci == 0) on_rest();
+      ++ci;
+      row0 = 0;
+    }
+  }
+};
+
+// One CTA per slab, one CTA per SM (all of its TMEM): sixteen data warps and
+// one that stages the images and issues the products.  (An issue blocks while
+// the tensor cores are busy, and a data warp that issued a tile kept the
+// other fifteen waiting.)  With 17 warps a thread has 96 registers, so the
+// accumulators are taken two strings at a time.
+__global__ void __launch_bounds__(kCta, 1)
+    k_sweep_fx(const __grid_constant__ Args g, const __grid_constant__ Mat X) {
+  extern __shared__ __align__(128) unsigned char smraw[];
+  __shared__ __align__(8) uint64_t s_mbar[4];
+  __shared__ uint32_t s_tmem;
+  __shared__ uint32_t s_max[kMaxVec][kWarps];
+  __shared__ float s_sum[kMaxVec][kWarps];
+  __shared__ Seg s_seg[kMaxSteps];
+  __shared__ int s_eb[kMaxVec];  // biased exponent of the scale, -1: not finite
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  double2* const state = g.st[blockIdx.y];
+  const int d = g.d, v0 = blockIdx.x * g.KV, nv = min(g.KV, g.nvec - v0);
+  unsigned char* simg = smraw;
+  uint16_t* ix_first = reinterpret_cast<uint16_t*>(smraw + kImgBytes);
+  uint16_t* ix_rest = reinterpret_cast<uint16_t*>(smraw + kImgBytes + g.cap_first);
+  longlong2* slab = reinterpret_cast<longlong2*>(smraw + kImgBytes + g.cap_first + g.cap_rest);
+  const uint32_t bar_first = tc::smem_u32(&s_mbar[0]), bar_rest = tc::smem_u32(&s_mbar[1]);
+  const uint32_t bar_mma = tc::smem_u32(&s_mbar[2]), bar_ready = tc::smem_u32(&s_mbar[3]);
+  if (tid == 0) {
+    for (int i = 0; i < 3; ++i) tc::mbar_init(tc::smem_u32(&s_mbar[i]), 1);
+    tc::mbar_init(bar_ready, kWarps);
+    tc::mbar_fence_init();
+  }
+  if (warp == 0) tc::tmem_alloc(tc::smem_u32(&s_tmem), 512);
+  for (int i = tid; i < g.nsteps; i += kCta) s_seg[i] = g.seg[g.a[i]];
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  if (warp == kWarps) {
+    if (lane == 0) {
+      // a step's images and gather addresses: class 3, then the other
+      // classes, each copy issued once the step before has used its half
+      auto stage_first = [&](int st) {
+        const Seg& q = s_seg[st];
+        const uint32_t len = 2u * (uint32_t)(q.start[1] - q.start[0]);
+        tc::mbar_expect_tx(bar_first, kImgFirst + len);
+        tc::bulk_g2s(tc::smem_u32(simg), g.img + (size_t)st * kStepBytes, kImgFirst, bar_first);
+        if (len) tc::bulk_g2s(tc::smem_u32(ix_first), g.idx + q.start[0], len, bar_first);
+      };
+      auto stage_rest = [&](int st) {
+        const Seg& q = s_seg[st];
+        const uint32_t len = 2u * (uint32_t)(q.start[5] - q.start[1]);
+        tc::mbar_expect_tx(bar_rest, kImgBytes - kImgFirst + len);
+        tc::bulk_g2s(tc::smem_u32(simg) + kImgFirst, g.img + (size_t)st * kStepBytes + kImgFirst,
+                     kImgBytes - kImgFirst, bar_rest);
+        if (len) tc::bulk_g2s(tc::smem_u32(ix_rest), g.idx + q.start[1], len, bar_rest);
+      };
+      const uint32_t tbase = s_tmem, bimg = tc::smem_u32(simg);
+      uint32_t ph = 0, phr = 0;  // phases of the products and of the data warps
+      stage_first(0);
+      stage_rest(0);
+      for (int st = 0; st < g.nsteps; ++st) {
+        const Seg& sg = s_seg[st];
+        const uint32_t phs = (uint32_t)st & 1u;
+        const bool more = st + 1 < g.nsteps;
+        bool ahead = false;  // the next step's class 3 copy is under way
+        if (!tc::mbar_wait(bar_first, phs)) timeout(g.status);
+        Walk wk;
+        // leaving class 3: its products are done and its addresses read (a
+        // step without any has not been seen by every data warp yet)
+        auto leave3 = [&]() {
+          ahead = more && sg.cnt[0] > 0;
+          if (ahead) stage_first(st + 1);
+          if (!tc::mbar_wait(bar_rest, phs)) timeout(g.status);
+        };
+        wk.settle(sg, nv, leave3);
+        while (wk.ci < 5) {
+          if (!tc::mbar_wait(bar_ready, phr)) timeout(g.status);
+          phr ^= 1u;
+          tc::fence_after();
+          const uint32_t b0 = bimg + img_offset(cls(wk.ci));
+          if (wk.ci == 0) issue<3>(tbase, b0, bar_mma);
+          else if (wk.ci < 3) issue<2>(tbase, b0, bar_mma);
+          else issue<1>(tbase, b0, bar_mma);
+          if (!tc::mbar_wait(bar_mma, ph)) timeout(g.status);
+          ph ^= 1u;
+          wk.row0 += tc::kRows;
+          wk.settle(sg, nv, leave3);
+        }
+        // the data warps have ended the step
+        if (!tc::mbar_wait(bar_ready, phr)) timeout(g.status);
+        phr ^= 1u;
+        if (more && !ahead) stage_first(st + 1);
+        if (more) stage_rest(st + 1);
+      }
+    }
+    return;
+  }
+  // ---- load
+  double2* raw = reinterpret_cast<double2*>(slab);
+  auto cp16 = [&](double2* dst, const double2* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src)
+                 : "memory");
+  };
+  if (g.dir == 1) {
+    for (int kv = 0; kv < nv; ++kv) {
+      const double2* src = state + (int64_t)(v0 + kv) * g.d_b;
+      for (int e = tid; e < d; e += kThreads) cp16(raw + (size_t)kv * d + e, src + e);
+    }
+  } else {
+    for (int i = tid; i < d * nv; i += kThreads) {
+      const int e = i / nv, kv = i - e * nv;
+      cp16(raw + (size_t)kv * d + e, state + (int64_t)e * g.d_b + v0 + kv);
+    }
+  }
+  // zeros in the A columns no tile writes (their B rows are zero, but a NaN
+  // left in TMEM would not be)
+  {
+    const uint32_t z[4] = {0, 0, 0, 0};
+    const uint32_t l0 = s_tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    for (int c = 4 * (warp >> 2); c < kColD; c += 16) tc::tmem_st4(l0 + c, z);
+    tc::wait_st();
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  sync_data();
+  // ---- scale of each vector: the exponent of its largest part, then its
+  // 2-norm in FP32 relative to that; `per` warps share a vector
+  const int per = nv >= kWarps ? 1 : kWarps / nv, ngrp = kWarps / per;
+  const int kv1 = warp / per, sub = warp - kv1 * per;
+  if (kv1 < ngrp)
+    for (int kv = kv1; kv < nv; kv += ngrp) {
+      uint32_t mx = 0;
+#pragma unroll 4
+    for (int e = sub * 32 + lane; e < d; e += 32 * per) {
+        const double2 x = raw[(size_t)kv * d + e];
+        mx = max(mx, (uint32_t)exp_field(x.x));
+        mx = max(mx, (uint32_t)exp_field(x.y));
+      }
+      mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+      if (lane == 0) s_max[kv][sub] = mx;
+    }
+  sync_data();
+  auto scaled = [](double x, int f) {  // about |x| 2^(1023 - f), 0 when far below
+    const int q = exp_field(x) - f + 127;
+    return q > 1 ? __int_as_float((q << 23) | ((__double2hiint(x) & 0xFFFFF) << 3)) : 0.f;
+  };
+  if (kv1 < ngrp)
+    for (int kv = kv1; kv < nv; kv += ngrp) {
+      uint32_t f = 1;
+      for (int i = 0; i < per; ++i) f = max(f, s_max[kv][i]);
+      float s = 0.f;
+#pragma unroll 4
+    for (int e = sub * 32 + lane; e < d; e += 32 * per) {
+        const double2 x = raw[(size_t)kv * d + e];
+        const float a = scaled(x.x, (int)f), b = scaled(x.y, (int)f);
+        s = fmaf(a, a, fmaf(b, b, s));
+      }
+#pragma unroll
+      for (int k = 16; k > 0; k >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, k);
+      if (lane == 0) s_sum[kv][sub] = s;
+    }
+  sync_data();
+  if (kv1 < ngrp)
+    for (int kv = kv1; kv < nv; kv += ngrp) {
+      uint32_t f = 1;
+      float s = 0.f;
+      for (int i = 0; i < per; ++i) {
+        f = max(f, s_max[kv][i]);
+        s += s_sum[kv][i];
+      }
+      // norm = 2^(f - 1023) sqrt(s) < 2^(eb - 1023); s < 2^20
+      const float r = fmaxf(sqrtf(s) * 1.001f, 1.0f);
+      const int k = ((__float_as_int(r) >> 23) & 0xFF) - 126;  // r < 2^k
+      const bool finite = f < 0x7FF;
+      const int eb = (int)f + k;
+      if (sub == 0 && lane == 0) s_eb[kv] = finite ? eb : -1;
+#pragma unroll 4
+    for (int e = sub * 32 + lane; e < d; e += 32 * per) {
+        const double2 x = raw[(size_t)kv * d + e];
+        slab[(size_t)kv * d + e] = finite ? make_longlong2(from_double(x.x, eb), from_double(x.y, eb))
+                                          : make_longlong2(0, 0);
+      }
+    }
+  Thread t;
+  t.wg = warp >> 2;
+  t.row = (warp & 3) * 32 + lane;
+  t.lane0 = s_tmem + ((uint32_t)((warp & 3) * 32) << 16);
+  uint32_t ph_mma = 0;
+  sync_data();
+  // ---- window steps.  The tiles of a step touch different strings, so
+  // they run as a pipeline: while the products of one tile run, the warps
+  // join and scatter the tile before it and gather the tile after it.
+  for (int st = 0; st < g.nsteps; ++st) {
+    const Seg& sg = s_seg[st];
+    const uint32_t ph = (uint32_t)st & 1u;
+    Walk wk;
+    auto leave3 = [&]() {
+      if (!tc::mbar_wait(bar_rest, ph)) timeout(g.status);
+    };
+    Item cur, nxt;
+    uint32_t w[5][kDig];
+    // a warp whose 32 rows lie past the class's last, or that owns no
+    // string of the class, leaves the tile alone
+    auto active = [&]() {
+      return wk.ci < 5 && wk.row0 + (warp & 3) * 32 < sg.cnt[wk.ci] * nv &&
+             (wk.ci < 3 || t.wg < 3);
+    };
+    auto load = [&](Item& it) {  // gathers the next tile
+      const int ci = wk.ci, cnt = sg.cnt[ci], rows = cnt * nv;
+      const uint16_t* ix = ci == 0 ? ix_first : ix_rest + (sg.start[ci] - sg.start[1]);
+      if (ci == 0) gather<3>(t, slab, d, ix, cnt, rows, wk.row0, it, w);
+      else if (ci < 3) gather<2>(t, slab, d, ix, cnt, rows, wk.row0, it, w);
+      else gather<1>(t, slab, d, ix, cnt, rows, wk.row0, it, w);
+    };
+    auto put = [&](int c) {
+      if (c == 0) put_digits<3>(t, w);
+      else if (c < 3) put_digits<2>(t, w);
+      else put_digits<1>(t, w);
+    };
+    auto ready = [&]() {
+      tc::wait_st();
+      tc::fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(bar_ready);
+    };
+    if (!tc::mbar_wait(bar_first, ph)) timeout(g.status);
+    wk.settle(sg, nv, leave3);
+    int cc = wk.ci;  // class of the tile whose products run
+    bool ac = active();
+    if (cc < 5) {
+      if (ac) {
+        load(cur);
+        put(cc);
+      }
+      ready();
+    }
+    while (cc < 5) {
+      wk.row0 += tc::kRows;
+      wk.settle(sg, nv, leave3);
+      const int cn = wk.ci;
+      const bool an = active();
+      if (an) load(nxt);
+      if (!tc::mbar_wait(bar_mma, ph_mma)) timeout(g.status);
+      ph_mma ^= 1u;
+      tc::fence_after();
+      if (an) put(cn);
+      uint32_t f[kSum][4];
+      if (ac) {
+        if (cc == 0) finish_fifth(t, slab, cur);
+        if (cc == 0) take<3>(t, 0, f);
+        else if (cc < 3) take<2>(t, 0, f);
+        else take<1>(t, 0, f);
+        if (cc < 3) {
+          scatter(slab, cur, 0, f);
+          if (cc == 0) take<3>(t, 2, f);
+          else take<2>(t, 2, f);
+        }
+      }
+      if (cn < 5) ready();
+      if (ac) scatter(slab, cur, cc < 3 ? 2 : 0, f);
+      cur = nxt;
+      cc = cn;
+      ac = an;
+    }
+    ready();
+    if (g.full[st]) {
+      const longlong2 z = __ldg(reinterpret_cast<const longlong2*>(
+          g.img + (size_t)st * kStepBytes + kImgBytes));
+      const int cnt = sg.cnt[5];
+      for (int i = tid; i < cnt * nv; i += kThreads) {
+        const int kv = i / cnt, o = i - kv * cnt;
+        longlong2* c = slab + (size_t)kv * d + __ldg(g.idx + sg.start[5] + o);
+        const longlong2 x = *c;
+        *c = cmul_fx(x, z);
+      }
+    }
+    sync_data();
+  }
+  if (warp == 0) {
+    tc::fence_after();
+    tc::tmem_dealloc(s_tmem, 512);
+  }
+  // ---- phases, store.  The cross tables go where the images were (every
+  // copy has landed and been read).
+  const int tper = g.nchunk * 256;
+  double2* tab = reinterpret_cast<double2*>(slab + (size_t)g.KV * d);
+  if (g.has_x) {
+    double* w = reinterpret_cast<double*>(simg);
+    for (int i = tid; i < nv * g.norb; i += kThreads) {
+      const int kv = i / g.norb, x = i - kv * g.norb;
+      double s = 0;
+      for (uint32_t m = g.masks_other[v0 + kv]; m; m &= m - 1) {
+        const int y = __ffs(m) - 1;
+        s += g.dir == 1 ? X.v[y * g.norb + x] : X.v[x * g.norb + y];
+      }
+      w[kv * kMaxOrb + x] = s;
+    }
+    sync_data();
+    for (int i = tid; i < nv * tper; i += kThreads) {
+      const int kv = i / tper, e = i - kv * tper, c = e >> 8;
+      double s = 0;
+      for (int v = e & 255; v; v &= v - 1) {
+        const int x = 8 * c + __ffs(v) - 1;
+        if (x < g.norb) s += w[kv * kMaxOrb + x];
+      }
+      tab[i] = expi<double>(s);
+    }
+    sync_data();
+  }
+  auto finish = [&](int kv, int e) {
+    const int eb = s_eb[kv];
+    const longlong2 c = slab[(size_t)kv * d + e];
+    double2 v = make_double2(to_double(c.x, eb), to_double(c.y, eb));
+    if (eb < 0) v.x = v.y = __longlong_as_double(0x7FF8000000000000ll);
+    if (g.ea_other) v = cmul<double>(v, __ldg(g.ea_other + v0 + kv));
+    if (g.ea_this) v = cmul<double>(v, __ldg(g.ea_this + e));
+    if (g.has_x) {
+      const uint32_t m = __ldg(g.masks_this + e);
+      for (int k = 0; k < g.nchunk; ++k)
+        v = cmul<double>(v, tab[kv * tper + k * 256 + ((m >> (8 * k)) & 255)]);
+    }
+    return v;
+  };
+  if (g.dir == 1) {
+    for (int kv = 0; kv < nv; ++kv)
+      for (int e = tid; e < d; e += kThreads)
+        state[(int64_t)(v0 + kv) * g.d_b + e] = finish(kv, e);
+  } else {
+    for (int i = tid; i < d * nv; i += kThreads) {
+      const int e = i / nv, kv = i - e * nv;
+      state[(int64_t)e * g.d_b + v0 + kv] = finish(kv, e);
+    }
+  }
+}
+
+// ------------------------------------------------------------------ host
+// Bytes of the staged gather addresses, of class 3 and of the classes 2, 4, 1
+// and 5 together: the orbits of class m are the (n - m)-subsets of the N - 6
+// orbitals outside, at every window position.
+static void caps(int N, int n, int (&out)[2]) {
+  out[0] = out[1] = 0;
+  for (int i = 0; i < 5; ++i) {
+    const int m = cls(i), k = n - m;
+    int64_t c = k < 0 || k > N - tc::kW ? 0 : 1;
+    for (int j = 1; c && j <= k; ++j) c = c * (N - tc::kW - k + j) / j;
+    const int64_t b = (c * 4 * grp_pad(m) * 2 + 15) / 16 * 16;
+    out[i > 0] += (int)std::min<int64_t>(b, 1 << 24);
+  }
+  for (int& x : out) x = (x + 127) / 128 * 128;
+}
+
+// Gather addresses of the steps, per window position: the classes 3, 2, 4,
+// 1, 5 and 6, each as its four column groups of `count` orbit rows (class 6:
+// one address per orbit); the orbits of a class in window_tables_host's
+// order, whose aligned groups of eight read distinct banks.
+static void build_index(Space* sp) {
+  if (sp->fx_seg) return;
+  const int N = sp->norb, n = sp->nocc, npos = N - tc::kW + 1;
+  std::vector<uint32_t> orbits;
+  std::vector<int> off;
+  std::vector<uint16_t> offs;
+  std::vector<uint8_t> okey;
+  window_tables_host(N, n, tc::kW, orbits, off, offs, okey);
+  std::vector<uint8_t> list[7];
+  for (int x = 0; x < 64; ++x) list[__builtin_popcount(x)].push_back((uint8_t)x);
+  std::vector<Seg> seg(npos);
+  std::vector<uint16_t> idx;
+  for (int a = 0; a < npos; ++a) {
+    for (int ci = 0; ci < 5; ++ci) {
+      const int m = cls(ci), P = grp_pad(m);
+      std::vector<uint32_t> os;
+      for (int k = off[a]; k < off[a + 1]; ++k)
+        if ((int)(orbits[k] >> 24) == m) os.push_back(orbits[k]);
+      while (idx.size() % 8) idx.push_back(0);
+      seg[a].start[ci] = (int)idx.size();
+      seg[a].cnt[ci] = (int)os.size();
+      for (int g = 0; g < 4; ++g)
+        for (uint32_t o : os) {
+          const uint16_t* F = offs.data() + (((size_t)a * (n + 1) + ((o >> 16) & 0xFF)) << tc::kW);
+          for (int j = 0; j < P; ++j) {
+            const int s = grp_string(m, g, j);
+            idx.push_back(s < 0 ? (uint16_t)0xFFFF : (uint16_t)((o & 0xFFFF) + F[list[m][s]]));
+          }
+        }
+    }
+    // class 6: the strings that fill the window
+    while (idx.size() % 8) idx.push_back(0);
+    seg[a].start[5] = (int)idx.size();
+    int cnt = 0;
+    const uint32_t win = 63u << a;
+    int64_t r = 0;
+    if (n >= 6) {  // strings in ascending order, as addresses are
+      uint64_t x = (1ull << n) - 1;
+      for (; !(x >> N); ++r) {
+        if (((uint32_t)x & win) == win) {
+          idx.push_back((uint16_t)r);
+          ++cnt;
+        }
+        const uint64_t c = x & (~x + 1), y = x + c;
+        x = (((y ^ x) >> 2) / c) | y;
+      }
+    }
+    seg[a].cnt[5] = cnt;
+  }
+  while (idx.size() % 8) idx.push_back(0);
+  FS_CUDA(cudaMalloc(&sp->fx_idx, std::max<size_t>(idx.size(), 8) * sizeof(uint16_t)));
+  FS_CUDA(cudaMemcpy(sp->fx_idx, idx.data(), idx.size() * sizeof(uint16_t),
+                     cudaMemcpyHostToDevice));
+  sp->fx_seg_h = seg;
+  Seg* ds = nullptr;
+  FS_CUDA(cudaMalloc(&ds, seg.size() * sizeof(Seg)));
+  FS_CUDA(cudaMemcpy(ds, seg.data(), seg.size() * sizeof(Seg), cudaMemcpyHostToDevice));
+  sp->fx_seg = ds;
+}
+
+}  // namespace fx
+
+// Host fixed point with 62 fraction bits.
+static inline int64_t hmul(int64_t a, int64_t b) {
+  return (int64_t)(((__int128)a * b + ((__int128)1 << 61)) >> 62);
+}
+static inline int64_t hfix(double x) { return (int64_t)std::llrint(std::ldexp(x, 62)); }
+// Scales x (n reals in fixed point, 2-norm 1 up to FP64 rounding) to 2-norm 1.
+static void hunit(int64_t* x, int n) {
+  __int128 s = (__int128)1 << 124;
+  for (int i = 0; i < n; ++i) s -= (__int128)x[i] * x[i];
+  const int64_t h = (int64_t)(s >> 63);  // (1 - norm^2) / 2
+  for (int i = 0; i < n; ++i) x[i] += hmul(x[i], h);
+}
+
+// The steps of a program with their unitaries V (row-major 6 x 6 complex,
+// fixed point; products of FP64 matrices would put an error of some 2^-52
+// into each entry, the same for every amplitude), the diagonal layer
+// multiplied into the last step that covers each orbital.  False when a
+// phase falls outside every window or the program has too many steps.
+static bool fx_steps(const RotProgram& rp, int N, std::vector<WinStep>& steps,
+                     std::vector<std::array<int64_t, 72>>* V, uint8_t* full) {
+  steps = schedule_windows(rp, N, tc::kW);
+  if (steps.empty() || (int)steps.size() > fx::kMaxSteps) return false;
+  std::vector<int> last(N, -1);
+  for (size_t s = 0; s < steps.size(); ++s)
+    for (int p = steps[s].a; p < steps[s].a + tc::kW; ++p) last[p] = (int)s;
+  for (int p = 0; p < N; ++p)
+    if (last[p] < 0 && rp.phase[p] != zd(1.0)) return false;
+  if (!V) return true;
+  V->resize(steps.size());
+  for (size_t s = 0; s < steps.size(); ++s) {
+    const int a = steps[s].a;
+    auto& M = (*V)[s];
+    M.fill(0);
+    for (int i = 0; i < 6; ++i) M[14 * i] = (int64_t)1 << 62;
+    for (int k : steps[s].givens) {
+      const Givens& G = rp.g[k];
+      int64_t g[3] = {hfix(G.c), hfix(G.s.real()), hfix(G.s.imag())};
+      hunit(g, 3);
+      int64_t* x = M.data() + 12 * (G.p - a);
+      for (int j = 0; j < 6; ++j) {
+        const int64_t ur = x[2 * j], ui = x[2 * j + 1], vr = x[12 + 2 * j], vi = x[13 + 2 * j];
+        x[2 * j] = hmul(g[0], ur) + hmul(g[1], vr) - hmul(g[2], vi);
+        x[2 * j + 1] = hmul(g[0], ui) + hmul(g[1], vi) + hmul(g[2], vr);
+        x[12 + 2 * j] = hmul(g[0], vr) - hmul(g[1], ur) - hmul(g[2], ui);
+        x[13 + 2 * j] = hmul(g[0], vi) - hmul(g[1], ui) + hmul(g[2], ur);
+      }
+    }
+    full[s] = 0;
+    for (int p = a; p < a + tc::kW; ++p) {
+      if (last[p] != (int)s || rp.phase[p] == zd(1.0)) continue;
+      int64_t z[2] = {hfix(rp.phase[p].real()), hfix(rp.phase[p].imag())};
+      hunit(z, 2);
+      int64_t* x = M.data() + 12 * (p - a);
+      for (int j = 0; j < 6; ++j) {
+        const int64_t re = hmul(x[2 * j], z[0]) - hmul(x[2 * j + 1], z[1]);
+        x[2 * j + 1] = hmul(x[2 * j], z[1]) + hmul(x[2 * j + 1], z[0]);
+        x[2 * j] = re;
+      }
+      full[s] = 1;
+    }
+  }
+  return true;
+}
+
+bool fx_supported(const Ctx* ctx, const Space* sthis, const Space* sother, int dtype,
+                  const RotProgram& rp) {
+  if (dtype != FS_C128 || ctx->sweep_engine == FS_SWEEP_CUDA_CORE || ctx->prop.major < 10)
+    return false;
+  if (sthis->norb < tc::kW || sthis->dim < 2) return false;
+  int caps[2];
+  fx::caps(sthis->norb, sthis->nocc, caps);
+  const size_t tab = (size_t)((sthis->norb + 7) / 8) * 256 * 16;
+  if (fx::kImgBytes + (size_t)caps[0] + caps[1] + (size_t)sthis->dim * 16 + tab >
+      (size_t)ctx->prop.sharedMemPerBlockOptin - fx::kStaticBytes)
+    return false;
+  if (sthis->dim * sother->dim < fx::kMinAmps) return false;
+  std::vector<WinStep> steps;
+  return fx_steps(rp, sthis->norb, steps, nullptr, nullptr) &&
+         rp.g.size() >= fx::kMinGivensPerStep * steps.size();
+}
+
+void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0, void* st1,
+                     const RotProgram& rp, const PhaseDev& ph, cudaStream_t st) {
+  const Space* sthis = dir == 0 ? sa : sb;
+  const Space* sother = dir == 0 ? sb : sa;
+  std::vector<WinStep> steps;
+  std::vector<std::array<int64_t, 72>> V;
+  fx::Args g{};
+  FS_REQUIRE(fx_steps(rp, sthis->norb, steps, &V, g.full), FS_ERR_ARG,
+             "program has no window steps");
+  fx::build_index(const_cast<Space*>(sthis));
+  g.st[0] = (double2*)st0;
+  g.st[1] = (double2*)st1;
+  const int nst = st1 ? 2 : 1;
+  g.d_b = sb->dim;
+  g.dir = dir;
+  g.d = (int)sthis->dim;
+  g.nvec = (int)sother->dim;
+  g.nsteps = (int)steps.size();
+  g.norb = sthis->norb;
+  g.nchunk = (sthis->norb + 7) / 8;
+  g.has_x = ph.has_x;
+  g.seg = (const fx::Seg*)sthis->fx_seg;
+  g.idx = sthis->fx_idx;
+  g.masks_this = sthis->masks;
+  g.masks_other = sother->masks;
+  g.ea_this = (const double2*)(dir == 0 ? ph.ea_a : ph.ea_b);
+  g.ea_other = (const double2*)(dir == 0 ? ph.ea_b : ph.ea_a);
+  g.status = ctx->d_status;
+  fx::StepMats sm;
+  for (int s = 0; s < g.nsteps; ++s) {
+    g.a[s] = (uint8_t)steps[s].a;
+    std::copy(V[s].begin(), V[s].end(), sm.v[s]);
+  }
+  // vectors per slab: the width with the least modelled time, a wave of
+  // slabs costing its tiles (class 3 the most) and its amplitudes
+  const size_t tab = ph.has_x ? (size_t)g.nchunk * 256 * 16 : 0;
+  int caps[2];
+  fx::caps(sthis->norb, sthis->nocc, caps);
+  g.cap_first = caps[0];
+  g.cap_rest = caps[1];
+  const size_t fixed = fx::kImgBytes + (size_t)caps[0] + caps[1];
+  const size_t avail = (size_t)ctx->prop.sharedMemPerBlockOptin - fx::kStaticBytes - fixed;
+  const int kvmax =
+      std::max(1, std::min<int>(fx::kMaxVec, (int)(avail / ((size_t)g.d * 16 + tab))));
+  const int sms = ctx->prop.multiProcessorCount;
+  double best = 0;
+  for (int kv = 1; kv <= kvmax; ++kv) {
+    static const double w[5] = {1.0, 0.75, 0.75, 0.4, 0.4};
+    double c = 0;
+    for (int s = 0; s < g.nsteps; ++s) {
+      const fx::Seg& sg = sthis->fx_seg_h[g.a[s]];
+      for (int i = 0; i < 5; ++i) c += w[i] * ((sg.cnt[i] * kv + tc::kRows - 1) / tc::kRows);
+    }
+    c += 4.0 + 1e-3 * g.d * kv;
+    const int slabs = nst * ((g.nvec + kv - 1) / kv);
+    c *= (slabs + sms - 1) / sms;
+    if (kv == 1 || c < best) {
+      best = c;
+      g.KV = kv;
+    }
+  }
+  unsigned char* img =
+      (unsigned char*)scratch(ctx, "fx_images", (size_t)g.nsteps * fx::kStepBytes);
+  g.img = img;
+  {
+    ProfScope ps("fx_images", st);
+    fx::k_fx_images<<<dim3(g.nsteps, 2), 512, 0, st>>>(sm, img);
+    FS_CUDA(cudaGetLastError());
+  }
+  // more than half an SM's shared memory: the CTA owns all TMEM of its SM
+  const size_t smem = std::max(fixed + (size_t)g.KV * ((size_t)g.d * 16 + tab),
+                               (size_t)ctx->prop.sharedMemPerMultiprocessor / 2 + 1024);
+  FS_CUDA(cudaFuncSetAttribute(fx::k_sweep_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)smem));
+  ProfScope ps(dir == 0 ? "sweep_alpha_fx" : "sweep_beta_fx", st);
+  fx::k_sweep_fx<<<dim3((g.nvec + g.KV - 1) / g.KV, nst), fx::kCta, smem, st>>>(g, ph.X);
+  FS_CUDA(cudaGetLastError());
+}
+
+}  // namespace fs

@@ -242,6 +242,8 @@ void free_space(Space* s) {
   cudaFree(s->trec);
   cudaFree(s->gpq);
   cudaFree(s->gsrc);
+  cudaFree(s->fx_seg);
+  cudaFree(s->fx_idx);
   for (int b = 0; b < 4; ++b) {
     cudaFree(s->tgrec[b]);
     cudaFree(s->tgoff[b]);
