@@ -300,10 +300,11 @@ int fs_apply_quad_ham_evolution(fs_ctx *ctx, void *vec, int dtype, const double 
  * with REAL tensors: one_body = h (N x N doubles), two_body = h_pqrs (N^4
  * doubles, index ((p*N + q)*N + r)*N + s).  `vec` and `out` are distinct
  * device states of the same sector and dtype; `vec` is read only, `out` is
- * overwritten.  The work runs in blocks whose N^2-fold intermediates use at
- * most `workspace_bytes` of scratch (0: min(8 GiB, a quarter of free
- * memory)).  The contractions over the two-body tensor are cuBLAS GEMMs in
- * the state's precision; everything else runs in the library's kernels.
+ * overwritten.  The work runs in blocks whose intermediates (one amplitude
+ * per single excitation of a string, n (N - n) + n of them) use at most
+ * `workspace_bytes` of scratch (0: min(8 GiB, a quarter of free memory; a
+ * single row or column of the state where that is more).  All of it runs in
+ * the library's kernels, in the state's precision.
  * N <= 32.  Asynchronous on `stream`. */
 int fs_apply_molecular_hamiltonian(fs_ctx *ctx, const void *vec, void *out, int dtype,
                                    const double *one_body, const double *two_body,

@@ -198,6 +198,7 @@ struct Space {
   // per string t, ne = n(N-n)+n entries (pq = p*N+q, src = E_qp t | sign<<31)
   uint16_t* gpq = nullptr;
   uint32_t* gsrc = nullptr;
+  uint16_t* gslot = nullptr;  // place of (q, p) in the list of src
   int ne = 0;
 };
 

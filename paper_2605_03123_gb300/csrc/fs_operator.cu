@@ -8,255 +8,266 @@
 //         + sum_pq E^a_pq [sum_rs V_pqrs E^a_rs + W_pqrs E^b_rs]
 //         + sum_pq E^b_pq [sum_rs V_pqrs E^b_rs],
 //   k_pq = h_pq - 1/2 sum_r h_prrq,  V = h / 2,  W_pqrs = (h_pqrs + h_rspq) / 2.
-// Each bracket is a contraction over rs: with D_rs = E_rs psi it is the
-// GEMM G = V D (a real matrix times the complex vectors viewed as pairs of
-// reals): complex64 on the tcgen05 tensor cores (gemm_tc: D transposed and
-// split into exact BF16 triples, V split on the host; FP32 accuracy),
-// complex128 as a tiled FP64 GEMM on the CUDA cores; and the outer E_pq is a
-// gather through the single-excitation table.  The beta part runs on
-// blocks of rows (a beta excitation stays in its row), the alpha and mixed
-// parts on blocks of columns (an alpha excitation stays in its column);
-// the block size bounds the N^2 x block intermediates.
-#include <cuda_bf16.h>
-
+// A string of one spin is reached by ne = n (N - n) + n excitations and left
+// by as many, so each bracket is needed, and has nonzero terms, for ne of the
+// N^2 excitations only.  The products are taken over those lists, per string,
+// on the FP32 and FP64 units: N = 12 (6,6) needs 42 of 144 on each side, an
+// eighth of the multiply-adds of full N^2 x N^2 products and of the
+// intermediates.  (The full products, complex64 on the tensor cores and
+// complex128 in FP64, took 5.7 ms at N = 12 (6,6) in complex64 and 8.8 ms at
+// N = 10 (5,5) in complex128; now 1.38 and 0.89 ms, bound by the products:
+// FP64 rate, and in complex64 the shared-memory reads of the mixed part.)
+//   same spin: F[l][s] = sum_k V[pq_l][rs_k] sign_k psi[src_k] + k_{pq_l} psi[s]
+//              for the excitations pq_l out of string s, rs_k into it; then
+//              out[t] += sum_k sign_k F[l(k)][src_k];
+//   mixed:     Y[k][i][j] = sum_l W[pq_l][rs_k] sign_l psi[src_l(i)][j] for the
+//              alpha excitations into i and the beta excitations out of j,
+//              then the same outer sum along j.
+// The alpha same-spin part runs on blocks of columns, the beta one on
+// transposed blocks of rows (the rotated spin along rows, so that a warp reads
+// neighbouring columns), the mixed one on the same blocks of rows; the block
+// size bounds the ne-fold intermediates.
 #include <algorithm>
 
 #include "fs_common.cuh"
 #include "fs_internal.h"
-#include "fs_tc.cuh"
 
 namespace fs {
 
-// D[rs][t][c] = (E_rs X)[t][col0 + c] for all rs, the rows t of X being
-// strings of the excited spin: sign * X[E_sr t][col0 + c] or 0.  One CTA per
-// target row.
+// acc += w x, w real.
+__device__ __forceinline__ void axpy(float2& acc, float w, float2 x) {
+  acc = __ffma2_rn(make_float2(w, w), x, acc);
+}
+__device__ __forceinline__ void axpy(double2& acc, double w, double2 x) {
+  acc.x = fma(w, x.x, acc.x);
+  acc.y = fma(w, x.y, acc.y);
+}
+__device__ __forceinline__ int swap_pq(int pq, int N) {
+  const int p = pq / N;
+  return (pq - p * N) * N + p;
+}
+
+// V = h / 2 and W[pq][rs] = (h_pqrs + h_rspq) / 2 in the state's precision.
 template <typename R>
-__global__ void __launch_bounds__(256)
-    k_excite_rows(cx_t<R>* D, const cx_t<R>* X, int64_t ldx, int64_t col0, int ncol,
-                  int64_t nrows, const uint16_t* gpq, const uint32_t* gsrc, int ne, int NN,
-                  int64_t dstride) {
-  extern __shared__ int ent[];  // NN: entry index of rs in row t's table, or -1
-  for (int64_t t = blockIdx.x; t < nrows; t += gridDim.x) {
-    for (int k = threadIdx.x; k < NN; k += blockDim.x) ent[k] = -1;
-    __syncthreads();
-    for (int k = threadIdx.x; k < ne; k += blockDim.x) ent[gpq[t * ne + k]] = k;
-    __syncthreads();
-    for (int rs = 0; rs < NN; ++rs) {
-      const int k = ent[rs];
-      cx_t<R>* d = D + rs * dstride + t * ncol;
-      if (k < 0) {
-        for (int c = threadIdx.x; c < ncol; c += blockDim.x) d[c] = mk<R>(0, 0);
-      } else {
-        const uint32_t v = gsrc[t * ne + k];
-        const R sg = (v >> 31) ? R(-1) : R(1);
-        const cx_t<R>* x = X + (int64_t)(v & 0x7FFFFFFFu) * ldx + col0;
-        for (int c = threadIdx.x; c < ncol; c += blockDim.x)
-          d[c] = mk<R>(sg * x[c].x, sg * x[c].y);
-      }
-    }
-    __syncthreads();
+__global__ void k_op_weights(const double* h2, R* V, R* W, int NN) {
+  const int64_t n = (int64_t)NN * NN;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const int pq = (int)(i / NN), rs = (int)(i - (int64_t)pq * NN);
+    const double a = h2[i], b = h2[(int64_t)rs * NN + pq];
+    V[i] = (R)(0.5 * a);
+    W[i] = (R)(0.5 * (a + b));
   }
 }
 
-// D[rs][ii][c] = (E_rs X)[row0 + ii][col0 + c] with the columns of X
-// strings of the excited spin: sign * X[row0 + ii][E_sr (col0 + c)] or 0.
-// One thread per output element; its column's table is walked in rs order.
+// Same-spin products of string s = blockIdx.x over columns of X (rows are
+// strings): F[l][s][c] for the excitations l out of s.  A thread owns `CT`
+// columns (128 apart) and 16 excitations at a time; the weights of those,
+// signs folded in, are in shared memory and reach a warp by broadcast, so a
+// product costs one multiply-add per part (FP32: one two-lane instruction)
+// and a sixteenth of a load.
+constexpr int kOpL = 16;
+template <typename R, int CT>
+__global__ void __launch_bounds__(128)
+    k_op_same(cx_t<R>* F, int64_t fstride, const cx_t<R>* X, int64_t ldx, int64_t col0,
+              int64_t ncol, const uint16_t* gpq, const uint32_t* gsrc, int ne, int N,
+              const R* V, const __grid_constant__ Mat kmat) {
+  using C = cx_t<R>;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  R* wt = reinterpret_cast<R*>(smraw);                             // [ne][kOpL]
+  uint32_t* src = reinterpret_cast<uint32_t*>(wt + (size_t)ne * kOpL);  // [ne]
+  const int64_t s = blockIdx.x;
+  const int NN = N * N;
+  const uint16_t* pq = gpq + s * ne;
+  for (int k = threadIdx.x; k < ne; k += 128) src[k] = gsrc[s * ne + k];
+  for (int l0 = 0; l0 < ne; l0 += kOpL) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < ne * kOpL; e += 128) {
+      const int k = e / kOpL, l = l0 + (e - k * kOpL);
+      R w = 0;
+      if (l < ne) {
+        w = V[(int64_t)swap_pq(pq[l], N) * NN + pq[k]];
+        if (src[k] >> 31) w = -w;
+      }
+      wt[e] = w;
+    }
+    __syncthreads();
+    for (int64_t c0 = blockIdx.y * (int64_t)(128 * CT); c0 < ncol;
+         c0 += gridDim.y * (int64_t)(128 * CT)) {
+      C acc[kOpL][CT];
+#pragma unroll
+      for (int l = 0; l < kOpL; ++l)
+#pragma unroll
+        for (int u = 0; u < CT; ++u) acc[l][u] = mk<R>(0, 0);
+      int64_t c[CT];
+      bool in[CT];
+#pragma unroll
+      for (int u = 0; u < CT; ++u) {
+        c[u] = c0 + threadIdx.x + 128 * u;
+        in[u] = c[u] < ncol;
+      }
+      if (in[0]) {
+#pragma unroll 2
+        for (int k = 0; k < ne; ++k) {
+          const C* xr = X + (int64_t)(src[k] & 0x7FFFFFFFu) * ldx + col0;
+          C x[CT];
+#pragma unroll
+          for (int u = 0; u < CT; ++u) x[u] = in[u] ? xr[c[u]] : mk<R>(0, 0);
+          const R* w = wt + k * kOpL;
+#pragma unroll
+          for (int l = 0; l < kOpL; ++l)
+#pragma unroll
+            for (int u = 0; u < CT; ++u) axpy(acc[l][u], w[l], x[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < CT; ++u) {
+          if (!in[u]) continue;
+          const C x = X[s * ldx + col0 + c[u]];
+#pragma unroll
+          for (int l = 0; l < kOpL; ++l) {
+            if (l0 + l >= ne) break;
+            axpy(acc[l][u], (R)kmat.v[swap_pq(pq[l0 + l], N)], x);
+            F[(l0 + l) * fstride + s * ncol + c[u]] = acc[l][u];
+          }
+        }
+      }
+    }
+  }
+}
+
+// Mixed products of alpha string row0 + blockIdx.x: Y[k][ii][j] for the beta
+// excitations k out of j (lanes over j).  The row's weights W[pq_l][.],
+// signs folded in, are in shared memory (lcap rows at a time); a lane reads
+// its own entry of each, which its neighbours mostly share.
+template <typename R>
+__global__ void __launch_bounds__(128)
+    k_op_mixed(cx_t<R>* Y, int64_t ystride, const cx_t<R>* X, int64_t db, int64_t row0,
+               const uint16_t* apq, const uint32_t* asrc, int nea, const uint16_t* bpq, int neb,
+               int N, const R* W, int lcap) {
+  using C = cx_t<R>;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  R* wt = reinterpret_cast<R*>(smraw);  // [lcap][NN]
+  const int NN = N * N;
+  const int64_t i = row0 + blockIdx.x;
+  const uint16_t* pq = apq + i * nea;
+  const uint32_t* src = asrc + i * nea;
+  for (int64_t j0 = blockIdx.y * 128ll; j0 < db; j0 += gridDim.y * 128ll) {
+    const int64_t j = j0 + threadIdx.x;
+    for (int k0 = 0; k0 < neb; k0 += kOpL) {
+      C acc[kOpL];
+      int rs[kOpL];
+#pragma unroll
+      for (int k = 0; k < kOpL; ++k) {
+        acc[k] = mk<R>(0, 0);
+        rs[k] = j < db && k0 + k < neb ? swap_pq(bpq[j * neb + k0 + k], N) : 0;
+      }
+      for (int l0 = 0; l0 < nea; l0 += lcap) {
+        const int nl = min(lcap, nea - l0);
+        if (nea > lcap || (k0 == 0 && j0 == blockIdx.y * 128ll)) {
+          __syncthreads();
+          for (int e = threadIdx.x; e < nl * NN; e += 128) {
+            const int l = e / NN;
+            const R w = W[(int64_t)pq[l0 + l] * NN + (e - l * NN)];
+            wt[e] = (src[l0 + l] >> 31) ? -w : w;
+          }
+          __syncthreads();
+        }
+        if (j < db) {
+#pragma unroll 2
+          for (int l = 0; l < nl; ++l) {
+            const C x = X[(int64_t)(src[l0 + l] & 0x7FFFFFFFu) * db + j];
+            const R* w = wt + l * NN;
+#pragma unroll
+            for (int k = 0; k < kOpL; ++k) axpy(acc[k], w[rs[k]], x);
+          }
+        }
+      }
+      if (j < db)
+#pragma unroll
+        for (int k = 0; k < kOpL; ++k)
+          if (k0 + k < neb) Y[(k0 + k) * ystride + (int64_t)blockIdx.x * db + j] = acc[k];
+    }
+  }
+}
+
+// out[row0 + ii][t] = c psi[row0 + ii][t] + sum_k sign_k Y[slot_k][ii][src_k]
+// over the beta excitations k into t.
 template <typename R>
 __global__ void __launch_bounds__(256)
-    k_excite_cols(cx_t<R>* D, const cx_t<R>* X, int64_t ldx, int64_t row0, int64_t nrow,
-                  int64_t col0, int64_t ncol, const uint16_t* gpq, const uint32_t* gsrc, int ne,
-                  int NN, int64_t dstride) {
-  const int64_t total = nrow * ncol;
+    k_op_gather_cols(cx_t<R>* out, const cx_t<R>* X, int64_t db, int64_t row0, int64_t nrow,
+                     const cx_t<R>* Y, int64_t ystride, const uint16_t* gslot,
+                     const uint32_t* gsrc, int ne, double constant) {
+  const int64_t total = nrow * db;
+  const R cst = (R)constant;
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
        idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t ii = idx / ncol, col = col0 + (idx - ii * ncol);
-    const cx_t<R>* x = X + (row0 + ii) * ldx;
-    const uint16_t* tp = gpq + col * ne;
-    const uint32_t* ts = gsrc + col * ne;
-    int k = 0;
-    int next = ne > 0 ? tp[0] : NN;
-    for (int rs = 0; rs < NN; ++rs) {
-      cx_t<R> v = mk<R>(0, 0);
-      if (rs == next) {
-        const uint32_t s = ts[k];
-        const cx_t<R> a = x[s & 0x7FFFFFFFu];
-        v = (s >> 31) ? mk<R>(-a.x, -a.y) : a;
-        ++k;
-        next = k < ne ? tp[k] : NN;
-      }
-      D[rs * dstride + idx] = v;
+    const int64_t ii = idx / db, t = idx - ii * db;
+    const cx_t<R> x = X[(row0 + ii) * db + t];
+    cx_t<R> acc = mk<R>(cst * x.x, cst * x.y);
+    const cx_t<R>* y = Y + ii * db;
+#pragma unroll 4
+    for (int k = 0; k < ne; ++k) {
+      const uint32_t v = gsrc[t * ne + k];
+      axpy(acc, (v >> 31) ? R(-1) : R(1), y[gslot[t * ne + k] * ystride + (v & 0x7FFFFFFFu)]);
     }
+    out[(row0 + ii) * db + t] = acc;
   }
 }
 
-// out[t][col0 + c] (+)= sum over row t's table entries (pq, src, sign) of
-// sign * (G[pq][src][c] + k_pq X[src][col0 + c]): the outer E_pq along rows.
+// out[t][col0 + c] += sum_k sign_k F[slot_k][src_k][c] over the excitations k
+// into row t.
 template <typename R>
 __global__ void __launch_bounds__(256)
-    k_gather_rows(cx_t<R>* out, int64_t ldo, int64_t col0, int ncol, int64_t nrows,
-                  const cx_t<R>* G, int64_t gstride, const cx_t<R>* X, int64_t ldx,
-                  const uint16_t* gpq, const uint32_t* gsrc, int ne,
-                  const __grid_constant__ Mat kmat) {
-  for (int64_t t = blockIdx.x; t < nrows; t += gridDim.x) {
-    for (int c = threadIdx.x; c < ncol; c += blockDim.x) {
+    k_op_gather_rows(cx_t<R>* out, int64_t ldo, int64_t col0, int64_t ncol, int64_t nrows,
+                     const cx_t<R>* F, int64_t fstride, const uint16_t* gslot,
+                     const uint32_t* gsrc, int ne) {
+  for (int64_t t = blockIdx.x; t < nrows; t += gridDim.x)
+    for (int64_t c = blockIdx.y * 256ll + threadIdx.x; c < ncol; c += gridDim.y * 256ll) {
       cx_t<R> acc = out[t * ldo + col0 + c];
+#pragma unroll 4
       for (int k = 0; k < ne; ++k) {
         const uint32_t v = gsrc[t * ne + k];
-        const int pq = gpq[t * ne + k];
-        const int64_t src = v & 0x7FFFFFFFu;
-        const R sg = (v >> 31) ? R(-1) : R(1), kk = (R)kmat.v[pq];
-        const cx_t<R> g = G[pq * gstride + src * ncol + c];
-        const cx_t<R> x = X[src * ldx + col0 + c];
-        acc.x += sg * (g.x + kk * x.x);
-        acc.y += sg * (g.y + kk * x.y);
+        axpy(acc, (v >> 31) ? R(-1) : R(1),
+             F[gslot[t * ne + k] * fstride + (int64_t)(v & 0x7FFFFFFFu) * ncol + c]);
       }
       out[t * ldo + col0 + c] = acc;
     }
-  }
 }
 
-// out[row0 + ii][j] = c X[row0 + ii][j] + sum over column j's entries of
-// sign * (G[pq][ii][src] + k_pq X[row0 + ii][src]): the outer E_pq along
-// columns, which also initialises the output.
+// The same sums for a transposed block (row t, columns ii), added to
+// out[row0 + ii][t] through a 32 x 32 tile.
 template <typename R>
 __global__ void __launch_bounds__(256)
-    k_gather_cols(cx_t<R>* out, int64_t ldo, int64_t row0, int64_t nrow, int64_t ncol,
-                  const cx_t<R>* G, int64_t gstride, const cx_t<R>* X, int64_t ldx,
-                  const uint16_t* gpq, const uint32_t* gsrc, int ne,
-                  const __grid_constant__ Mat kmat, double constant) {
-  const int64_t total = nrow * ncol;
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t ii = idx / ncol, j = idx - ii * ncol;
-    const cx_t<R>* x = X + (row0 + ii) * ldx;
-    const R cst = (R)constant;
-    cx_t<R> acc = mk<R>(cst * x[j].x, cst * x[j].y);
-    for (int k = 0; k < ne; ++k) {
-      const uint32_t v = gsrc[j * ne + k];
-      const int pq = gpq[j * ne + k];
-      const int64_t src = v & 0x7FFFFFFFu;
-      const R sg = (v >> 31) ? R(-1) : R(1), kk = (R)kmat.v[pq];
-      const cx_t<R> g = G[pq * gstride + ii * ncol + src];
-      acc.x += sg * (g.x + kk * x[src].x);
-      acc.y += sg * (g.y + kk * x[src].y);
-    }
-    out[(row0 + ii) * ldo + j] = acc;
-  }
-}
-
-// The left operand of the tensor-core contraction: A_q[(2 p + c) * lda + k]
-// = piece q of component c (0 = Re, 1 = Im) of D[k][p], for k < K rows of D
-// (K x X complex, row stride X) and positions p < X; columns K .. lda - 1
-// are zeroed.  32 x 32 tiles through shared memory, so both the reads of D
-// and the writes of the planes run along contiguous memory.
-__global__ void __launch_bounds__(256)
-    k_transpose_split(const float2* D, int K, int64_t X, __nv_bfloat16* A0, __nv_bfloat16* A1,
-                      __nv_bfloat16* A2, int64_t lda) {
-  __shared__ float2 tile[32][33];
-  const int64_t p0 = (int64_t)blockIdx.x * 32;
-  const int k0 = blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 8 rows of 32
-  for (int r = ty; r < 32; r += 8) {
-    const int k = k0 + r;
-    const int64_t p = p0 + tx;
-    tile[r][tx] = (k < K && p < X) ? D[(int64_t)k * X + p] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  __nv_bfloat16* planes[3] = {A0, A1, A2};
-  for (int r = ty; r < 32; r += 8) {  // r: position within the tile; tx: k
-    const int64_t p = p0 + r;
-    const int k = k0 + tx;
-    if (p >= X || k >= (int)lda) continue;
-    const float2 v = tile[tx][r];
-    uint32_t w[3];
-    tc::split_bf16x3(v.x, v.y, w[0], w[1], w[2]);  // low half Re, high half Im
-    for (int q = 0; q < 3; ++q) {
-      planes[q][(2 * p) * lda + k] = __ushort_as_bfloat16((unsigned short)(w[q] & 0xFFFFu));
-      planes[q][(2 * p + 1) * lda + k] = __ushort_as_bfloat16((unsigned short)(w[q] >> 16));
-    }
-  }
-}
-
-// G[m][n] = sum_k V[m][k] D[k][n], real FP64 (row-major, leading dimensions
-// ldv, ldd, ldg): 64 x 64 tiles, 256 threads, 4 x 4 outputs per thread.
-constexpr int kRT = 64, kRK = 16;
-__global__ void __launch_bounds__(256)
-    k_rgemm_f64(const double* V, int64_t ldv, const double* D, int64_t ldd, double* G,
-                int64_t ldg, int M, int64_t N, int K) {
-  __shared__ double sa[kRK][kRT + 1];
-  __shared__ double sb[kRK][kRT + 1];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m0 = blockIdx.y * kRT;
-  const int64_t n0 = (int64_t)blockIdx.x * kRT;
-  double acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += kRK) {
-    for (int e = threadIdx.x; e < kRK * kRT; e += 256) {
-      const int kk = e / kRT, mm = e - kk * kRT;
-      const int gk = k0 + kk;
-      sa[kk][mm] = (m0 + mm < M && gk < K) ? V[(int64_t)(m0 + mm) * ldv + gk] : 0.0;
-      sb[kk][mm] = (n0 + mm < N && gk < K) ? D[(int64_t)gk * ldd + n0 + mm] : 0.0;
+    k_op_gather_t(cx_t<R>* out, int64_t ldo, int64_t row0, int64_t nrow, int64_t nt,
+                  const cx_t<R>* F, int64_t fstride, const uint16_t* gslot, const uint32_t* gsrc,
+                  int ne) {
+  __shared__ cx_t<R> tile[32][33];
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t t0 = blockIdx.x * 32ll;
+  for (int64_t i0 = blockIdx.y * 32ll; i0 < nrow; i0 += gridDim.y * 32ll) {
+    for (int r = ty; r < 32; r += 8) {
+      const int64_t t = t0 + r, ii = i0 + tx;
+      cx_t<R> acc = mk<R>(0, 0);
+      if (t < nt && ii < nrow) {
+#pragma unroll 4
+        for (int k = 0; k < ne; ++k) {
+          const uint32_t v = gsrc[t * ne + k];
+          axpy(acc, (v >> 31) ? R(-1) : R(1),
+               F[gslot[t * ne + k] * fstride + (int64_t)(v & 0x7FFFFFFFu) * nrow + ii]);
+        }
+      }
+      tile[r][tx] = acc;
     }
     __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < kRK; ++kk) {
-      double a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = sa[kk][ty * 4 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = sb[kk][tx * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    for (int r = ty; r < 32; r += 8) {
+      const int64_t ii = i0 + r, t = t0 + tx;
+      if (t < nt && ii < nrow) {
+        cx_t<R>* o = out + (row0 + ii) * ldo + t;
+        const cx_t<R> v = tile[tx][r];
+        *o = mk<R>(o->x + v.x, o->y + v.y);
+      }
     }
     __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int m = m0 + ty * 4 + i;
-      const int64_t n = n0 + tx * 4 + j;
-      if (m < M && n < N) G[(int64_t)m * ldg + n] = acc[i][j];
-    }
-}
-
-// G (row-major [n][2X] reals) = V (row-major [n][k] reals, leading dimension
-// ldv; for complex64 its three BF16 planes Vp with the same layout) x
-// D (k rows of X complex).  Ap: scratch for the transposed planes of D.
-template <typename R>
-static void contract(Ctx* ctx, int64_t X, int n, int k, const void* D, const R* Vd,
-                     const uint16_t* Vp, int ldv, int ldvp, void* G, uint16_t* Ap,
-                     cudaStream_t st) {
-  FS_REQUIRE(2 * X <= 0x7FFFFFFF, FS_ERR_UNSUPPORTED, "operator block too large for one GEMM");
-  if constexpr (sizeof(R) == 4) {
-    const int64_t lda = (k + 7) / 8 * 8;
-    const size_t plane = (size_t)2 * X * lda;
-    dim3 grid((unsigned)((X + 31) / 32), (unsigned)((lda + 31) / 32));
-    k_transpose_split<<<grid, 256, 0, st>>>((const float2*)D, k, X, (__nv_bfloat16*)Ap,
-                                            (__nv_bfloat16*)(Ap + plane),
-                                            (__nv_bfloat16*)(Ap + 2 * plane), lda);
-    FS_CUDA(cudaGetLastError());
-    GemmTc g{};
-    for (int q = 0; q < 3; ++q) {
-      g.A[q] = Ap + q * plane;
-      g.B[q] = Vp + (size_t)q * n * ldvp;
-    }
-    g.M = (int)(2 * X);
-    g.N = n;
-    g.K = k;
-    g.lda = lda;
-    g.ldb = ldvp;
-    g.out = G;
-    g.mode = GEMM_REAL_T;
-    g.ldo = 2 * X;
-    g.status = ctx->d_status;
-    gemm_tc(g, st);
-  } else {
-    dim3 grid((unsigned)((2 * X + kRT - 1) / kRT), (unsigned)((n + kRT - 1) / kRT));
-    k_rgemm_f64<<<grid, 256, 0, st>>>(Vd, ldv, (const double*)D, 2 * X, (double*)G, 2 * X, n,
-                                      2 * X, k);
-    FS_CUDA(cudaGetLastError());
   }
 }
 
@@ -265,52 +276,29 @@ static void molecular_hamiltonian_t(Ctx* ctx, Space* sa, Space* sb, const void* 
                                     const double* h1, const double* h2, double constant,
                                     int64_t ws, cudaStream_t st) {
   using C = cx_t<R>;
+  constexpr int CT = sizeof(R) == 4 ? 2 : 1;
+  constexpr int dt = sizeof(R) == 4 ? FS_C64 : FS_C128;
   const int N = sa->norb, NN = N * N;
   const C* vec = (const C*)vec_;
   C* out = (C*)out_;
   const int64_t da = sa->dim, db = sb->dim;
   build_gather_table(sa, st);
   build_gather_table(sb, st);
-  // host: k, and V = [h/2 | W] as the row-major NN x 2NN real matrix
+  const int nea = sa->ne, neb = sb->ne;
   Mat kmat{};
-  std::vector<R> V((size_t)NN * 2 * NN);
   for (int p = 0; p < N; ++p)
     for (int q = 0; q < N; ++q) {
       double s = h1[p * N + q];
       for (int r = 0; r < N; ++r) s -= 0.5 * h2[((size_t)(p * N + r) * N + r) * N + q];
       kmat.v[p * N + q] = s;
     }
-  for (int pq = 0; pq < NN; ++pq)
-    for (int rs = 0; rs < NN; ++rs) {
-      const double a = h2[(size_t)pq * NN + rs], b = h2[(size_t)rs * NN + pq];
-      V[(size_t)pq * 2 * NN + rs] = (R)(0.5 * a);
-      V[(size_t)pq * 2 * NN + NN + rs] = (R)(0.5 * (a + b));
-    }
-  R* Vd = (R*)scratch(ctx, "op_V", V.size() * sizeof(R));
-  FS_CUDA(cudaMemcpyAsync(Vd, V.data(), V.size() * sizeof(R), cudaMemcpyHostToDevice, st));
-  uint16_t* Vp = nullptr;
-  std::vector<uint16_t> Vh;
-  const int ldvp = (2 * NN + 7) / 8 * 8;
-  if (sizeof(R) == 4) {
-    // three BF16 planes of V from FP64 (each the nearest BF16 of the
-    // remainder), rows padded to a multiple of 8 entries (16 bytes)
-    const size_t nv = (size_t)NN * ldvp;
-    Vh.assign(3 * nv, 0);
-    for (int pq = 0; pq < NN; ++pq)
-      for (int rs = 0; rs < 2 * NN; ++rs) {
-        const double a = h2[(size_t)pq * NN + rs % NN], b = h2[(size_t)(rs % NN) * NN + pq];
-        double r = rs < NN ? 0.5 * a : 0.5 * (a + b);
-        for (int q = 0; q < 3; ++q) {
-          const __nv_bfloat16 v = __float2bfloat16_rn((float)r);
-          Vh[q * nv + (size_t)pq * ldvp + rs] = __bfloat16_as_ushort(v);
-          r -= (double)__bfloat162float(v);
-        }
-      }
-    Vp = (uint16_t*)scratch(ctx, "op_Vp", Vh.size() * sizeof(uint16_t));
-    FS_CUDA(cudaMemcpyAsync(Vp, Vh.data(), Vh.size() * sizeof(uint16_t), cudaMemcpyHostToDevice,
-                            st));
-  }
-  // block sizes from the workspace budget (D and G together)
+  const size_t nw = (size_t)NN * NN;
+  double* hd = (double*)scratch(ctx, "op_h2", nw * sizeof(double));
+  R* V = (R*)scratch(ctx, "op_V", 2 * nw * sizeof(R));
+  R* W = V + nw;
+  FS_CUDA(cudaMemcpyAsync(hd, h2, nw * sizeof(double), cudaMemcpyHostToDevice, st));
+  // block sizes from the workspace budget: rows take the mixed and the beta
+  // products and the transposed block, columns the alpha products
   const size_t csz = sizeof(C);
   size_t budget = (size_t)ws;
   if (ws <= 0) {
@@ -318,63 +306,71 @@ static void molecular_hamiltonian_t(Ctx* ctx, Space* sa, Space* sb, const void* 
     FS_CUDA(cudaMemGetInfo(&fr, &tot));
     budget = std::min<size_t>((size_t)8 << 30, fr / 4);
   }
-  // per position: D (2 N^2 complex), G (N^2 complex) and, for complex64, the
-  // transposed BF16 planes of D (3 x 2 x 2 N^2 x 2 bytes)
-  const size_t per = (size_t)3 * NN * csz + (sizeof(R) == 4 ? (size_t)24 * NN : 0);
-  const int64_t nr = std::max<int64_t>(1, std::min<int64_t>(da, budget / (per * db)));
-  const int64_t nc = std::max<int64_t>(1, std::min<int64_t>(db, budget / (per * da)));
-  const int64_t xmax = std::max(nr * db, nc * da);
-  C* D = (C*)scratch(ctx, "op_D", (size_t)2 * NN * xmax * csz);
-  C* G = (C*)scratch(ctx, "op_G", (size_t)NN * xmax * csz);
-  uint16_t* Ap = sizeof(R) == 4
-                     ? (uint16_t*)scratch(ctx, "op_Dp", (size_t)3 * 2 * xmax * (2 * NN + 8) * 2)
-                     : nullptr;
+  const size_t per_row = (size_t)(2 * neb + 1) * csz * db;
+  const size_t per_col = (size_t)std::max(nea, 1) * csz * da;
+  const int64_t nr = std::max<int64_t>(1, std::min<int64_t>(da, budget / per_row));
+  const int64_t nc = std::max<int64_t>(1, std::min<int64_t>(db, budget / per_col));
+  C* buf = (C*)scratch(ctx, "op_F", std::max(nr * per_row, nc * per_col));
   const int sms = ctx->prop.multiProcessorCount;
-  // beta part on row blocks; also writes c psi and the beta one-body term
+  const size_t smax = (size_t)ctx->prop.sharedMemPerBlockOptin;
+  auto same_smem = [&](int ne) { return (size_t)ne * (kOpL * sizeof(R) + 4); };
+  const int lcap = (int)std::max<size_t>(1, std::min<size_t>(std::max(nea, 1),
+                                                             (size_t)64 * 1024 / (NN * sizeof(R))));
+  const size_t mixed_smem = (size_t)lcap * NN * sizeof(R);
+  FS_REQUIRE(same_smem(std::max(nea, neb)) <= smax && mixed_smem <= smax, FS_ERR_UNSUPPORTED,
+             "operator action: weights exceed shared memory");
+  FS_CUDA(cudaFuncSetAttribute(k_op_same<R, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)std::max<size_t>(same_smem(std::max(nea, neb)), 16)));
+  FS_CUDA(cudaFuncSetAttribute(k_op_mixed<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)mixed_smem));
+  {
+    ProfScope ps("op_weights", st);
+    k_op_weights<R><<<(unsigned)std::min<size_t>((nw + 255) / 256, 8 * sms), 256, 0, st>>>(
+        hd, V, W, NN);
+    FS_CUDA(cudaGetLastError());
+  }
+  auto ytiles = [](int64_t n, int64_t w) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + w - 1) / w, 65535));
+  };
+  // mixed and beta parts on row blocks; also writes c psi
   for (int64_t i0 = 0; i0 < da; i0 += nr) {
     const int64_t nrow = std::min(nr, da - i0), X = nrow * db;
-    {
-      ProfScope ps("op_excite", st);
-      const unsigned grid = (unsigned)std::min<int64_t>((X + 255) / 256, 32 * sms);
-      k_excite_cols<R><<<grid, 256, 0, st>>>(D, vec, db, i0, nrow, 0, db, sb->gpq, sb->gsrc,
-                                             sb->ne, NN, X);
+    C* Y = buf;
+    C* G = buf + (size_t)neb * X;
+    C* xt = G + (size_t)neb * X;
+    if (neb > 0) {
+      launch_transpose(vec + i0 * db, xt, nrow, db, dt, st);
+      ProfScope ps("op_products", st, 2);
+      k_op_mixed<R><<<dim3((unsigned)nrow, ytiles(db, 128)), 128, mixed_smem, st>>>(
+          Y, X, vec, db, i0, sa->gpq, sa->gsrc, nea, sb->gpq, neb, N, W, lcap);
+      FS_CUDA(cudaGetLastError());
+      k_op_same<R, CT><<<dim3((unsigned)db, ytiles(nrow, 128 * CT)), 128, same_smem(neb), st>>>(
+          G, X, xt, nrow, 0, nrow, sb->gpq, sb->gsrc, neb, N, V, kmat);
       FS_CUDA(cudaGetLastError());
     }
-    {
-      ProfScope ps("op_gemm", st, sizeof(R) == 4 ? 2 : 1);
-      contract<R>(ctx, X, NN, NN, D, Vd, Vp, 2 * NN, ldvp, G, Ap, st);
-    }
-    {
-      ProfScope ps("op_gather", st);
-      const unsigned grid = (unsigned)std::min<int64_t>((X + 255) / 256, 32 * sms);
-      k_gather_cols<R><<<grid, 256, 0, st>>>(out, db, i0, nrow, db, G, X, vec, db, sb->gpq,
-                                             sb->gsrc, sb->ne, kmat, constant);
+    ProfScope ps("op_gather", st, neb > 0 ? 2 : 1);
+    k_op_gather_cols<R><<<(unsigned)std::min<int64_t>((X + 255) / 256, 32 * sms), 256, 0, st>>>(
+        out, vec, db, i0, nrow, Y, X, sb->gslot, sb->gsrc, neb, constant);
+    FS_CUDA(cudaGetLastError());
+    if (neb > 0) {
+      k_op_gather_t<R><<<dim3((unsigned)((db + 31) / 32), ytiles(nrow, 32)), 256, 0, st>>>(
+          out, db, i0, nrow, db, G, X, sb->gslot, sb->gsrc, neb);
       FS_CUDA(cudaGetLastError());
     }
   }
-  // alpha and mixed parts on column blocks, added to the output
-  for (int64_t j0 = 0; j0 < db; j0 += nc) {
+  // alpha part on column blocks, added to the output
+  for (int64_t j0 = 0; nea > 0 && j0 < db; j0 += nc) {
     const int64_t ncol = std::min(nc, db - j0), X = da * ncol;
     {
-      ProfScope ps("op_excite", st, 2);
-      const unsigned g1 = (unsigned)std::min<int64_t>(da, 32 * sms);
-      k_excite_rows<R><<<g1, 256, NN * sizeof(int), st>>>(D, vec, db, j0, (int)ncol, da, sa->gpq,
-                                                          sa->gsrc, sa->ne, NN, X);
+      ProfScope ps("op_products", st);
+      k_op_same<R, CT><<<dim3((unsigned)da, ytiles(ncol, 128 * CT)), 128, same_smem(nea), st>>>(
+          buf, X, vec, db, j0, ncol, sa->gpq, sa->gsrc, nea, N, V, kmat);
       FS_CUDA(cudaGetLastError());
-      const unsigned g2 = (unsigned)std::min<int64_t>((X + 255) / 256, 32 * sms);
-      k_excite_cols<R><<<g2, 256, 0, st>>>(D + (int64_t)NN * X, vec, db, 0, da, j0, ncol, sb->gpq,
-                                           sb->gsrc, sb->ne, NN, X);
-      FS_CUDA(cudaGetLastError());
-    }
-    {
-      ProfScope ps("op_gemm", st, sizeof(R) == 4 ? 2 : 1);
-      contract<R>(ctx, X, NN, 2 * NN, D, Vd, Vp, 2 * NN, ldvp, G, Ap, st);
     }
     {
       ProfScope ps("op_gather", st);
-      const unsigned grid = (unsigned)std::min<int64_t>(da, 32 * sms);
-      k_gather_rows<R><<<grid, 256, 0, st>>>(out, db, j0, (int)ncol, da, G, X, vec, db, sa->gpq,
-                                             sa->gsrc, sa->ne, kmat);
+      k_op_gather_rows<R><<<dim3((unsigned)std::min<int64_t>(da, 32 * sms), ytiles(ncol, 256)), 256,
+                            0, st>>>(out, db, j0, ncol, da, buf, X, sa->gslot, sa->gsrc, nea);
       FS_CUDA(cudaGetLastError());
     }
   }

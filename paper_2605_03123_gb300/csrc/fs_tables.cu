@@ -170,6 +170,23 @@ __global__ void k_gather_table(uint16_t* pq_out, uint32_t* src_out, const uint32
   }
 }
 
+// slot[t * ne + k]: the place, in the list of src = E_qp t, of the excitation
+// (q, p) (lists ascend in p * N + q): the index under which src keeps what it
+// sends along E_pq.
+__global__ void k_gather_slots(uint16_t* slot, const uint16_t* pq, const uint32_t* src, int64_t n,
+                               int norb, int ne) {
+  const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  const int p = pq[e] / norb, qp = (pq[e] - p * norb) * norb + p;
+  const uint16_t* list = pq + (int64_t)(src[e] & 0x7FFFFFFFu) * ne;
+  int lo = 0, hi = ne - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (list[mid] < qp) lo = mid + 1; else hi = mid;
+  }
+  slot[e] = (uint16_t)lo;
+}
+
 static int64_t choose(int n, int k) { return (int64_t)binom_host(n, k); }
 
 void build_gather_table(Space* sp, cudaStream_t st) {
@@ -179,10 +196,15 @@ void build_gather_table(Space* sp, cudaStream_t st) {
   const size_t cnt = (size_t)sp->dim * std::max(sp->ne, 1);
   FS_CUDA(cudaMalloc(&sp->gpq, cnt * sizeof(uint16_t)));
   FS_CUDA(cudaMalloc(&sp->gsrc, cnt * sizeof(uint32_t)));
+  FS_CUDA(cudaMalloc(&sp->gslot, cnt * sizeof(uint16_t)));
   if (sp->ne > 0) {
     k_gather_table<<<(unsigned)((sp->dim + 127) / 128), 128, 0, st>>>(sp->gpq, sp->gsrc,
                                                                     sp->masks, sp->dim, N,
                                                                     sp->ne);
+    FS_CUDA(cudaGetLastError());
+    const int64_t n = sp->dim * sp->ne;
+    k_gather_slots<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(sp->gslot, sp->gpq, sp->gsrc, n, N,
+                                                              sp->ne);
     FS_CUDA(cudaGetLastError());
   }
 }
@@ -242,6 +264,7 @@ void free_space(Space* s) {
   cudaFree(s->trec);
   cudaFree(s->gpq);
   cudaFree(s->gsrc);
+  cudaFree(s->gslot);
   cudaFree(s->fx_seg);
   cudaFree(s->fx_idx);
   for (int b = 0; b < 4; ++b) {
