@@ -21,6 +21,7 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include "fs_internal.h"
 #include "fs_tc.cuh"
 
 namespace fs {
@@ -108,8 +109,20 @@ __device__ __forceinline__ long long from_double(double x, int eb) {
   if (f != 0) m |= 0x0010000000000000ull;
   m <<= 10;                        // |x| 2^(62 - e), e = max(f, 1) - 1023
   const int r = eb - (f ? f : 1);     // >= 1
-  unsigned long long q = r < 63 ? (m + (1ull << (r - 1))) >> r : 0ull;
+  unsigned long long q = r >= 1 && r < 63 ? (m + (1ull << (r - 1))) >> r : 0ull;
   return x < 0 ? -(long long)q : (long long)q;
+}
+// About |x| 2^(1023 - f) in FP32 (0 when far below): x relative to the
+// exponent field f of the largest of its fellows.
+__device__ __forceinline__ float rel_abs(double x, int f) {
+  const int q = exp_field(x) - f + 127;
+  return q > 1 ? __int_as_float((q << 23) | ((__double2hiint(x) & 0xFFFFF) << 3)) : 0.f;
+}
+// Biased exponent eb = E + 1023 with 2-norm < 2^E, from the largest exponent
+// field f and the sum s of the squares of rel_abs.
+__device__ __forceinline__ int norm_exponent(int f, float s) {
+  const float r = fmaxf(sqrtf(s) * 1.001f, 1.0f);
+  return f + ((__float_as_int(r) >> 23) & 0xFF) - 126;  // r < 2^(eb - f)
 }
 // X 2^(E - 62), eb = E + 1023, rounded to 53 bits.  Built from integers (the
 // 64-bit conversion instruction runs on the FP64 units).
@@ -124,6 +137,79 @@ __device__ __forceinline__ double to_double(long long X, int eb) {
     return __longlong_as_double((long long)(v | ((unsigned long long)X & (1ull << 63))));
   }
   return scalbn(__ll2double_rn(X), eb - 1023 - kFrac);  // zeros, out of range
+}
+
+// ------------------------------------------------- phases in fixed point
+// Products of phases on the integer units: two of them cost less than the
+// four FP64 multiply-adds of one on GB300 (two issue slots a clock and SM).
+// a b up to 2^-60, both with 62 fraction bits and |a b| <= 1.
+__device__ __forceinline__ long long mul60(long long a, long long b) {
+  return (long long)((unsigned long long)__mul64hi(a, b) << 2);
+}
+__device__ __forceinline__ longlong2 phase_mul(longlong2 x, longlong2 y) {
+  return make_longlong2(mul60(x.x, y.x) - mul60(x.y, y.y), mul60(x.x, y.y) + mul60(x.y, y.x));
+}
+// (x.x + i x.y) times a phase, rounded at the last bit.
+__device__ __forceinline__ longlong2 cmul_fx(longlong2 x, longlong2 y) {
+  return make_longlong2(mul(x.x, y.x) - mul(x.y, y.y), mul(x.x, y.y) + mul(x.y, y.x));
+}
+__device__ __forceinline__ bool not_finite(double2 z) {
+  return exp_field(z.x) == 0x7FF || exp_field(z.y) == 0x7FF;
+}
+__device__ __forceinline__ double2 nan2() {
+  return make_double2(__longlong_as_double(0x7FF8000000000000ll),
+                      __longlong_as_double(0x7FF8000000000000ll));
+}
+__device__ __forceinline__ longlong2 phase_from(double2 z) {  // |z| <= 1 + rounding
+  return make_longlong2(from_double(z.x, 1024) << 1, from_double(z.y, 1024) << 1);
+}
+__device__ __forceinline__ double2 phase_to(longlong2 z) {
+  return make_double2(to_double(z.x, 1023), to_double(z.y, 1023));
+}
+// Cross-phase tables of the vectors v0 .. v0 + nv - 1 of the other spin (the
+// complex128 form of build_cross_tables): tab[kv][c][v] = exp(i sum over the
+// bits b of v of w(8 c + b)), w(x) = sum_{y in I} X[y][x] (this = beta) or
+// X[x][y].  One sincos per vector and orbital, then products: pairs of half
+// bytes, which are products of single orbitals.  work: nv (32 + 32 nchunk)
+// entries; bad: per vector, the orbitals whose angle is not finite (a string
+// that holds one has no phase).  Ends with a barrier (`sync`).
+template <typename Sync>
+__device__ void cross_tables(const uint32_t* masks_other, int dir, int norb, int nchunk,
+                             const Mat& X, int v0, int nv, longlong2* tab, longlong2* work,
+                             uint32_t* bad, int tid, int nthr, Sync&& sync) {
+  longlong2* one = work;                  // [nv][32] exp(i w(x))
+  longlong2* half = work + nv * 32;       // [nv][nchunk][2][16]
+  for (int i = tid; i < nv; i += nthr) bad[i] = 0;
+  sync();
+  for (int i = tid; i < nv * 32; i += nthr) {
+    const int kv = i >> 5, x = i & 31;
+    double s = 0, c = 1, sn = 0;
+    if (x < norb) {
+      for (uint32_t m = masks_other[v0 + kv]; m; m &= m - 1) {
+        const int y = __ffs(m) - 1;
+        s += dir == 1 ? X.v[y * norb + x] : X.v[x * norb + y];
+      }
+      if (exp_field(s) == 0x7FF) atomicOr(bad + kv, 1u << x);
+      sincos(s - 6.283185307179586 * rint(s * 0.15915494309189535), &sn, &c);
+    }
+    one[i] = phase_from(make_double2(c, sn));
+  }
+  sync();
+  for (int i = tid; i < nv * nchunk * 32; i += nthr) {
+    const int kv = i / (nchunk * 32), r = i - kv * nchunk * 32;  // r = (c, h, v)
+    const longlong2* e = one + kv * 32 + (r >> 4) * 4;
+    longlong2 z = make_longlong2(1ll << 62, 0);
+    for (int b = 0; b < 4; ++b)
+      if ((r >> b) & 1) z = phase_mul(z, e[b]);
+    half[i] = z;
+  }
+  sync();
+  for (int i = tid; i < nv * nchunk * 256; i += nthr) {
+    const int v = i & 255;
+    const longlong2* h = half + (i >> 8) * 32;
+    tab[i] = phase_mul(h[16 + (v >> 4)], h[v & 15]);
+  }
+  sync();
 }
 
 }  // namespace fx

@@ -519,6 +519,15 @@ bool fx_supported(const Ctx* ctx, const Space* sthis, const Space* sother, int d
 void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0, void* st1,
                      const RotProgram& rp, const PhaseDev& ph, cudaStream_t st);
 
+// The reductions behind a reverse fixed-point sweep (fs_trans_fx.cu): T += the
+// transition sums of this spin (its pass tables are built), if supported.
+bool trans_fx_supported(const Ctx* ctx, const Space* sthis);
+void launch_trans_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, const void* psi,
+                     const void* g, double* T, cudaStream_t st);
+// Then W and the second phase of both states, as launch_sweep's reverse mode.
+void launch_rev_phase(const Space* sa, const Space* sb, void* psi, void* cot, int dtype,
+                      const RevArgs& rev, const PhaseDev& ph, cudaStream_t st);
+
 // dJ from W = Im(conj(g) psi) of one diagonal-Coulomb gate (t = 1):
 //   dJ_ab[p][q] += sum_{ij} W_ij occ_a(i)_p occ_b(j)_q
 //   dJ_aa[p][q] += 1/2 sum_{ij} W_ij (occ_a(i)_p occ_a(i)_q + occ_b(j)_p occ_b(j)_q)

@@ -9,6 +9,7 @@
 // the slab is written back once, multiplied by the configuration phases
 // (the diagonal layer of the decomposition, and optionally a fused
 // diagonal-Coulomb / number-operator evolution, §3.2.1-§3.2.2).
+#include "fs_fx.cuh"
 #include "fs_sweep_kern.cuh"
 
 namespace fs {
@@ -491,9 +492,17 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
       launch_sweep_fx(ctx, sa, sb, dir, st0, nullptr, rp, ph, st);
       return;
     }
-    // reverse: both states rotated, then the reductions and the second phase
-    // as a sweep without rotations
+    // reverse: both states rotated, the transition sums, then W and the second
+    // phase (as a sweep without rotations where the sums do not fit one CTA)
     launch_sweep_fx(ctx, sa, sb, dir, st0, st1, rp, PhaseDev{}, st);
+    Space* sthis = const_cast<Space*>(dir == 0 ? sa : sb);
+    if (sthis->norb >= 4 && sthis->nocc >= 1) build_tpass_tables(sthis);
+    if (rev->T && trans_fx_supported(ctx, sthis)) {
+      launch_trans_fx(ctx, sa, sb, dir, st0, st1, rev->T, st);
+      if (rev->W || rev->ea2_a || rev->ea2_b || ph.has_x)
+        launch_rev_phase(sa, sb, st0, st1, dtype, *rev, ph, st);
+      return;
+    }
     RotProgram none;
     none.phase.assign(sa->norb, zd(1.0));
     launch_sweep(ctx, sa, sb, dir, st0, st1, nst, dtype, none, ph, st, rev, false);
@@ -830,16 +839,15 @@ void launch_sweep_batch(Ctx* ctx, int dtype, int nst, const SweepJob* jobs, int 
 }
 
 // ------------------------------------------------------------------ phase
-// One streaming pass: psi[i][j] *= ea_a[i] ea_b[j] exp(i sum X[p][q]) with
-// the cross tables built per row from the alpha string.
-template <typename R>
+// One streaming pass (complex64 outside the reach of k_phase_tc): psi[i][j] *=
+// ea_a[i] ea_b[j] exp(i sum X[p][q]) with the cross tables built per row from
+// the alpha string.
 __global__ void __launch_bounds__(256)
-    k_phase(cx_t<R>* vec, int64_t da, int64_t db, const uint32_t* ma,
+    k_phase(float2* vec, int64_t da, int64_t db, const uint32_t* ma,
             const uint32_t* mb, int norb, int nchunk, const void* ea_a,
             const void* ea_b, int has_x, const __grid_constant__ Mat X) {
-  using C = cx_t<R>;
   __shared__ double w[kMaxOrb];
-  __shared__ C tab[4 * 256];
+  __shared__ float2 tab[4 * 256];
   SweepGeom g{};
   g.dir = 1;
   g.norb = norb;
@@ -847,19 +855,78 @@ __global__ void __launch_bounds__(256)
   g.has_x = has_x;
   g.masks_other = ma;
   for (int64_t i = blockIdx.x; i < da; i += gridDim.x) {
-    C fa = ld_ea<R>(ea_a, i);
+    float2 fa = ld_ea<float>(ea_a, i);
     if (has_x) {
       __syncthreads();
-      build_cross_tables<R>(g, X, (int)i, 1, w, tab, threadIdx.x, blockDim.x);
+      build_cross_tables<float>(g, X, (int)i, 1, w, tab, threadIdx.x, blockDim.x);
     }
-    C* row = vec + i * db;
+    float2* row = vec + i * db;
     for (int64_t j = threadIdx.x; j < db; j += blockDim.x) {
-      C f = cmul<R>(fa, ld_ea<R>(ea_b, j));
+      float2 f = cmul<float>(fa, ld_ea<float>(ea_b, j));
       if (has_x) {
         uint32_t m = __ldg(mb + j);
-        for (int c = 0; c < nchunk; ++c) f = cmul<R>(f, tab[c * 256 + ((m >> (8 * c)) & 255)]);
+        for (int c = 0; c < nchunk; ++c) f = cmul<float>(f, tab[c * 256 + ((m >> (8 * c)) & 255)]);
       }
-      row[j] = cmul<R>(f, row[j]);
+      row[j] = cmul<float>(f, row[j]);
+    }
+  }
+}
+
+// The complex128 pass, and the one behind the transition sums of a reverse
+// sweep: with a second state, W = Im(conj(g) psi) first (unless null), then
+// both states times ea_a[i] ea_b[j] exp(i sum X[p][q]).  The phase of an
+// amplitude is a product of fixed-point factors on the integer units and
+// meets the state in FP64 (four multiply-adds a state, where the FP64 product
+// of all factors took sixteen and its tables 512 sincos a row: N = 14 (7,7)
+// 465 us, now 217; what is left is those and the integer
+// products).
+__global__ void __launch_bounds__(256)
+    k_phase_fx(double2* psi, double2* cot, double* W, int64_t da, int64_t db, const uint32_t* ma,
+               const uint32_t* mb, int norb, int nchunk, const double2* ea_a,
+               const double2* ea_b, int has_x, const __grid_constant__ Mat X) {
+  __shared__ longlong2 tab[4 * 256], work[32 + 32 * 4];
+  __shared__ uint32_t bad_x;
+  for (int64_t i = blockIdx.x; i < da; i += gridDim.x) {
+    longlong2 fa = make_longlong2(1ll << 62, 0);
+    bool bad_a = false;
+    if (ea_a) {
+      const double2 z = __ldg(ea_a + i);
+      bad_a = fx::not_finite(z);
+      fa = fx::phase_from(z);
+    }
+    if (has_x) {
+      __syncthreads();
+      fx::cross_tables(ma, 1, norb, nchunk, X, (int)i, 1, tab, work, &bad_x, threadIdx.x, blockDim.x,
+                       [] { __syncthreads(); });
+      // the row's own factor joins the last table
+      for (int v = threadIdx.x; v < 256; v += blockDim.x)
+        tab[(nchunk - 1) * 256 + v] = fx::phase_mul(tab[(nchunk - 1) * 256 + v], fa);
+      __syncthreads();
+    }
+    for (int64_t j = threadIdx.x; j < db; j += blockDim.x) {
+      const double2 p = psi[i * db + j];
+      longlong2 f = make_longlong2(1ll << 62, 0);
+      bool bad = bad_a;
+      if (ea_b) {
+        const double2 z = __ldg(ea_b + j);
+        bad = bad || fx::not_finite(z);
+        f = fx::phase_from(z);
+      }
+      if (has_x) {
+        const uint32_t m = __ldg(mb + j);
+        bad = bad || (m & bad_x);
+        for (int k = 0; k < nchunk; ++k)
+          f = fx::phase_mul(f, tab[k * 256 + ((m >> (8 * k)) & 255)]);
+      } else {
+        f = fx::phase_mul(f, fa);
+      }
+      const double2 z = bad ? fx::nan2() : fx::phase_to(f);
+      psi[i * db + j] = cmul<double>(z, p);
+      if (cot) {
+        const double2 c = cot[i * db + j];
+        if (W) W[i * db + j] = c.x * p.y - c.y * p.x;
+        cot[i * db + j] = cmul<double>(z, c);
+      }
     }
   }
 }
@@ -870,13 +937,24 @@ void launch_phase(const Space* sa, const Space* sb, void* vec, int dtype,
   int nchunk = (sa->norb + 7) / 8;
   unsigned grid = (unsigned)std::min<int64_t>(sa->dim, 4096);
   if (dtype == FS_C64)
-    k_phase<float><<<grid, 256, 0, st>>>((float2*)vec, sa->dim, sb->dim, sa->masks,
+    k_phase<<<grid, 256, 0, st>>>((float2*)vec, sa->dim, sb->dim, sa->masks,
                                          sb->masks, sa->norb, nchunk, ph.ea_a,
                                          ph.ea_b, ph.has_x, ph.X);
   else
-    k_phase<double><<<grid, 256, 0, st>>>((double2*)vec, sa->dim, sb->dim, sa->masks,
-                                          sb->masks, sa->norb, nchunk, ph.ea_a,
-                                          ph.ea_b, ph.has_x, ph.X);
+    k_phase_fx<<<grid, 256, 0, st>>>((double2*)vec, nullptr, nullptr, sa->dim, sb->dim, sa->masks,
+                                     sb->masks, sa->norb, nchunk, (const double2*)ph.ea_a,
+                                     (const double2*)ph.ea_b, ph.has_x, ph.X);
+  FS_CUDA(cudaGetLastError());
+}
+
+void launch_rev_phase(const Space* sa, const Space* sb, void* psi, void* cot, int dtype,
+                      const RevArgs& rev, const PhaseDev& ph, cudaStream_t st) {
+  FS_REQUIRE(dtype == FS_C128, FS_ERR_ARG, "reverse phase pass: complex128");
+  ProfScope ps("rev_phase_f64", st);
+  k_phase_fx<<<(unsigned)std::min<int64_t>(sa->dim, 4096), 256, 0, st>>>(
+      (double2*)psi, (double2*)cot, (double*)rev.W, sa->dim, sb->dim, sa->masks, sb->masks,
+      sa->norb, (sa->norb + 7) / 8, (const double2*)rev.ea2_a, (const double2*)rev.ea2_b, ph.has_x,
+      ph.X);
   FS_CUDA(cudaGetLastError());
 }
 
@@ -911,8 +989,8 @@ void preload_phase_kernels() {
   cudaFuncAttributes fa;
   FS_CUDA(cudaFuncGetAttributes(&fa, k_string_phase<float>));
   FS_CUDA(cudaFuncGetAttributes(&fa, k_string_phase<double>));
-  FS_CUDA(cudaFuncGetAttributes(&fa, k_phase<float>));
-  FS_CUDA(cudaFuncGetAttributes(&fa, k_phase<double>));
+  FS_CUDA(cudaFuncGetAttributes(&fa, k_phase));
+  FS_CUDA(cudaFuncGetAttributes(&fa, k_phase_fx));
 }
 
 void launch_string_phase(const Space* sp, void* out, int dtype, const StrPhase& f,

@@ -19,7 +19,7 @@
 // the step's images in shared memory accumulate in seven TMEM accumulators;
 // the warps read those back, join them and scatter the new amplitudes.
 //
-// Measured (one GB300, one spin, complex128): N = 14 (7,7) 1.64 ms against
+// Measured (one GB300, one spin, complex128): N = 14 (7,7) 1.52 ms against
 // 6.74 ms of the FP64 sweep, which runs at 0.8 of the FP64 rate (2 FMA per
 // clock and SM); N = 12 (6,6) 0.105 against 0.80 ms; N = 8 (4,4) 32 + 18
 // (images) against 45 us.  Bound by the integer and FP32 instructions of the
@@ -73,10 +73,6 @@ __host__ __device__ constexpr uint32_t idesc(int n) {
 struct StepMats {
   long long v[kMaxSteps][72];  // V of each step, row-major 6 x 6 complex, fixed point
 };
-
-__device__ __forceinline__ longlong2 cmul_fx(longlong2 x, longlong2 y) {
-  return make_longlong2(mul(x.x, y.x) - mul(x.y, y.y), mul(x.x, y.y) + mul(x.y, y.x));
-}
 
 // Per step, the compound matrices C_m(V)[S', S] = det V[S', S] by Laplace
 // expansion along the first row of S', in fixed point (integer multiplies:
@@ -293,7 +289,7 @@ struct Args {
   int cap_first, cap_rest;  // bytes of the staged addresses: class 3; the others
   const unsigned char* img;
   const uint32_t *masks_this, *masks_other;
-  const double2 *ea_this, *ea_other;
+  const double2 *ea_this, *ea_other;  // phases
   int* status;
   uint8_t a[kMaxSteps];     // window position of each step
   uint8_t full[kMaxSteps];  // class 6 moves in this step (det V != 1)
@@ -455,10 +451,6 @@ __global__ void __launch_bounds__(kCta, 1)
       if (lane == 0) s_max[kv][sub] = mx;
     }
   sync_data();
-  auto scaled = [](double x, int f) {  // about |x| 2^(1023 - f), 0 when far below
-    const int q = exp_field(x) - f + 127;
-    return q > 1 ? __int_as_float((q << 23) | ((__double2hiint(x) & 0xFFFFF) << 3)) : 0.f;
-  };
   if (kv1 < ngrp)
     for (int kv = kv1; kv < nv; kv += ngrp) {
       uint32_t f = 1;
@@ -467,7 +459,7 @@ __global__ void __launch_bounds__(kCta, 1)
 #pragma unroll 4
     for (int e = sub * 32 + lane; e < d; e += 32 * per) {
         const double2 x = raw[(size_t)kv * d + e];
-        const float a = scaled(x.x, (int)f), b = scaled(x.y, (int)f);
+        const float a = rel_abs(x.x, (int)f), b = rel_abs(x.y, (int)f);
         s = fmaf(a, a, fmaf(b, b, s));
       }
 #pragma unroll
@@ -483,11 +475,8 @@ __global__ void __launch_bounds__(kCta, 1)
         f = max(f, s_max[kv][i]);
         s += s_sum[kv][i];
       }
-      // norm = 2^(f - 1023) sqrt(s) < 2^(eb - 1023); s < 2^20
-      const float r = fmaxf(sqrtf(s) * 1.001f, 1.0f);
-      const int k = ((__float_as_int(r) >> 23) & 0xFF) - 126;  // r < 2^k
       const bool finite = f < 0x7FF;
-      const int eb = (int)f + k;
+      const int eb = norm_exponent((int)f, s);
       if (sub == 0 && lane == 0) s_eb[kv] = finite ? eb : -1;
 #pragma unroll 4
     for (int e = sub * 32 + lane; e < d; e += 32 * per) {
@@ -598,43 +587,32 @@ __global__ void __launch_bounds__(kCta, 1)
   // ---- phases, store.  The cross tables go where the images were (every
   // copy has landed and been read).
   const int tper = g.nchunk * 256;
-  double2* tab = reinterpret_cast<double2*>(slab + (size_t)g.KV * d);
-  if (g.has_x) {
-    double* w = reinterpret_cast<double*>(simg);
-    for (int i = tid; i < nv * g.norb; i += kThreads) {
-      const int kv = i / g.norb, x = i - kv * g.norb;
-      double s = 0;
-      for (uint32_t m = g.masks_other[v0 + kv]; m; m &= m - 1) {
-        const int y = __ffs(m) - 1;
-        s += g.dir == 1 ? X.v[y * g.norb + x] : X.v[x * g.norb + y];
-      }
-      w[kv * kMaxOrb + x] = s;
-    }
-    sync_data();
-    for (int i = tid; i < nv * tper; i += kThreads) {
-      const int kv = i / tper, e = i - kv * tper, c = e >> 8;
-      double s = 0;
-      for (int v = e & 255; v; v &= v - 1) {
-        const int x = 8 * c + __ffs(v) - 1;
-        if (x < g.norb) s += w[kv * kMaxOrb + x];
-      }
-      tab[i] = expi<double>(s);
-    }
-    sync_data();
-  }
+  longlong2* tab = slab + (size_t)g.KV * d;
+  if (g.has_x)
+    cross_tables(g.masks_other, g.dir, g.norb, g.nchunk, X, v0, nv, tab,
+                 reinterpret_cast<longlong2*>(simg), &s_max[0][0], tid, kThreads, [] { sync_data(); });
   auto finish = [&](int kv, int e) {
     const int eb = s_eb[kv];
-    const longlong2 c = slab[(size_t)kv * d + e];
-    double2 v = make_double2(to_double(c.x, eb), to_double(c.y, eb));
-    if (eb < 0) v.x = v.y = __longlong_as_double(0x7FF8000000000000ll);
-    if (g.ea_other) v = cmul<double>(v, __ldg(g.ea_other + v0 + kv));
-    if (g.ea_this) v = cmul<double>(v, __ldg(g.ea_this + e));
-    if (g.has_x) {
-      const uint32_t m = __ldg(g.masks_this + e);
-      for (int k = 0; k < g.nchunk; ++k)
-        v = cmul<double>(v, tab[kv * tper + k * 256 + ((m >> (8 * k)) & 255)]);
+    longlong2 c = slab[(size_t)kv * d + e];
+    bool bad = eb < 0;
+    if (g.has_x || g.ea_this || g.ea_other) {
+      longlong2 f = make_longlong2(1ll << 62, 0);
+      auto factor = [&](double2 z) {
+        bad = bad || not_finite(z);
+        f = phase_mul(f, phase_from(z));
+      };
+      if (g.ea_this) factor(__ldg(g.ea_this + e));
+      if (g.ea_other) factor(__ldg(g.ea_other + v0 + kv));
+      if (g.has_x) {
+        const uint32_t m = __ldg(g.masks_this + e);
+        bad = bad || (m & (&s_max[0][0])[kv]);
+        for (int k = 0; k < g.nchunk; ++k)
+          f = phase_mul(f, tab[kv * tper + k * 256 + ((m >> (8 * k)) & 255)]);
+      }
+      c = cmul_fx(c, f);
     }
-    return v;
+    double2 v = make_double2(to_double(c.x, eb), to_double(c.y, eb));
+    return bad ? nan2() : v;
   };
   if (g.dir == 1) {
     for (int kv = 0; kv < nv; ++kv)

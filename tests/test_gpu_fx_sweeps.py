@@ -136,3 +136,22 @@ def test_vjp_against_oracle(lib, ctx, norb, nelec):
         assert np.max(np.abs(a - b)) <= 1e-10 * max(1.0, np.max(np.abs(b)))
     assert np.max(np.abs(c.cpu().numpy() - grads[3])) < TOL
     assert np.max(np.abs(x.cpu().numpy() - v)) < TOL
+
+
+def test_phase_of_non_finite_coupling_stays_with_its_strings(lib, ctx):
+    """The complex128 phase passes: a coupling that is not a number reaches the
+    configurations that hold both its orbitals, and no others."""
+    norb, nelec = 9, (4, 5)
+    g = inputs.rng(41990)
+    v = inputs.random_state(norb, nelec, g)
+    Ja, Jb = inputs.random_symmetric(norb, 1.0, g), inputs.random_symmetric(norb, 1.0, g)
+    ref = oracle.apply_diag_coulomb_evolution(v, Ja, Jb, Ja, 0.4, norb, nelec)
+    Jb = Jb.copy()
+    Jb[2, 7] = np.nan
+    x = torch.from_numpy(v).cuda()
+    lib.apply_diag_coulomb_evolution_(x, Ja, Jb, 0.4, norb, nelec, ctx=ctx)
+    ma, mb = lib.string_table(norb, 4, ctx=ctx), lib.string_table(norb, 5, ctx=ctx)
+    hit = (((ma >> 2) & 1)[:, None] & ((mb >> 7) & 1)[None, :]).astype(bool)
+    out = x.cpu().numpy()
+    assert np.isnan(out[hit]).all()
+    assert np.max(np.abs(out[~hit] - ref[~hit])) < TOL
