@@ -234,7 +234,9 @@ __global__ void __launch_bounds__(1024)
   __syncthreads();
   if (threadIdx.x == 0) {
     T e = A::zero();
-    for (int k = 0; k < (int)blockDim.x; ++k) {
+    // chunks past the last tile hold zeros, which no later one needs
+    const int used = (int)min((int64_t)blockDim.x, (ntiles + chunk - 1) / chunk);
+    for (int k = 0; k < used; ++k) {
       const T x = tot[k];
       tot[k] = e;
       e = A::add(e, x);
@@ -383,6 +385,274 @@ __global__ void __launch_bounds__(256)
   }
 }
 
+// ------------------------------------------- many shots per group
+// With at least as many shots as groups the shots are ordered by group first,
+// so that a group is read and summed once for all of them (one warp per shot
+// reads 2 KB of the state for each: 1e6 shots from N = 15 (7,8), 162k groups,
+// 860 us; ordered, 225 us: locating 75, ordering 20, picking 130).  The decisions are those of k_sample_state: the
+// same sums in the same order, compared in the same way.
+struct ShotRec {  // located: rank inside its group; ordered: shot index
+  uint32_t g, r;
+  float2 x;  // the target inside the group (dfl, or the bits of a double)
+};
+__device__ __forceinline__ float2 pack_acc(dfl a) { return make_float2(a.h, a.l); }
+__device__ __forceinline__ float2 pack_acc(double a) {
+  return make_float2(__int_as_float(__double2loint(a)), __int_as_float(__double2hiint(a)));
+}
+__device__ __forceinline__ void unpack_acc(float2 p, dfl& a) { a = dfl{p.x, p.y}; }
+__device__ __forceinline__ void unpack_acc(float2 p, double& a) {
+  a = __hiloint2double(__float_as_int(p.y), __float_as_int(p.x));
+}
+
+// First k in [lo, hi) with a[k] > x (>= when ge); a[hi - 1] satisfies it.
+template <typename A>
+__device__ __forceinline__ int thread_search(const typename A::T* a, int lo, int hi,
+                                             typename A::T x, bool ge) {
+  while (hi - lo > 1) {
+    const int mid = lo + ((hi - lo) >> 1) - 1;  // the last of the first half
+    const typename A::T y = a[mid];
+    if (ge ? A::ge(y, x) : A::gt(y, x)) hi = mid + 1; else lo = mid + 1;
+  }
+  return lo;
+}
+
+// Tile and group of every shot (one thread each, as k_sample_state finds
+// them), its target inside the group and its rank among the group's shots.
+constexpr int kTilesShared = 2048;
+template <typename R>
+__global__ void __launch_bounds__(256)
+    k_shot_groups(int ngroups, int ntiles, const typename Acc<R>::T* __restrict__ gc,
+                  const typename Acc<R>::T* __restrict__ tcg, const double* __restrict__ u,
+                  int64_t shots, uint32_t* count, ShotRec* rec) {
+  using A = Acc<R>;
+  using T = typename A::T;
+  __shared__ T stc[kTilesShared];
+  const T* tc = tcg;
+  if (ntiles <= kTilesShared) {
+    for (int i = threadIdx.x; i < ntiles; i += 256) stc[i] = tcg[i];
+    __syncthreads();
+    tc = stc;
+  }
+  const int64_t s = blockIdx.x * 256ll + threadIdx.x;
+  if (s >= shots) return;
+  const T total = tc[ntiles - 1];
+  if (!(A::finite(total) && A::pos(total))) {  // no shot has a group: any order will do
+    rec[s] = ShotRec{0u, (uint32_t)s, make_float2(0.f, 0.f)};
+    return;
+  }
+  R uh = 0, ul = 0;
+  {
+    const double x = u[s];
+    if (x == x) {
+      uh = (R)x;
+      ul = (R)(x - (double)uh);
+    }
+  }
+  T x = A::scale(uh, ul, total);
+  if (!A::pos(x)) x = A::zero();
+  bool ge = false;
+  if (!A::gt(total, x)) {
+    x = total;
+    ge = true;
+  }
+  const int t = thread_search<A>(tc, 0, ntiles, x, ge);
+  T xt = t > 0 ? A::add(x, A::neg(tc[t - 1])) : x;
+  if (!A::pos(xt)) xt = A::zero();
+  const int g0 = t * kTileGroups, g1 = min(ngroups, g0 + kTileGroups);
+  const T ttot = gc[g1 - 1];
+  ge = false;
+  if (!A::gt(ttot, xt)) {
+    xt = ttot;
+    ge = true;
+  }
+  const int g = thread_search<A>(gc, g0, g1, xt, ge);
+  T xg = g > g0 ? A::add(xt, A::neg(gc[g - 1])) : xt;
+  if (!A::pos(xg)) xg = A::zero();
+  ShotRec r;
+  r.g = (uint32_t)g;
+  r.r = atomicAdd(count + g, 1u);
+  r.x = pack_acc(xg);
+  rec[s] = r;
+}
+
+// Exclusive prefix of the groups' shot counts in blocks of 1024, and the
+// blocks' totals; k_order adds the totals of the blocks before.
+__global__ void __launch_bounds__(1024)
+    k_count_prefix(uint32_t* count, uint32_t* block_total, int64_t n) {
+  __shared__ uint32_t ws[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t i = blockIdx.x * 1024ll + threadIdx.x;
+  const uint32_t c = i < n ? count[i] : 0u;
+  uint32_t v = c;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, v, d);
+    if (lane >= d) v += y;
+  }
+  if (lane == 31) ws[warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t w = ws[lane];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, w, d);
+      if (lane >= d) w += y;
+    }
+    ws[lane] = w;
+  }
+  __syncthreads();
+  const uint32_t before = warp ? ws[warp - 1] : 0u;
+  if (i < n) count[i] = before + v - c;
+  if (threadIdx.x == 1023) block_total[blockIdx.x] = before + v;
+}
+// One CTA: block totals to their exclusive prefix.
+__global__ void __launch_bounds__(1024) k_block_prefix(uint32_t* total, int64_t n) {
+  __shared__ uint32_t ws[32];
+  __shared__ uint32_t carry;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) carry = 0;
+  for (int64_t b = 0; b < n; b += 1024) {
+    __syncthreads();
+    const int64_t i = b + threadIdx.x;
+    const uint32_t c = i < n ? total[i] : 0u;
+    uint32_t v = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, v, d);
+      if (lane >= d) v += y;
+    }
+    if (lane == 31) ws[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+      uint32_t w = ws[lane];
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, w, d);
+        if (lane >= d) w += y;
+      }
+      ws[lane] = w;
+    }
+    __syncthreads();
+    const uint32_t at = carry + (warp ? ws[warp - 1] : 0u) + v;
+    if (i < n) total[i] = at - c;
+    __syncthreads();
+    if (threadIdx.x == 1023) carry = at;
+  }
+}
+__global__ void __launch_bounds__(256)
+    k_order(const ShotRec* __restrict__ rec, int64_t shots, const uint32_t* __restrict__ count,
+            const uint32_t* __restrict__ block, ShotRec* __restrict__ ordered) {
+  const int64_t s = blockIdx.x * 256ll + threadIdx.x;
+  if (s >= shots) return;
+  ShotRec r = rec[s];
+  const uint32_t at = block[r.g >> 10] + count[r.g] + r.r;
+  r.r = (uint32_t)s;
+  ordered[at] = r;
+}
+
+// One warp per 64 ordered shots, group by group: the group's 256 amplitudes
+// are summed as in k_sample_state and kept in shared memory, then each lane
+// decides one shot.
+template <typename R>
+__global__ void __launch_bounds__(256)
+    k_pick(const cx_t<R>* __restrict__ v, int64_t n, int64_t ntiles,
+           const typename Acc<R>::T* __restrict__ tc, const ShotRec* __restrict__ rec,
+           int64_t shots, int64_t* __restrict__ out) {
+  using A = Acc<R>;
+  using T = typename A::T;
+  __shared__ T srun[8][8][32];  // [warp][k][lane]: running sums of a lane's slice
+  __shared__ T sincl[8][32], sexcl[8][32];
+  __shared__ uint8_t smass[8][32];  // which of the slice's eight hold mass
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const T total = tc[ntiles - 1];
+  const bool usable = A::finite(total) && A::pos(total);
+  const int64_t w = blockIdx.x * 8ll + warp;
+  int64_t at = w * 64;
+  const int64_t end = min(shots, at + 64);
+  if (!usable) {
+    for (int64_t s = at + lane; s < end; s += 32) out[s] = -1;
+    return;
+  }
+  uint32_t have = 0xFFFFFFFFu;  // the group in shared memory
+  unsigned has = 0;
+  while (at < end) {
+    ShotRec r{};
+    const bool in = at + lane < end;
+    if (in) r = rec[at + lane];
+    const uint32_t g = __shfl_sync(0xffffffffu, r.g, 0);
+    const unsigned same = __ballot_sync(0xffffffffu, in && r.g == g);
+    const int cnt = same == 0xffffffffu ? 32 : __ffs(~same) - 1;
+    if (g != have) {
+      __syncwarp();
+      const int64_t a0 = (int64_t)g * kGroup + 8 * lane;
+      const int64_t left = n - a0;
+      const int c = left <= 0 ? 0 : (left >= 8 ? 8 : (int)left);
+      cx_t<R> z[8];
+      if (c == 8) {
+        if constexpr (sizeof(R) == 4) {
+          const float4* p4 = reinterpret_cast<const float4*>(v + a0);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float4 q = p4[k];
+            z[2 * k] = make_float2(q.x, q.y);
+            z[2 * k + 1] = make_float2(q.z, q.w);
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) z[k] = v[a0 + k];
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) z[k] = k < c ? v[a0 + k] : cx_t<R>{};
+      }
+      T own = A::zero();
+      unsigned mass = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const T p = k < c ? A::prob(z[k]) : A::zero();
+        mass |= (A::pos(p) ? 1u : 0u) << k;
+        own = A::add(own, p);
+        srun[warp][k][lane] = own;
+      }
+      smass[warp][lane] = (uint8_t)mass;
+      T incl = own;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const T y = A::shfl_up(incl, d);
+        if (lane >= d) incl = A::add(y, incl);
+      }
+      T excl = A::shfl_up(incl, 1);
+      if (lane == 0) excl = A::zero();
+      sincl[warp][lane] = incl;
+      sexcl[warp][lane] = excl;
+      has = __ballot_sync(0xffffffffu, A::pos(own));
+      have = g;
+      __syncwarp();
+    }
+    if (lane < cnt) {
+      T xg;
+      unpack_acc(r.x, xg);
+      // the first slice that crosses the target: sums ascend over the slices
+      int f = 0;
+#pragma unroll
+      for (int h = 16; h > 0; h >>= 1)
+        if (!A::gt(sincl[warp][f + h - 1], xg)) f += h;
+      const bool scan = A::gt(sincl[warp][f], xg) && ((has >> f) & 1u);
+      if (!scan) f = has ? 31 - __clz(has) : 0;  // the last slice that holds mass
+      const unsigned mass = smass[warp][f];
+      int pick = -1;
+      T xl = A::add(xg, A::neg(sexcl[warp][f]));
+      if (!A::pos(xl)) xl = A::zero();
+#pragma unroll
+      for (int k = 7; k >= 0; --k)
+        if (scan && ((mass >> k) & 1u) && A::gt(srun[warp][k][f], xl)) pick = k;
+      if (pick < 0) pick = 31 - __clz(mass);  // -1 without mass
+      out[r.r] = pick < 0 ? -1 : (int64_t)g * kGroup + 8 * f + pick;
+    }
+    at += cnt;
+  }
+}
+
 // ------------------------------------------------- Slater determinants
 // K[p][q] = sum_j Phi[p][j] conj(Phi[q][j]) (FP64), Phi = U[:, occ] (N x n).
 __global__ void k_projector(double2* __restrict__ K, const double2* __restrict__ Phi, int N,
@@ -519,51 +789,68 @@ __global__ void __launch_bounds__(256)
 }
 
 // ------------------------------------------------------------- launch
+template <typename R>
+static void sample_state_t(Ctx* ctx, const cx_t<R>* vec, int64_t n, const double* u, int64_t shots,
+                           int64_t* out, cudaStream_t st) {
+  using T = typename Acc<R>::T;
+  static_assert(sizeof(T) == 8, "prefix tables hold 8 bytes per entry");
+  const int64_t ngroups = (n + kGroup - 1) / kGroup;
+  const int64_t ntiles = (ngroups + kTileGroups - 1) / kTileGroups;
+  T* gc = (T*)scratch(ctx, "sample_cdf", (size_t)(ngroups + 2 * ntiles) * sizeof(T));
+  T* ts = gc + ngroups;
+  T* tc = ts + ntiles;
+  const int sms = ctx->prop.multiProcessorCount;
+  {
+    ProfScope ps("sample_cdf", st);
+    k_cdf_groups<R><<<(unsigned)std::min<int64_t>(ntiles, (int64_t)1 << 30), 256, 0, st>>>(
+        vec, n, ngroups, ntiles, gc, ts);
+    FS_CUDA(cudaGetLastError());
+  }
+  {
+    ProfScope ps("sample_cdf_tiles", st);
+    k_cdf_tiles<R><<<1, 1024, 0, st>>>(ts, ntiles, tc);
+    FS_CUDA(cudaGetLastError());
+  }
+  // Ordered by group where the groups get at least one shot each on average
+  // (fewer: as many groups to read as shots, and the ordering on top); 2^24
+  // shots at a time bound its scratch to 0.5 GB, group counts to 32 bits.
+  constexpr int64_t kOrdered = (int64_t)1 << 24;
+  if (shots >= ngroups && ngroups <= kOrdered) {
+    ProfScope ps("sample_search", st, 6);
+    const int64_t cap = std::min(shots, kOrdered), nblk = (ngroups + 1023) / 1024;
+    uint32_t* count = (uint32_t*)scratch(ctx, "sample_count", (size_t)(ngroups + nblk) * 4);
+    ShotRec* rec = (ShotRec*)scratch(ctx, "sample_shots", 2 * (size_t)cap * sizeof(ShotRec));
+    for (int64_t s0 = 0; s0 < shots; s0 += cap) {
+      const int64_t c = std::min(cap, shots - s0);
+      const unsigned grid = (unsigned)((c + 255) / 256);
+      FS_CUDA(cudaMemsetAsync(count, 0, (size_t)ngroups * 4, st));
+      k_shot_groups<R><<<grid, 256, 0, st>>>((int)ngroups, (int)ntiles, gc, tc, u + s0, c, count, rec);
+      FS_CUDA(cudaGetLastError());
+      k_count_prefix<<<(unsigned)nblk, 1024, 0, st>>>(count, count + ngroups, ngroups);
+      FS_CUDA(cudaGetLastError());
+      k_block_prefix<<<1, 1024, 0, st>>>(count + ngroups, nblk);
+      FS_CUDA(cudaGetLastError());
+      k_order<<<grid, 256, 0, st>>>(rec, c, count, count + ngroups, rec + cap);
+      FS_CUDA(cudaGetLastError());
+      k_pick<R><<<(unsigned)((c + 511) / 512), 256, 0, st>>>(vec, n, ntiles, tc, rec + cap, c,
+                                                           out + s0);
+      FS_CUDA(cudaGetLastError());
+    }
+    return;
+  }
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((shots + 7) / 8, (int64_t)sms * 16));
+  ProfScope ps("sample_search", st);
+  k_sample_state<R><<<grid, 256, 0, st>>>(vec, n, ngroups, ntiles, gc, tc, u, shots, out);
+  FS_CUDA(cudaGetLastError());
+}
+
 void sample_state(Ctx* ctx, const void* vec, int dtype, int64_t n, const double* u,
                   int64_t shots, int64_t* out, cudaStream_t st) {
   if (shots == 0) return;
-  const int64_t ngroups = (n + kGroup - 1) / kGroup;
-  const int64_t ntiles = (ngroups + kTileGroups - 1) / kTileGroups;
-  const size_t acc = 8;  // dfl and double are both 8 bytes
-  char* ws = (char*)scratch(ctx, "sample_cdf", (size_t)(ngroups + 2 * ntiles) * acc);
-  const int sms = ctx->prop.multiProcessorCount;
-  const unsigned g1 = (unsigned)std::min<int64_t>(ntiles, (int64_t)1 << 30);
-  const int g3 = (int)std::max<int64_t>(
-      1, std::min<int64_t>((shots + 7) / 8, (int64_t)sms * 16));
-  if (dtype == FS_C64) {
-    using T = Acc<float>::T;
-    T* gc = (T*)ws;
-    T* ts = gc + ngroups;
-    T* tc = ts + ntiles;
-    {
-      ProfScope ps("sample_cdf", st);
-      k_cdf_groups<float><<<g1, 256, 0, st>>>((const float2*)vec, n, ngroups, ntiles, gc, ts);
-    }
-    {
-      ProfScope ps("sample_cdf_tiles", st);
-      k_cdf_tiles<float><<<1, 1024, 0, st>>>(ts, ntiles, tc);
-    }
-    ProfScope ps("sample_search", st);
-    k_sample_state<float><<<g3, 256, 0, st>>>((const float2*)vec, n, ngroups, ntiles, gc, tc, u,
-                                              shots, out);
-  } else {
-    using T = Acc<double>::T;
-    T* gc = (T*)ws;
-    T* ts = gc + ngroups;
-    T* tc = ts + ntiles;
-    {
-      ProfScope ps("sample_cdf", st);
-      k_cdf_groups<double><<<g1, 256, 0, st>>>((const double2*)vec, n, ngroups, ntiles, gc, ts);
-    }
-    {
-      ProfScope ps("sample_cdf_tiles", st);
-      k_cdf_tiles<double><<<1, 1024, 0, st>>>(ts, ntiles, tc);
-    }
-    ProfScope ps("sample_search", st);
-    k_sample_state<double><<<g3, 256, 0, st>>>((const double2*)vec, n, ngroups, ntiles, gc, tc,
-                                               u, shots, out);
-  }
-  FS_CUDA(cudaGetLastError());
+  if (dtype == FS_C64)
+    sample_state_t<float>(ctx, (const float2*)vec, n, u, shots, out, st);
+  else
+    sample_state_t<double>(ctx, (const double2*)vec, n, u, shots, out, st);
 }
 
 void sample_slater(Ctx* ctx, const std::vector<zd>& Phi, int N, int n, const double* u,

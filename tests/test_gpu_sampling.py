@@ -195,3 +195,28 @@ def test_sample_slater_spinful_and_edges(lib):
     with pytest.raises(lib.FsError) as e:
         lib.sample_slater(N, [0, 1], Ua * 1.01, shots=3)
     assert e.value.code == -2
+
+
+@pytest.mark.parametrize("dt", ["c128", "c64"])
+@pytest.mark.parametrize("norb,nelec,shots", [(5, (2, 2), 4000), (8, (4, 4), 20), (10, (5, 4), 250),
+                                              (12, (6, 5), 6000), (12, (6, 5), 2800)])
+def test_shots_ordered_by_group_match_one_by_one(lib, dt, norb, nelec, shots):
+    """With at least a shot per group of 256 amplitudes the shots are ordered
+    by group first: every one is the configuration it gets alone, on states
+    with empty groups and tails, and at the ends of the uniform's range."""
+    g = inputs.rng(1590 + norb + shots)
+    v = inputs.random_state(norb, nelec, g)
+    flat = v.reshape(-1)
+    flat[flat.size // 3:flat.size // 2] = 0
+    flat[-5:] = 0
+    x = dev(v, dt)
+    u = torch.from_numpy(np.concatenate([g.random(shots - 5),
+                                         [0.0, 1.0, -1.0, np.nan, np.nextafter(1.0, 0.0)]])).cuda()
+    got = lib.sample_state(x, norb, nelec, uniforms=u)
+    few = max(1, (flat.size + 255) // 256 - 1)  # fewer shots than groups: one warp each
+    alone = torch.cat([lib.sample_state(x, norb, nelec, uniforms=u[i:i + few])
+                       for i in range(0, shots, few)])
+    assert torch.equal(got, alone)
+    bad = x.clone()
+    bad.view(-1)[7] = float("inf")
+    assert (lib.sample_state(bad, norb, nelec, uniforms=u) == -1).all()
