@@ -15,7 +15,7 @@
 // eighth of the multiply-adds of full N^2 x N^2 products and of the
 // intermediates.  (The full products, complex64 on the tensor cores and
 // complex128 in FP64, took 5.7 ms at N = 12 (6,6) in complex64 and 8.8 ms at
-// N = 10 (5,5) in complex128; now 1.38 and 0.89 ms, bound by the products:
+// N = 10 (5,5) in complex128; now 1.19 and 0.89 ms, bound by the products:
 // FP64 rate, and in complex64 the shared-memory reads of the mixed part.)
 //   same spin: F[l][s] = sum_k V[pq_l][rs_k] sign_k psi[src_k] + k_{pq_l} psi[s]
 //              for the excitations pq_l out of string s, rs_k into it; then
@@ -61,84 +61,157 @@ __global__ void k_op_weights(const double* h2, R* V, R* W, int NN) {
 }
 
 // Same-spin products of string s = blockIdx.x over columns of X (rows are
-// strings): F[l][s][c] for the excitations l out of s.  A thread owns `CT`
-// columns (128 apart) and 16 excitations at a time; the weights of those,
-// signs folded in, are in shared memory and reach a warp by broadcast, so a
-// product costs one multiply-add per part (FP32: one two-lane instruction)
-// and a sixteenth of a load.
-constexpr int kOpL = 16;
-template <typename R, int CT>
+// strings): F[l][s][c] for the excitations l out of s, L of them at a time
+// (the whole list where the registers allow: every pass reads the ne rows of
+// X again).  Their weights, signs folded in, are in shared memory.
+//   complex128: a thread owns one column and all L excitations; bound by the
+//     FP64 rate (N = 10 (5,5): 0.76 of it).
+//   complex64: a thread owns L / 4 excitations of four columns, so that a
+//     weight is read for four products (two-lane multiply-adds), from a
+//     tile of X in shared memory.  N = 12 (6,6), ne = 42: 232 us; with one
+//     column per thread, read from L2 as needed, 320 us.
+template <typename R>
+__host__ __device__ constexpr int op_rows() {  // rows of X staged at a time
+  return sizeof(R) == 4 ? 48 : 32;
+}
+__device__ __forceinline__ void cp_async_x(float2* dst, const float2* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_x(double2* dst, const double2* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+template <typename R, int L>
 __global__ void __launch_bounds__(128)
     k_op_same(cx_t<R>* F, int64_t fstride, const cx_t<R>* X, int64_t ldx, int64_t col0,
               int64_t ncol, const uint16_t* gpq, const uint32_t* gsrc, int ne, int N,
               const R* V, const __grid_constant__ Mat kmat) {
   using C = cx_t<R>;
+  constexpr int LG = sizeof(R) == 4 ? 4 : 1;  // lane groups along l
+  constexpr int TL = L / LG, TC = LG;         // excitations and columns of a thread
+  constexpr int CW = 32 / LG;                 // columns of a warp per TC
+  constexpr int KB = op_rows<R>();
   extern __shared__ __align__(16) unsigned char smraw[];
-  R* wt = reinterpret_cast<R*>(smraw);                             // [ne][kOpL]
-  uint32_t* src = reinterpret_cast<uint32_t*>(wt + (size_t)ne * kOpL);  // [ne]
+  C* xs = reinterpret_cast<C*>(smraw);       // [KB][128]: a tile of X
+  R* wt = reinterpret_cast<R*>(xs + KB * 128);  // [ne][L]
+  uint32_t* src = reinterpret_cast<uint32_t*>(wt + (size_t)ne * L);  // [ne]
+  uint32_t* pq = src + ne;                                           // [ne] into s | out of s << 16
   const int64_t s = blockIdx.x;
   const int NN = N * N;
-  const uint16_t* pq = gpq + s * ne;
-  for (int k = threadIdx.x; k < ne; k += 128) src[k] = gsrc[s * ne + k];
-  for (int l0 = 0; l0 < ne; l0 += kOpL) {
+  const int lane = threadIdx.x & 31, lg = lane / CW;
+  for (int k = threadIdx.x; k < ne; k += 128) {
+    src[k] = gsrc[s * ne + k];
+    const int q = gpq[s * ne + k];
+    pq[k] = (uint32_t)q | ((uint32_t)swap_pq(q, N) << 16);
+  }
+  for (int l0 = 0; l0 < ne; l0 += L) {
     __syncthreads();
-    for (int e = threadIdx.x; e < ne * kOpL; e += 128) {
-      const int k = e / kOpL, l = l0 + (e - k * kOpL);
+#pragma unroll 8
+    for (int e = threadIdx.x; e < ne * L; e += 128) {
+      const int k = e / L, l = l0 + (e - k * L);
       R w = 0;
       if (l < ne) {
-        w = V[(int64_t)swap_pq(pq[l], N) * NN + pq[k]];
+        w = V[(int64_t)(pq[l] >> 16) * NN + (pq[k] & 0xFFFFu)];
         if (src[k] >> 31) w = -w;
       }
       wt[e] = w;
     }
     __syncthreads();
-    for (int64_t c0 = blockIdx.y * (int64_t)(128 * CT); c0 < ncol;
-         c0 += gridDim.y * (int64_t)(128 * CT)) {
-      C acc[kOpL][CT];
+    const int lb = lg * TL;  // this thread's first excitation of the pass
+    for (int64_t cb = blockIdx.y * 128ll; cb < ncol; cb += gridDim.y * 128ll) {
+      C acc[TL][TC];
 #pragma unroll
-      for (int l = 0; l < kOpL; ++l)
+      for (int l = 0; l < TL; ++l)
 #pragma unroll
-        for (int u = 0; u < CT; ++u) acc[l][u] = mk<R>(0, 0);
-      int64_t c[CT];
-      bool in[CT];
-#pragma unroll
-      for (int u = 0; u < CT; ++u) {
-        c[u] = c0 + threadIdx.x + 128 * u;
-        in[u] = c[u] < ncol;
-      }
-      if (in[0]) {
+        for (int u = 0; u < TC; ++u) acc[l][u] = mk<R>(0, 0);
+      const int cw = (threadIdx.x >> 5) * 32 + lane % CW;  // first column in the tile
+      for (int k0 = 0; k0 < ne; k0 += KB) {
+        const int nk = min(KB, ne - k0);
+        __syncthreads();
+        if (cb + threadIdx.x < ncol)
+          for (int k = 0; k < nk; ++k)
+            cp_async_x(xs + k * 128 + threadIdx.x,
+                       X + (int64_t)(src[k0 + k] & 0x7FFFFFFFu) * ldx + col0 + cb + threadIdx.x);
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
 #pragma unroll 2
-        for (int k = 0; k < ne; ++k) {
-          const C* xr = X + (int64_t)(src[k] & 0x7FFFFFFFu) * ldx + col0;
-          C x[CT];
+        for (int k = 0; k < nk; ++k) {
+          C x[TC];
 #pragma unroll
-          for (int u = 0; u < CT; ++u) x[u] = in[u] ? xr[c[u]] : mk<R>(0, 0);
-          const R* w = wt + k * kOpL;
+          for (int u = 0; u < TC; ++u) x[u] = xs[k * 128 + cw + CW * u];
+          const R* w = wt + (k0 + k) * L + lb;
 #pragma unroll
-          for (int l = 0; l < kOpL; ++l)
+          for (int l = 0; l < TL; ++l)
 #pragma unroll
-            for (int u = 0; u < CT; ++u) axpy(acc[l][u], w[l], x[u]);
+            for (int u = 0; u < TC; ++u) axpy(acc[l][u], w[l], x[u]);
         }
+      }
 #pragma unroll
-        for (int u = 0; u < CT; ++u) {
-          if (!in[u]) continue;
-          const C x = X[s * ldx + col0 + c[u]];
+      for (int u = 0; u < TC; ++u) {
+        const int64_t c = cb + cw + CW * u;
+        if (c >= ncol) continue;
+        const C x = X[s * ldx + col0 + c];
 #pragma unroll
-          for (int l = 0; l < kOpL; ++l) {
-            if (l0 + l >= ne) break;
-            axpy(acc[l][u], (R)kmat.v[swap_pq(pq[l0 + l], N)], x);
-            F[(l0 + l) * fstride + s * ncol + c[u]] = acc[l][u];
-          }
+        for (int l = 0; l < TL; ++l) {
+          if (l0 + lb + l >= ne) break;
+          axpy(acc[l][u], (R)kmat.v[pq[l0 + lb + l] >> 16], x);
+          F[(l0 + lb + l) * fstride + s * ncol + c] = acc[l][u];
         }
       }
     }
   }
 }
 
+// Excitations per pass: the smallest of the compiled widths that covers the
+// list in the fewest passes (complex128 at most 32: four registers each).
+template <typename R>
+static int same_width(int ne) {
+  const int most = sizeof(R) == 4 ? 48 : 32;
+  const int passes = (ne + most - 1) / most;
+  int L = 16;
+  while (L < most && passes * L < ne) L += 16;
+  return L;
+}
+template <typename R>
+static size_t same_smem(int ne) {
+  return (size_t)op_rows<R>() * 128 * sizeof(cx_t<R>) +
+         (size_t)ne * (same_width<R>(ne) * sizeof(R) + 8);
+}
+template <typename R, int L>
+static void same_launch(cx_t<R>* F, int64_t fstride, const cx_t<R>* X, int64_t ldx, int64_t col0,
+                        int64_t ncol, const Space* sp, int N, const R* V, const Mat& kmat,
+                        cudaStream_t st) {
+  const size_t smem = same_smem<R>(sp->ne);
+  FS_CUDA(cudaFuncSetAttribute(k_op_same<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)smem));
+  // four column tiles per CTA: the weights of a string (2000 scattered reads at
+  // N = 12) cost as much as one tile's products
+  const unsigned ty = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ncol + 511) / 512, 65535));
+  k_op_same<R, L><<<dim3((unsigned)sp->dim, ty), 128, smem, st>>>(
+      F, fstride, X, ldx, col0, ncol, sp->gpq, sp->gsrc, sp->ne, N, V, kmat);
+  FS_CUDA(cudaGetLastError());
+}
+template <typename R>
+static void same_products(cx_t<R>* F, int64_t fstride, const cx_t<R>* X, int64_t ldx, int64_t col0,
+                          int64_t ncol, const Space* sp, int N, const R* V, const Mat& kmat,
+                          cudaStream_t st) {
+  switch (same_width<R>(sp->ne)) {
+    case 16: same_launch<R, 16>(F, fstride, X, ldx, col0, ncol, sp, N, V, kmat, st); break;
+    case 32: same_launch<R, 32>(F, fstride, X, ldx, col0, ncol, sp, N, V, kmat, st); break;
+    default:
+      if constexpr (sizeof(R) == 4)
+        same_launch<R, 48>(F, fstride, X, ldx, col0, ncol, sp, N, V, kmat, st);
+      break;
+  }
+}
+
+constexpr int kOpL = 16;  // excitations per pass of the mixed products
 // Mixed products of alpha string row0 + blockIdx.x: Y[k][ii][j] for the beta
 // excitations k out of j (lanes over j).  The row's weights W[pq_l][.],
-// signs folded in, are in shared memory (lcap rows at a time); a lane reads
-// its own entry of each, which its neighbours mostly share.
+// signs folded in, are in shared memory (lcap excitations l at a time, two
+// side by side); a lane reads its own entry of each, which its neighbours
+// mostly share.  Those reads bound the complex64 form.
 template <typename R>
 __global__ void __launch_bounds__(128)
     k_op_mixed(cx_t<R>* Y, int64_t ystride, const cx_t<R>* X, int64_t db, int64_t row0,
@@ -146,7 +219,7 @@ __global__ void __launch_bounds__(128)
                int N, const R* W, int lcap) {
   using C = cx_t<R>;
   extern __shared__ __align__(16) unsigned char smraw[];
-  R* wt = reinterpret_cast<R*>(smraw);  // [lcap][NN]
+  C* wt = reinterpret_cast<C*>(smraw);  // [lcap / 2][NN], l even in x, odd in y
   const int NN = N * N;
   const int64_t i = row0 + blockIdx.x;
   const uint16_t* pq = apq + i * nea;
@@ -165,20 +238,29 @@ __global__ void __launch_bounds__(128)
         const int nl = min(lcap, nea - l0);
         if (nea > lcap || (k0 == 0 && j0 == blockIdx.y * 128ll)) {
           __syncthreads();
-          for (int e = threadIdx.x; e < nl * NN; e += 128) {
-            const int l = e / NN;
-            const R w = W[(int64_t)pq[l0 + l] * NN + (e - l * NN)];
-            wt[e] = (src[l0 + l] >> 31) ? -w : w;
+          const int np = (nl + 1) / 2;
+          for (int e = threadIdx.x; e < np * NN; e += 128) {
+            const int h = e / NN, r = e - h * NN, l = l0 + 2 * h;
+            auto at = [&](int q) {
+              const R w = W[(int64_t)pq[q] * NN + r];
+              return (src[q] >> 31) ? -w : w;
+            };
+            wt[e] = mk<R>(at(l), l + 1 < nea ? at(l + 1) : R(0));
           }
           __syncthreads();
         }
         if (j < db) {
-#pragma unroll 2
-          for (int l = 0; l < nl; ++l) {
+          for (int l = 0; l < nl; l += 2) {
             const C x = X[(int64_t)(src[l0 + l] & 0x7FFFFFFFu) * db + j];
-            const R* w = wt + l * NN;
+            C y = mk<R>(0, 0);
+            if (l + 1 < nl) y = X[(int64_t)(src[l0 + l + 1] & 0x7FFFFFFFu) * db + j];
+            const C* w = wt + (l >> 1) * NN;
 #pragma unroll
-            for (int k = 0; k < kOpL; ++k) axpy(acc[k], w[rs[k]], x);
+            for (int k = 0; k < kOpL; ++k) {
+              const C v = w[rs[k]];
+              axpy(acc[k], v.x, x);
+              axpy(acc[k], v.y, y);
+            }
           }
         }
       }
@@ -276,7 +358,6 @@ static void molecular_hamiltonian_t(Ctx* ctx, Space* sa, Space* sb, const void* 
                                     const double* h1, const double* h2, double constant,
                                     int64_t ws, cudaStream_t st) {
   using C = cx_t<R>;
-  constexpr int CT = sizeof(R) == 4 ? 2 : 1;
   constexpr int dt = sizeof(R) == 4 ? FS_C64 : FS_C128;
   const int N = sa->norb, NN = N * N;
   const C* vec = (const C*)vec_;
@@ -313,14 +394,11 @@ static void molecular_hamiltonian_t(Ctx* ctx, Space* sa, Space* sb, const void* 
   C* buf = (C*)scratch(ctx, "op_F", std::max(nr * per_row, nc * per_col));
   const int sms = ctx->prop.multiProcessorCount;
   const size_t smax = (size_t)ctx->prop.sharedMemPerBlockOptin;
-  auto same_smem = [&](int ne) { return (size_t)ne * (kOpL * sizeof(R) + 4); };
-  const int lcap = (int)std::max<size_t>(1, std::min<size_t>(std::max(nea, 1),
-                                                             (size_t)64 * 1024 / (NN * sizeof(R))));
+  const int lcap = 2 * (int)std::max<size_t>(1, std::min<size_t>((nea + 1) / 2,
+                                                                 (size_t)32 * 1024 / (NN * sizeof(R))));
   const size_t mixed_smem = (size_t)lcap * NN * sizeof(R);
-  FS_REQUIRE(same_smem(std::max(nea, neb)) <= smax && mixed_smem <= smax, FS_ERR_UNSUPPORTED,
+  FS_REQUIRE(same_smem<R>(nea) <= smax && same_smem<R>(neb) <= smax && mixed_smem <= smax, FS_ERR_UNSUPPORTED,
              "operator action: weights exceed shared memory");
-  FS_CUDA(cudaFuncSetAttribute(k_op_same<R, CT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)std::max<size_t>(same_smem(std::max(nea, neb)), 16)));
   FS_CUDA(cudaFuncSetAttribute(k_op_mixed<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)mixed_smem));
   {
@@ -344,9 +422,7 @@ static void molecular_hamiltonian_t(Ctx* ctx, Space* sa, Space* sb, const void* 
       k_op_mixed<R><<<dim3((unsigned)nrow, ytiles(db, 128)), 128, mixed_smem, st>>>(
           Y, X, vec, db, i0, sa->gpq, sa->gsrc, nea, sb->gpq, neb, N, W, lcap);
       FS_CUDA(cudaGetLastError());
-      k_op_same<R, CT><<<dim3((unsigned)db, ytiles(nrow, 128 * CT)), 128, same_smem(neb), st>>>(
-          G, X, xt, nrow, 0, nrow, sb->gpq, sb->gsrc, neb, N, V, kmat);
-      FS_CUDA(cudaGetLastError());
+      same_products<R>(G, X, xt, nrow, 0, nrow, sb, N, V, kmat, st);
     }
     ProfScope ps("op_gather", st, neb > 0 ? 2 : 1);
     k_op_gather_cols<R><<<(unsigned)std::min<int64_t>((X + 255) / 256, 32 * sms), 256, 0, st>>>(
@@ -363,9 +439,7 @@ static void molecular_hamiltonian_t(Ctx* ctx, Space* sa, Space* sb, const void* 
     const int64_t ncol = std::min(nc, db - j0), X = da * ncol;
     {
       ProfScope ps("op_products", st);
-      k_op_same<R, CT><<<dim3((unsigned)da, ytiles(ncol, 128 * CT)), 128, same_smem(nea), st>>>(
-          buf, X, vec, db, j0, ncol, sa->gpq, sa->gsrc, nea, N, V, kmat);
-      FS_CUDA(cudaGetLastError());
+      same_products<R>(buf, X, vec, db, j0, ncol, sa, N, V, kmat, st);
     }
     {
       ProfScope ps("op_gather", st);
