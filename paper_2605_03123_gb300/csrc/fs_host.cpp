@@ -365,6 +365,30 @@ void window_tables_host(int N, int n, int W, std::vector<uint32_t>& orbits,
 
 namespace fs {
 
+void window_rows_host(int n, int W, const std::vector<uint32_t>& orbits,
+                      const std::vector<int>& off, const std::vector<uint16_t>& offs,
+                      std::vector<uint32_t>& chunk, std::vector<uint16_t>& rows) {
+  std::vector<std::vector<int>> masks(W + 1);
+  for (int x = 0; x < (1 << W); ++x) masks[__builtin_popcount(x)].push_back(x);
+  chunk.clear();
+  rows.clear();
+  for (size_t a = 0; a + 1 < off.size(); ++a)
+    for (int c = off[a]; c < off[a + 1]; c += 32) {
+      int m = 0;  // the chunk's class: that of its orbits, empty ones aside
+      for (int l = 0; l < 32 && !m; ++l) m = (int)(orbits[c + l] >> 24);
+      const size_t start = rows.size(), ns = masks[m].size(), nu = (ns + 7) / 8;
+      chunk.push_back((uint32_t)(start / 8) | ((uint32_t)m << 24));
+      rows.resize(start + nu * 32 * 8, (uint16_t)0xFFFF);
+      for (int l = 0; l < 32; ++l) {
+        const uint32_t d = orbits[c + l];
+        if (!(d >> 24)) continue;
+        const uint16_t* F = offs.data() + ((a * (n + 1) + ((d >> 16) & 0xFF)) << W);
+        for (size_t k = 0; k < ns; ++k)
+          rows[start + ((k / 8) * 32 + l) * 8 + k % 8] = (uint16_t)((d & 0xFFFF) + F[masks[m][k]]);
+      }
+    }
+}
+
 // Subsets of four orbitals covering every unordered orbital pair (greedy:
 // repeatedly the subset covering the most uncovered pairs), each pair and
 // each diagonal assigned to exactly one subset; and, per subset Q, the

@@ -70,6 +70,13 @@ std::vector<WinStep> schedule_windows(const RotProgram& rp, int N, int W);
 void window_tables_host(int N, int n, int W, std::vector<uint32_t>& orbits,
                         std::vector<int>& off, std::vector<uint16_t>& offs,
                         std::vector<uint8_t>& okey);
+// The gather addresses of those orbits, chunk by chunk of 32 (one class each):
+// string k of the orbit of lane l is the 16-bit half k % 2 of word k / 2 % 4 of
+// the 16-byte unit chunk[c] % 2^24 + 32 (k / 8) + l; rows of empty orbits and
+// the places past C(W, m) hold 0xFFFF.
+void window_rows_host(int n, int W, const std::vector<uint32_t>& orbits,
+                      const std::vector<int>& off, const std::vector<uint16_t>& offs,
+                      std::vector<uint32_t>& chunk, std::vector<uint16_t>& rows);
 // The orbits regrouped for clusters of 2^b CTAs: per window position a,
 // group r (occupation of the top b orbitals, the strings of cluster rank r)
 // at gorb[goff[a * 9 + r] .. goff[a * 9 + r + 1]), class order kept inside,
@@ -175,6 +182,11 @@ struct Space {
     TcSeg* tc_seg[2] = {};
     uint16_t* tc_idx[2] = {};
     int tc_seg_max[2] = {};  // largest segment, bytes
+    // gather addresses of the packed sweeps (W = 6): chunk c of 32 orbits of
+    // the padded list holds class m in pk_chunk[c] >> 24 and its rows from
+    // 16-byte unit pk_chunk[c] & 0xFFFFFF on
+    uint32_t* pk_chunk = nullptr;
+    uint4* pk_rows = nullptr;
     std::vector<uint32_t> orb_h;
     std::vector<int> off_h;
     std::vector<uint8_t> okey_h;
@@ -410,7 +422,7 @@ struct SweepGeom {
   int dir;      // 0: alpha, vectors are columns; 1: beta, vectors are rows
   int d;        // vector length (strings of the rotated spin)
   int nvec;     // number of vectors (strings of the other spin)
-  int lgKV;     // log2 of vectors per slab
+  int KV;       // vectors per slab
   int chunk;    // vector elements held by one CTA of the cluster (maximum)
   // cluster rank r holds elements [cb[r], cb[r + 1]) of each vector; with
   // `blocked`, rank r holds exactly the strings whose occupation of the top
@@ -453,6 +465,8 @@ struct SweepGeom {
   const int* tgoff;
   const uint16_t* offs;    // [npos][nocc + 1][1 << W] in-window rank offsets
   int offs_stride;         // (nocc + 1) << W
+  const uint32_t* pk_chunk;  // packed sweeps: see Space::Win
+  const uint4* pk_rows;
   // tensor-core window steps (W = 6): per step the B images of classes
   // m = 1..5 (tc::kStepBytes each step); gather-index segments per window
   // position (seg_full[a]) and, for blocked clusters, per position and rank

@@ -183,6 +183,17 @@ static void build_window_tables(Space* sp, int W) {
     FS_CUDA(cudaMemcpy(wt.orbits, orbits.data(), orbits.size() * 4, cudaMemcpyHostToDevice));
   FS_CUDA(cudaMemcpy(wt.off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice));
   FS_CUDA(cudaMemcpy(wt.offs, offs.data(), offs.size() * 2, cudaMemcpyHostToDevice));
+  if (W == window_width<float, 1>()) {  // packed sweeps
+    std::vector<uint32_t> chunk;
+    std::vector<uint16_t> rows;
+    window_rows_host(sp->nocc, W, orbits, off, offs, chunk, rows);
+    FS_CUDA(cudaMalloc(&wt.pk_chunk, std::max<size_t>(chunk.size(), 1) * 4));
+    FS_CUDA(cudaMalloc(&wt.pk_rows, std::max<size_t>(rows.size(), 8) * 2));
+    if (!chunk.empty()) {
+      FS_CUDA(cudaMemcpy(wt.pk_chunk, chunk.data(), chunk.size() * 4, cudaMemcpyHostToDevice));
+      FS_CUDA(cudaMemcpy(wt.pk_rows, rows.data(), rows.size() * 2, cudaMemcpyHostToDevice));
+    }
+  }
   wt.built = true;
 }
 
@@ -290,6 +301,8 @@ static void set_window_geom(SweepGeom& g, Space* sp, int W) {
     g.orb_grp = wt.gorb[g.lgcs];
     g.orb_goff = wt.goff[g.lgcs];
   }
+  g.pk_chunk = wt.pk_chunk;
+  g.pk_rows = wt.pk_rows;
   g.offs = wt.offs;
   g.offs_stride = (sp->nocc + 1) << W;
 }
@@ -408,7 +421,7 @@ static void dispatch_prog(Space* sthis, int CS, const SweepGeom& g0, const RotPr
       auto prog = make_wprog<R>(rp, sthis->norb, W);
       if constexpr (sizeof(R) == 4) {
         // slabs of an even number of vectors: packed vector pairs
-        if (CS == 1 && g.lgKV >= 1) {
+        if (CS == 1 && g.KV % 2 == 0) {
           if (two_per_sm)
             launch_sweep_t<R, 1, 1, false, W, 256, false, WProg<R>, false, true>(g, prog, X,
                                                                                nslabs, smem, st);
@@ -579,7 +592,7 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
       int want = std::max(1, gt.nvec / (2 * ctx->prop.multiProcessorCount));
       int lg = 0;
       while ((2 << lg) <= std::min(want, kMaxKV) && smem_tc(gt.chunk, 2 << lg) <= maxsm) ++lg;
-      gt.lgKV = lg;
+      gt.KV = 1 << lg;
       if (gt.blocked && gt.npass > 0) {
         build_tpass_groups(const_cast<Space*>(sthis), gt.lgcs);
         gt.trec_grp = sthis->tgrec[gt.lgcs];
@@ -617,7 +630,29 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
   int lg = 0;
   while ((2 << lg) <= std::min(want, kMaxKV) && smem_for(CS, 2 << lg) <= budget) ++lg;
   if (pair_slab && lg == 0) lg = 1;
-  g.lgKV = lg;
+  int KV = 1 << lg;
+  if (dtype == FS_C64 && CS == 1 && sthis->norb >= window_width<float, 1>() && sthis->dim > 1) {
+    // packed slabs take any width (pairs of vectors when forward): the one
+    // with the least modelled time.  A slab costs its vectors and a fixed part
+    // worth c0 of them; slabs run in waves of two per SM (forward slabs that
+    // fit half an SM) or one, and a last wave of at most one per SM runs 0.6
+    // as long.  N = 12 (6,6), 924 vectors: 4 forward (was 2), 7 reverse (2).
+    const int unit = nst == 1 ? 2 : 1, slots = (two_per_sm ? 2 : 1) * ctx->prop.multiProcessorCount;
+    const double c0 = 450.0 / g.d + 0.1;
+    double best = -1;
+    for (int kv = unit; kv <= kMaxKV && kv < g.nvec + unit; kv += unit) {
+      if (smem_for(1, kv) > budget) break;
+      const int slabs = (g.nvec + kv - 1) / kv, last = slabs % slots;
+      const double waves = slabs / slots + (last == 0 ? 0.0
+                                            : two_per_sm && last <= slots / 2 ? 0.6 : 1.0);
+      const double c = waves * (kv + c0);
+      if (best < 0 || c < best) {
+        best = c;
+        KV = kv;
+      }
+    }
+  }
+  g.KV = KV;
   set_cluster_layout(g, sthis, CS, [&](int chunk) {
     return (size_t)(chunk * csz * nst + tab_per_kv + fixed) + tsum <= maxsm;
   });
@@ -626,7 +661,6 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
     g.trec_grp = sthis->tgrec[g.lgcs];
     g.tgoff = sthis->tgoff[g.lgcs];
   }
-  const int KV = 1 << lg;
   const int nslabs = (g.nvec + KV - 1) / KV;
   const size_t smem = std::max<size_t>(
       (size_t)KV * ((size_t)g.chunk * csz * nst + tab_per_kv + fixed) + tsum, 16);
@@ -691,7 +725,7 @@ static int tune_batch_slab(Ctx* ctx, const SweepGeom& g0, const std::vector<unsi
   std::vector<float> ms(lgmax + 1, 0.f);
   int best = lgmin;
   for (int lg = lgmin; lg <= lgmax; ++lg) {
-    g.lgKV = lg;
+    g.KV = 1 << lg;
     SweepJob j{};
     j.g = g;
     j.prog = dprog;
@@ -799,7 +833,7 @@ void plan_batch_sweep(Ctx* ctx, Space* sa, Space* sb, int dir, void* st0, void* 
     while ((2 << lg) <= std::min(want, kMaxKV) && lg < lgmax) ++lg;
   }
   lg = std::max(lg, lgmin);
-  g.lgKV = lg;
+  g.KV = 1 << lg;
   out.nslabs = (g.nvec + (1 << lg) - 1) >> lg;
   out.smem = smem_for(1 << lg);
   out.pk = lgmin > 0;

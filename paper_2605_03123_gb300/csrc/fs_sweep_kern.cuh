@@ -557,17 +557,22 @@ __device__ __forceinline__ void win_pairs_pk(float2 (&vr)[NS], float2 (&vi)[NS],
                                   std::make_integer_sequence<int, win_npairs(W, M, U)>{});
 }
 // One orbit of a window step in a packed slab, packed set kc (cell stride
-// per string KC).
+// per string KC), its string addresses in the row q (two per word).  Reading
+// them as up to three 16-byte words per orbit replaces one 2-byte read of the
+// in-window offsets per string: with the 16-byte cell reads and writes those
+// kept the load/store units as busy as the multiply-adds keep theirs.
 template <int W, int M>
-__device__ __forceinline__ void win_orbit_pk(uint32_t desc, const uint16_t* F, float* smf, int KC,
-                                             int kc, const WProg<float>& prog, int ga, int gb) {
+__device__ __forceinline__ void win_orbit_pk(const uint4 (&q)[3], float* smf, int KC, int kc,
+                                             const WProg<float>& prog, int ga, int gb) {
   constexpr int NS = cbinom(W, M);
-  const int RO = desc & 0xFFFF, clo = (desc >> 16) & 0xFF;
-  const uint16_t* Fc = F + (clo << W);
+  if ((q[0].x & 0xFFFFu) == 0xFFFFu) return;  // an empty lane
   int ad[NS];
-  win_offsets<W, M>(Fc, ad, std::make_integer_sequence<int, NS>{});
 #pragma unroll
-  for (int k = 0; k < NS; ++k) ad[k] = (RO + ad[k]) * KC;
+  for (int k = 0; k < NS; ++k) {
+    const uint4& u = q[k / 8];
+    const uint32_t w = (k / 2) % 4 == 0 ? u.x : (k / 2) % 4 == 1 ? u.y : (k / 2) % 4 == 2 ? u.z : u.w;
+    ad[k] = (int)((w >> (16 * (k & 1))) & 0xFFFFu) * KC;
+  }
   {
     float2 vr[NS], vi[NS];
 #pragma unroll
@@ -858,7 +863,7 @@ __device__ __forceinline__ cx_t<R> ld_ea(const void* p, int64_t i) {
 // phase the first half of the CTA rotates state 0 and the second half state
 // 1, each half synchronising on its own named barrier.
 template <typename R, int CS, int NST, bool VJP, int W, int NT, bool SPLIT, typename P,
-          bool TC = false, bool PK = false>
+          bool TC = false, bool PK = false, bool AHEAD = true>
 __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, const Mat& X,
                                            const int slab, const int rank,
                                            unsigned char* smraw) {
@@ -869,7 +874,7 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
   constexpr int kThreads = NT;
   using C = cx_t<R>;
   C* sm = reinterpret_cast<C*>(smraw);
-  const int KV = 1 << g.lgKV;
+  const int KV = g.KV;
   const int v0 = slab * KV;
   const int kv_eff = min(KV, g.nvec - v0);
   // element ranges of the cluster ranks (registers; rank is runtime)
@@ -887,7 +892,7 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
   const int tid = threadIdx.x;
   const size_t st_stride = (size_t)g.chunk * KV;  // elements per state
   C* tab = sm + NST * st_stride;                  // cross tables, KV sets
-  double* w = reinterpret_cast<double*>(tab + (g.has_x ? ((size_t)g.nchunk * 256 << g.lgKV) : 0));
+  double* w = reinterpret_cast<double*>(tab + (g.has_x ? (size_t)g.nchunk * 256 * g.KV : 0));
 
   C* base[CS];
   if constexpr (CS > 1) {
@@ -935,8 +940,9 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
           cp_async_4(smf + r + 2, src + 1);
         }
       } else {
-        for (int idx = tid; idx < (nel << g.lgKV); idx += kThreads) {
-          const int el = idx >> g.lgKV, kv = idx & (KV - 1);
+        DivWalk dw(tid, kThreads, KV);
+        for (int idx = tid; idx < nel * KV; idx += kThreads, dw.next()) {
+          const int el = dw.a, kv = dw.b;
           if (kv >= kv_eff) continue;
           const size_t r = pk_re<NST>(s, el, KV, kv);
           const float* src = gf + 2 * ((int64_t)(e0 + el) * g.d_b + v0 + kv);
@@ -953,8 +959,9 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
         cp_async_elem(ss + (size_t)el * KV + kv, gs + (int64_t)(v0 + kv) * g.d_b + e0 + el);
       }
     } else {
-      for (int idx = tid; idx < (nel << g.lgKV); idx += kThreads) {
-        int el = idx >> g.lgKV, kv = idx & (KV - 1);
+      DivWalk dw(tid, kThreads, KV);
+      for (int idx = tid; idx < nel * KV; idx += kThreads, dw.next()) {
+        const int el = dw.a, kv = dw.b;
         if (kv < kv_eff)
           cp_async_elem(ss + (size_t)el * KV + kv, gs + (int64_t)(e0 + el) * g.d_b + v0 + kv);
       }
@@ -974,14 +981,14 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
     unsigned char* bsm = smraw + (((sb + 127u) & ~127u) - s0);
     tc_window_steps<CS, NST>(g, prog, base, cbr, KV, kv_eff, st_stride, rank, bsm);
   } else if constexpr (W == 0) {
-    const int items = g.npp << g.lgKV;
+    const int items = g.npp * KV;
     const int per = (items + CS - 1) / CS;
     const int lo = rank * per, hi = min(items, lo + per);
     for (int k = 0; k < prog.m; ++k) {
       const uint32_t* list = g.pairs + (int64_t)prog.p[k] * g.npp;
       const R c = prog.c[k], sr = prog.sr[k], si = prog.si[k];
       for (int it = lo + tid; it < hi; it += kThreads) {
-        int t = it >> g.lgKV, kv = it & (KV - 1);
+        const int t = it / KV, kv = it - t * KV;
         if (kv >= kv_eff) continue;
         uint32_t pr = __ldg(list + t);
         int src = pr & 0xFFFF, dst = pr >> 16;
@@ -1083,46 +1090,66 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
         const int KC = NST == 1 ? (KV >> 1) : KV;
         const int nk = NST == 1 ? (kv_eff + 1) >> 1 : kv_eff;
         const int nit = (hi - lo) * nk;
-        // the descriptor of the next round is loaded while this one runs
-        auto item_orbit = [&](int it) {
+        // AHEAD: the address rows of the next round are loaded while this
+        // one runs (not in the batched kernels, whose program is read through
+        // a pointer: they would spill)
+        const uint32_t* chunks = g.pk_chunk + (lo >> 5);
+        auto rows_of = [&](int it, uint32_t& m, uint4 (&q)[3]) {
           const int ch = it >> 5, oc = nk == 1 ? ch : ch / nk;
-          return lo + (oc << 5) + (it & 31);
+          const uint32_t c = __ldg(chunks + oc);
+          const uint4* r = g.pk_rows + (c & 0xFFFFFFu) + (it & 31);
+          m = c >> 24;
+          q[0] = __ldg(r);
+          if (m > 1 && m < 5) q[1] = __ldg(r + 32);
+          if (m == 3) q[2] = __ldg(r + 64);
         };
-        int it_next = dealt_round<kThreads>(0, nit, 0, 0, 1) ? dealt_item<kThreads>(0, nit, 0, tid, 0, 1) : -1;
-        uint32_t desc_next = it_next >= 0 ? __ldg(olist + item_orbit(it_next)) : 0u;
+        auto item_of = [&](int rd) {
+          return dealt_round<kThreads>(0, nit, rd, 0, 1)
+                     ? dealt_item<kThreads>(0, nit, rd, tid, 0, 1)
+                     : -1;
+        };
+        int it = item_of(0);
+        uint32_t m = 0;
+        uint4 q[3];
+        if (AHEAD && it >= 0) rows_of(it, m, q);
         for (int rd = 0; dealt_round<kThreads>(0, nit, rd, 0, 1); ++rd) {
-          const int it = it_next;
-          const uint32_t desc = desc_next;
-          it_next = dealt_round<kThreads>(0, nit, rd + 1, 0, 1)
-                        ? dealt_item<kThreads>(0, nit, rd + 1, tid, 0, 1)
-                        : -1;
-          if (it_next >= 0) desc_next = __ldg(olist + item_orbit(it_next));
-          if (it < 0) continue;
-          const int ch = it >> 5, oc = nk == 1 ? ch : ch / nk;
-          const int kc = ch - oc * nk;
-          switch (desc >> 24) {
-            case 1: win_orbit_pk<W, 1>(desc, F, smf, KC, kc, prog, ga, gb); break;
-            case 2: win_orbit_pk<W, 2>(desc, F, smf, KC, kc, prog, ga, gb); break;
-            case 3: win_orbit_pk<W, 3>(desc, F, smf, KC, kc, prog, ga, gb); break;
-            case 4: if constexpr (W > 4) win_orbit_pk<W, 4>(desc, F, smf, KC, kc, prog, ga, gb); break;
-            case 5: if constexpr (W > 5) win_orbit_pk<W, 5>(desc, F, smf, KC, kc, prog, ga, gb); break;
-            default: break;
+          const int it_next = item_of(rd + 1);
+          uint32_t m_next = 0;
+          uint4 q_next[3];
+          if (AHEAD && it_next >= 0) rows_of(it_next, m_next, q_next);
+          if (!AHEAD && it >= 0) rows_of(it, m, q);
+          if (it >= 0) {
+            const int ch = it >> 5, oc = nk == 1 ? ch : ch / nk;
+            const int kc = ch - oc * nk;
+            switch (m) {
+              case 1: win_orbit_pk<W, 1>(q, smf, KC, kc, prog, ga, gb); break;
+              case 2: win_orbit_pk<W, 2>(q, smf, KC, kc, prog, ga, gb); break;
+              case 3: win_orbit_pk<W, 3>(q, smf, KC, kc, prog, ga, gb); break;
+              case 4: if constexpr (W > 4) win_orbit_pk<W, 4>(q, smf, KC, kc, prog, ga, gb); break;
+              case 5: if constexpr (W > 5) win_orbit_pk<W, 5>(q, smf, KC, kc, prog, ga, gb); break;
+              default: break;
+            }
+          }
+          it = it_next;
+          if (AHEAD) {
+            m = m_next;
+#pragma unroll
+            for (int u = 0; u < 3; ++u) q[u] = q_next[u];
           }
         }
-        __syncthreads();
-        continue;
-      }
-      for (int rd = 0; dealt_round<kThreads>(lo, hi, rd, drank, dcs); ++rd) {
-        const int o = dealt_item<kThreads>(lo, hi, rd, tid, drank, dcs);
-        if (o < 0) continue;
-        const uint32_t desc = __ldg(olist + o);
-        switch (desc >> 24) {
-          case 1: win_orbit<R, CS, NST, W, 1>(desc, F, base, st_stride, cbr, KV, kv_eff, prog, ga, gb, pid); break;
-          case 2: win_orbit<R, CS, NST, W, 2>(desc, F, base, st_stride, cbr, KV, kv_eff, prog, ga, gb, pid); break;
-          case 3: win_orbit<R, CS, NST, W, 3>(desc, F, base, st_stride, cbr, KV, kv_eff, prog, ga, gb, pid); break;
-          case 4: if constexpr (W > 4) win_orbit<R, CS, NST, W, 4>(desc, F, base, st_stride, cbr, KV, kv_eff, prog, ga, gb, pid); break;
-          case 5: if constexpr (W > 5) win_orbit<R, CS, NST, W, 5>(desc, F, base, st_stride, cbr, KV, kv_eff, prog, ga, gb, pid); break;
-          default: break;
+      } else {
+        for (int rd = 0; dealt_round<kThreads>(lo, hi, rd, drank, dcs); ++rd) {
+          const int o = dealt_item<kThreads>(lo, hi, rd, tid, drank, dcs);
+          if (o < 0) continue;
+          const uint32_t desc = __ldg(olist + o);
+          switch (desc >> 24) {
+            case 1: win_orbit<R, CS, NST, W, 1>(desc, F, base, st_stride, cbr, KV, kv_eff, prog, ga, gb, pid); break;
+            case 2: win_orbit<R, CS, NST, W, 2>(desc, F, base, st_stride, cbr, KV, kv_eff, prog, ga, gb, pid); break;
+            case 3: win_orbit<R, CS, NST, W, 3>(desc, F, base, st_stride, cbr, KV, kv_eff, prog, ga, gb, pid); break;
+            case 4: if constexpr (W > 4) win_orbit<R, CS, NST, W, 4>(desc, F, base, st_stride, cbr, KV, kv_eff, prog, ga, gb, pid); break;
+            case 5: if constexpr (W > 5) win_orbit<R, CS, NST, W, 5>(desc, F, base, st_stride, cbr, KV, kv_eff, prog, ga, gb, pid); break;
+            default: break;
+          }
         }
       }
       if constexpr (CS > 1) cg::this_cluster().sync(); else __syncthreads();
@@ -1133,16 +1160,16 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
   if constexpr (!VJP) {
     // ---- epilogue: phases, store
     if (g.has_x) build_cross_tables<R>(g, X, v0, kv_eff, w, tab, tid, kThreads);
-    const int tot = g.dir == 1 ? kv_eff * nel : (nel << g.lgKV);
-    DivWalk dw(tid, kThreads, nel > 0 ? nel : 1);
+    const int tot = g.dir == 1 ? kv_eff * nel : nel * KV;
+    DivWalk dw(tid, kThreads, g.dir != 1 ? KV : nel > 0 ? nel : 1);
     for (int idx = tid; idx < tot; idx += kThreads, dw.next()) {
       int kv, el;
       if (g.dir == 1) {
         kv = dw.a;
         el = dw.b;
       } else {
-        el = idx >> g.lgKV;
-        kv = idx & (KV - 1);
+        el = dw.a;
+        kv = dw.b;
         if (kv >= kv_eff) continue;
       }
       const int o = v0 + kv, e = e0 + el;
@@ -1165,8 +1192,9 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
   } else {
     // ---- reverse-mode epilogue
     // (a) the diagonal layer of the (inverse) rotation, in shared memory
-    for (int idx = tid; idx < (nel << g.lgKV); idx += kThreads) {
-      int el = idx >> g.lgKV, kv = idx & (KV - 1);
+    DivWalk dk(tid, kThreads, KV);
+    for (int idx = tid; idx < nel * KV; idx += kThreads, dk.next()) {
+      const int el = dk.a, kv = dk.b;
       if (kv >= kv_eff) continue;
       C f = cmul<R>(ld_ea<R>(g.ea_other, v0 + kv), ld_ea<R>(g.ea_this, e0 + el));
 #pragma unroll
@@ -1178,7 +1206,7 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
     if (g.T && g.npass > 0) {
       // subset passes: per-thread partial sums of the 16 local slots, one
       // warp reduction per pass, per-CTA sums in shared memory
-      R* tsm = reinterpret_cast<R*>(w + (g.has_x ? (kMaxOrb << g.lgKV) : 0));
+      R* tsm = reinterpret_cast<R*>(w + (g.has_x ? kMaxOrb * g.KV : 0));
       for (int i = tid; i < g.npass * 32; i += kThreads) tsm[i] = 0;
       __syncthreads();
       const int lane = tid & 31;
@@ -1341,16 +1369,16 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
     // (c) W = Im(conj(g) psi) (invariant under the diagonal gate that
     //     follows), then the second phase, then store both states
     if (g.has_x) build_cross_tables<R>(g, X, v0, kv_eff, w, tab, tid, kThreads);
-    const int tot = g.dir == 1 ? kv_eff * nel : (nel << g.lgKV);
-    DivWalk dw(tid, kThreads, nel > 0 ? nel : 1);
+    const int tot = g.dir == 1 ? kv_eff * nel : nel * KV;
+    DivWalk dw(tid, kThreads, g.dir != 1 ? KV : nel > 0 ? nel : 1);
     for (int idx = tid; idx < tot; idx += kThreads, dw.next()) {
       int kv, el;
       if (g.dir == 1) {
         kv = dw.a;
         el = dw.b;
       } else {
-        el = idx >> g.lgKV;
-        kv = idx & (KV - 1);
+        el = dw.a;
+        kv = dw.b;
         if (kv >= kv_eff) continue;
       }
       const int o = v0 + kv, e = e0 + el;
@@ -1405,7 +1433,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
     const int it = s_item;
     if (it >= total) break;
     const SweepJob& J = jobs[s_job];
-    sweep_body<R, 1, NST, VJP, W, NT, SPLIT, WProg<R>, false, PK>(
+    sweep_body<R, 1, NST, VJP, W, NT, SPLIT, WProg<R>, false, PK, false>(
         J.g, *reinterpret_cast<const WProg<R>*>(J.prog),
                                              *J.X, it - J.item0, 0, smraw);
     __syncthreads();

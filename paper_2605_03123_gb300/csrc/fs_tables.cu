@@ -275,6 +275,12 @@ void free_space(Space* s) {
     cudaFree(w.orbits);
     cudaFree(w.off);
     cudaFree(w.offs);
+    cudaFree(w.pk_chunk);
+    cudaFree(w.pk_rows);
+    for (int b = 0; b < 2; ++b) {
+      cudaFree(w.tc_seg[b]);
+      cudaFree(w.tc_idx[b]);
+    }
     for (int b = 0; b < 4; ++b) {
       cudaFree(w.gorb[b]);
       cudaFree(w.goff[b]);
