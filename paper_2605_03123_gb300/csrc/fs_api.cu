@@ -78,28 +78,6 @@ static Mat real_mat(const double* p, int n, double scale) {
   return m;
 }
 
-static StrPhase phase_of(const RotProgram* rp, const double* J, double t, const double* lam,
-                         int n) {
-  StrPhase f;
-  f.t = t;
-  if (rp) {
-    f.use_d = 1;
-    for (int p = 0; p < n; ++p) {
-      f.d[2 * p] = rp->phase[p].real();
-      f.d[2 * p + 1] = rp->phase[p].imag();
-    }
-  }
-  if (J) {
-    f.use_j = 1;
-    for (int k = 0; k < n * n; ++k) f.J.v[k] = J[k];
-  }
-  if (lam) {
-    f.use_lam = 1;
-    for (int p = 0; p < n; ++p) f.lam[p] = lam[p];
-  }
-  return f;
-}
-
 // A diagonal-Coulomb evolution fused into the epilogue of a beta sweep:
 // same-spin matrix J (J_bb = J_aa), mixed matrix J_ab, time t.
 struct Fused {
@@ -120,29 +98,28 @@ static void rotate(Ctx* ctx, Space* sa, Space* sb, void* v0, void* v1, int nst, 
   void* ea_a = scratch(ctx, "ea_a", sa->dim * csz);
   void* ea_b = scratch(ctx, "ea_b", sb->dim * csz);
   void* ea_o = scratch(ctx, "ea_o", sa->dim * csz);
-  const bool fa = fx_supported(ctx, sa, sb, dtype, pa), fb = fx_supported(ctx, sb, sa, dtype, pb);
-  PhaseDev ph;
-  if (!fa) {
-    launch_string_phase(sa, ea_a, dtype, phase_of(&pa, nullptr, 0, nullptr, n), st);
+  const FxPair fx = fx_prepare(ctx, sa, sb, dtype, pa, pb, st);
+  StringPhases tables(n);
+  PhaseDev ph, phb;
+  if (!fx.a()) {
+    tables.add(sa, ea_a, &pa, nullptr, 0);
     ph.ea_a = ea_a;
   }
-  launch_sweep(ctx, sa, sb, 0, v0, v1, nst, dtype, pa, ph, st, nullptr, fa);
-  PhaseDev phb;
-  const RotProgram* db = fb ? nullptr : &pb;
   if (dc) {
-    launch_string_phase(sb, ea_b, dtype,
-                        phase_of(db, dc->J_bb ? dc->J_bb : dc->J_aa, dc->t, nullptr, n), st);
+    tables.add(sb, ea_b, fx.b() ? nullptr : &pb, dc->J_bb ? dc->J_bb : dc->J_aa, dc->t);
+    tables.add(sa, ea_o, nullptr, dc->J_aa, dc->t);
     phb.ea_b = ea_b;
-    launch_string_phase(sa, ea_o, dtype, phase_of(nullptr, dc->J_aa, dc->t, nullptr, n), st);
     phb.ea_a = ea_o;
     phb.has_x = 1;
     // mixed terms (p in I_a, q in I_b) and (p in I_b, q in I_a), J_ba = J_ab^T
     phb.X = real_mat(dc->J_ab, n, -dc->t);
-  } else if (!fb) {
-    launch_string_phase(sb, ea_b, dtype, phase_of(&pb, nullptr, 0, nullptr, n), st);
+  } else if (!fx.b()) {
+    tables.add(sb, ea_b, &pb, nullptr, 0);
     phb.ea_b = ea_b;
   }
-  launch_sweep(ctx, sa, sb, 1, v0, v1, nst, dtype, pb, phb, st, nullptr, fb);
+  tables.launch(dtype, st);
+  launch_sweep(ctx, sa, sb, 0, v0, v1, nst, dtype, pa, ph, st, nullptr, fx.a());
+  launch_sweep(ctx, sa, sb, 1, v0, v1, nst, dtype, pb, phb, st, nullptr, fx.b());
 }
 
 // The same rotation (and fused diagonal-Coulomb evolution) with every sweep a
@@ -162,53 +139,51 @@ static void rotate_alternating(Ctx* ctx, Space* sa, Space* sb, void* vec, void* 
   void* eo_a = scratch(ctx, "alt_eo_a", sa->dim * csz);
   void* eo_b = scratch(ctx, "alt_eo_b", sb->dim * csz);
   const double* Jbb = dc ? (dc->J_bb ? dc->J_bb : dc->J_aa) : nullptr;
-  const bool fa = fx_supported(ctx, sa, sb, dtype, pa), fb = fx_supported(ctx, sb, sa, dtype, pb);
-  const RotProgram *da = fa ? nullptr : &pa, *db = fb ? nullptr : &pb;
+  const FxPair fx = fx_prepare(ctx, sa, sb, dtype, pa, pb, st);
+  const RotProgram *da = fx.a() ? nullptr : &pa, *db = fx.b() ? nullptr : &pb;
+  StringPhases tables(n);
+  PhaseDev p1, p2;  // of the first and of the second sweep
   if (!trans) {
-    PhaseDev p1;
-    if (!fb) {
-      launch_string_phase(sb, ea_b, dtype, phase_of(&pb, nullptr, 0, nullptr, n), st);
+    if (db) {
+      tables.add(sb, ea_b, db, nullptr, 0);
       p1.ea_b = ea_b;
     }
-    launch_sweep(ctx, sa, sb, 1, vec, nullptr, 1, dtype, pb, p1, st, nullptr, fb);
-    launch_transpose(vec, tv, sa->dim, sb->dim, dtype, st);
     // alpha on rows of tv: spaces swapped, this spin (alpha) in the b slot
-    PhaseDev p2;
     if (dc) {
-      launch_string_phase(sa, ea_a, dtype, phase_of(da, dc->J_aa, dc->t, nullptr, n), st);
-      p2.ea_b = ea_a;
-      launch_string_phase(sb, eo_b, dtype, phase_of(nullptr, Jbb, dc->t, nullptr, n), st);
+      tables.add(sa, ea_a, da, dc->J_aa, dc->t);
+      tables.add(sb, eo_b, nullptr, Jbb, dc->t);
       p2.ea_a = eo_b;
       p2.has_x = 1;
       for (int p = 0; p < n; ++p)
         for (int q = 0; q < n; ++q) p2.X.v[q * n + p] = -dc->t * dc->J_ab[p * n + q];
-    } else if (!fa) {
-      launch_string_phase(sa, ea_a, dtype, phase_of(&pa, nullptr, 0, nullptr, n), st);
-      p2.ea_b = ea_a;
+    } else if (da) {
+      tables.add(sa, ea_a, da, nullptr, 0);
     }
-    launch_sweep(ctx, sb, sa, 1, tv, nullptr, 1, dtype, pa, p2, st, nullptr, fa);
+    if (dc || da) p2.ea_b = ea_a;
+    tables.launch(dtype, st);
+    launch_sweep(ctx, sa, sb, 1, vec, nullptr, 1, dtype, pb, p1, st, nullptr, fx.b());
+    launch_transpose(vec, tv, sa->dim, sb->dim, dtype, st);
+    launch_sweep(ctx, sb, sa, 1, tv, nullptr, 1, dtype, pa, p2, st, nullptr, fx.a());
     trans = true;
   } else {
-    PhaseDev p1;
-    if (!fa) {
-      launch_string_phase(sa, ea_a, dtype, phase_of(&pa, nullptr, 0, nullptr, n), st);
+    if (da) {
+      tables.add(sa, ea_a, da, nullptr, 0);
       p1.ea_b = ea_a;
     }
-    launch_sweep(ctx, sb, sa, 1, tv, nullptr, 1, dtype, pa, p1, st, nullptr, fa);
-    launch_transpose(tv, vec, sb->dim, sa->dim, dtype, st);
-    PhaseDev p2;
     if (dc) {
-      launch_string_phase(sb, ea_b, dtype, phase_of(db, Jbb, dc->t, nullptr, n), st);
-      p2.ea_b = ea_b;
-      launch_string_phase(sa, eo_a, dtype, phase_of(nullptr, dc->J_aa, dc->t, nullptr, n), st);
+      tables.add(sb, ea_b, db, Jbb, dc->t);
+      tables.add(sa, eo_a, nullptr, dc->J_aa, dc->t);
       p2.ea_a = eo_a;
       p2.has_x = 1;
       p2.X = real_mat(dc->J_ab, n, -dc->t);
-    } else if (!fb) {
-      launch_string_phase(sb, ea_b, dtype, phase_of(&pb, nullptr, 0, nullptr, n), st);
-      p2.ea_b = ea_b;
+    } else if (db) {
+      tables.add(sb, ea_b, db, nullptr, 0);
     }
-    launch_sweep(ctx, sa, sb, 1, vec, nullptr, 1, dtype, pb, p2, st, nullptr, fb);
+    if (dc || db) p2.ea_b = ea_b;
+    tables.launch(dtype, st);
+    launch_sweep(ctx, sb, sa, 1, tv, nullptr, 1, dtype, pa, p1, st, nullptr, fx.a());
+    launch_transpose(tv, vec, sb->dim, sa->dim, dtype, st);
+    launch_sweep(ctx, sa, sb, 1, vec, nullptr, 1, dtype, pb, p2, st, nullptr, fx.b());
     trans = false;
   }
 }
@@ -227,20 +202,23 @@ static bool alternate_layouts(Ctx* ctx, Space* sa, Space* sb, int dtype, int ext
 }
 
 // Standalone diagonal phase pass (number-operator sum and/or diagonal Coulomb).
-static void phase_pass(Ctx* ctx, Space* sa, Space* sb, void* vec, int dtype,
-                       const StrPhase& fa, const StrPhase& fb, const double* J_ab,
-                       double xscale, cudaStream_t st) {
+// (couplings J_aa, J_bb, J_ab or orbital energies lam_a, lam_b, at time t).
+static void phase_pass(Ctx* ctx, Space* sa, Space* sb, void* vec, int dtype, const double* J_aa,
+                       const double* J_bb, const double* J_ab, const double* lam_a,
+                       const double* lam_b, double t, cudaStream_t st) {
   const size_t csz = dtype == FS_C64 ? 8 : 16;
   void* ea_a = scratch(ctx, "ea_a", sa->dim * csz);
   void* ea_b = scratch(ctx, "ea_b", sb->dim * csz);
-  launch_string_phase(sa, ea_a, dtype, fa, st);
-  launch_string_phase(sb, ea_b, dtype, fb, st);
+  StringPhases tables(sa->norb);
+  tables.add(sa, ea_a, nullptr, J_aa, t, lam_a);
+  tables.add(sb, ea_b, nullptr, J_bb, t, lam_b);
+  tables.launch(dtype, st);
   PhaseDev ph;
   ph.ea_a = ea_a;
   ph.ea_b = ea_b;
   if (J_ab) {
     ph.has_x = 1;
-    ph.X = real_mat(J_ab, sa->norb, xscale);
+    ph.X = real_mat(J_ab, sa->norb, -t);
   }
   if (ph.has_x && phase_tc_supported(dtype, sa, sb, vec))
     launch_phase_tc(ctx, sa, sb, vec, ph, st);
@@ -357,8 +335,9 @@ static void run_gates(Ctx* ctx, Space* sa, Space* sb, void* vec, int dtype,
   bool pending = false;
   auto flush = [&](const GateOp* dc) {
     if (pending) {
-      RotProgram pa = decompose_adjacent(n, Pa.data());
-      RotProgram pb = decompose_adjacent(n, Pb.data());
+      const bool same = Pa == Pb;  // one program for both spins
+      const RotProgram pa = decompose_adjacent(n, Pa.data());
+      const RotProgram pb = same ? RotProgram{} : decompose_adjacent(n, Pb.data());
       Fused f;
       if (dc) {
         f.J_aa = dc->J_aa;
@@ -366,11 +345,10 @@ static void run_gates(Ctx* ctx, Space* sa, Space* sb, void* vec, int dtype,
         f.J_bb = dc->J_bb;
         f.t = dc->t;
       }
-      rotate(ctx, sa, sb, vec, nullptr, 1, dtype, pa, pb, dc ? &f : nullptr, st);
+      rotate(ctx, sa, sb, vec, nullptr, 1, dtype, pa, same ? pa : pb, dc ? &f : nullptr, st);
     } else if (dc) {
-      phase_pass(ctx, sa, sb, vec, dtype, phase_of(nullptr, dc->J_aa, dc->t, nullptr, n),
-                 phase_of(nullptr, dc->J_bb ? dc->J_bb : dc->J_aa, dc->t, nullptr, n), dc->J_ab,
-                 -dc->t, st);
+      phase_pass(ctx, sa, sb, vec, dtype, dc->J_aa, dc->J_bb ? dc->J_bb : dc->J_aa, dc->J_ab,
+                 nullptr, nullptr, dc->t, st);
     }
     Pa = I;
     Pb = I;
@@ -663,9 +641,9 @@ int fs_apply_orbital_rotation(fs_ctx* ctx, void* vec, int dtype, const double* U
     cudaStream_t st = (cudaStream_t)stream;
     Space* sa = get_space(ctx, norb, na, st);
     Space* sb = get_space(ctx, norb, nb, st);
-    RotProgram pa = decompose_adjacent(norb, Ua.data());
-    RotProgram pb = U_b ? decompose_adjacent(norb, Ub.data()) : pa;
-    rotate_any(ctx, sa, sb, vec, dtype, Ua, Ub, pa, pb, st);
+    const RotProgram pa = decompose_adjacent(norb, Ua.data());
+    const RotProgram pb = U_b ? decompose_adjacent(norb, Ub.data()) : RotProgram{};
+    rotate_any(ctx, sa, sb, vec, dtype, Ua, Ub, pa, U_b ? pb : pa, st);
   });
 }
 
@@ -682,8 +660,8 @@ int fs_apply_num_op_sum_evolution(fs_ctx* ctx, void* vec, int dtype, const doubl
     cudaStream_t st = (cudaStream_t)stream;
     Space* sa = get_space(ctx, norb, na, st);
     Space* sb = get_space(ctx, norb, nb, st);
-    phase_pass(ctx, sa, sb, vec, dtype, phase_of(nullptr, nullptr, t, lam_a, norb),
-               phase_of(nullptr, nullptr, t, lam_b ? lam_b : lam_a, norb), nullptr, 0, st);
+    phase_pass(ctx, sa, sb, vec, dtype, nullptr, nullptr, nullptr, lam_a,
+               lam_b ? lam_b : lam_a, t, st);
   });
 }
 
@@ -701,8 +679,7 @@ int fs_apply_diag_coulomb_evolution(fs_ctx* ctx, void* vec, int dtype, const dou
     Space* sa = get_space(ctx, norb, na, st);
     Space* sb = get_space(ctx, norb, nb, st);
     // theta = -(t/2)[sum_{I_a} J_aa + sum_{I_b} J_bb + 2 sum_{p in I_a, q in I_b} J_ab]
-    phase_pass(ctx, sa, sb, vec, dtype, phase_of(nullptr, J_aa, t, nullptr, norb),
-               phase_of(nullptr, J_bb ? J_bb : J_aa, t, nullptr, norb), J_ab, -t, st);
+    phase_pass(ctx, sa, sb, vec, dtype, J_aa, J_bb ? J_bb : J_aa, J_ab, nullptr, nullptr, t, st);
   });
 }
 
@@ -735,8 +712,8 @@ int fs_lucj_forward(fs_ctx* ctx, const fs_lucj* op, void* vec, int dtype, void* 
         Rm.v[2 * q + 1] = Rs[0][q].imag();
       }
       launch_slater(ctx, sa, sb, vec, dtype, Rm, st);
-      phase_pass(ctx, sa, sb, vec, dtype, phase_of(nullptr, op->J_aa, 1.0, nullptr, n),
-                 phase_of(nullptr, op->J_aa, 1.0, nullptr, n), op->J_ab, -1.0, st);
+      phase_pass(ctx, sa, sb, vec, dtype, op->J_aa, op->J_aa, op->J_ab, nullptr, nullptr, 1.0,
+                 st);
       k0 = 1;
     }
     static const char* const kFwdT[] = {"vjp_tpsi"};
@@ -789,8 +766,8 @@ int fs_apply_num_interaction(fs_ctx* ctx, void* vec, int dtype, double theta, in
     cudaStream_t st = (cudaStream_t)stream;
     Space* sa = get_space(ctx, norb, na, st);
     Space* sb = get_space(ctx, norb, nb, st);
-    phase_pass(ctx, sa, sb, vec, dtype, phase_of(nullptr, nullptr, -theta, la.data(), norb),
-               phase_of(nullptr, nullptr, -theta, lb.data(), norb), nullptr, 0, st);
+    phase_pass(ctx, sa, sb, vec, dtype, nullptr, nullptr, nullptr, la.data(), lb.data(), -theta,
+               st);
   });
 }
 
@@ -826,9 +803,8 @@ int fs_apply_num_num_interaction(fs_ctx* ctx, void* vec, int dtype, double theta
     cudaStream_t st = (cudaStream_t)stream;
     Space* sa = get_space(ctx, norb, na, st);
     Space* sb = get_space(ctx, norb, nb, st);
-    phase_pass(ctx, sa, sb, vec, dtype, phase_of(nullptr, Jaa.data(), -theta, nullptr, norb),
-               phase_of(nullptr, Jbb.data(), -theta, nullptr, norb),
-               sigma == tau ? nullptr : Jab.data(), theta, st);
+    phase_pass(ctx, sa, sb, vec, dtype, Jaa.data(), Jbb.data(),
+               sigma == tau ? nullptr : Jab.data(), nullptr, nullptr, -theta, st);
   });
 }
 
@@ -907,9 +883,9 @@ int fs_apply_quad_ham_evolution(fs_ctx* ctx, void* vec, int dtype, const double*
     cudaStream_t st = (cudaStream_t)stream;
     Space* sa = get_space(ctx, norb, na, st);
     Space* sb = get_space(ctx, norb, nb, st);
-    RotProgram pa = decompose_adjacent(norb, Ua.data());
-    RotProgram pb = M_b ? decompose_adjacent(norb, Ub.data()) : pa;
-    rotate_any(ctx, sa, sb, vec, dtype, Ua, Ub, pa, pb, st);
+    const RotProgram pa = decompose_adjacent(norb, Ua.data());
+    const RotProgram pb = M_b ? decompose_adjacent(norb, Ub.data()) : RotProgram{};
+    rotate_any(ctx, sa, sb, vec, dtype, Ua, Ub, pa, M_b ? pb : pa, st);
   });
 }
 
@@ -1190,14 +1166,16 @@ static void lucj_vjp_impl(Ctx* ctx, const fs_lucj* op, void* vec, void* cot, int
     double* Tm = Tacc + (size_t)m * nn * 2;
     const double* Ja = m >= 1 ? op->J_aa + (size_t)(m - 1) * nn : nullptr;
     const double* Jab = m >= 1 ? op->J_ab + (size_t)(m - 1) * nn : nullptr;
+    const FxPair fx = fx_prepare(ctx, sa, sb, dtype, inv, inv, st);
+    const FxPlan *fa = fx.a(), *fb = fx.b();
+    StringPhases tables(n);
     if (m >= 1) {
-      launch_string_phase(sa, e2_a, dtype, phase_of(nullptr, Ja, -1.0, nullptr, n), st);
-      launch_string_phase(sb, e2_b, dtype, phase_of(nullptr, Ja, -1.0, nullptr, n), st);
+      tables.add(sa, e2_a, nullptr, Ja, -1.0);
+      tables.add(sb, e2_b, nullptr, Ja, -1.0);
     }
-    const bool fa = fx_supported(ctx, sa, sb, dtype, inv);
-    const bool fb = fx_supported(ctx, sb, sa, dtype, inv);
-    if (!fb) launch_string_phase(sb, ea_b, dtype, phase_of(&inv, nullptr, 0, nullptr, n), st);
-    if (!fa) launch_string_phase(sa, ea_a, dtype, phase_of(&inv, nullptr, 0, nullptr, n), st);
+    if (!fb) tables.add(sb, ea_b, &inv, nullptr, 0);
+    if (!fa) tables.add(sa, ea_a, &inv, nullptr, 0);
+    tables.launch(dtype, st);
     if (alpha_t && trans) {
       // alpha: undo on rows of the copies, T^alpha
       PhaseDev q1;

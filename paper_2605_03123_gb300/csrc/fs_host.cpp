@@ -10,24 +10,58 @@
 
 namespace fs {
 
-void mat_mul(int n, const zd* A, const zd* B, zd* C) {
-  // real arithmetic on the parts (std::complex products carry inf/nan
-  // recovery calls that make these small products several times slower)
-  std::vector<double> t((size_t)2 * n * n, 0.0);
-  const double* a = reinterpret_cast<const double*>(A);
-  const double* b = reinterpret_cast<const double*>(B);
-  for (int i = 0; i < n; ++i)
+// Small complex matrices with real and imaginary parts apart: their products
+// are four multiply-adds per element on contiguous rows, which the compiler
+// vectorises (std::complex products carry inf/nan recovery calls that make
+// them several times slower).
+namespace {
+struct Split {
+  int n;
+  std::vector<double> r, i;
+  explicit Split(int n_) : n(n_), r((size_t)n_ * n_, 0.0), i((size_t)n_ * n_, 0.0) {}
+  Split(int n_, const zd* A, double scale) : Split(n_) {
+    for (size_t k = 0; k < r.size(); ++k) {
+      r[k] = A[k].real() * scale;
+      i[k] = A[k].imag() * scale;
+    }
+  }
+  void store(zd* out) const {
+    for (size_t k = 0; k < r.size(); ++k) out[k] = zd(r[k], i[k]);
+  }
+};
+// C += A B
+void mul_add(const Split& A, const Split& B, Split& C) {
+  const int n = A.n;
+  for (int p = 0; p < n; ++p) {
+    double* cr = C.r.data() + (size_t)p * n;
+    double* ci = C.i.data() + (size_t)p * n;
     for (int k = 0; k < n; ++k) {
-      const double ar = a[2 * (i * n + k)], ai = a[2 * (i * n + k) + 1];
+      const double ar = A.r[(size_t)p * n + k], ai = A.i[(size_t)p * n + k];
       if (ar == 0.0 && ai == 0.0) continue;
-      double* ti = t.data() + (size_t)2 * i * n;
-      const double* bk = b + (size_t)2 * k * n;
+      const double* br = B.r.data() + (size_t)k * n;
+      const double* bi = B.i.data() + (size_t)k * n;
       for (int j = 0; j < n; ++j) {
-        ti[2 * j] += ar * bk[2 * j] - ai * bk[2 * j + 1];
-        ti[2 * j + 1] += ar * bk[2 * j + 1] + ai * bk[2 * j];
+        cr[j] += ar * br[j] - ai * bi[j];
+        ci[j] += ar * bi[j] + ai * br[j];
       }
     }
-  std::copy(t.begin(), t.end(), reinterpret_cast<double*>(C));
+  }
+}
+Split product(const Split& A, const Split& B) {
+  Split C(A.n);
+  mul_add(A, B, C);
+  return C;
+}
+void axpy(Split& C, double a, const Split& B) {
+  for (size_t k = 0; k < C.r.size(); ++k) {
+    C.r[k] += a * B.r[k];
+    C.i[k] += a * B.i[k];
+  }
+}
+}  // namespace
+
+void mat_mul(int n, const zd* A, const zd* B, zd* C) {
+  product(Split(n, A, 1.0), Split(n, B, 1.0)).store(C);
 }
 
 void mat_adjoint(int n, const zd* A, zd* out) {
@@ -47,60 +81,100 @@ static double norm1(int n, const zd* A) {
   return m;
 }
 
-// Scaling and squaring with a Taylor series: A / 2^s has 1-norm <= 1/2, and
-// the series is summed until a term no longer changes the sum in FP64.
+// Scaling and squaring with the Taylor polynomial of degree 18: A / 2^s has
+// 1-norm <= 1/2, where its remainder is below 2^-75.  The polynomial takes
+// seven products (powers 2, 3, 4 and four steps of Horner's rule in the
+// fourth power) instead of seventeen.
+static int taylor_scale(double nrm) {
+  return nrm > 0.5 ? (int)std::ceil(std::log2(nrm / 0.5)) : 0;
+}
+static const double* taylor_coef() {
+  static const std::array<double, 20> c = [] {
+    std::array<double, 20> t;
+    t[0] = 1.0;
+    for (int k = 1; k < 20; ++k) t[k] = t[k - 1] / k;
+    return t;
+  }();
+  return c.data();
+}
+constexpr int kTaylor = 18;
+
 void expm(int n, const zd* A, zd* out) {
-  const size_t nn = (size_t)n * n;
-  double nrm = norm1(n, A);
-  int s = 0;
-  if (nrm > 0.5) s = (int)std::ceil(std::log2(nrm / 0.5));
-  double scale = std::ldexp(1.0, -s);
-  std::vector<zd> B(nn), term(nn), sum(nn, zd(0)), tmp(nn);
-  for (size_t k = 0; k < nn; ++k) B[k] = A[k] * scale;
-  for (int i = 0; i < n; ++i) {
-    sum[i * n + i] = 1.0;
-    term[i * n + i] = 1.0;
+  const int s = taylor_scale(norm1(n, A));
+  const double* c = taylor_coef();
+  const Split B(n, A, std::ldexp(1.0, -s)), B2 = product(B, B), B3 = product(B2, B),
+              B4 = product(B2, B2);
+  auto block = [&](int k) {  // c_k + c_{k+1} B + c_{k+2} B^2 + c_{k+3} B^3
+    Split P(n);
+    for (int p = 0; p < n; ++p) P.r[(size_t)p * n + p] = c[k];
+    if (k + 1 <= kTaylor) axpy(P, c[k + 1], B);
+    if (k + 2 <= kTaylor) axpy(P, c[k + 2], B2);
+    if (k + 3 <= kTaylor) axpy(P, c[k + 3], B3);
+    return P;
+  };
+  Split E = block(16);
+  for (int k = 12; k >= 0; k -= 4) {
+    Split P = block(k);
+    mul_add(E, B4, P);
+    E = std::move(P);
   }
-  for (int k = 1; k <= 40; ++k) {
-    mat_mul(n, term.data(), B.data(), tmp.data());
-    double tn = 0;
-    for (size_t q = 0; q < nn; ++q) {
-      term[q] = tmp[q] / (double)k;
-      sum[q] += term[q];
-      tn = std::max(tn, std::abs(term[q]));
-    }
-    if (tn < 1e-18) break;
-  }
-  for (int k = 0; k < s; ++k) mat_mul(n, sum.data(), sum.data(), sum.data());
-  std::copy(sum.begin(), sum.end(), out);
+  for (int k = 0; k < s; ++k) E = product(E, E);
+  E.store(out);
 }
 
 // For the real inner product <A, B> = Re tr(A^dag B), the adjoint of the
-// Frechet derivative of expm at K is the Frechet derivative at K^dag; the
-// latter is the upper-right block of expm([[K^dag, H], [0, K^dag]]).
+// Frechet derivative of expm at K is the Frechet derivative at K^dag, the
+// upper-right block of expm([[K^dag, H], [0, K^dag]]).  The same polynomial
+// on such block matrices, of which only the diagonal block X and the
+// upper-right block L are held: (X, L) (Y, M) = (X Y, X M + L Y).
 void expm_frechet_adjoint(int n, const zd* K, const zd* H, zd* out) {
-  const int m = 2 * n;
-  std::vector<zd> B((size_t)m * m, zd(0)), E((size_t)m * m);
-  for (int i = 0; i < n; ++i)
-    for (int j = 0; j < n; ++j) {
-      zd kd = std::conj(K[j * n + i]);
-      B[i * m + j] = kd;
-      B[(n + i) * m + n + j] = kd;
-      B[i * m + n + j] = H[i * n + j];
+  struct Pair {
+    Split X, L;
+  };
+  auto mul = [](const Pair& a, const Pair& b) {
+    Pair p{product(a.X, b.X), product(a.X, b.L)};
+    mul_add(a.L, b.X, p.L);
+    return p;
+  };
+  std::vector<zd> Kd((size_t)n * n);
+  mat_adjoint(n, K, Kd.data());
+  const int s = taylor_scale(norm1(n, Kd.data()));
+  const double sc = std::ldexp(1.0, -s);
+  const double* c = taylor_coef();
+  const Pair B{Split(n, Kd.data(), sc), Split(n, H, sc)};
+  const Pair B2 = mul(B, B), B3 = mul(B2, B), B4 = mul(B2, B2);
+  auto block = [&](int k) {
+    Pair P{Split(n), Split(n)};
+    for (int p = 0; p < n; ++p) P.X.r[(size_t)p * n + p] = c[k];
+    const Pair* b[3] = {&B, &B2, &B3};
+    for (int j = 1; j <= 3 && k + j <= kTaylor; ++j) {
+      axpy(P.X, c[k + j], b[j - 1]->X);
+      axpy(P.L, c[k + j], b[j - 1]->L);
     }
-  expm(m, B.data(), E.data());
-  for (int i = 0; i < n; ++i)
-    for (int j = 0; j < n; ++j) out[i * n + j] = E[i * m + n + j];
+    return P;
+  };
+  Pair E = block(16);
+  for (int k = 12; k >= 0; k -= 4) {
+    Pair P = block(k);
+    mul_add(E.X, B4.X, P.X);
+    mul_add(E.X, B4.L, P.L);
+    mul_add(E.L, B4.X, P.L);
+    E = std::move(P);
+  }
+  for (int k = 0; k < s; ++k) E = mul(E, E);
+  E.L.store(out);
 }
 
 double unitarity_error(int n, const zd* U) {
+  std::vector<zd> ad((size_t)n * n);
+  mat_adjoint(n, U, ad.data());
+  const Split P = product(Split(n, ad.data(), 1.0), Split(n, U, 1.0));
   double e = 0;
   for (int i = 0; i < n; ++i)
     for (int j = 0; j < n; ++j) {
-      zd s = 0;
-      for (int k = 0; k < n; ++k) s += std::conj(U[k * n + i]) * U[k * n + j];
-      if (i == j) s -= 1.0;
-      e = std::max(e, std::abs(s));
+      const double d = std::hypot(P.r[(size_t)i * n + j] - (i == j ? 1.0 : 0.0),
+                                  P.i[(size_t)i * n + j]);
+      e = std::max(e, d);
     }
   return e;
 }
@@ -129,11 +203,16 @@ RotProgram decompose_adjacent(int n, const zd* U) {
         c = std::abs(b) / rho;
         s = -std::conj(a) * b / (std::abs(b) * rho);
       }
-      // A <- A G^dag on columns (j, j+1): G^dag = [[c, -s], [s*, c]]
-      for (int i = 0; i < n; ++i) {
-        zd x = A[i * n + j], y = A[i * n + j + 1];
-        A[i * n + j] = c * x + std::conj(s) * y;
-        A[i * n + j + 1] = -s * x + c * y;
+      // A <- A G^dag on columns (j, j+1): G^dag = [[c, -s], [s*, c]], in real
+      // arithmetic (see Split)
+      const double sr = s.real(), si = s.imag();
+      double* col = reinterpret_cast<double*>(A.data() + j);
+      for (int i = 0; i < n; ++i, col += 2 * n) {
+        const double xr = col[0], xi = col[1], yr = col[2], yi = col[3];
+        col[0] = c * xr + (sr * yr + si * yi);
+        col[1] = c * xi + (sr * yi - si * yr);
+        col[2] = c * yr - (sr * xr - si * xi);
+        col[3] = c * yi - (sr * xi + si * xr);
       }
       A[r * n + j] = 0.0;
       prog.g.push_back(Givens{j, c, s});
@@ -180,6 +259,18 @@ std::vector<WinStep> schedule_windows(const RotProgram& rp, int N, int W) {
     steps.push_back(best);
   }
   return steps;
+}
+
+const std::vector<WinStep>& window_schedule(Ctx* ctx, const RotProgram& rp, int N, int W) {
+  Ctx::Schedule& s = ctx->schedules[{N, W}];
+  bool same = s.p.size() == rp.g.size() && !s.steps.empty();
+  for (size_t k = 0; same && k < s.p.size(); ++k) same = s.p[k] == rp.g[k].p;
+  if (!same) {
+    s.p.clear();
+    s.steps = schedule_windows(rp, N, W);
+    for (const Givens& g : rp.g) s.p.push_back(g.p);
+  }
+  return s.steps;
 }
 
 // Top-3 group of a configuration: the occupation of orbitals N-1, N-2, N-3

@@ -59,6 +59,11 @@ struct WinStep {
   std::vector<int> givens;
 };
 std::vector<WinStep> schedule_windows(const RotProgram& rp, int N, int W);
+struct Ctx;
+// The same through the context, which keeps the last schedule per (N, W): the
+// programs of dense rotations differ in their coefficients only (the sequence
+// of orbital pairs is compared).
+const std::vector<WinStep>& window_schedule(Ctx* ctx, const RotProgram& rp, int N, int W);
 // Orbit tables of the strings of n electrons in N orbitals for windows of W
 // adjacent orbitals: for each window position a, orbits[off[a] .. off[a+1])
 // hold R_O | c_lo << 16 | m << 24 grouped by m (classes in descending order
@@ -246,6 +251,11 @@ struct Ctx {
   std::map<std::pair<int, int>, Space*> spaces;
   std::map<std::string, Scratch> scratch;
   int* d_status = nullptr;  // device status word
+  struct Schedule {
+    std::vector<int> p;  // first orbitals of the rotations, in program order
+    std::vector<WinStep> steps;
+  };
+  std::map<std::pair<int, int>, Schedule> schedules;  // see window_schedule
   // small results the host needs right away (transition sums, coupling
   // gradients) land in a mapped pinned buffer, written by a kernel: a copy
   // through a copy engine would wait behind the caller's own large copies
@@ -327,13 +337,6 @@ struct Mat {
 struct CMat {
   double v[2 * kMaxOrb * kMaxOrb];
 };
-struct StrPhase {  // per-string factor recipe, see launch_string_phase
-  int use_d = 0, use_j = 0, use_lam = 0;
-  double t = 0;
-  double d[2 * kMaxOrb];
-  double lam[kMaxOrb];
-  Mat J;
-};
 
 // Phase of one configuration, factored as
 //   f(i, j) = ea_a[i] * ea_b[j] * exp(i sum_{p in I_a, q in I_b} X[p][q])
@@ -346,10 +349,40 @@ struct PhaseDev {
   Mat X;
 };
 
-// Per-string factors: out[e] = prod_{p in I} d_p * exp(i(-(t/2) sum_{p,q in I} J[p][q]
-//                                                    - t sum_{p in I} lam[p])).
-void launch_string_phase(const Space* sp, void* out, int dtype, const StrPhase& f,
-                         cudaStream_t st);
+// Per-string factor tables of one or two gates, filled by one launch:
+//   out[e] = prod_{p in I} d_p * exp(i(-(t/2) sum_{p,q in I} J[p][q]
+//                                      - t sum_{p in I} lam[p])).
+// Every angle is held as a 64-bit fraction of a turn (sums are exact modulo
+// 2 pi); entries that are not finite are listed apart and make the factor of
+// every string that holds them not a number.
+struct StrJobs {  // kernel parameter
+  struct Job {
+    const uint32_t* masks;
+    void* out;
+    int64_t dim;
+    int lin, quad;  // indices below, -1: none
+  } job[4];
+  int njobs, norb;
+  int64_t lin[2][kMaxOrb];
+  int64_t quad[2][kMaxOrb * kMaxOrb];
+  uint32_t bad_lin[2], bad_quad[2][kMaxOrb];
+};
+class StringPhases {
+ public:
+  explicit StringPhases(int norb);
+  // rp: its diagonal layer (d); J, lam: host, norb x norb and norb; all may be
+  // null
+  void add(const Space* sp, void* out, const RotProgram* rp, const double* J, double t,
+           const double* lam = nullptr);
+  void launch(int dtype, cudaStream_t st);
+
+ private:
+  StrJobs p_;
+  const void* lin_key_[2] = {};
+  const void* quad_key_[2] = {};
+  double lin_t_[2] = {}, quad_t_[2] = {};
+  int nlin_ = 0, nquad_ = 0;
+};
 
 // Window program: step s applies Givens g0[s] .. g0[s+1]-1, all acting on
 // orbitals inside the window [a[s], a[s] + W); u = p - a[s] is the local
@@ -514,6 +547,24 @@ struct RevArgs {
   void* W = nullptr;    // [d_a][d_b] real Im(conj(g) psi), or null
 };
 
+// A program prepared for the complex128 fixed-point sweep (fs_sweep_fx.cu):
+// window steps, and their images on the device.  launch_sweep with such a plan
+// applies the program's diagonal layer too, so `ph` must not hold it.
+struct FxPlan {
+  int nsteps = 0;
+  uint8_t a[fx::kMaxSteps], full[fx::kMaxSteps];
+  const unsigned char* img = nullptr;
+};
+// The plans of a rotation's two spins (null: the spin takes the FP64 or FP32
+// sweep), with one launch for the images of both.  They live in the context's
+// scratch until the next call.
+struct FxPair {
+  FxPlan plan[2];
+  int use[2] = {-1, -1};  // plan of each spin, -1: none
+  const FxPlan* a() const { return use[0] < 0 ? nullptr : &plan[use[0]]; }
+  const FxPlan* b() const { return use[1] < 0 ? nullptr : &plan[use[1]]; }
+};
+
 // Givens sweep over one spin: dir 0 rotates alpha (columns of the state),
 // dir 1 rotates beta (rows).  With nst == 1 the epilogue multiplies by the
 // phase `ph` (strings of both spins, cross matrix ph.X).  With nst == 2
@@ -523,15 +574,12 @@ struct RevArgs {
 void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir,
                   void* st0, void* st1, int nst, int dtype,
                   const RotProgram& prog, const PhaseDev& ph, cudaStream_t st,
-                  const RevArgs* rev = nullptr, bool fx = false);
-// Whether the complex128 fixed-point sweep (fs_sweep_fx.cu) takes a program:
-// launch_sweep with fx = true then applies the program's diagonal layer too,
-// so `ph` must not hold it.
-bool fx_supported(const Ctx* ctx, const Space* sthis, const Space* sother, int dtype,
-                  const RotProgram& rp);
+                  const RevArgs* rev = nullptr, const FxPlan* fx = nullptr);
+FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const RotProgram& pa,
+                  const RotProgram& pb, cudaStream_t st);
 // That sweep, on st0 and (unless null) st1, with the phase `ph` behind it.
 void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0, void* st1,
-                     const RotProgram& rp, const PhaseDev& ph, cudaStream_t st);
+                     const FxPlan& plan, const PhaseDev& ph, cudaStream_t st);
 
 // The reductions behind a reverse fixed-point sweep (fs_trans_fx.cu): T += the
 // transition sums of this spin (its pass tables are built), if supported.
@@ -624,7 +672,7 @@ void split_planes(const void* X, int64_t rows, int cols, int64_t ldx, void* cons
                   int64_t ldk, cudaStream_t st);
 
 // Force the module loads of the kernels the allocation-free entry point
-// launches (k_masks; k_string_phase and k_phase in both precisions), so
+// launches (k_masks; the string and state phases in both precisions), so
 // that none of them loads lazily on a later call.
 void preload_mask_kernel();
 void preload_phase_kernels();

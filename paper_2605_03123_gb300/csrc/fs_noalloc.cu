@@ -107,15 +107,10 @@ extern "C" int fs_apply_diag_coulomb_evolution_noalloc(void* vec, int dtype, con
     launch_masks(sa.masks, norb, n_alpha, st);
     launch_masks(sb.masks, norb, n_beta, st);
     // theta = -(t/2)[sum_{I_a} J_aa + sum_{I_b} J_bb + 2 sum_{p in I_a, q in I_b} J_ab]
-    StrPhase pa, pb;
-    pa.use_j = pb.use_j = 1;
-    pa.t = pb.t = t;
-    for (int k = 0; k < norb * norb; ++k) {
-      pa.J.v[k] = J_aa[k];
-      pb.J.v[k] = (J_bb ? J_bb : J_aa)[k];
-    }
-    launch_string_phase(&sa, fa, dtype, pa, st);
-    launch_string_phase(&sb, fb, dtype, pb, st);
+    StringPhases sp(norb);
+    sp.add(&sa, fa, nullptr, J_aa, t);
+    sp.add(&sb, fb, nullptr, J_bb ? J_bb : J_aa, t);
+    sp.launch(dtype, st);
     PhaseDev ph;
     ph.ea_a = fa;
     ph.ea_b = fb;

@@ -257,9 +257,9 @@ static int match_pattern(int W, const std::vector<int>& u) {
 }
 
 template <typename R>
-static WProg<R> make_wprog(const RotProgram& rp, int N, int W) {
+static WProg<R> make_wprog(Ctx* ctx, const RotProgram& rp, int N, int W) {
   WProg<R> w;
-  std::vector<WinStep> steps = schedule_windows(rp, N, W);
+  const std::vector<WinStep>& steps = window_schedule(ctx, rp, N, W);
   int ng = 0;
   for (size_t st = 0; st < steps.size(); ++st) {
     w.a[st] = (int8_t)steps[st].a;
@@ -391,8 +391,8 @@ static void dispatch_tc(Ctx* ctx, Space* sthis, int CS, const SweepGeom& g0, con
     g.tc_seg_grp = wt.tc_seg[1];
     g.tc_idx_grp = wt.tc_idx[1];
   }
-  const WProg<double> wpd = make_wprog<double>(rp, sthis->norb, tc::kW);
-  const WProg<float> wpf = make_wprog<float>(rp, sthis->norb, tc::kW);
+  const WProg<double> wpd = make_wprog<double>(ctx, rp, sthis->norb, tc::kW);
+  const WProg<float> wpf = make_wprog<float>(ctx, rp, sthis->norb, tc::kW);
   unsigned char* img = (unsigned char*)scratch(
       ctx, "tc_steps", (size_t)std::max(1, wpd.nsteps) * tc::kStepBytes);
   if (wpd.nsteps > 0) {
@@ -410,7 +410,7 @@ static void dispatch_tc(Ctx* ctx, Space* sthis, int CS, const SweepGeom& g0, con
 }
 
 template <typename R, int NST, bool VJP>
-static void dispatch_prog(Space* sthis, int CS, const SweepGeom& g0, const RotProgram& rp,
+static void dispatch_prog(Ctx* ctx, Space* sthis, int CS, const SweepGeom& g0, const RotProgram& rp,
                           const Mat& X, int nslabs, size_t smem, bool two_per_sm,
                           cudaStream_t st) {
   if constexpr (NST == 1) {
@@ -418,7 +418,7 @@ static void dispatch_prog(Space* sthis, int CS, const SweepGeom& g0, const RotPr
     if (sthis->norb >= W && sthis->dim > 1) {
       SweepGeom g = g0;
       set_window_geom(g, sthis, W);
-      auto prog = make_wprog<R>(rp, sthis->norb, W);
+      auto prog = make_wprog<R>(ctx, rp, sthis->norb, W);
       if constexpr (sizeof(R) == 4) {
         // slabs of an even number of vectors: packed vector pairs
         if (CS == 1 && g.KV % 2 == 0) {
@@ -443,7 +443,7 @@ static void dispatch_prog(Space* sthis, int CS, const SweepGeom& g0, const RotPr
     if (CS == 1 && sthis->norb >= WS && sthis->dim > 1) {
       SweepGeom g = g0;
       set_window_geom(g, sthis, WS);
-      auto prog = make_wprog<R>(rp, sthis->norb, WS);
+      auto prog = make_wprog<R>(ctx, rp, sthis->norb, WS);
       if constexpr (sizeof(R) == 4)
         // complex64: psi and g of an orbit in one thread, packed per string
         // (W = 6; shared addresses and coefficients, two-lane updates)
@@ -456,7 +456,7 @@ static void dispatch_prog(Space* sthis, int CS, const SweepGeom& g0, const RotPr
     if (sthis->norb >= WJ && sthis->dim > 1) {
       SweepGeom g = g0;
       set_window_geom(g, sthis, WJ);
-      auto prog = make_wprog<R>(rp, sthis->norb, WJ);
+      auto prog = make_wprog<R>(ctx, rp, sthis->norb, WJ);
       dispatch_cs<R, NST, VJP, WJ, 512>(CS, g, prog, X, nslabs, smem, st);
       return;
     }
@@ -499,15 +499,15 @@ static void set_cluster_layout(SweepGeom& g, const Space* sp, int CS, Fits&& fit
 
 void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0,
                   void* st1, int nst, int dtype, const RotProgram& rp,
-                  const PhaseDev& ph, cudaStream_t st, const RevArgs* rev, bool fx) {
+                  const PhaseDev& ph, cudaStream_t st, const RevArgs* rev, const FxPlan* fx) {
   if (fx) {
     if (nst == 1) {
-      launch_sweep_fx(ctx, sa, sb, dir, st0, nullptr, rp, ph, st);
+      launch_sweep_fx(ctx, sa, sb, dir, st0, nullptr, *fx, ph, st);
       return;
     }
     // reverse: both states rotated, the transition sums, then W and the second
     // phase (as a sweep without rotations where the sums do not fit one CTA)
-    launch_sweep_fx(ctx, sa, sb, dir, st0, st1, rp, PhaseDev{}, st);
+    launch_sweep_fx(ctx, sa, sb, dir, st0, st1, *fx, PhaseDev{}, st);
     Space* sthis = const_cast<Space*>(dir == 0 ? sa : sb);
     if (sthis->norb >= 4 && sthis->nocc >= 1) build_tpass_tables(sthis);
     if (rev->T && trans_fx_supported(ctx, sthis)) {
@@ -518,7 +518,7 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
     }
     RotProgram none;
     none.phase.assign(sa->norb, zd(1.0));
-    launch_sweep(ctx, sa, sb, dir, st0, st1, nst, dtype, none, ph, st, rev, false);
+    launch_sweep(ctx, sa, sb, dir, st0, st1, nst, dtype, none, ph, st, rev);
     return;
   }
   FS_REQUIRE((nst == 2) == (rev != nullptr), FS_ERR_ARG, "reverse mode needs two states");
@@ -666,11 +666,11 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
       (size_t)KV * ((size_t)g.chunk * csz * nst + tab_per_kv + fixed) + tsum, 16);
   Space* sw = const_cast<Space*>(sthis);
   if (dtype == FS_C64) {
-    if (nst == 1) dispatch_prog<float, 1, false>(sw, CS, g, rp, ph.X, nslabs, smem, two_per_sm, st);
-    else dispatch_prog<float, 2, true>(sw, CS, g, rp, ph.X, nslabs, smem, false, st);
+    if (nst == 1) dispatch_prog<float, 1, false>(ctx, sw, CS, g, rp, ph.X, nslabs, smem, two_per_sm, st);
+    else dispatch_prog<float, 2, true>(ctx, sw, CS, g, rp, ph.X, nslabs, smem, false, st);
   } else {
-    if (nst == 1) dispatch_prog<double, 1, false>(sw, CS, g, rp, ph.X, nslabs, smem, two_per_sm, st);
-    else dispatch_prog<double, 2, true>(sw, CS, g, rp, ph.X, nslabs, smem, false, st);
+    if (nst == 1) dispatch_prog<double, 1, false>(ctx, sw, CS, g, rp, ph.X, nslabs, smem, two_per_sm, st);
+    else dispatch_prog<double, 2, true>(ctx, sw, CS, g, rp, ph.X, nslabs, smem, false, st);
   }
 }
 
@@ -804,10 +804,10 @@ void plan_batch_sweep(Ctx* ctx, Space* sa, Space* sb, int dir, void* st0, void* 
   g.cb[1] = g.d;
   out.prog.resize(wprog_bytes(dtype));
   if (dtype == FS_C64) {
-    auto w = make_wprog<float>(rp, sthis->norb, W);
+    auto w = make_wprog<float>(ctx, rp, sthis->norb, W);
     memcpy(out.prog.data(), &w, sizeof(w));
   } else {
-    auto w = make_wprog<double>(rp, sthis->norb, W);
+    auto w = make_wprog<double>(ctx, rp, sthis->norb, W);
     memcpy(out.prog.data(), &w, sizeof(w));
   }
   // slab width: the widest that fits the budget (at most 64 vectors), or the
@@ -992,52 +992,114 @@ void launch_rev_phase(const Space* sa, const Space* sb, void* psi, void* cot, in
   FS_CUDA(cudaGetLastError());
 }
 
-// Per-string factors (FP64 arithmetic, stored in the state precision).
+// Per-string factors, one launch for up to four tables: the angle as a sum of
+// 64-bit fractions of a turn (integers, exact modulo 2 pi), one FP64 sincos
+// per string, stored in the state precision.  The products and sums of FP64
+// angles it replaces were a chain of some hundred FP64 instructions, 8 us a
+// table at N = 12.
 template <typename R>
-__global__ void k_string_phase(cx_t<R>* out, const uint32_t* masks, int64_t dim,
-                               int norb, const __grid_constant__ StrPhase f) {
-  int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (e >= dim) return;
-  uint32_t m = masks[e];
-  double re = 1, im = 0, ang = 0;
-  for (int p = 0; p < norb; ++p) {
-    if (!((m >> p) & 1u)) continue;
-    if (f.use_d) {
-      double dr = f.d[2 * p], di = f.d[2 * p + 1];
-      double nr = re * dr - im * di;
-      im = re * di + im * dr;
-      re = nr;
+__global__ void __launch_bounds__(128) k_string_phases(const __grid_constant__ StrJobs f) {
+  __shared__ int64_t quad[kMaxOrb * kMaxOrb];
+  const StrJobs::Job& J = f.job[blockIdx.y];
+  const int N = f.norb;
+  if (blockIdx.x * 128ll >= J.dim) return;
+  if (J.quad >= 0)
+    for (int k = threadIdx.x; k < N * N; k += 128) quad[k] = f.quad[J.quad][k];
+  __syncthreads();
+  const int64_t e = blockIdx.x * 128ll + threadIdx.x;
+  if (e >= J.dim) return;
+  const uint32_t m = J.masks[e];
+  int64_t turn = 0;
+  bool bad = J.lin >= 0 && (m & f.bad_lin[J.lin]);
+  for (uint32_t b = m; b; b &= b - 1) {
+    const int p = __ffs(b) - 1;
+    if (J.lin >= 0) turn += f.lin[J.lin][p];
+    if (J.quad >= 0) {
+      bad = bad || (m & f.bad_quad[J.quad][p]);
+      for (uint32_t c = m; c; c &= c - 1) turn += quad[p * N + __ffs(c) - 1];
     }
-    if (f.use_lam) ang -= f.t * f.lam[p];
-    if (f.use_j)
-      for (int q = 0; q < norb; ++q)
-        if ((m >> q) & 1u) ang -= 0.5 * f.t * f.J.v[p * norb + q];
   }
-  double r = ang - 6.283185307179586 * rint(ang * 0.15915494309189535);
   double s, c;
-  sincos(r, &s, &c);
-  out[e] = mk<R>((R)(re * c - im * s), (R)(re * s + im * c));
+  sincos((double)turn * 3.4061215800865545e-19, &s, &c);  // 2 pi / 2^64
+  if (bad) s = c = __longlong_as_double(0x7FF8000000000000ll);
+  reinterpret_cast<cx_t<R>*>(J.out)[e] = mk<R>((R)c, (R)s);
+}
+
+// x radians as a 64-bit fraction of a turn (modulo one turn).
+static int64_t turns(double x) {
+  constexpr double hi = 0x1.45f306dc9c883p-3, lo = -0x1.6b01ec5417056p-57;  // 1 / (2 pi)
+  const double r = x * hi;
+  double f = (r - std::rint(r)) + (std::fma(x, hi, -r) + x * lo);
+  f -= std::rint(f);
+  return (int64_t)((uint64_t)std::llrint(std::ldexp(f, 63)) << 1);
+}
+
+StringPhases::StringPhases(int norb) {
+  p_.njobs = 0;
+  p_.norb = norb;
+}
+
+void StringPhases::add(const Space* sp, void* out, const RotProgram* rp, const double* J, double t,
+                       const double* lam) {
+  const int n = p_.norb;
+  FS_REQUIRE(p_.njobs < 4, FS_ERR_ARG, "too many string tables");
+  StrJobs::Job& j = p_.job[p_.njobs++];
+  j = StrJobs::Job{sp->masks, out, sp->dim, -1, -1};
+  if (rp || lam) {
+    const void* key = rp ? (const void*)rp : (const void*)lam;
+    int k = 0;
+    while (k < nlin_ && !(lin_key_[k] == key && lin_t_[k] == t)) ++k;
+    if (k == nlin_) {
+      FS_REQUIRE(nlin_ < 2 && !(rp && lam), FS_ERR_ARG, "too many orbital phases");
+      lin_key_[nlin_] = key;
+      lin_t_[nlin_++] = t;
+      p_.bad_lin[k] = 0;
+      for (int q = 0; q < n; ++q) {
+        const double x = rp ? std::arg(rp->phase[q]) : -t * lam[q];
+        if (!std::isfinite(x)) p_.bad_lin[k] |= 1u << q;
+        p_.lin[k][q] = std::isfinite(x) ? turns(x) : 0;
+      }
+    }
+    j.lin = k;
+  }
+  if (J) {
+    int k = 0;
+    while (k < nquad_ && !(quad_key_[k] == J && quad_t_[k] == t)) ++k;
+    if (k == nquad_) {
+      FS_REQUIRE(nquad_ < 2, FS_ERR_ARG, "too many coupling matrices");
+      quad_key_[nquad_] = J;
+      quad_t_[nquad_++] = t;
+      for (int q = 0; q < n; ++q) p_.bad_quad[k][q] = 0;
+      for (int q = 0; q < n * n; ++q) {
+        const double x = -0.5 * t * J[q];
+        if (!std::isfinite(x)) p_.bad_quad[k][q / n] |= 1u << (q % n);
+        p_.quad[k][q] = std::isfinite(x) ? turns(x) : 0;
+      }
+    }
+    j.quad = k;
+  }
+}
+
+void StringPhases::launch(int dtype, cudaStream_t st) {
+  if (p_.njobs == 0) return;
+  ProfScope ps("string_phase", st);
+  int64_t d = 0;
+  for (int k = 0; k < p_.njobs; ++k) d = std::max(d, p_.job[k].dim);
+  const dim3 grid((unsigned)((d + 127) / 128), (unsigned)p_.njobs);
+  if (dtype == FS_C64)
+    k_string_phases<float><<<grid, 128, 0, st>>>(p_);
+  else
+    k_string_phases<double><<<grid, 128, 0, st>>>(p_);
+  FS_CUDA(cudaGetLastError());
+  p_.njobs = nlin_ = nquad_ = 0;
 }
 
 void preload_phase_kernels() {
   cudaFuncAttributes fa;
-  FS_CUDA(cudaFuncGetAttributes(&fa, k_string_phase<float>));
-  FS_CUDA(cudaFuncGetAttributes(&fa, k_string_phase<double>));
+  FS_CUDA(cudaFuncGetAttributes(&fa, k_string_phases<float>));
+  FS_CUDA(cudaFuncGetAttributes(&fa, k_string_phases<double>));
   FS_CUDA(cudaFuncGetAttributes(&fa, k_phase));
   FS_CUDA(cudaFuncGetAttributes(&fa, k_phase_fx));
-}
-
-void launch_string_phase(const Space* sp, void* out, int dtype, const StrPhase& f,
-                         cudaStream_t st) {
-  ProfScope ps("string_phase", st);
-  unsigned grid = (unsigned)((sp->dim + 127) / 128);
-  if (dtype == FS_C64)
-    k_string_phase<float><<<grid, 128, 0, st>>>((float2*)out, sp->masks, sp->dim,
-                                                 sp->norb, f);
-  else
-    k_string_phase<double><<<grid, 128, 0, st>>>((double2*)out, sp->masks, sp->dim,
-                                                  sp->norb, f);
-  FS_CUDA(cudaGetLastError());
 }
 
 // ----------------------------------------------- Hartree-Fock closed form

@@ -721,25 +721,29 @@ static void hunit(int64_t* x, int n) {
   for (int i = 0; i < n; ++i) x[i] += hmul(x[i], h);
 }
 
-// The steps of a program with their unitaries V (row-major 6 x 6 complex,
-// fixed point; products of FP64 matrices would put an error of some 2^-52
-// into each entry, the same for every amplitude), the diagonal layer
-// multiplied into the last step that covers each orbital.  False when a
-// phase falls outside every window or the program has too many steps.
-static bool fx_steps(const RotProgram& rp, int N, std::vector<WinStep>& steps,
-                     std::vector<std::array<int64_t, 72>>* V, uint8_t* full) {
-  steps = schedule_windows(rp, N, tc::kW);
-  if (steps.empty() || (int)steps.size() > fx::kMaxSteps) return false;
+// The steps of a program (into plan and, as unitaries V, row-major 6 x 6
+// complex fixed point, into V: products of FP64 matrices would put an error
+// of some 2^-52 into each entry, the same for every amplitude), the diagonal
+// layer multiplied into the last step that covers each orbital.  False when
+// the program does not suit the sweep: a phase falls outside every window, or
+// it has too many steps, or too few rotations a step.
+static bool fx_steps(Ctx* ctx, const RotProgram& rp, int N, FxPlan& plan,
+                     std::vector<std::array<int64_t, 72>>& V) {
+  const std::vector<WinStep>& steps = window_schedule(ctx, rp, N, tc::kW);
+  if (steps.empty() || (int)steps.size() > fx::kMaxSteps ||
+      rp.g.size() < fx::kMinGivensPerStep * steps.size())
+    return false;
   std::vector<int> last(N, -1);
   for (size_t s = 0; s < steps.size(); ++s)
     for (int p = steps[s].a; p < steps[s].a + tc::kW; ++p) last[p] = (int)s;
   for (int p = 0; p < N; ++p)
     if (last[p] < 0 && rp.phase[p] != zd(1.0)) return false;
-  if (!V) return true;
-  V->resize(steps.size());
+  plan.nsteps = (int)steps.size();
+  V.resize(steps.size());
   for (size_t s = 0; s < steps.size(); ++s) {
     const int a = steps[s].a;
-    auto& M = (*V)[s];
+    plan.a[s] = (uint8_t)a;
+    auto& M = V[s];
     M.fill(0);
     for (int i = 0; i < 6; ++i) M[14 * i] = (int64_t)1 << 62;
     for (int k : steps[s].givens) {
@@ -755,7 +759,7 @@ static bool fx_steps(const RotProgram& rp, int N, std::vector<WinStep>& steps,
         x[13 + 2 * j] = hmul(g[0], vi) - hmul(g[1], ui) + hmul(g[2], ur);
       }
     }
-    full[s] = 0;
+    plan.full[s] = 0;
     for (int p = a; p < a + tc::kW; ++p) {
       if (last[p] != (int)s || rp.phase[p] == zd(1.0)) continue;
       int64_t z[2] = {hfix(rp.phase[p].real()), hfix(rp.phase[p].imag())};
@@ -766,39 +770,78 @@ static bool fx_steps(const RotProgram& rp, int N, std::vector<WinStep>& steps,
         x[2 * j + 1] = hmul(x[2 * j], z[1]) + hmul(x[2 * j + 1], z[0]);
         x[2 * j] = re;
       }
-      full[s] = 1;
+      plan.full[s] = 1;
     }
   }
   return true;
 }
 
-bool fx_supported(const Ctx* ctx, const Space* sthis, const Space* sother, int dtype,
-                  const RotProgram& rp) {
-  if (dtype != FS_C128 || ctx->sweep_engine == FS_SWEEP_CUDA_CORE || ctx->prop.major < 10)
+// Sectors the sweep takes: a window of orbitals, a vector and its step's
+// images in one SM's shared memory, and enough amplitudes.
+static bool fx_sector(const Ctx* ctx, const Space* sthis, const Space* sother) {
+  if (sthis->norb < tc::kW || sthis->dim < 2 || sthis->dim * sother->dim < fx::kMinAmps)
     return false;
-  if (sthis->norb < tc::kW || sthis->dim < 2) return false;
   int caps[2];
   fx::caps(sthis->norb, sthis->nocc, caps);
   const size_t tab = (size_t)((sthis->norb + 7) / 8) * 256 * 16;
-  if (fx::kImgBytes + (size_t)caps[0] + caps[1] + (size_t)sthis->dim * 16 + tab >
-      (size_t)ctx->prop.sharedMemPerBlockOptin - fx::kStaticBytes)
-    return false;
-  if (sthis->dim * sother->dim < fx::kMinAmps) return false;
-  std::vector<WinStep> steps;
-  return fx_steps(rp, sthis->norb, steps, nullptr, nullptr) &&
-         rp.g.size() >= fx::kMinGivensPerStep * steps.size();
+  return fx::kImgBytes + (size_t)caps[0] + caps[1] + (size_t)sthis->dim * 16 + tab <=
+         (size_t)ctx->prop.sharedMemPerBlockOptin - fx::kStaticBytes;
+}
+
+FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const RotProgram& pa,
+                  const RotProgram& pb, cudaStream_t st) {
+  FxPair r;
+  if (dtype != FS_C128 || ctx->sweep_engine == FS_SWEEP_CUDA_CORE || ctx->prop.major < 10)
+    return r;
+  const bool sect[2] = {fx_sector(ctx, sa, sb), fx_sector(ctx, sb, sa)};
+  const RotProgram* rp[2] = {&pa, &pb};
+  const bool shared = &pa == &pb;  // one program for both spins
+  bool ok[2] = {false, false};
+  std::vector<std::array<int64_t, 72>> V[2];
+  for (int s = 0; s < 2; ++s) {
+    if (shared ? s == 0 && (sect[0] || sect[1]) : sect[s])
+      ok[s] = fx_steps(ctx, *rp[s], sa->norb, r.plan[s], V[s]);
+  }
+  const int n0 = ok[0] ? r.plan[0].nsteps : 0, n1 = ok[1] ? r.plan[1].nsteps : 0;
+  if (n0 + n1 == 0) return r;
+  unsigned char* img =
+      (unsigned char*)scratch(ctx, "fx_images", (size_t)(n0 + n1) * fx::kStepBytes);
+  r.plan[0].img = img;
+  r.plan[1].img = img + (size_t)n0 * fx::kStepBytes;
+  {
+    ProfScope ps("fx_images", st, n0 + n1 > fx::kMaxSteps ? 2 : 1);
+    fx::StepMats sm;
+    int k = 0, at = 0;
+    auto flush = [&]() {
+      if (k == 0) return;
+      fx::k_fx_images<<<dim3(k, 2), 512, 0, st>>>(sm, img + (size_t)at * fx::kStepBytes);
+      FS_CUDA(cudaGetLastError());
+      at += k;
+      k = 0;
+    };
+    for (int s = 0; s < 2; ++s) {
+      if (!ok[s]) continue;
+      if (k + r.plan[s].nsteps > fx::kMaxSteps) flush();
+      for (int q = 0; q < r.plan[s].nsteps; ++q, ++k) std::copy(V[s][q].begin(), V[s][q].end(), sm.v[k]);
+    }
+    flush();
+  }
+  if (shared) {
+    for (int s = 0; s < 2; ++s)
+      if (ok[0] && sect[s]) r.use[s] = 0;
+  } else {
+    for (int s = 0; s < 2; ++s)
+      if (ok[s]) r.use[s] = s;
+  }
+  return r;
 }
 
 void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0, void* st1,
-                     const RotProgram& rp, const PhaseDev& ph, cudaStream_t st) {
+                     const FxPlan& plan, const PhaseDev& ph, cudaStream_t st) {
   const Space* sthis = dir == 0 ? sa : sb;
   const Space* sother = dir == 0 ? sb : sa;
-  std::vector<WinStep> steps;
-  std::vector<std::array<int64_t, 72>> V;
-  fx::Args g{};
-  FS_REQUIRE(fx_steps(rp, sthis->norb, steps, &V, g.full), FS_ERR_ARG,
-             "program has no window steps");
   fx::build_index(const_cast<Space*>(sthis));
+  fx::Args g{};
   g.st[0] = (double2*)st0;
   g.st[1] = (double2*)st1;
   const int nst = st1 ? 2 : 1;
@@ -806,7 +849,10 @@ void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* 
   g.dir = dir;
   g.d = (int)sthis->dim;
   g.nvec = (int)sother->dim;
-  g.nsteps = (int)steps.size();
+  g.nsteps = plan.nsteps;
+  std::copy(plan.a, plan.a + plan.nsteps, g.a);
+  std::copy(plan.full, plan.full + plan.nsteps, g.full);
+  g.img = plan.img;
   g.norb = sthis->norb;
   g.nchunk = (sthis->norb + 7) / 8;
   g.has_x = ph.has_x;
@@ -817,11 +863,6 @@ void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* 
   g.ea_this = (const double2*)(dir == 0 ? ph.ea_a : ph.ea_b);
   g.ea_other = (const double2*)(dir == 0 ? ph.ea_b : ph.ea_a);
   g.status = ctx->d_status;
-  fx::StepMats sm;
-  for (int s = 0; s < g.nsteps; ++s) {
-    g.a[s] = (uint8_t)steps[s].a;
-    std::copy(V[s].begin(), V[s].end(), sm.v[s]);
-  }
   // vectors per slab: the width with the least modelled time, a wave of
   // slabs costing its tiles (class 3 the most) and its amplitudes
   const size_t tab = ph.has_x ? (size_t)g.nchunk * 256 * 16 : 0;
@@ -849,14 +890,6 @@ void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* 
       best = c;
       g.KV = kv;
     }
-  }
-  unsigned char* img =
-      (unsigned char*)scratch(ctx, "fx_images", (size_t)g.nsteps * fx::kStepBytes);
-  g.img = img;
-  {
-    ProfScope ps("fx_images", st);
-    fx::k_fx_images<<<dim3(g.nsteps, 2), 512, 0, st>>>(sm, img);
-    FS_CUDA(cudaGetLastError());
   }
   // more than half an SM's shared memory: the CTA owns all TMEM of its SM
   const size_t smem = std::max(fixed + (size_t)g.KV * ((size_t)g.d * 16 + tab),
