@@ -110,9 +110,11 @@ int fs_set_rotation_path(fs_ctx *ctx, int path);
  *                       fixed-point digits (62 fraction bits relative to
  *                       each vector's 2-norm, so at least as accurate as
  *                       FP64 arithmetic) where the sector and the program
- *                       allow it, else in FP64 on the CUDA cores.  There, a
- *                       vector that holds a non-finite amplitude comes out
- *                       not a number throughout;
+ *                       allow it, else in FP64 on the CUDA cores, as the
+ *                       rotations of small spaces (up to a few hundred
+ *                       strings), where that is faster.  In digits a vector
+ *                       that holds a non-finite amplitude comes out not a
+ *                       number throughout;
  *   FS_SWEEP_CUDA_CORE: every Givens rotation as FP32 / FP64 FMAs on CUDA
  *                       cores;
  *   FS_SWEEP_TENSOR:    complex64 too: each window step of 6 adjacent
@@ -123,7 +125,7 @@ int fs_set_rotation_path(fs_ctx *ctx, int path);
  *                       accuracy); falls back to the CUDA cores where the
  *                       tensor path does not apply (fewer than 6 orbitals,
  *                       vectors spanning more than 2 CTAs).  complex128 as
- *                       under FS_SWEEP_AUTO.
+ *                       under FS_SWEEP_AUTO, small spaces too.
  * Results agree to the rounding of the dtype.  FS_ERR_ARG for another
  * value. */
 enum { FS_SWEEP_AUTO = 0, FS_SWEEP_CUDA_CORE = 1, FS_SWEEP_TENSOR = 2 };

@@ -98,10 +98,14 @@ static void rotate(Ctx* ctx, Space* sa, Space* sb, void* v0, void* v1, int nst, 
   void* ea_a = scratch(ctx, "ea_a", sa->dim * csz);
   void* ea_b = scratch(ctx, "ea_b", sb->dim * csz);
   void* ea_o = scratch(ctx, "ea_o", sa->dim * csz);
-  const FxPair fx = fx_prepare(ctx, sa, sb, dtype, pa, pb, st);
+  const FxPair fx = fx_prepare(ctx, sa, sb, dtype, pa, pb, true, st);
+  // small spaces: a sweep of its own, which takes the diagonal layer itself
+  // where no other table of that spin is built
+  const bool qa = nst == 1 && !fx.a() && pairs_supported(ctx, sa, sb, dtype, pa);
+  const bool qb = nst == 1 && !fx.b() && pairs_supported(ctx, sb, sa, dtype, pb);
   StringPhases tables(n);
   PhaseDev ph, phb;
-  if (!fx.a()) {
+  if (!fx.a() && !qa) {
     tables.add(sa, ea_a, &pa, nullptr, 0);
     ph.ea_a = ea_a;
   }
@@ -113,13 +117,19 @@ static void rotate(Ctx* ctx, Space* sa, Space* sb, void* v0, void* v1, int nst, 
     phb.has_x = 1;
     // mixed terms (p in I_a, q in I_b) and (p in I_b, q in I_a), J_ba = J_ab^T
     phb.X = real_mat(dc->J_ab, n, -dc->t);
-  } else if (!fx.b()) {
+  } else if (!fx.b() && !qb) {
     tables.add(sb, ea_b, &pb, nullptr, 0);
     phb.ea_b = ea_b;
   }
   tables.launch(dtype, st);
-  launch_sweep(ctx, sa, sb, 0, v0, v1, nst, dtype, pa, ph, st, nullptr, fx.a());
-  launch_sweep(ctx, sa, sb, 1, v0, v1, nst, dtype, pb, phb, st, nullptr, fx.b());
+  if (qa)
+    launch_sweep_pairs(ctx, sa, sb, 0, v0, pa, true, ph, st);
+  else
+    launch_sweep(ctx, sa, sb, 0, v0, v1, nst, dtype, pa, ph, st, nullptr, fx.a());
+  if (qb)
+    launch_sweep_pairs(ctx, sa, sb, 1, v0, pb, !dc, phb, st);
+  else
+    launch_sweep(ctx, sa, sb, 1, v0, v1, nst, dtype, pb, phb, st, nullptr, fx.b());
 }
 
 // The same rotation (and fused diagonal-Coulomb evolution) with every sweep a
@@ -139,7 +149,7 @@ static void rotate_alternating(Ctx* ctx, Space* sa, Space* sb, void* vec, void* 
   void* eo_a = scratch(ctx, "alt_eo_a", sa->dim * csz);
   void* eo_b = scratch(ctx, "alt_eo_b", sb->dim * csz);
   const double* Jbb = dc ? (dc->J_bb ? dc->J_bb : dc->J_aa) : nullptr;
-  const FxPair fx = fx_prepare(ctx, sa, sb, dtype, pa, pb, st);
+  const FxPair fx = fx_prepare(ctx, sa, sb, dtype, pa, pb, true, st);
   const RotProgram *da = fx.a() ? nullptr : &pa, *db = fx.b() ? nullptr : &pb;
   StringPhases tables(n);
   PhaseDev p1, p2;  // of the first and of the second sweep
@@ -1166,7 +1176,7 @@ static void lucj_vjp_impl(Ctx* ctx, const fs_lucj* op, void* vec, void* cot, int
     double* Tm = Tacc + (size_t)m * nn * 2;
     const double* Ja = m >= 1 ? op->J_aa + (size_t)(m - 1) * nn : nullptr;
     const double* Jab = m >= 1 ? op->J_ab + (size_t)(m - 1) * nn : nullptr;
-    const FxPair fx = fx_prepare(ctx, sa, sb, dtype, inv, inv, st);
+    const FxPair fx = fx_prepare(ctx, sa, sb, dtype, inv, inv, false, st);
     const FxPlan *fa = fx.a(), *fb = fx.b();
     StringPhases tables(n);
     if (m >= 1) {

@@ -367,6 +367,8 @@ struct StrJobs {  // kernel parameter
   int64_t quad[2][kMaxOrb * kMaxOrb];
   uint32_t bad_lin[2], bad_quad[2][kMaxOrb];
 };
+// x radians as a 64-bit fraction of a turn (modulo one turn; x finite).
+int64_t angle_turns(double x);
 class StringPhases {
  public:
   explicit StringPhases(int norb);
@@ -565,6 +567,17 @@ struct FxPair {
   const FxPlan* b() const { return use[1] < 0 ? nullptr : &plan[use[1]]; }
 };
 
+// The complex128 sweep of small spaces (fs_sweep_pairs.cu): whether it takes a
+// forward sweep, and that sweep; diag: it applies the program's diagonal layer
+// too (then `ph` must not hold it).
+namespace pairs {
+constexpr int kMaxM = 192;  // rotations of a program
+}
+bool pairs_supported(const Ctx* ctx, const Space* sthis, const Space* sother, int dtype,
+                     const RotProgram& rp);
+void launch_sweep_pairs(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* vec,
+                        const RotProgram& rp, bool diag, const PhaseDev& ph, cudaStream_t st);
+
 // Givens sweep over one spin: dir 0 rotates alpha (columns of the state),
 // dir 1 rotates beta (rows).  With nst == 1 the epilogue multiplies by the
 // phase `ph` (strings of both spins, cross matrix ph.X).  With nst == 2
@@ -575,8 +588,9 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir,
                   void* st0, void* st1, int nst, int dtype,
                   const RotProgram& prog, const PhaseDev& ph, cudaStream_t st,
                   const RevArgs* rev = nullptr, const FxPlan* fx = nullptr);
+// forward: spins that the small-space sweep takes get no plan.
 FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const RotProgram& pa,
-                  const RotProgram& pb, cudaStream_t st);
+                  const RotProgram& pb, bool forward, cudaStream_t st);
 // That sweep, on st0 and (unless null) st1, with the phase `ph` behind it.
 void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0, void* st1,
                      const FxPlan& plan, const PhaseDev& ph, cudaStream_t st);

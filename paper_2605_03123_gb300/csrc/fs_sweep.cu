@@ -1025,8 +1025,7 @@ __global__ void __launch_bounds__(128) k_string_phases(const __grid_constant__ S
   reinterpret_cast<cx_t<R>*>(J.out)[e] = mk<R>((R)c, (R)s);
 }
 
-// x radians as a 64-bit fraction of a turn (modulo one turn).
-static int64_t turns(double x) {
+int64_t angle_turns(double x) {
   constexpr double hi = 0x1.45f306dc9c883p-3, lo = -0x1.6b01ec5417056p-57;  // 1 / (2 pi)
   const double r = x * hi;
   double f = (r - std::rint(r)) + (std::fma(x, hi, -r) + x * lo);
@@ -1057,7 +1056,7 @@ void StringPhases::add(const Space* sp, void* out, const RotProgram* rp, const d
       for (int q = 0; q < n; ++q) {
         const double x = rp ? std::arg(rp->phase[q]) : -t * lam[q];
         if (!std::isfinite(x)) p_.bad_lin[k] |= 1u << q;
-        p_.lin[k][q] = std::isfinite(x) ? turns(x) : 0;
+        p_.lin[k][q] = std::isfinite(x) ? angle_turns(x) : 0;
       }
     }
     j.lin = k;
@@ -1073,7 +1072,7 @@ void StringPhases::add(const Space* sp, void* out, const RotProgram* rp, const d
       for (int q = 0; q < n * n; ++q) {
         const double x = -0.5 * t * J[q];
         if (!std::isfinite(x)) p_.bad_quad[k][q / n] |= 1u << (q % n);
-        p_.quad[k][q] = std::isfinite(x) ? turns(x) : 0;
+        p_.quad[k][q] = std::isfinite(x) ? angle_turns(x) : 0;
       }
     }
     j.quad = k;

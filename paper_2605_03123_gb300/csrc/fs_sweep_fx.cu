@@ -789,12 +789,15 @@ static bool fx_sector(const Ctx* ctx, const Space* sthis, const Space* sother) {
 }
 
 FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const RotProgram& pa,
-                  const RotProgram& pb, cudaStream_t st) {
+                  const RotProgram& pb, bool forward, cudaStream_t st) {
   FxPair r;
   if (dtype != FS_C128 || ctx->sweep_engine == FS_SWEEP_CUDA_CORE || ctx->prop.major < 10)
     return r;
-  const bool sect[2] = {fx_sector(ctx, sa, sb), fx_sector(ctx, sb, sa)};
   const RotProgram* rp[2] = {&pa, &pb};
+  bool sect[2] = {fx_sector(ctx, sa, sb), fx_sector(ctx, sb, sa)};
+  if (forward)
+    for (int s = 0; s < 2; ++s)
+      sect[s] = sect[s] && !pairs_supported(ctx, s ? sb : sa, s ? sa : sb, dtype, *rp[s]);
   const bool shared = &pa == &pb;  // one program for both spins
   bool ok[2] = {false, false};
   std::vector<std::array<int64_t, 72>> V[2];

@@ -55,6 +55,7 @@ def test_against_oracle_and_fp64_sweeps(lib, ctx, norb, nelec):
     ref = oracle.apply_orbital_rotation(v, Ua, Ub, norb, nelec)
     x = torch.from_numpy(v).cuda()
     y = x.clone()
+    ctx.set_sweep_engine(lib.FS_SWEEP_TENSOR)
     used = _kernels(ctx, lambda: lib.apply_orbital_rotation_(x, Ua, norb, nelec, U_b=Ub, ctx=ctx))
     assert ctx.sync_status() == 0
     assert v.size < 400 or any(k.endswith("_fx") for k in used), used
@@ -65,10 +66,12 @@ def test_against_oracle_and_fp64_sweeps(lib, ctx, norb, nelec):
     assert float((x - y).abs().max()) < TOL
 
 
+@pytest.mark.parametrize("engine", ["FS_SWEEP_AUTO", "FS_SWEEP_TENSOR"])
 @pytest.mark.parametrize("scale", [1e-305, 1e-150, 1e150])
-def test_scales_and_zero_vectors(lib, ctx, scale):
+def test_scales_and_zero_vectors(lib, ctx, scale, engine):
     """Each vector keeps its own scale: rows of very different size (and zero
     rows and columns) come out as accurate as a rotation of each alone."""
+    ctx.set_sweep_engine(getattr(lib, engine))
     norb, nelec = 9, (4, 5)
     g = inputs.rng(41900)
     U = inputs.haar_unitary(norb, g)
@@ -87,7 +90,9 @@ def test_scales_and_zero_vectors(lib, ctx, scale):
     assert not out[3].any()
 
 
-def test_not_finite_vectors_stay_apart(lib, ctx):
+@pytest.mark.parametrize("engine", ["FS_SWEEP_AUTO", "FS_SWEEP_TENSOR"])
+def test_not_finite_vectors_stay_apart(lib, ctx, engine):
+    ctx.set_sweep_engine(getattr(lib, engine))
     norb, nelec = 8, (4, 4)
     g = inputs.rng(41950)
     U = inputs.haar_unitary(norb, g)
@@ -155,3 +160,32 @@ def test_phase_of_non_finite_coupling_stays_with_its_strings(lib, ctx):
     out = x.cpu().numpy()
     assert np.isnan(out[hit]).all()
     assert np.max(np.abs(out[~hit] - ref[~hit])) < TOL
+
+
+@pytest.mark.parametrize("norb,nelec", [(2, (1, 1)), (4, (2, 1)), (5, (4, 3)), (8, (4, 4)),
+                                        (9, (5, 4)), (9, (1, 8)), (12, (2, 1)), (17, (1, 2))])
+def test_small_spaces_against_fp64_window_sweeps(lib, ctx, norb, nelec):
+    """The sweep of small spaces applies the same rotations in the same order
+    with the same FP64 operations as the window sweeps: only the phases behind
+    them round differently.  Also with its own cross tables (a diagonal gate
+    fused behind the rotation)."""
+    g = inputs.rng(42000 + 41 * norb + nelec[0])
+    Ua, Ub = inputs.haar_unitary(norb, g), inputs.haar_unitary(norb, g)
+    h, J = inputs.random_symmetric(norb, 0.7, g), inputs.random_symmetric(norb, 0.7, g)
+    v = inputs.random_state(norb, nelec, g)
+    ref = oracle.apply_orbital_rotation(v, Ua, Ub, norb, nelec)
+    tref = oracle.simulate_trotter_diag_coulomb(v, h, J, J, J, 0.6, norb, nelec, 2, 1)
+    out = []
+    for engine in (lib.FS_SWEEP_AUTO, lib.FS_SWEEP_CUDA_CORE):
+        ctx.set_sweep_engine(engine)
+        x = torch.from_numpy(v).cuda()
+        used = _kernels(ctx, lambda: lib.apply_orbital_rotation_(x, Ua, norb, nelec, U_b=Ub, ctx=ctx))
+        # N = 17 has too many rotations for a sweep one rotation at a time
+        taken = engine == lib.FS_SWEEP_AUTO and norb <= 12
+        assert any("pairs" in k for k in used) == taken, used
+        y = torch.from_numpy(v).cuda()
+        lib.simulate_trotter_diag_coulomb_(y, h, J, J, 0.6, norb, nelec, n_steps=2, order=1, ctx=ctx)
+        assert np.max(np.abs(y.cpu().numpy() - tref)) < TOL
+        out.append(x.cpu().numpy())
+    assert np.max(np.abs(out[0] - ref)) < TOL
+    assert np.max(np.abs(out[0] - out[1])) < 1e-14 * norb
