@@ -81,13 +81,40 @@ static double norm1(int n, const zd* A) {
   return m;
 }
 
-// Scaling and squaring with the Taylor polynomial of degree 18: A / 2^s has
-// 1-norm <= 1/2, where its remainder is below 2^-75.  The polynomial takes
-// seven products (powers 2, 3, 4 and four steps of Horner's rule in the
-// fourth power) instead of seventeen.
 static int taylor_scale(double nrm) {
   return nrm > 0.5 ? (int)std::ceil(std::log2(nrm / 0.5)) : 0;
 }
+
+// Scaling and squaring with a Taylor series: A / 2^s has 1-norm <= 1/2, and
+// the series is summed term by term until a term no longer changes the sum in
+// FP64.  (A form with fewer products rounds differently: the FP32 coefficients
+// and phases made from a matrix 1e-15 away differ in a last place here and
+// there, and a long FP32 sweep in all of its last places.)
+void expm(int n, const zd* A, zd* out) {
+  const int s = taylor_scale(norm1(n, A));
+  const Split B(n, A, std::ldexp(1.0, -s));
+  Split term(n), sum(n);
+  for (int i = 0; i < n; ++i) term.r[(size_t)i * n + i] = sum.r[(size_t)i * n + i] = 1.0;
+  for (int k = 1; k <= 40; ++k) {
+    Split next = product(term, B);
+    bool small = true;  // no entry of modulus 1e-18 or more
+    for (size_t q = 0; q < next.r.size(); ++q) {
+      next.r[q] /= (double)k;
+      next.i[q] /= (double)k;
+      sum.r[q] += next.r[q];
+      sum.i[q] += next.i[q];
+    }
+    for (size_t q = 0; q < next.r.size() && small; ++q)
+      small = std::hypot(next.r[q], next.i[q]) < 1e-18;
+    term = std::move(next);
+    if (small) break;
+  }
+  for (int k = 0; k < s; ++k) sum = product(sum, sum);
+  sum.store(out);
+}
+
+// Taylor polynomial of degree 18 (remainder below 2^-75 at 1-norm 1/2) in
+// seven products: powers 2, 3, 4 and four steps of Horner's rule in the fourth.
 static const double* taylor_coef() {
   static const std::array<double, 20> c = [] {
     std::array<double, 20> t;
@@ -99,32 +126,9 @@ static const double* taylor_coef() {
 }
 constexpr int kTaylor = 18;
 
-void expm(int n, const zd* A, zd* out) {
-  const int s = taylor_scale(norm1(n, A));
-  const double* c = taylor_coef();
-  const Split B(n, A, std::ldexp(1.0, -s)), B2 = product(B, B), B3 = product(B2, B),
-              B4 = product(B2, B2);
-  auto block = [&](int k) {  // c_k + c_{k+1} B + c_{k+2} B^2 + c_{k+3} B^3
-    Split P(n);
-    for (int p = 0; p < n; ++p) P.r[(size_t)p * n + p] = c[k];
-    if (k + 1 <= kTaylor) axpy(P, c[k + 1], B);
-    if (k + 2 <= kTaylor) axpy(P, c[k + 2], B2);
-    if (k + 3 <= kTaylor) axpy(P, c[k + 3], B3);
-    return P;
-  };
-  Split E = block(16);
-  for (int k = 12; k >= 0; k -= 4) {
-    Split P = block(k);
-    mul_add(E, B4, P);
-    E = std::move(P);
-  }
-  for (int k = 0; k < s; ++k) E = product(E, E);
-  E.store(out);
-}
-
 // For the real inner product <A, B> = Re tr(A^dag B), the adjoint of the
 // Frechet derivative of expm at K is the Frechet derivative at K^dag, the
-// upper-right block of expm([[K^dag, H], [0, K^dag]]).  The same polynomial
+// upper-right block of expm([[K^dag, H], [0, K^dag]]).  That polynomial
 // on such block matrices, of which only the diagonal block X and the
 // upper-right block L are held: (X, L) (Y, M) = (X Y, X M + L Y).
 void expm_frechet_adjoint(int n, const zd* K, const zd* H, zd* out) {
@@ -203,16 +207,11 @@ RotProgram decompose_adjacent(int n, const zd* U) {
         c = std::abs(b) / rho;
         s = -std::conj(a) * b / (std::abs(b) * rho);
       }
-      // A <- A G^dag on columns (j, j+1): G^dag = [[c, -s], [s*, c]], in real
-      // arithmetic (see Split)
-      const double sr = s.real(), si = s.imag();
-      double* col = reinterpret_cast<double*>(A.data() + j);
-      for (int i = 0; i < n; ++i, col += 2 * n) {
-        const double xr = col[0], xi = col[1], yr = col[2], yi = col[3];
-        col[0] = c * xr + (sr * yr + si * yi);
-        col[1] = c * xi + (sr * yi - si * yr);
-        col[2] = c * yr - (sr * xr - si * xi);
-        col[3] = c * yi - (sr * xi + si * xr);
+      // A <- A G^dag on columns (j, j+1): G^dag = [[c, -s], [s*, c]]
+      for (int i = 0; i < n; ++i) {
+        zd x = A[i * n + j], y = A[i * n + j + 1];
+        A[i * n + j] = c * x + std::conj(s) * y;
+        A[i * n + j + 1] = -s * x + c * y;
       }
       A[r * n + j] = 0.0;
       prog.g.push_back(Givens{j, c, s});
@@ -458,26 +457,44 @@ namespace fs {
 
 void window_rows_host(int n, int W, const std::vector<uint32_t>& orbits,
                       const std::vector<int>& off, const std::vector<uint16_t>& offs,
-                      std::vector<uint32_t>& chunk, std::vector<uint16_t>& rows) {
+                      std::vector<uint2>& cls, std::vector<uint16_t>& rows) {
   std::vector<std::vector<int>> masks(W + 1);
   for (int x = 0; x < (1 << W); ++x) masks[__builtin_popcount(x)].push_back(x);
-  chunk.clear();
+  cls.clear();
   rows.clear();
-  for (size_t a = 0; a + 1 < off.size(); ++a)
-    for (int c = off[a]; c < off[a + 1]; c += 32) {
-      int m = 0;  // the chunk's class: that of its orbits, empty ones aside
-      for (int l = 0; l < 32 && !m; ++l) m = (int)(orbits[c + l] >> 24);
-      const size_t start = rows.size(), ns = masks[m].size(), nu = (ns + 7) / 8;
-      chunk.push_back((uint32_t)(start / 8) | ((uint32_t)m << 24));
-      rows.resize(start + nu * 32 * 8, (uint16_t)0xFFFF);
-      for (int l = 0; l < 32; ++l) {
-        const uint32_t d = orbits[c + l];
-        if (!(d >> 24)) continue;
+  for (size_t a = 0; a + 1 < off.size(); ++a) {
+    int c = off[a];
+    for (int i = 0; i < W - 1; ++i) {
+      uint2 e{};
+      const uint32_t m = c < off[a + 1] ? orbits[c] >> 24 : 0;
+      const size_t start = rows.size();
+      e.x = (uint32_t)(start / 8) | (m << 24);
+      while (c + (int)e.y < off[a + 1] && m && orbits[c + e.y] >> 24 == m) ++e.y;
+      cls.push_back(e);
+      const size_t ns = masks[m].size(), nu = (ns + 7) / 8, us = (e.y + 7) / 8 * 8;
+      rows.resize(start + us * nu * 8, (uint16_t)0xFFFF);
+      for (uint32_t o = 0; o < e.y; ++o) {
+        const uint32_t d = orbits[c + o];
         const uint16_t* F = offs.data() + ((a * (n + 1) + ((d >> 16) & 0xFF)) << W);
         for (size_t k = 0; k < ns; ++k)
-          rows[start + ((k / 8) * 32 + l) * 8 + k % 8] = (uint16_t)((d & 0xFFFF) + F[masks[m][k]]);
+          rows[start + ((k / 8) * us + o) * 8 + k % 8] = (uint16_t)((d & 0xFFFF) + F[masks[m][k]]);
       }
+      c += (int)(e.y + 31) / 32 * 32;  // past the class's padding
     }
+  }
+}
+
+void window_chunks_host(int W, int nk, const std::vector<uint2>& cls, std::vector<int>& off,
+                        std::vector<uint4>& chunk) {
+  chunk.clear();
+  off.assign(1, 0);
+  for (size_t i = 0; i < cls.size(); ++i) {
+    const uint32_t cnt = cls[i].y, us = (cnt + 7) / 8 * 8;
+    for (uint32_t k = 0; k < cnt * (uint32_t)nk; k += 32)
+      chunk.push_back(uint4{cls[i].x, cnt | us << 16, k % cnt | (k / cnt) << 16,
+                            (1u << 31) / cnt + 1});
+    if (i % (W - 1) == (size_t)W - 2) off.push_back((int)chunk.size());
+  }
 }
 
 // Subsets of four orbitals covering every unordered orbital pair (greedy:
