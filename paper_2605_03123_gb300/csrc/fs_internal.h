@@ -75,13 +75,19 @@ const std::vector<WinStep>& window_schedule(Ctx* ctx, const RotProgram& rp, int 
 void window_tables_host(int N, int n, int W, std::vector<uint32_t>& orbits,
                         std::vector<int>& off, std::vector<uint16_t>& offs,
                         std::vector<uint8_t>& okey);
-// The gather addresses of those orbits, chunk by chunk of 32 (one class each):
-// string k of the orbit of lane l is the 16-bit half k % 2 of word k / 2 % 4 of
-// the 16-byte unit chunk[c] % 2^24 + 32 (k / 8) + l; rows of empty orbits and
-// the places past C(W, m) hold 0xFFFF.
+// The gather addresses of those orbits.  Per window position, W - 1 classes in
+// their order (absent ones empty): cls = (first unit | m << 24, orbits y); string
+// k of orbit o is the 16-bit half k % 2 of word k / 2 % 4 of the 16-byte unit
+// first + (k / 8) us + o, us = y rounded up to 8.
 void window_rows_host(int n, int W, const std::vector<uint32_t>& orbits,
                       const std::vector<int>& off, const std::vector<uint16_t>& offs,
-                      std::vector<uint32_t>& chunk, std::vector<uint16_t>& rows);
+                      std::vector<uint2>& cls, std::vector<uint16_t>& rows);
+// The (packed set, orbit) items of those classes for slabs of nk sets, orbit
+// first, in chunks of 32 of one class: (first unit | m << 24, y | us << 16,
+// orbit | set << 16 of the first item, 2^31 / y + 1: the high word of twice
+// its product with i is i / y).
+void window_chunks_host(int W, int nk, const std::vector<uint2>& cls, std::vector<int>& off,
+                        std::vector<uint4>& chunk);
 // The orbits regrouped for clusters of 2^b CTAs: per window position a,
 // group r (occupation of the top b orbitals, the strings of cluster rank r)
 // at gorb[goff[a * 9 + r] .. goff[a * 9 + r + 1]), class order kept inside,
@@ -187,10 +193,15 @@ struct Space {
     TcSeg* tc_seg[2] = {};
     uint16_t* tc_idx[2] = {};
     int tc_seg_max[2] = {};  // largest segment, bytes
-    // gather addresses of the packed sweeps (W = 6): chunk c of 32 orbits of
-    // the padded list holds class m in pk_chunk[c] >> 24 and its rows from
-    // 16-byte unit pk_chunk[c] & 0xFFFFFF on
-    uint32_t* pk_chunk = nullptr;
+    // packed sweeps (W = 6): the orbits' gather addresses (window_rows_host)
+    // and, per number of packed sets in a slab, the work of a step in chunks
+    // of 32 items (window_chunks_host), window position a's from off[a] on
+    struct Chunks {
+      uint4* chunk = nullptr;
+      int* off = nullptr;
+    };
+    std::map<int, Chunks> pk_chunks;
+    std::vector<uint2> pk_cls;
     uint4* pk_rows = nullptr;
     std::vector<uint32_t> orb_h;
     std::vector<int> off_h;
@@ -500,7 +511,10 @@ struct SweepGeom {
   const int* tgoff;
   const uint16_t* offs;    // [npos][nocc + 1][1 << W] in-window rank offsets
   int offs_stride;         // (nocc + 1) << W
-  const uint32_t* pk_chunk;  // packed sweeps: see Space::Win
+  const uint4* pk_chunk;  // packed sweeps: see Space::Win
+  const int* pk_off;
+  int nv;    // vectors per packed slab (its pitch: KV)
+  int tgrp;  // vectors per FP32 partial of the transition sums (packed slabs)
   const uint4* pk_rows;
   // tensor-core window steps (W = 6): per step the B images of classes
   // m = 1..5 (tc::kStepBytes each step); gather-index segments per window

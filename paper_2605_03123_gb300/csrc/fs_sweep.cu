@@ -184,15 +184,11 @@ static void build_window_tables(Space* sp, int W) {
   FS_CUDA(cudaMemcpy(wt.off, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice));
   FS_CUDA(cudaMemcpy(wt.offs, offs.data(), offs.size() * 2, cudaMemcpyHostToDevice));
   if (W == window_width<float, 1>()) {  // packed sweeps
-    std::vector<uint32_t> chunk;
     std::vector<uint16_t> rows;
-    window_rows_host(sp->nocc, W, orbits, off, offs, chunk, rows);
-    FS_CUDA(cudaMalloc(&wt.pk_chunk, std::max<size_t>(chunk.size(), 1) * 4));
+    window_rows_host(sp->nocc, W, orbits, off, offs, wt.pk_cls, rows);
     FS_CUDA(cudaMalloc(&wt.pk_rows, std::max<size_t>(rows.size(), 8) * 2));
-    if (!chunk.empty()) {
-      FS_CUDA(cudaMemcpy(wt.pk_chunk, chunk.data(), chunk.size() * 4, cudaMemcpyHostToDevice));
+    if (!rows.empty())
       FS_CUDA(cudaMemcpy(wt.pk_rows, rows.data(), rows.size() * 2, cudaMemcpyHostToDevice));
-    }
   }
   wt.built = true;
 }
@@ -301,10 +297,39 @@ static void set_window_geom(SweepGeom& g, Space* sp, int W) {
     g.orb_grp = wt.gorb[g.lgcs];
     g.orb_goff = wt.goff[g.lgcs];
   }
-  g.pk_chunk = wt.pk_chunk;
-  g.pk_rows = wt.pk_rows;
   g.offs = wt.offs;
   g.offs_stride = (sp->nocc + 1) << W;
+}
+
+// The packed tables of a slab of nk sets (at most one set of tables per width;
+// built on first use, as the window tables are).
+static void set_packed_geom(SweepGeom& g, Space* sp, int W, int nk) {
+  Space::Win& wt = sp->win[W];
+  Space::Win::Chunks& c = wt.pk_chunks[nk];
+  if (!c.off) {
+    std::vector<int> off;
+    std::vector<uint4> chunk;
+    window_chunks_host(W, nk, wt.pk_cls, off, chunk);
+    if (!c.chunk) FS_CUDA(cudaMalloc(&c.chunk, std::max<size_t>(chunk.size(), 1) * sizeof(uint4)));
+    if (!chunk.empty())
+      FS_CUDA(cudaMemcpy(c.chunk, chunk.data(), chunk.size() * sizeof(uint4),
+                         cudaMemcpyHostToDevice));
+    int* o = nullptr;
+    FS_CUDA(cudaMalloc(&o, off.size() * sizeof(int)));
+    FS_CUDA(cudaMemcpy(o, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice));
+    c.off = o;
+  }
+  g.pk_chunk = c.chunk;
+  g.pk_off = c.off;
+  g.pk_rows = wt.pk_rows;
+}
+
+// Pitch of a packed slab of nv vectors: an odd number of 16-byte cells per
+// string, so that the eight lanes of a phase, whose strings lie in distinct
+// banks, keep them distinct (reverse sweep of N = 12 (6,6), 8 vectors a slab:
+// 131 to 135 us at a pitch of 8, 84 to 104 at 9).
+static int packed_pitch(int nst, int nv) {
+  return nst == 2 ? (nv > 1 ? nv | 1 : nv) : nv > 2 ? 2 * (nv / 2 | 1) : nv;
 }
 
 // Kernel choice: window sweeps when the orbitals allow a window; forward
@@ -422,6 +447,7 @@ static void dispatch_prog(Ctx* ctx, Space* sthis, int CS, const SweepGeom& g0, c
       if constexpr (sizeof(R) == 4) {
         // slabs of an even number of vectors: packed vector pairs
         if (CS == 1 && g.KV % 2 == 0) {
+          set_packed_geom(g, sthis, W, g.nv / 2);
           if (two_per_sm)
             launch_sweep_t<R, 1, 1, false, W, 256, false, WProg<R>, false, true>(g, prog, X,
                                                                                nslabs, smem, st);
@@ -444,13 +470,15 @@ static void dispatch_prog(Ctx* ctx, Space* sthis, int CS, const SweepGeom& g0, c
       SweepGeom g = g0;
       set_window_geom(g, sthis, WS);
       auto prog = make_wprog<R>(ctx, rp, sthis->norb, WS);
-      if constexpr (sizeof(R) == 4)
+      if constexpr (sizeof(R) == 4) {
         // complex64: psi and g of an orbit in one thread, packed per string
         // (W = 6; shared addresses and coefficients, two-lane updates)
+        set_packed_geom(g, sthis, WS, g.nv);
         launch_sweep_t<R, 1, NST, VJP, WS, 512, false, WProg<R>, false, true>(g, prog, X, nslabs,
                                                                               smem, st);
-      else
+      } else {
         launch_sweep_t<R, 1, NST, VJP, WS, 512, true>(g, prog, X, nslabs, smem, st);
+      }
       return;
     }
     if (sthis->norb >= WJ && sthis->dim > 1) {
@@ -631,17 +659,22 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
   while ((2 << lg) <= std::min(want, kMaxKV) && smem_for(CS, 2 << lg) <= budget) ++lg;
   if (pair_slab && lg == 0) lg = 1;
   int KV = 1 << lg;
+  g.tgrp = KV;
   if (dtype == FS_C64 && CS == 1 && sthis->norb >= window_width<float, 1>() && sthis->dim > 1) {
-    // packed slabs take any width (pairs of vectors when forward): the one
-    // with the least modelled time.  A slab costs its vectors and a fixed part
-    // worth c0 of them; slabs run in waves of two per SM (forward slabs that
-    // fit half an SM) or one, and a last wave of at most one per SM runs 0.6
-    // as long.  N = 12 (6,6), 924 vectors: 4 forward (was 2), 7 reverse (2).
-    const int unit = nst == 1 ? 2 : 1, slots = (two_per_sm ? 2 : 1) * ctx->prop.multiProcessorCount;
+    // packed slabs take any width (pairs of vectors when forward; reverse,
+    // multiples of the power of two above, which stays the length of the FP32
+    // sums: longer ones move the gradients by some 1.5e-7): the one with the
+    // least modelled time.  A slab costs its vectors and a fixed part worth c0
+    // of them; slabs run in waves of two per SM (forward slabs that fit half an
+    // SM) or one, and a last wave of at most one per SM runs 0.6 as long.
+    // N = 12 (6,6), 924 vectors: 4 forward, 8 reverse (84 to 104 us a sweep;
+    // 2: 127 to 160, 4: 98 to 120).
+    const int unit = nst == 1 ? 2 : g.tgrp, slots = (two_per_sm ? 2 : 1) * ctx->prop.multiProcessorCount;
     const double c0 = 450.0 / g.d + 0.1;
     double best = -1;
     for (int kv = unit; kv <= kMaxKV && kv < g.nvec + unit; kv += unit) {
-      if (smem_for(1, kv) > budget) break;
+      // (pass sums per g.tgrp vectors)
+      if (smem_for(1, kv) + (kv / unit - 1) * (nst == 1 ? 0 : tsum) > budget) break;
       const int slabs = (g.nvec + kv - 1) / kv, last = slabs % slots;
       const double waves = slabs / slots + (last == 0 ? 0.0
                                             : two_per_sm && last <= slots / 2 ? 0.6 : 1.0);
@@ -652,6 +685,12 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
       }
     }
   }
+  g.nv = KV;
+  const int nslabs = (g.nvec + KV - 1) / KV;
+  if (dtype == FS_C64 && CS == 1) {
+    const int p = packed_pitch(nst, KV);
+    if (smem_for(1, p) + tsum * (KV / g.tgrp) <= budget) KV = p;
+  }
   g.KV = KV;
   set_cluster_layout(g, sthis, CS, [&](int chunk) {
     return (size_t)(chunk * csz * nst + tab_per_kv + fixed) + tsum <= maxsm;
@@ -661,9 +700,8 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
     g.trec_grp = sthis->tgrec[g.lgcs];
     g.tgoff = sthis->tgoff[g.lgcs];
   }
-  const int nslabs = (g.nvec + KV - 1) / KV;
   const size_t smem = std::max<size_t>(
-      (size_t)KV * ((size_t)g.chunk * csz * nst + tab_per_kv + fixed) + tsum, 16);
+      (size_t)KV * ((size_t)g.chunk * csz * nst + tab_per_kv + fixed) + tsum * ((g.nv + g.tgrp - 1) / g.tgrp), 16);
   Space* sw = const_cast<Space*>(sthis);
   if (dtype == FS_C64) {
     if (nst == 1) dispatch_prog<float, 1, false>(ctx, sw, CS, g, rp, ph.X, nslabs, smem, two_per_sm, st);
@@ -691,12 +729,13 @@ int batch_window(int dtype, int nst) {
 // one-job launch of the batched kernel, on scratch states (and scratch W
 // and T for the reverse sweeps), for every slab width 2^0 .. 2^lgmax that
 // fits the stage's budget; CUDA events on a private stream, the fastest
-// mean of two launches after one warm-up wins and is cached per sector and
-// sweep kind.  Runs before any capture.
-template <typename SmemFor>
-static int tune_batch_slab(Ctx* ctx, const SweepGeom& g0, const std::vector<unsigned char>& prog,
+// mean of two launches after one warm-up wins (the narrower slab, whose FP32
+// sums are shorter, unless the wider one gains 5 %) and is cached per sector
+// and sweep kind.  Runs before any capture.
+template <typename SmemFor, typename Pitch>
+static int tune_batch_slab(Ctx* ctx, Space* sthis, int W, const SweepGeom& g0, const std::vector<unsigned char>& prog,
                            int nst, int dtype, bool rev, int lgmin, int lgmax,
-                           SmemFor&& smem_for, const std::array<int, 8>& key) {
+                           SmemFor&& smem_for, Pitch&& pitch_for, const std::array<int, 8>& key) {
   if (!ctx->tune_stream)
     FS_CUDA(cudaStreamCreateWithFlags(&ctx->tune_stream, cudaStreamNonBlocking));
   cudaStream_t ts = ctx->tune_stream;
@@ -725,14 +764,17 @@ static int tune_batch_slab(Ctx* ctx, const SweepGeom& g0, const std::vector<unsi
   std::vector<float> ms(lgmax + 1, 0.f);
   int best = lgmin;
   for (int lg = lgmin; lg <= lgmax; ++lg) {
-    g.KV = 1 << lg;
+    g.nv = g.tgrp = 1 << lg;
+    g.KV = pitch_for(1 << lg);
+    if (dtype == FS_C64 && (nst == 2 || lgmin > 0))
+      set_packed_geom(g, sthis, W, nst == 2 ? g.nv : g.nv / 2);
     SweepJob j{};
     j.g = g;
     j.prog = dprog;
     j.X = dX;
     j.item0 = 0;
     const int nslabs = (g.nvec + (1 << lg) - 1) >> lg;
-    const size_t smem = smem_for(1 << lg);
+    const size_t smem = smem_for(g.KV);
     FS_CUDA(cudaMemcpyAsync(djob, &j, sizeof(j), cudaMemcpyHostToDevice, ts));
     const bool pk = lgmin > 0;
     launch_sweep_batch(ctx, dtype, nst, nullptr, 0, 0, nullptr, smem, ts, pk);  // attribute
@@ -746,7 +788,7 @@ static int tune_batch_slab(Ctx* ctx, const SweepGeom& g0, const std::vector<unsi
     FS_CUDA(cudaEventSynchronize(e1));
     FS_CUDA(cudaEventElapsedTime(&tot, e0, e1));
     ms[lg] = tot / 2;
-    if (ms[lg] < ms[best]) best = lg;
+    if (ms[lg] < 0.95f * ms[best]) best = lg;
   }
   FS_CUDA(cudaEventDestroy(e0));
   FS_CUDA(cudaEventDestroy(e1));
@@ -817,6 +859,10 @@ void plan_batch_sweep(Ctx* ctx, Space* sa, Space* sb, int dir, void* st0, void* 
   // complex64 forward sweeps: at least two vectors per slab, run as packed
   // vector pairs
   const int lgmin = dtype == FS_C64 && nst == 1 && lgmax >= 1 ? 1 : 0;
+  auto pitch_for = [&](int nv) {
+    const int p = dtype == FS_C64 && (nst == 2 || lgmin > 0) ? packed_pitch(nst, nv) : nv;
+    return smem_for(p) <= budget ? p : nv;
+  };
   const std::array<int, 8> key = {sthis->norb, sthis->nocc, sother->nocc, dtype, nst,
                                   rev != nullptr, ph.has_x, (int)(budget >> 10)};
   int lg = -1;
@@ -824,8 +870,8 @@ void plan_batch_sweep(Ctx* ctx, Space* sa, Space* sb, int dir, void* st0, void* 
   if (it != ctx->sweep_tune.end()) {
     lg = std::min(it->second, lgmax);
   } else if (ctx->batch_tuning && lgmax > lgmin) {
-    lg = tune_batch_slab(ctx, g, out.prog, nst, dtype, rev != nullptr, lgmin, lgmax, smem_for,
-                         key);
+    lg = tune_batch_slab(ctx, sthis, W, g, out.prog, nst, dtype, rev != nullptr, lgmin, lgmax, smem_for,
+                         pitch_for, key);
   }
   if (lg < 0) {  // untuned: about eight slabs per circuit
     const int want = std::max(1, g.nvec / 8);
@@ -833,9 +879,12 @@ void plan_batch_sweep(Ctx* ctx, Space* sa, Space* sb, int dir, void* st0, void* 
     while ((2 << lg) <= std::min(want, kMaxKV) && lg < lgmax) ++lg;
   }
   lg = std::max(lg, lgmin);
-  g.KV = 1 << lg;
+  g.nv = g.tgrp = 1 << lg;
+  g.KV = pitch_for(1 << lg);
+  if (dtype == FS_C64 && (nst == 2 || lgmin > 0))
+    set_packed_geom(g, sthis, W, nst == 2 ? g.nv : g.nv / 2);
   out.nslabs = (g.nvec + (1 << lg) - 1) >> lg;
-  out.smem = smem_for(1 << lg);
+  out.smem = smem_for(g.KV);
   out.pk = lgmin > 0;
 }
 

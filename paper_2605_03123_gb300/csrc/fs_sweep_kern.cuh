@@ -565,7 +565,6 @@ template <int W, int M>
 __device__ __forceinline__ void win_orbit_pk(const uint4 (&q)[3], float* smf, int KC, int kc,
                                              const WProg<float>& prog, int ga, int gb) {
   constexpr int NS = cbinom(W, M);
-  if ((q[0].x & 0xFFFFu) == 0xFFFFu) return;  // an empty lane
   int ad[NS];
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
@@ -875,8 +874,10 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
   using C = cx_t<R>;
   C* sm = reinterpret_cast<C*>(smraw);
   const int KV = g.KV;
-  const int v0 = slab * KV;
-  const int kv_eff = min(KV, g.nvec - v0);
+  // packed slabs hold g.nv vectors at a pitch of KV
+  const int nvs = PK ? g.nv : KV;
+  const int v0 = slab * nvs;
+  const int kv_eff = min(nvs, g.nvec - v0);
   // element ranges of the cluster ranks (registers; rank is runtime)
   int cbr[CS + 1];
 #pragma unroll
@@ -1084,24 +1085,33 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
       }
       if constexpr (PK) {
         // packed cells (vector pairs of one state, or psi and g); the work
-        // items are (orbit, packed set) pairs, chunk by chunk of 32 orbits
-        // (a class boundary never falls inside a chunk), so that short
-        // vectors with few orbits per step still fill the CTA
+        // items of a class are its (packed set, orbit) pairs, orbit first,
+        // 32 to a warp: at N = 12 a class has 6 .. 20 orbits, and a warp of
+        // one set's orbits left half of its lanes idle (N = 12 (6,6)
+        // forward sweeps 43 -> 35 us, N = 16 (3,8) alpha 459 -> 219)
         const int KC = NST == 1 ? (KV >> 1) : KV;
         const int nk = NST == 1 ? (kv_eff + 1) >> 1 : kv_eff;
-        const int nit = (hi - lo) * nk;
+        const int ch0 = __ldg(g.pk_off + a), nit = (__ldg(g.pk_off + a + 1) - ch0) * 32;
+        const uint4* chunks = g.pk_chunk + ch0;
         // AHEAD: the address rows of the next round are loaded while this
         // one runs (not in the batched kernels, whose program is read through
         // a pointer: they would spill)
-        const uint32_t* chunks = g.pk_chunk + (lo >> 5);
-        auto rows_of = [&](int it, uint32_t& m, uint4 (&q)[3]) {
-          const int ch = it >> 5, oc = nk == 1 ? ch : ch / nk;
-          const uint32_t c = __ldg(chunks + oc);
-          const uint4* r = g.pk_rows + (c & 0xFFFFFFu) + (it & 31);
-          m = c >> 24;
-          q[0] = __ldg(r);
-          if (m > 1 && m < 5) q[1] = __ldg(r + 32);
-          if (m == 3) q[2] = __ldg(r + 64);
+        auto rows_of = [&](int it, uint32_t& m, int& kc, uint4 (&q)[3]) {
+          const uint4 e = __ldg(chunks + (it >> 5));
+          const int cnt = (int)(e.y & 0xFFFFu);
+          int o = (int)(e.z & 0xFFFFu) + (it & 31);
+          kc = (int)(e.z >> 16);
+          if (KC > 1) {
+            const int t = (int)__umulhi((uint32_t)(2 * o), e.w);  // o / cnt
+            kc += t;
+            o -= t * cnt;
+          }
+          m = o < cnt && kc < nk ? e.x >> 24 : 0;
+          const uint4* r = g.pk_rows + (e.x & 0xFFFFFFu) + o;
+          const uint32_t us = e.y >> 16;
+          if (m > 0) q[0] = __ldg(r);
+          if (m > 1 && m < 5) q[1] = __ldg(r + us);
+          if (m == 3) q[2] = __ldg(r + 2 * us);
         };
         auto item_of = [&](int rd) {
           return dealt_round<kThreads>(0, nit, rd, 0, 1)
@@ -1110,17 +1120,17 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
         };
         int it = item_of(0);
         uint32_t m = 0;
+        int kc = 0;
         uint4 q[3];
-        if (AHEAD && it >= 0) rows_of(it, m, q);
+        if (AHEAD && it >= 0) rows_of(it, m, kc, q);
         for (int rd = 0; dealt_round<kThreads>(0, nit, rd, 0, 1); ++rd) {
           const int it_next = item_of(rd + 1);
           uint32_t m_next = 0;
+          int kc_next = 0;
           uint4 q_next[3];
-          if (AHEAD && it_next >= 0) rows_of(it_next, m_next, q_next);
-          if (!AHEAD && it >= 0) rows_of(it, m, q);
+          if (AHEAD && it_next >= 0) rows_of(it_next, m_next, kc_next, q_next);
+          if (!AHEAD && it >= 0) rows_of(it, m, kc, q);
           if (it >= 0) {
-            const int ch = it >> 5, oc = nk == 1 ? ch : ch / nk;
-            const int kc = ch - oc * nk;
             switch (m) {
               case 1: win_orbit_pk<W, 1>(q, smf, KC, kc, prog, ga, gb); break;
               case 2: win_orbit_pk<W, 2>(q, smf, KC, kc, prog, ga, gb); break;
@@ -1133,6 +1143,7 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
           it = it_next;
           if (AHEAD) {
             m = m_next;
+            kc = kc_next;
 #pragma unroll
             for (int u = 0; u < 3; ++u) q[u] = q_next[u];
           }
@@ -1206,8 +1217,11 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
     if (g.T && g.npass > 0) {
       // subset passes: per-thread partial sums of the 16 local slots, one
       // warp reduction per pass, per-CTA sums in shared memory
+      // (packed slabs: per group of g.tgrp vectors, so that the FP32 sums do
+      // not grow with the slab's width)
       R* tsm = reinterpret_cast<R*>(w + (g.has_x ? kMaxOrb * g.KV : 0));
-      for (int i = tid; i < g.npass * 32; i += kThreads) tsm[i] = 0;
+      const int ngrp = CS == 1 && PK ? (kv_eff + g.tgrp - 1) / g.tgrp : 1;
+      for (int i = tid; i < g.npass * 32 * ngrp; i += kThreads) tsm[i] = 0;
       __syncthreads();
       const int lane = tid & 31;
       if constexpr (CS == 1 && PK) {
@@ -1217,9 +1231,11 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
         // reduces once per unit; units are dealt round-robin over the
         // warps in pass order, so the passes that also own diagonals (the
         // first ones of the covering) fall on different warps
-        const int warp = tid >> 5, nkv = kv_eff;
-        for (int u = warp; u < g.npass * 4; u += kThreads / 32) {
-          const int ip = u >> 2, qq = u & 3;
+        const int warp = tid >> 5;
+        for (int u = warp; u < g.npass * 4 * ngrp; u += kThreads / 32) {
+          const int gi = ngrp == 1 ? 0 : u / (g.npass * 4), ui = u - gi * g.npass * 4;
+          const int ip = ui >> 2, qq = ui & 3;
+          const int kvb = gi * g.tgrp, nkv = min(g.tgrp, kv_eff - kvb);
           const TPassDev pd = g.tpass[ip];
           R acc[32];
 #pragma unroll
@@ -1234,7 +1250,7 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
           DivWalk cw(qq, 4, nkv);
           uint4 rnext = qq < nch ? rec_of(cw.a) : make_uint4(0, 0, 0, 0);
           for (int ch = qq; ch < nch; ch += 4) {
-            const int kv0 = cw.b;
+            const int kv0 = kvb + cw.b;
             cw.next();
             TRecord rc;
             *reinterpret_cast<uint4*>(&rc) = rnext;
@@ -1242,7 +1258,8 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
             t_record<R, CS, PK>((pd.keep & 0x8421u) != 0, rc, base, st_stride, cbr, KV, kv0, kv0 + 1, acc, pd.keep);
           }
           const R v = warp_transpose_sum<R>(acc, lane);
-          if (pd.keep & (1u << (lane >> 1))) atomicAdd(tsm + ip * 32 + lane, v);
+          if (pd.keep & (1u << (lane >> 1)))
+            atomicAdd(tsm + (gi * g.npass + ip) * 32 + lane, v);
         }
       } else {
       for (int ip = 0; ip < g.npass; ++ip) {
@@ -1289,7 +1306,9 @@ __device__ __forceinline__ void sweep_body(const SweepGeom& g, const P& prog, co
         const int slot = (i & 31) >> 1;
         if (!(pd.keep & (1u << slot))) continue;
         const int p = pd.q[slot >> 2], q = pd.q[slot & 3];
-        atomicAdd(g.T + 2 * (p * g.norb + q) + (i & 1), (double)tsm[i]);
+        double v = (double)tsm[i];
+        for (int gi = 1; gi < ngrp; ++gi) v += (double)tsm[gi * g.npass * 32 + i];
+        atomicAdd(g.T + 2 * (p * g.norb + q) + (i & 1), v);
       }
     } else if (g.T) {
       const int lane = tid & 31;
