@@ -328,6 +328,7 @@ static void set_packed_geom(SweepGeom& g, Space* sp, int W, int nk) {
 // string, so that the eight lanes of a phase, whose strings lie in distinct
 // banks, keep them distinct (reverse sweep of N = 12 (6,6), 8 vectors a slab:
 // 131 to 135 us at a pitch of 8, 84 to 104 at 9).
+constexpr size_t kStaticSlack = 1024;  // for a kernel's static shared memory
 static int packed_pitch(int nst, int nv) {
   return nst == 2 ? (nv > 1 ? nv | 1 : nv) : nv > 2 ? 2 * (nv / 2 | 1) : nv;
 }
@@ -674,7 +675,9 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
     double best = -1;
     for (int kv = unit; kv <= kMaxKV && kv < g.nvec + unit; kv += unit) {
       // (pass sums per g.tgrp vectors)
-      if (smem_for(1, kv) + (kv / unit - 1) * (nst == 1 ? 0 : tsum) > budget) break;
+      if (smem_for(1, kv) + (nst == 1 || kv == unit ? 0 : (kv / unit - 1) * tsum + kStaticSlack) >
+          budget)
+        break;
       const int slabs = (g.nvec + kv - 1) / kv, last = slabs % slots;
       const double waves = slabs / slots + (last == 0 ? 0.0
                                             : two_per_sm && last <= slots / 2 ? 0.6 : 1.0);
@@ -689,7 +692,7 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
   const int nslabs = (g.nvec + KV - 1) / KV;
   if (dtype == FS_C64 && CS == 1) {
     const int p = packed_pitch(nst, KV);
-    if (smem_for(1, p) + tsum * (KV / g.tgrp) <= budget) KV = p;
+    if (smem_for(1, p) + tsum * (KV / g.tgrp - 1) + kStaticSlack <= budget) KV = p;
   }
   g.KV = KV;
   set_cluster_layout(g, sthis, CS, [&](int chunk) {
@@ -729,13 +732,13 @@ int batch_window(int dtype, int nst) {
 // one-job launch of the batched kernel, on scratch states (and scratch W
 // and T for the reverse sweeps), for every slab width 2^0 .. 2^lgmax that
 // fits the stage's budget; CUDA events on a private stream, the fastest
-// mean of two launches after one warm-up wins (the narrower slab, whose FP32
-// sums are shorter, unless the wider one gains 5 %) and is cached per sector
-// and sweep kind.  Runs before any capture.
-template <typename SmemFor, typename Pitch>
+// mean of two launches after one warm-up wins and is cached per sector and
+// sweep kind.  Runs before any capture.
+template <typename SmemFor, typename Pitch, typename Group>
 static int tune_batch_slab(Ctx* ctx, Space* sthis, int W, const SweepGeom& g0, const std::vector<unsigned char>& prog,
                            int nst, int dtype, bool rev, int lgmin, int lgmax,
-                           SmemFor&& smem_for, Pitch&& pitch_for, const std::array<int, 8>& key) {
+                           SmemFor&& smem_for, Pitch&& pitch_for, Group&& group_for,
+                           const std::array<int, 8>& key) {
   if (!ctx->tune_stream)
     FS_CUDA(cudaStreamCreateWithFlags(&ctx->tune_stream, cudaStreamNonBlocking));
   cudaStream_t ts = ctx->tune_stream;
@@ -764,8 +767,9 @@ static int tune_batch_slab(Ctx* ctx, Space* sthis, int W, const SweepGeom& g0, c
   std::vector<float> ms(lgmax + 1, 0.f);
   int best = lgmin;
   for (int lg = lgmin; lg <= lgmax; ++lg) {
-    g.nv = g.tgrp = 1 << lg;
-    g.KV = pitch_for(1 << lg);
+    g.nv = 1 << lg;
+    g.tgrp = group_for(g.nv);
+    g.KV = pitch_for(g.nv);
     if (dtype == FS_C64 && (nst == 2 || lgmin > 0))
       set_packed_geom(g, sthis, W, nst == 2 ? g.nv : g.nv / 2);
     SweepJob j{};
@@ -774,7 +778,7 @@ static int tune_batch_slab(Ctx* ctx, Space* sthis, int W, const SweepGeom& g0, c
     j.X = dX;
     j.item0 = 0;
     const int nslabs = (g.nvec + (1 << lg) - 1) >> lg;
-    const size_t smem = smem_for(g.KV);
+    const size_t smem = smem_for(g.KV, g.nv);
     FS_CUDA(cudaMemcpyAsync(djob, &j, sizeof(j), cudaMemcpyHostToDevice, ts));
     const bool pk = lgmin > 0;
     launch_sweep_batch(ctx, dtype, nst, nullptr, 0, 0, nullptr, smem, ts, pk);  // attribute
@@ -788,7 +792,7 @@ static int tune_batch_slab(Ctx* ctx, Space* sthis, int W, const SweepGeom& g0, c
     FS_CUDA(cudaEventSynchronize(e1));
     FS_CUDA(cudaEventElapsedTime(&tot, e0, e1));
     ms[lg] = tot / 2;
-    if (ms[lg] < 0.95f * ms[best]) best = lg;
+    if (ms[lg] < ms[best]) best = lg;
   }
   FS_CUDA(cudaEventDestroy(e0));
   FS_CUDA(cudaEventDestroy(e1));
@@ -837,10 +841,16 @@ void plan_batch_sweep(Ctx* ctx, Space* sa, Space* sb, int dir, void* st0, void* 
   const size_t tab_per_kv = ph.has_x ? g.nchunk * 256 * csz : 0;
   const size_t fixed = ph.has_x ? kMaxOrb * sizeof(double) : 0;
   const size_t tsum = (size_t)g.npass * 32 * (csz / 2);
-  auto smem_for = [&](int KV) {
-    return (size_t)KV * ((size_t)g.d * csz * nst + tab_per_kv + fixed) + tsum;
+  // FP32 transition sums run over a slab, in small spaces over each vector:
+  // there widths 1 and 2 tie (N = 8: 20.2 us both), and the gradients must not
+  // hang on which of them the autotuner met first
+  auto group_for = [&](int nv) { return dtype == FS_C64 && nst == 2 && g.d < 128 ? 1 : nv; };
+  // shared memory of nv vectors at a pitch of KV
+  auto smem_for = [&](int KV, int nv) {
+    return (size_t)KV * ((size_t)g.d * csz * nst + tab_per_kv + fixed) +
+           tsum * (size_t)(nv / group_for(nv));
   };
-  FS_REQUIRE(smem_for(1) <= budget, FS_ERR_UNSUPPORTED, "batched sweep slab does not fit");
+  FS_REQUIRE(smem_for(1, 1) <= budget, FS_ERR_UNSUPPORTED, "batched sweep slab does not fit");
   g.chunk = g.d;
   g.cb[0] = 0;
   g.cb[1] = g.d;
@@ -855,13 +865,15 @@ void plan_batch_sweep(Ctx* ctx, Space* sa, Space* sb, int dir, void* st0, void* 
   // slab width: the widest that fits the budget (at most 64 vectors), or the
   // autotuned width for this sector and sweep kind
   int lgmax = 0;
-  while ((2 << lgmax) <= std::min(g.nvec, kMaxKV) && smem_for(2 << lgmax) <= budget) ++lgmax;
+  while ((2 << lgmax) <= std::min(g.nvec, kMaxKV) &&
+         smem_for(2 << lgmax, 2 << lgmax) + (group_for(2) < 2 ? kStaticSlack : 0) <= budget)
+    ++lgmax;
   // complex64 forward sweeps: at least two vectors per slab, run as packed
   // vector pairs
   const int lgmin = dtype == FS_C64 && nst == 1 && lgmax >= 1 ? 1 : 0;
   auto pitch_for = [&](int nv) {
     const int p = dtype == FS_C64 && (nst == 2 || lgmin > 0) ? packed_pitch(nst, nv) : nv;
-    return smem_for(p) <= budget ? p : nv;
+    return smem_for(p, nv) + kStaticSlack <= budget ? p : nv;
   };
   const std::array<int, 8> key = {sthis->norb, sthis->nocc, sother->nocc, dtype, nst,
                                   rev != nullptr, ph.has_x, (int)(budget >> 10)};
@@ -871,7 +883,7 @@ void plan_batch_sweep(Ctx* ctx, Space* sa, Space* sb, int dir, void* st0, void* 
     lg = std::min(it->second, lgmax);
   } else if (ctx->batch_tuning && lgmax > lgmin) {
     lg = tune_batch_slab(ctx, sthis, W, g, out.prog, nst, dtype, rev != nullptr, lgmin, lgmax, smem_for,
-                         pitch_for, key);
+                         pitch_for, group_for, key);
   }
   if (lg < 0) {  // untuned: about eight slabs per circuit
     const int want = std::max(1, g.nvec / 8);
@@ -879,12 +891,13 @@ void plan_batch_sweep(Ctx* ctx, Space* sa, Space* sb, int dir, void* st0, void* 
     while ((2 << lg) <= std::min(want, kMaxKV) && lg < lgmax) ++lg;
   }
   lg = std::max(lg, lgmin);
-  g.nv = g.tgrp = 1 << lg;
-  g.KV = pitch_for(1 << lg);
+  g.nv = 1 << lg;
+  g.tgrp = group_for(g.nv);
+  g.KV = pitch_for(g.nv);
   if (dtype == FS_C64 && (nst == 2 || lgmin > 0))
     set_packed_geom(g, sthis, W, nst == 2 ? g.nv : g.nv / 2);
   out.nslabs = (g.nvec + (1 << lg) - 1) >> lg;
-  out.smem = smem_for(g.KV);
+  out.smem = smem_for(g.KV, g.nv);
   out.pk = lgmin > 0;
 }
 
