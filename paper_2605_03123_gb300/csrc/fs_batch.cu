@@ -28,7 +28,7 @@ __device__ __forceinline__ int find_job(const Job* jobs, int njobs, int64_t it) 
   return lo;
 }
 
-// Per-string factors (see launch_string_phase), one recipe per job.
+// Per-string factors (see StringPhases), one recipe per job.
 struct BStr {
   const uint32_t* masks;
   void* out;

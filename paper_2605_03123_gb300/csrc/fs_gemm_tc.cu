@@ -1,6 +1,5 @@
-// FP32-accurate GEMM on the tcgen05 tensor cores, for the dense contractions
-// of the library (the minor-matrix rotation, §2.3; the two-body contraction
-// of the operator action).
+// FP32-accurate GEMM on the tcgen05 tensor cores, for the dense contraction
+// of the library (the minor-matrix rotation, §2.3).
 //
 //   C[m][n] = sum_k A[m][k] B[n][k],   m < M, n < N, k < K,
 //
@@ -163,15 +162,6 @@ __global__ void __launch_bounds__(gtc::THREADS, 1)
           const float x0 = __uint_as_float(vv[jj >> 3][jj & 7]);
           const float x1 = __uint_as_float(vv[(jj + 1) >> 3][(jj + 1) & 7]);
           switch (g.mode) {
-            case GEMM_REAL:
-              if (n < g.N) reinterpret_cast<float*>(g.out)[(int64_t)m * g.ldo + n] = x0;
-              if (n + 1 < g.N) reinterpret_cast<float*>(g.out)[(int64_t)m * g.ldo + n + 1] = x1;
-              break;
-            case GEMM_REAL_T:
-              if (n < g.N) reinterpret_cast<float*>(g.out)[(int64_t)n * g.ldo + m] = x0;
-              if (n + 1 < g.N)
-                reinterpret_cast<float*>(g.out)[(int64_t)(n + 1) * g.ldo + m] = x1;
-              break;
             case GEMM_CPLX_T:
               if (n + 1 < g.N)
                 reinterpret_cast<float2*>(g.out)[(int64_t)(n >> 1) * g.ldo + m] =

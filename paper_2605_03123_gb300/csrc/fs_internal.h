@@ -194,14 +194,12 @@ struct Space {
     uint16_t* tc_idx[2] = {};
     int tc_seg_max[2] = {};  // largest segment, bytes
     // packed sweeps (W = 6): the orbits' gather addresses (window_rows_host)
-    // and, per number of packed sets in a slab, the work of a step in chunks
-    // of 32 items (window_chunks_host), window position a's from off[a] on
-    struct Chunks {
-      uint4* chunk = nullptr;
-      int* off = nullptr;
-    };
-    std::map<int, Chunks> pk_chunks;
-    std::vector<uint2> pk_cls;
+    // and, for every number nk of packed sets that a slab can hold, the work
+    // of a step in chunks of 32 items (window_chunks_host): from pk_at[nk - 1]
+    // on, window position a's from pk_off[(nk - 1) (npos + 1) + a] on
+    uint4* pk_chunk = nullptr;
+    int* pk_off = nullptr;
+    std::vector<int> pk_at;
     uint4* pk_rows = nullptr;
     std::vector<uint32_t> orb_h;
     std::vector<int> off_h;
@@ -673,13 +671,11 @@ void launch_masks(uint32_t* out, int norb, int nocc, cudaStream_t st);
 // C[m][n] = sum_k A[m][k] B[n][k] on the tcgen05 tensor cores with both
 // operands as three exact BF16 pieces (K contiguous, rows a multiple of 16
 // bytes apart), FP32 accuracy (fs_gemm_tc.cu).  Output forms:
-//   GEMM_REAL:          float out[m * ldo + n];
-//   GEMM_REAL_T:        float out[n * ldo + m];
 //   GEMM_CPLX_T:        N even, (C[m][2j], C[m][2j+1]) is the complex
 //                       float2 out[j * ldo + m];
 //   GEMM_CPLX_T_PLANES: as GEMM_CPLX_T, written as the three BF16 planes
 //                       outp[p] (row j, columns 2m, 2m + 1; row stride ldp).
-enum { GEMM_REAL = 0, GEMM_REAL_T = 1, GEMM_CPLX_T = 2, GEMM_CPLX_T_PLANES = 3 };
+enum { GEMM_CPLX_T = 0, GEMM_CPLX_T_PLANES = 1 };
 struct GemmTc {
   const uint16_t* A[3];
   const uint16_t* B[3];

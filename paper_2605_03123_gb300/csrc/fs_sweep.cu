@@ -185,10 +185,30 @@ static void build_window_tables(Space* sp, int W) {
   FS_CUDA(cudaMemcpy(wt.offs, offs.data(), offs.size() * 2, cudaMemcpyHostToDevice));
   if (W == window_width<float, 1>()) {  // packed sweeps
     std::vector<uint16_t> rows;
-    window_rows_host(sp->nocc, W, orbits, off, offs, wt.pk_cls, rows);
+    std::vector<uint2> cls;
+    window_rows_host(sp->nocc, W, orbits, off, offs, cls, rows);
+    // every width whose cells fit the 227 KB of a CTA, so that no later call
+    // allocates
+    wt.pk_at.clear();
+    std::vector<uint4> all, chunk;
+    std::vector<int> alloff, coff;
+    const int nkmax = (int)std::min<int64_t>(kMaxKV, std::max<int64_t>(1, 232448 / (16 * sp->dim)));
+    for (int nk = 1; nk <= nkmax; ++nk) {
+      window_chunks_host(W, nk, cls, coff, chunk);
+      wt.pk_at.push_back((int)all.size());
+      all.insert(all.end(), chunk.begin(), chunk.end());
+      alloff.insert(alloff.end(), coff.begin(), coff.end());
+    }
     FS_CUDA(cudaMalloc(&wt.pk_rows, std::max<size_t>(rows.size(), 8) * 2));
     if (!rows.empty())
       FS_CUDA(cudaMemcpy(wt.pk_rows, rows.data(), rows.size() * 2, cudaMemcpyHostToDevice));
+    FS_CUDA(cudaMalloc(&wt.pk_chunk, std::max<size_t>(all.size(), 1) * sizeof(uint4)));
+    if (!all.empty())
+      FS_CUDA(cudaMemcpy(wt.pk_chunk, all.data(), all.size() * sizeof(uint4),
+                         cudaMemcpyHostToDevice));
+    FS_CUDA(cudaMalloc(&wt.pk_off, alloff.size() * sizeof(int)));
+    FS_CUDA(cudaMemcpy(wt.pk_off, alloff.data(), alloff.size() * sizeof(int),
+                       cudaMemcpyHostToDevice));
   }
   wt.built = true;
 }
@@ -301,26 +321,12 @@ static void set_window_geom(SweepGeom& g, Space* sp, int W) {
   g.offs_stride = (sp->nocc + 1) << W;
 }
 
-// The packed tables of a slab of nk sets (at most one set of tables per width;
-// built on first use, as the window tables are).
-static void set_packed_geom(SweepGeom& g, Space* sp, int W, int nk) {
-  Space::Win& wt = sp->win[W];
-  Space::Win::Chunks& c = wt.pk_chunks[nk];
-  if (!c.off) {
-    std::vector<int> off;
-    std::vector<uint4> chunk;
-    window_chunks_host(W, nk, wt.pk_cls, off, chunk);
-    if (!c.chunk) FS_CUDA(cudaMalloc(&c.chunk, std::max<size_t>(chunk.size(), 1) * sizeof(uint4)));
-    if (!chunk.empty())
-      FS_CUDA(cudaMemcpy(c.chunk, chunk.data(), chunk.size() * sizeof(uint4),
-                         cudaMemcpyHostToDevice));
-    int* o = nullptr;
-    FS_CUDA(cudaMalloc(&o, off.size() * sizeof(int)));
-    FS_CUDA(cudaMemcpy(o, off.data(), off.size() * sizeof(int), cudaMemcpyHostToDevice));
-    c.off = o;
-  }
-  g.pk_chunk = c.chunk;
-  g.pk_off = c.off;
+// The packed tables of a slab of nk sets.
+static void set_packed_geom(SweepGeom& g, const Space* sp, int W, int nk) {
+  const Space::Win& wt = sp->win[W];
+  FS_REQUIRE(nk >= 1 && nk <= (int)wt.pk_at.size(), FS_ERR_UNSUPPORTED, "packed slab too wide");
+  g.pk_chunk = wt.pk_chunk + wt.pk_at[nk - 1];
+  g.pk_off = wt.pk_off + (size_t)(nk - 1) * (sp->norb - W + 2);
   g.pk_rows = wt.pk_rows;
 }
 

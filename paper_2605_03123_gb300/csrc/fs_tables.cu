@@ -275,10 +275,8 @@ void free_space(Space* s) {
     cudaFree(w.orbits);
     cudaFree(w.off);
     cudaFree(w.offs);
-    for (auto& c : w.pk_chunks) {
-      cudaFree(c.second.chunk);
-      cudaFree(c.second.off);
-    }
+    cudaFree(w.pk_chunk);
+    cudaFree(w.pk_off);
     cudaFree(w.pk_rows);
     for (int b = 0; b < 2; ++b) {
       cudaFree(w.tc_seg[b]);
