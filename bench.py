@@ -681,7 +681,7 @@ def run_trotter(args, ctx):
 def run_operator_action(args, ctx):
     """H psi for a molecular Hamiltonian with random real symmetric tensors
     (8-fold symmetric h_pqrs) at N=12 (6,6) and N=16 (4,4): milliseconds per
-    application and the GEMM rate (2 * N^2 * 3N^2 * 2 * dim flops)."""
+    application."""
     import torch
     from paper_2605_03123_gb300 import fsgpu, inputs
     res = {"unit": "ms per application"}
@@ -700,8 +700,7 @@ def run_operator_action(args, ctx):
             f = lambda: fsgpu.apply_molecular_hamiltonian(v, h1, h2, N, ne, out=o, ctx=ctx)
             f()
             ms = _timed(f, steps=2)
-            flops = 2 * N * N * 3 * N * N * 2 * dim
-            row[name] = {"ms": ms, "gemm_tflops": flops / (ms / 1e3) / 1e12}
+            row[name] = {"ms": ms}
             del v, o
         res["norb%d_nelec%d_%d" % (N, ne[0], ne[1])] = row
         del v0
