@@ -222,6 +222,13 @@ RotProgram decompose_adjacent(int n, const zd* U) {
   return prog;
 }
 
+bool RotProgram::finite() const {
+  auto ok = [](zd z) { return std::isfinite(z.real()) && std::isfinite(z.imag()); };
+  return std::all_of(phase.begin(), phase.end(), ok) &&
+         std::all_of(g.begin(), g.end(),
+                     [&](const Givens& x) { return std::isfinite(x.c) && ok(x.s); });
+}
+
 // Greedy grouping of a Givens sequence into window steps: repeatedly take
 // the window [a, a+W) that admits the most rotations whose earlier
 // neighbours (rotations sharing an orbital and preceding them) are done or

@@ -42,6 +42,9 @@ struct Givens {
 struct RotProgram {
   std::vector<Givens> g;
   std::vector<zd> phase;
+  // no entry is infinite or not a number (a matrix with NaNs passes the
+  // unitarity check)
+  bool finite() const;
 };
 
 void mat_mul(int n, const zd* A, const zd* B, zd* C);            // C = A B

@@ -726,12 +726,13 @@ static void hunit(int64_t* x, int n) {
 // of some 2^-52 into each entry, the same for every amplitude), the diagonal
 // layer multiplied into the last step that covers each orbital.  False when
 // the program does not suit the sweep: a phase falls outside every window, or
-// it has too many steps, or too few rotations a step.
+// it has too many steps, or too few rotations a step, or an entry that no
+// integer stands for (infinite, or not a number).
 static bool fx_steps(Ctx* ctx, const RotProgram& rp, int N, FxPlan& plan,
                      std::vector<std::array<int64_t, 72>>& V) {
   const std::vector<WinStep>& steps = window_schedule(ctx, rp, N, tc::kW);
   if (steps.empty() || (int)steps.size() > fx::kMaxSteps ||
-      rp.g.size() < fx::kMinGivensPerStep * steps.size())
+      rp.g.size() < fx::kMinGivensPerStep * steps.size() || !rp.finite())
     return false;
   std::vector<int> last(N, -1);
   for (size_t s = 0; s < steps.size(); ++s)

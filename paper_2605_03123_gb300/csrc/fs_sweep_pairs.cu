@@ -117,7 +117,8 @@ bool pairs_supported(const Ctx* ctx, const Space* sthis, const Space* sother, in
   if (dtype != FS_C128 || ctx->sweep_engine != FS_SWEEP_AUTO) return false;
   if (sthis->dim < 2 || sthis->dim > 512 || (int)rp.g.size() > pairs::kMaxM || rp.g.empty())
     return false;
-  if (sother->dim > 65535) return false;
+  // the diagonal layer is held as angles in integers
+  if (sother->dim > 65535 || !rp.finite()) return false;
   // modelled clocks: a rotation is a chain of about 350, or the FP64 issue of
   // its components on four units for the vectors of an SM.  The digit sweep
   // is flat at about 60 us with its images up to a few hundred vectors; the
