@@ -107,14 +107,24 @@ int fs_set_rotation_path(fs_ctx *ctx, int path);
  *   FS_SWEEP_AUTO:      complex64 on the CUDA cores (measured faster on GB300
  *                       at the benchmarked sectors, see FS_SWEEP_TENSOR);
  *                       complex128 on the tcgen05 tensor cores as exact
- *                       fixed-point digits (62 fraction bits relative to
- *                       each vector's 2-norm, so at least as accurate as
- *                       FP64 arithmetic) where the sector and the program
+ *                       fixed-point digits where the sector and the program
  *                       allow it, else in FP64 on the CUDA cores, as the
  *                       rotations of small spaces (up to a few hundred
- *                       strings), where that is faster.  In digits a vector
- *                       that holds a non-finite amplitude comes out not a
- *                       number throughout;
+ *                       strings), where that is faster.  Digits hold an
+ *                       amplitude to 2^-62 of its vector's 2-norm (one spin's
+ *                       strings at one string of the other) and round there
+ *                       once per window step, an absolute error, where FP64
+ *                       rounds at 2^-53 of the amplitudes mixed.  Vectors
+ *                       for which that is too coarse are rotated in FP64:
+ *                       under a rotation that leaves blocks of orbitals
+ *                       apart those with a nonzero amplitude below 2^-30 of
+ *                       the norm or a sixteenth of them below 2^-12, under
+ *                       any other those that come out with one below 2^-30
+ *                       or a sixteenth below 2^-22, and those with an
+ *                       infinity or a NaN.  In a vector that stays in digits
+ *                       an amplitude may keep fewer than FP64's 53 bits by
+ *                       those that it lies below 2^-9 of the norm
+ *                       (FS_SWEEP_CUDA_CORE keeps them);
  *   FS_SWEEP_CUDA_CORE: every Givens rotation as FP32 / FP64 FMAs on CUDA
  *                       cores;
  *   FS_SWEEP_TENSOR:    complex64 too: each window step of 6 adjacent

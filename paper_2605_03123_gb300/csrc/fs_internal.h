@@ -571,6 +571,7 @@ struct FxPlan {
   int nsteps = 0;
   uint8_t a[fx::kMaxSteps], full[fx::kMaxSteps];
   const unsigned char* img = nullptr;
+  bool weak = false, joined = false;  // which vectors take FP64 (see fs_sweep_fx.cu)
 };
 // The plans of a rotation's two spins (null: the spin takes the FP64 or FP32
 // sweep), with one launch for the images of both.  They live in the context's
@@ -606,9 +607,11 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir,
 // forward: spins that the small-space sweep takes get no plan.
 FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const RotProgram& pa,
                   const RotProgram& pb, bool forward, cudaStream_t st);
-// That sweep, on st0 and (unless null) st1, with the phase `ph` behind it.
+// That sweep of the program rp, on st0 and (unless null) st1, with the phase
+// `ph` behind it.
 void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0, void* st1,
-                     const FxPlan& plan, const PhaseDev& ph, cudaStream_t st);
+                     const FxPlan& plan, const RotProgram& rp, const PhaseDev& ph,
+                     cudaStream_t st);
 
 // The reductions behind a reverse fixed-point sweep (fs_trans_fx.cu): T += the
 // transition sums of this spin (its pass tables are built), if supported.

@@ -537,12 +537,12 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
                   const PhaseDev& ph, cudaStream_t st, const RevArgs* rev, const FxPlan* fx) {
   if (fx) {
     if (nst == 1) {
-      launch_sweep_fx(ctx, sa, sb, dir, st0, nullptr, *fx, ph, st);
+      launch_sweep_fx(ctx, sa, sb, dir, st0, nullptr, *fx, rp, ph, st);
       return;
     }
     // reverse: both states rotated, the transition sums, then W and the second
     // phase (as a sweep without rotations where the sums do not fit one CTA)
-    launch_sweep_fx(ctx, sa, sb, dir, st0, st1, *fx, PhaseDev{}, st);
+    launch_sweep_fx(ctx, sa, sb, dir, st0, st1, *fx, rp, PhaseDev{}, st);
     Space* sthis = const_cast<Space*>(dir == 0 ? sa : sb);
     if (sthis->norb >= 4 && sthis->nocc >= 1) build_tpass_tables(sthis);
     if (rev->T && trans_fx_supported(ctx, sthis)) {

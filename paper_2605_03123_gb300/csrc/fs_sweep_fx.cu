@@ -19,6 +19,19 @@
 // the step's images in shared memory accumulate in seven TMEM accumulators;
 // the warps read those back, join them and scatter the new amplitudes.
 //
+// Integers keep an amplitude to some 2^-60 of its vector's norm, FP64
+// rotations to 2^-53 of the amplitudes that it is mixed with.  With all
+// amplitudes x_j in one range those are at least min |x_j| (the rows of a
+// rotation have 2-norm 1), and the digits keep more; a vector with a wide range
+// (a determinant and its weakly coupled excitations, a block of a
+// block-diagonal rotation that hardly counts) would lose its small ones, and
+// integers cannot carry infinities and NaNs.  The CTA sees both when it loads a
+// vector (see Range) and rotates such vectors in FP64 instead, one rotation
+// after another on the pairs of strings, behind the others.  All vectors of a
+// state so, both spins, against the FP64 sweeps: N = 11 (6,5) 0.20 against 0.25
+// ms, N = 13 (5,7) 1.33 against 1.55, N = 14 (7,7) 7.9 against 6.5 (two vectors a
+// CTA leave the FP64 units waiting at the barrier of each rotation).
+//
 // Measured (one GB300, one spin, complex128): N = 14 (7,7) 1.52 ms against
 // 6.74 ms of the FP64 sweep, which runs at 0.8 of the FP64 rate (2 FMA per
 // clock and SM); N = 12 (6,6) 0.105 against 0.80 ms; N = 8 (4,4) 32 + 18
@@ -280,6 +293,34 @@ __device__ __forceinline__ void scatter(longlong2* slab, const Item& it, int h,
   }
 }
 
+// What decides how a vector is rotated: its range, wide when a nonzero
+// amplitude lies below 2^-kTinyBits of its 2-norm (by the exponent of its larger
+// part), or a sixteenth of them below 2^-kSmallBits or 2^-kApartBits.
+//   A program that leaves blocks of orbitals apart keeps each block of a vector
+// to its own accuracy in FP64, so that a vector whose range is wide when it is
+// loaded goes to FP64 (kApartBits: below 2^-9 of the norm the digits' 62 bits are
+// fewer than FP64's 53, at 2^-12 three fewer; a random vector of 3432 strings
+// has 2^-6 on average and one amplitude in 2^10 there).
+//   A program that joins all orbitals brings the rounding of the large
+// amplitudes into the small ones in FP64 too.  There a wide range has to come
+// out of the rotation as well, and the line (kSmallBits) lies below what the
+// ansatz states near a determinant hold (12 orbitals, generators of 0.1: the last
+// sixteenth of a vector at 2^-15 to 2^-20), whose sweeps would take 5 to 8 times
+// as long.
+//   A vector that starts with zeros is judged by its result under both, since
+// what comes into them may be small (a determinant under a weak rotation); under
+// a program with a rotation weaker than 2^-kWeakBits, where amplitudes could
+// vanish altogether in between, it goes to FP64.
+constexpr int kTinyBits = 30, kSmallBits = 22, kApartBits = 12, kWeakBits = 12;
+// Orbitals are joined when the product of the rotations' moduli connects each
+// to each by at least 2^-kJoinBits (random unitaries 2^-5 to 2^-8, generators
+// with entries of 0.1 2^-6 to 2^-11, of 0.001 2^-12 to 2^-17).
+constexpr int kJoinBits = 12;
+struct Range {  // per vector: nonzero amplitudes << 16 | small ones (both below 2^14)
+  uint32_t in[kMaxVec], out[kMaxVec];
+  uint32_t tiny_in, tiny_out;  // bit per vector
+};
+
 struct Args {
   double2* st[2];  // blockIdx.y chooses: psi and the cotangent share a program
   int64_t d_b;
@@ -293,11 +334,97 @@ struct Args {
   int* status;
   uint8_t a[kMaxSteps];     // window position of each step
   uint8_t full[kMaxSteps];  // class 6 moves in this step (det V != 1)
+  // the program rotation by rotation, for vectors that take FP64
+  const uint32_t* pairs;  // adjacent pair lists
+  int npp, m, weak, joined;
+  long long phase[2 * kMaxOrb];  // the diagonal layer, fixed point
+  double c[kMaxGivens], sr[kMaxGivens], si[kMaxGivens];
+  int8_t p[kMaxGivens];
 };
+
+__device__ __forceinline__ bool not_zero(double2 x) {
+  return ((__double2hiint(x.x) | __double2hiint(x.y)) & 0x7FFFFFFF) | __double2loint(x.x) |
+         __double2loint(x.y);
+}
 
 // A barrier of the sixteen data warps.
 __device__ __forceinline__ void sync_data() {
   asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory");
+}
+
+// The vectors of `wide` (bit per vector of the slab) in FP64, by all data
+// threads: from the state into their cells, rotation by rotation over the pairs
+// of all of them (a pair list entry is read while the one before it is used),
+// with the phases back to the state.  dtab: where the images were, for the
+// diagonal layer (8 orbitals an entry); tab: the cross tables (null: none), bad_x the orbitals without an
+// angle there; at: scratch for the first cells of the vectors.
+static_assert((kMaxOrb + 7) / 8 * 256 * 16 <= kImgBytes, "");
+__device__ __noinline__ void rotate_fp64(const Args& g, uint32_t wide, double2* slab,
+                                         double2* state, longlong2* dtab, const longlong2* tab,
+                                         const uint32_t* bad_x, int* at, int v0, int nv, int tid) {
+  const int nw = __popc(wide), d = g.d, npp = g.npp, m = g.m, items = npp * nw;
+  auto each = [&](auto&& f) {  // (vector, element, its place in the state)
+    if (g.dir == 1) {
+      for (uint32_t w = wide; w; w &= w - 1) {
+        const int kv = __ffs(w) - 1;
+        for (int e = tid; e < d; e += kThreads) f(kv, e, (int64_t)(v0 + kv) * g.d_b + e);
+      }
+    } else {
+      for (int i = tid; i < d * nv; i += kThreads) {
+        const int e = i / nv, kv = i - e * nv;
+        if ((wide >> kv) & 1) f(kv, e, (int64_t)e * g.d_b + v0 + kv);
+      }
+    }
+  };
+  each([&](int kv, int e, int64_t s) { slab[(size_t)kv * d + e] = state[s]; });
+  if (tid < nv && ((wide >> tid) & 1)) at[__popc(wide & ((1u << tid) - 1))] = tid * d;
+  for (int i = tid; i < g.nchunk * 256; i += kThreads) {
+    const uint64_t mask = (uint64_t)(i & 255) << (i / 256 * 8) & ((1ull << g.norb) - 1);
+    longlong2 z = make_longlong2(1ll << 62, 0);
+    for (uint32_t b = (uint32_t)mask; b; b &= b - 1) {
+      const int p = __ffs(b) - 1;
+      z = phase_mul(z, make_longlong2(g.phase[2 * p], g.phase[2 * p + 1]));
+    }
+    dtab[i] = z;
+  }
+  sync_data();
+  const int first = tid % npp;
+  uint32_t next = tid < items ? __ldg(g.pairs + (int64_t)g.p[0] * npp + first) : 0u;
+  for (int k = 0; k < m; ++k) {
+    const uint32_t* l = g.pairs + (int64_t)g.p[k] * npp;
+    const double c = g.c[k], sr = g.sr[k], si = g.si[k];
+    int w = tid / npp;
+    for (int i = tid; i < items;) {
+      const uint32_t pr = next;
+      double2* x = slab + at[w];
+      i += kThreads;
+      if (i < items) {
+        w = i / npp;
+        next = __ldg(l + (i - w * npp));
+      } else if (k + 1 < m) {
+        next = __ldg(g.pairs + (int64_t)g.p[k + 1] * npp + first);
+      }
+      double2 a = x[pr & 0xFFFFu], b = x[pr >> 16];
+      givens2<double>(a, b, c, sr, si);
+      x[pr & 0xFFFFu] = a;
+      x[pr >> 16] = b;
+    }
+    sync_data();
+  }
+  each([&](int kv, int e, int64_t s) {
+    const uint32_t bits = __ldg(g.masks_this + e);
+    const longlong2* t = tab ? tab + kv * g.nchunk * 256 : nullptr;
+    longlong2 f = make_longlong2(1ll << 62, 0);
+    for (int k = 0; k < g.nchunk; ++k) {
+      const int v = k * 256 + ((bits >> (8 * k)) & 255);
+      f = k ? phase_mul(f, dtab[v]) : dtab[v];
+      if (t) f = phase_mul(f, t[v]);
+    }
+    double2 z = phase_to(f);
+    if (g.ea_this) z = cmul<double>(z, __ldg(g.ea_this + e));
+    if (g.ea_other) z = cmul<double>(z, __ldg(g.ea_other + v0 + kv));
+    state[s] = t && (bits & bad_x[kv]) ? nan2() : cmul<double>(z, slab[(size_t)kv * d + e]);
+  });
 }
 
 // Walks the tiles of a step: class cls(ci), rows row0 ..; ci = 5 past the
@@ -328,6 +455,7 @@ __global__ void __launch_bounds__(kCta, 1)
   __shared__ float s_sum[kMaxVec][kWarps];
   __shared__ Seg s_seg[kMaxSteps];
   __shared__ int s_eb[kMaxVec];  // biased exponent of the scale, -1: not finite
+  __shared__ Range s_range;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   double2* const state = g.st[blockIdx.y];
   const int d = g.d, v0 = blockIdx.x * g.KV, nv = min(g.KV, g.nvec - v0);
@@ -344,32 +472,62 @@ __global__ void __launch_bounds__(kCta, 1)
   }
   if (warp == 0) tc::tmem_alloc(tc::smem_u32(&s_tmem), 512);
   for (int i = tid; i < g.nsteps; i += kCta) s_seg[i] = g.seg[g.a[i]];
+  if (tid < kMaxVec) s_range.in[tid] = s_range.out[tid] = 0;
+  if (tid == 0) s_range.tiny_in = s_range.tiny_out = 0;
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
+  // bits per vector, the same in all threads: the vectors of a wide range as
+  // counted, of zeros throughout, and (the first, before any rotation) those
+  // that go to FP64 at once and those that are judged by their result
+  const uint32_t small_bits = g.joined ? kSmallBits : kApartBits;
+  auto wide_range = [&](const uint32_t (&count)[kMaxVec], uint32_t tiny) {
+    return tiny | __ballot_sync(0xFFFFFFFFu,
+                                lane < nv && (count[lane] & 0xFFFFu) * 16 > (uint32_t)d);
+  };
+  auto judge = [&](uint32_t& zero, uint32_t& later) {
+    const uint32_t nz = lane < nv ? s_range.in[lane] >> 16 : 0;
+    const bool fin = lane < nv && s_eb[lane] >= 0;
+    zero = __ballot_sync(0xFFFFFFFFu, fin && nz == 0);
+    const uint32_t some = __ballot_sync(0xFFFFFFFFu, fin && nz > 0 && nz < (uint32_t)d);
+    const uint32_t range = wide_range(s_range.in, s_range.tiny_in) & ~zero;
+    const uint32_t now = __ballot_sync(0xFFFFFFFFu, lane < nv && !fin) |
+                         (g.weak ? some : 0) | (g.joined ? 0 : range);
+    later = (some | range) & ~now;
+    return now;
+  };
+  const uint32_t all = nv == 32 ? 0xFFFFFFFFu : (1u << nv) - 1;
   if (warp == kWarps) {
+    // a step's images and gather addresses: class 3, then the other
+    // classes, each copy issued once the step before has used its half
+    auto stage_first = [&](int st) {
+      const Seg& q = s_seg[st];
+      const uint32_t len = 2u * (uint32_t)(q.start[1] - q.start[0]);
+      tc::mbar_expect_tx(bar_first, kImgFirst + len);
+      tc::bulk_g2s(tc::smem_u32(simg), g.img + (size_t)st * kStepBytes, kImgFirst, bar_first);
+      if (len) tc::bulk_g2s(tc::smem_u32(ix_first), g.idx + q.start[0], len, bar_first);
+    };
+    auto stage_rest = [&](int st) {
+      const Seg& q = s_seg[st];
+      const uint32_t len = 2u * (uint32_t)(q.start[5] - q.start[1]);
+      tc::mbar_expect_tx(bar_rest, kImgBytes - kImgFirst + len);
+      tc::bulk_g2s(tc::smem_u32(simg) + kImgFirst, g.img + (size_t)st * kStepBytes + kImgFirst,
+                   kImgBytes - kImgFirst, bar_rest);
+      if (len) tc::bulk_g2s(tc::smem_u32(ix_rest), g.idx + q.start[1], len, bar_rest);
+    };
     if (lane == 0) {
-      // a step's images and gather addresses: class 3, then the other
-      // classes, each copy issued once the step before has used its half
-      auto stage_first = [&](int st) {
-        const Seg& q = s_seg[st];
-        const uint32_t len = 2u * (uint32_t)(q.start[1] - q.start[0]);
-        tc::mbar_expect_tx(bar_first, kImgFirst + len);
-        tc::bulk_g2s(tc::smem_u32(simg), g.img + (size_t)st * kStepBytes, kImgFirst, bar_first);
-        if (len) tc::bulk_g2s(tc::smem_u32(ix_first), g.idx + q.start[0], len, bar_first);
-      };
-      auto stage_rest = [&](int st) {
-        const Seg& q = s_seg[st];
-        const uint32_t len = 2u * (uint32_t)(q.start[5] - q.start[1]);
-        tc::mbar_expect_tx(bar_rest, kImgBytes - kImgFirst + len);
-        tc::bulk_g2s(tc::smem_u32(simg) + kImgFirst, g.img + (size_t)st * kStepBytes + kImgFirst,
-                     kImgBytes - kImgFirst, bar_rest);
-        if (len) tc::bulk_g2s(tc::smem_u32(ix_rest), g.idx + q.start[1], len, bar_rest);
-      };
-      const uint32_t tbase = s_tmem, bimg = tc::smem_u32(simg);
-      uint32_t ph = 0, phr = 0;  // phases of the products and of the data warps
       stage_first(0);
       stage_rest(0);
+    }
+    __syncthreads();  // the vectors are loaded
+    uint32_t zero, later;
+    const bool skip = (judge(zero, later) | zero) == all;
+    if (lane == 0 && skip) {  // no tiles: the copies have to land all the same
+      if (!tc::mbar_wait(bar_first, 0)) timeout(g.status);
+      if (!tc::mbar_wait(bar_rest, 0)) timeout(g.status);
+    } else if (lane == 0) {
+      const uint32_t tbase = s_tmem, bimg = tc::smem_u32(simg);
+      uint32_t ph = 0, phr = 0;  // phases of the products and of the data warps
       for (int st = 0; st < g.nsteps; ++st) {
         const Seg& sg = s_seg[st];
         const uint32_t phs = (uint32_t)st & 1u;
@@ -478,11 +636,22 @@ __global__ void __launch_bounds__(kCta, 1)
       const bool finite = f < 0x7FF;
       const int eb = norm_exponent((int)f, s);
       if (sub == 0 && lane == 0) s_eb[kv] = finite ? eb : -1;
+      uint32_t count = 0, tiny = 0;
 #pragma unroll 4
     for (int e = sub * 32 + lane; e < d; e += 32 * per) {
         const double2 x = raw[(size_t)kv * d + e];
         slab[(size_t)kv * d + e] = finite ? make_longlong2(from_double(x.x, eb), from_double(x.y, eb))
                                           : make_longlong2(0, 0);
+        const int q = max(exp_field(x.x), exp_field(x.y));
+        const bool nz = q || not_zero(x);
+        count += nz ? 0x10000u + (q < eb - (int)small_bits) : 0u;
+        tiny |= nz && q < eb - kTinyBits;
+      }
+      count = __reduce_add_sync(0xFFFFFFFFu, count);
+      tiny = __reduce_or_sync(0xFFFFFFFFu, tiny);
+      if (lane == 0) {
+        atomicAdd(&s_range.in[kv], count);
+        if (tiny) atomicOr(&s_range.tiny_in, 1u << kv);
       }
     }
   Thread t;
@@ -490,11 +659,18 @@ __global__ void __launch_bounds__(kCta, 1)
   t.row = (warp & 3) * 32 + lane;
   t.lane0 = s_tmem + ((uint32_t)((warp & 3) * 32) << 16);
   uint32_t ph_mma = 0;
-  sync_data();
+  __syncthreads();  // with the issuing warp
+  uint32_t zero, later;
+  uint32_t wide = judge(zero, later);
+  const bool skip = (wide | zero) == all;
+  if (skip) {  // the tables below go where the copies land
+    if (!tc::mbar_wait(bar_first, 0)) timeout(g.status);
+    if (!tc::mbar_wait(bar_rest, 0)) timeout(g.status);
+  }
   // ---- window steps.  The tiles of a step touch different strings, so
   // they run as a pipeline: while the products of one tile run, the warps
   // join and scatter the tile before it and gather the tile after it.
-  for (int st = 0; st < g.nsteps; ++st) {
+  for (int st = 0; st < g.nsteps && !skip; ++st) {
     const Seg& sg = s_seg[st];
     const uint32_t ph = (uint32_t)st & 1u;
     Walk wk;
@@ -584,6 +760,26 @@ __global__ void __launch_bounds__(kCta, 1)
     tc::fence_after();
     tc::tmem_dealloc(s_tmem, 512);
   }
+  // ---- the range of the vectors that are judged by it now
+  if (later) {
+    for (int kv = 0; kv < nv; ++kv) {
+      if (!((later >> kv) & 1)) continue;
+      uint32_t count = 0, tiny = 0;
+      for (int e = tid; e < d; e += kThreads) {
+        const longlong2 x = slab[(size_t)kv * d + e];
+        const unsigned long long u =
+            (unsigned long long)(x.x < 0 ? -x.x : x.x) | (unsigned long long)(x.y < 0 ? -x.y : x.y);
+        count += u && u < 1ull << (kFrac - small_bits);
+        tiny |= u && u < 1ull << (kFrac - kTinyBits);
+      }
+      count = __reduce_add_sync(0xFFFFFFFFu, count);
+      tiny = __reduce_or_sync(0xFFFFFFFFu, tiny);
+      if (lane == 0 && count) atomicAdd(&s_range.out[kv], count);
+      if (lane == 0 && tiny) atomicOr(&s_range.tiny_out, 1u << kv);
+    }
+    sync_data();
+    wide |= later & wide_range(s_range.out, s_range.tiny_out);
+  }
   // ---- phases, store.  The cross tables go where the images were (every
   // copy has landed and been read).
   const int tper = g.nchunk * 256;
@@ -594,7 +790,7 @@ __global__ void __launch_bounds__(kCta, 1)
   auto finish = [&](int kv, int e) {
     const int eb = s_eb[kv];
     longlong2 c = slab[(size_t)kv * d + e];
-    bool bad = eb < 0;
+    bool bad = false;
     if (g.has_x || g.ea_this || g.ea_other) {
       longlong2 f = make_longlong2(1ll << 62, 0);
       auto factor = [&](double2 z) {
@@ -616,13 +812,21 @@ __global__ void __launch_bounds__(kCta, 1)
   };
   if (g.dir == 1) {
     for (int kv = 0; kv < nv; ++kv)
-      for (int e = tid; e < d; e += kThreads)
-        state[(int64_t)(v0 + kv) * g.d_b + e] = finish(kv, e);
+      if (!((wide >> kv) & 1))
+        for (int e = tid; e < d; e += kThreads)
+          state[(int64_t)(v0 + kv) * g.d_b + e] = finish(kv, e);
   } else {
     for (int i = tid; i < d * nv; i += kThreads) {
       const int e = i / nv, kv = i - e * nv;
-      state[(int64_t)e * g.d_b + v0 + kv] = finish(kv, e);
+      if (!((wide >> kv) & 1)) state[(int64_t)e * g.d_b + v0 + kv] = finish(kv, e);
     }
+  }
+  // ---- the others, still as they were in the state, in FP64
+  if (wide) {
+    sync_data();  // the tables are read
+    rotate_fp64(g, wide, raw, state, reinterpret_cast<longlong2*>(simg),
+                g.has_x ? tab : nullptr, &s_max[0][0], reinterpret_cast<int*>(&s_sum[0][0]), v0,
+                nv, tid);
   }
 }
 
@@ -721,6 +925,12 @@ static void hunit(int64_t* x, int n) {
   for (int i = 0; i < n; ++i) x[i] += hmul(x[i], h);
 }
 
+static void unit_phase(zd d, int64_t* z) {
+  z[0] = hfix(d.real());
+  z[1] = hfix(d.imag());
+  hunit(z, 2);
+}
+
 // The steps of a program (into plan and, as unitaries V, row-major 6 x 6
 // complex fixed point, into V: products of FP64 matrices would put an error
 // of some 2^-52 into each entry, the same for every amplitude), the diagonal
@@ -739,6 +949,22 @@ static bool fx_steps(Ctx* ctx, const RotProgram& rp, int N, FxPlan& plan,
     for (int p = steps[s].a; p < steps[s].a + tc::kW; ++p) last[p] = (int)s;
   for (int p = 0; p < N; ++p)
     if (last[p] < 0 && rp.phase[p] != zd(1.0)) return false;
+  // what the moduli of the rotations join (see Range)
+  std::vector<double> join((size_t)N * N, 0.0);
+  for (int p = 0; p < N; ++p) join[(size_t)p * N + p] = 1.0;
+  plan.weak = false;
+  for (const Givens& G : rp.g) {
+    const double c = std::abs(G.c), s = std::abs(G.s), weaker = std::min(c, s);
+    plan.weak = plan.weak || (weaker > 0 && weaker < std::ldexp(1.0, -fx::kWeakBits));
+    double* x = join.data() + (size_t)G.p * N;
+    for (int j = 0; j < N; ++j) {
+      const double u = x[j], v = x[N + j];
+      x[j] = c * u + s * v;
+      x[N + j] = s * u + c * v;
+    }
+  }
+  plan.joined =
+      *std::min_element(join.begin(), join.end()) >= std::ldexp(1.0, -fx::kJoinBits);
   plan.nsteps = (int)steps.size();
   V.resize(steps.size());
   for (size_t s = 0; s < steps.size(); ++s) {
@@ -763,8 +989,8 @@ static bool fx_steps(Ctx* ctx, const RotProgram& rp, int N, FxPlan& plan,
     plan.full[s] = 0;
     for (int p = a; p < a + tc::kW; ++p) {
       if (last[p] != (int)s || rp.phase[p] == zd(1.0)) continue;
-      int64_t z[2] = {hfix(rp.phase[p].real()), hfix(rp.phase[p].imag())};
-      hunit(z, 2);
+      int64_t z[2];
+      unit_phase(rp.phase[p], z);
       int64_t* x = M.data() + 12 * (p - a);
       for (int j = 0; j < 6; ++j) {
         const int64_t re = hmul(x[2 * j], z[0]) - hmul(x[2 * j + 1], z[1]);
@@ -841,7 +1067,8 @@ FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const R
 }
 
 void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0, void* st1,
-                     const FxPlan& plan, const PhaseDev& ph, cudaStream_t st) {
+                     const FxPlan& plan, const RotProgram& rp, const PhaseDev& ph,
+                     cudaStream_t st) {
   const Space* sthis = dir == 0 ? sa : sb;
   const Space* sother = dir == 0 ? sb : sa;
   fx::build_index(const_cast<Space*>(sthis));
@@ -857,6 +1084,25 @@ void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* 
   std::copy(plan.a, plan.a + plan.nsteps, g.a);
   std::copy(plan.full, plan.full + plan.nsteps, g.full);
   g.img = plan.img;
+  g.pairs = sthis->pairs;
+  g.npp = sthis->npp;
+  g.m = (int)rp.g.size();
+  FS_REQUIRE(g.m <= kMaxGivens, FS_ERR_ARG, "too many Givens rotations");
+  for (int k = 0; k < g.m; ++k) {
+    const Givens& G = rp.g[k];
+    g.p[k] = (int8_t)G.p;
+    g.c[k] = G.c;
+    g.sr[k] = G.s.real();
+    g.si[k] = G.s.imag();
+  }
+  g.weak = plan.weak;
+  g.joined = plan.joined;
+  for (int p = 0; p < sthis->norb; ++p) {
+    int64_t z[2];
+    unit_phase(rp.phase[p], z);
+    g.phase[2 * p] = z[0];
+    g.phase[2 * p + 1] = z[1];
+  }
   g.norb = sthis->norb;
   g.nchunk = (sthis->norb + 7) / 8;
   g.has_x = ph.has_x;
