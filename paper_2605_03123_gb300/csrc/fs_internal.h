@@ -608,16 +608,18 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir,
 FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const RotProgram& pa,
                   const RotProgram& pb, bool forward, cudaStream_t st);
 // That sweep of the program rp, on st0 and (unless null) st1, with the phase
-// `ph` behind it.
+// `ph` behind it.  scale (null: not wanted): per state and vector, the biased
+// exponent of a power of two above its 2-norm, -1 where it was rotated in FP64.
 void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0, void* st1,
                      const FxPlan& plan, const RotProgram& rp, const PhaseDev& ph,
-                     cudaStream_t st);
+                     cudaStream_t st, int* scale = nullptr);
 
 // The reductions behind a reverse fixed-point sweep (fs_trans_fx.cu): T += the
-// transition sums of this spin (its pass tables are built), if supported.
+// transition sums of this spin (its pass tables are built), if supported;
+// scale as that sweep wrote it.
 bool trans_fx_supported(const Ctx* ctx, const Space* sthis);
 void launch_trans_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, const void* psi,
-                     const void* g, double* T, cudaStream_t st);
+                     const void* g, const int* scale, double* T, cudaStream_t st);
 // Then W and the second phase of both states, as launch_sweep's reverse mode.
 void launch_rev_phase(const Space* sa, const Space* sb, void* psi, void* cot, int dtype,
                       const RevArgs& rev, const PhaseDev& ph, cudaStream_t st);

@@ -542,11 +542,15 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
     }
     // reverse: both states rotated, the transition sums, then W and the second
     // phase (as a sweep without rotations where the sums do not fit one CTA)
-    launch_sweep_fx(ctx, sa, sb, dir, st0, st1, *fx, rp, PhaseDev{}, st);
     Space* sthis = const_cast<Space*>(dir == 0 ? sa : sb);
     if (sthis->norb >= 4 && sthis->nocc >= 1) build_tpass_tables(sthis);
-    if (rev->T && trans_fx_supported(ctx, sthis)) {
-      launch_trans_fx(ctx, sa, sb, dir, st0, st1, rev->T, st);
+    const bool trans = rev->T && trans_fx_supported(ctx, sthis);
+    int* scale = nullptr;
+    if (trans)
+      scale = (int*)scratch(ctx, "fx_scale", 2 * (dir == 0 ? sb : sa)->dim * sizeof(int));
+    launch_sweep_fx(ctx, sa, sb, dir, st0, st1, *fx, rp, PhaseDev{}, st, scale);
+    if (trans) {
+      launch_trans_fx(ctx, sa, sb, dir, st0, st1, scale, rev->T, st);
       if (rev->W || rev->ea2_a || rev->ea2_b || ph.has_x)
         launch_rev_phase(sa, sb, st0, st1, dtype, *rev, ph, st);
       return;

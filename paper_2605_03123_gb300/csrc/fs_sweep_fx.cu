@@ -332,6 +332,7 @@ struct Args {
   const uint32_t *masks_this, *masks_other;
   const double2 *ea_this, *ea_other;  // phases
   int* status;
+  int* scale;  // null, or [2][nvec]: see launch_sweep_fx
   uint8_t a[kMaxSteps];     // window position of each step
   uint8_t full[kMaxSteps];  // class 6 moves in this step (det V != 1)
   // the program rotation by rotation, for vectors that take FP64
@@ -780,6 +781,8 @@ __global__ void __launch_bounds__(kCta, 1)
     sync_data();
     wide |= later & wide_range(s_range.out, s_range.tiny_out);
   }
+  if (g.scale && tid < nv)
+    g.scale[(int64_t)blockIdx.y * g.nvec + v0 + tid] = (wide >> tid) & 1 ? -1 : s_eb[tid];
   // ---- phases, store.  The cross tables go where the images were (every
   // copy has landed and been read).
   const int tper = g.nchunk * 256;
@@ -1068,7 +1071,7 @@ FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const R
 
 void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0, void* st1,
                      const FxPlan& plan, const RotProgram& rp, const PhaseDev& ph,
-                     cudaStream_t st) {
+                     cudaStream_t st, int* scale) {
   const Space* sthis = dir == 0 ? sa : sb;
   const Space* sother = dir == 0 ? sb : sa;
   fx::build_index(const_cast<Space*>(sthis));
@@ -1084,6 +1087,7 @@ void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* 
   std::copy(plan.a, plan.a + plan.nsteps, g.a);
   std::copy(plan.full, plan.full + plan.nsteps, g.full);
   g.img = plan.img;
+  g.scale = scale;
   g.pairs = sthis->pairs;
   g.npp = sthis->npp;
   g.m = (int)rp.g.size();

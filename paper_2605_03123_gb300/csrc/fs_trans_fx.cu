@@ -15,10 +15,18 @@ constexpr int kTThreads = 256;
 constexpr int kTWarps = kTThreads / 32;
 constexpr int kTUnits = 4;  // units per pass
 
+// A slab's products are held relative to the product of its two norms.  Where
+// no vector of it comes within 2^-kApart of that (psi and g in different
+// vectors), or one of its vectors was rotated in FP64, the slab is summed in
+// FP64: the digits keep 2^-57 of the norms, FP64 2^-53 of the amplitudes that
+// meet.  (KV equal vectors are 2^-8 apart at most, for KV = 64.)
+constexpr int kApart = 10;
+
 struct TransArgs {
   const double2* st[2];  // psi, g
   int64_t d_b;
   int dir, d, nvec, KV, npass, norb;
+  const int* scale;  // per state and vector, from launch_sweep_fx
   const TPassDev* tpass;
   const TRecord* trec;
   double* T;
@@ -119,6 +127,82 @@ __device__ __forceinline__ void unit(const TransArgs& a, const TPassDev& pd, int
   }
 }
 
+// The same of a slab in FP64: its cells hold the amplitudes, `sum` ([npass][32]
+// [2]) takes each slot's parts as doubles.
+template <int M, int J, bool DIAG, int NS>
+__device__ __forceinline__ void term64(const double2 (&ps)[NS], const double2 (&pg)[NS],
+                                       double (&t)[32]) {
+  constexpr int k = J / 16, a = (J / 4) % 4, b = J % 4;
+  if constexpr (k < NS) {
+    constexpr int S = sub_mask(M, k), slot = a * 4 + b;
+    if constexpr (((S >> b) & 1) && (a == b ? DIAG : !((S >> a) & 1))) {
+      constexpr int k2 = a == b ? k : sub_index(M, (S & ~(1 << b)) | (1 << a));
+      constexpr int lo = a < b ? a : b, hi = a < b ? b : a;
+      constexpr double sg = a != b && (popc4(S & ((1 << hi) - 1) & ~((2 << lo) - 1)) & 1) ? -1 : 1;
+      const double2 g = pg[k2], p = ps[k];
+      t[2 * slot] = fma(sg * g.x, p.x, fma(sg * g.y, p.y, t[2 * slot]));
+      t[2 * slot + 1] = fma(sg * g.x, p.y, fma(-sg * g.y, p.x, t[2 * slot + 1]));
+    }
+  }
+}
+template <int M, bool DIAG, int NS, int... J>
+__device__ __forceinline__ void terms64(const double2 (&ps)[NS], const double2 (&pg)[NS],
+                                        double (&t)[32], std::integer_sequence<int, J...>) {
+  (term64<M, J, DIAG, NS>(ps, pg, t), ...);
+}
+template <int M, bool DIAG>
+__device__ __forceinline__ void record64(const TRecord& rc, const double2* psi, const double2* g,
+                                         double (&t)[32]) {
+  constexpr int NS = sub_count(M);
+  double2 ps[NS], pg[NS];
+#pragma unroll
+  for (int k = 0; k < NS; ++k) {
+    const double f = (rc.flips >> k) & 1u ? -1.0 : 1.0;
+    ps[k] = psi[rc.addr[k]];
+    pg[k] = g[rc.addr[k]];
+    ps[k].x *= f;
+    ps[k].y *= f;
+    pg[k].x *= f;
+    pg[k].y *= f;
+  }
+  terms64<M, DIAG, NS>(ps, pg, t, std::make_integer_sequence<int, 6 * 16>{});
+}
+template <bool DIAG>
+__device__ __noinline__ void unit64(const TransArgs& a, const TPassDev& pd, int q, int nv,
+                                    const double2* psi, const double2* g, int lane,
+                                    unsigned long long* sum) {
+  double t[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) t[i] = 0;
+  const int nrec = (pd.rec1 - pd.rec0) >> 5, nch = nrec * nv;
+  for (int ch = q; ch < nch; ch += kTUnits) {
+    const int kv = ch / nrec, oc = ch - kv * nrec;
+    TRecord rc;
+    *reinterpret_cast<uint4*>(&rc) =
+        __ldg(reinterpret_cast<const uint4*>(a.trec + pd.rec0 + (oc << 5) + lane));
+    const double2* p0 = psi + (size_t)kv * a.d;
+    const double2* g0 = g + (size_t)kv * a.d;
+    switch (rc.m) {
+      case 1: record64<1, DIAG>(rc, p0, g0, t); break;
+      case 2: record64<2, DIAG>(rc, p0, g0, t); break;
+      case 3: record64<3, DIAG>(rc, p0, g0, t); break;
+      case 4: if constexpr (DIAG) record64<4, DIAG>(rc, p0, g0, t); break;
+      default: break;
+    }
+  }
+  // after the halving lane l holds the warp's sum of value l
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const bool up = lane & s;
+#pragma unroll
+    for (int i = 0; i < s; ++i) {
+      const double send = up ? t[i] : t[i + s], keep = up ? t[i + s] : t[i];
+      t[i] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, s);
+    }
+  }
+  if (pd.keep & (1u << (lane >> 1))) atomicAdd(reinterpret_cast<double*>(sum + 2 * lane), t[0]);
+}
+
 // One CTA per slab of KV vectors of both states.  The multiply-adds of the
 // sums (12 wide integer ones per complex product; FP64 would need 4, but
 // GB300 issues two of those per clock and SM) bound it: N = 12 (6,6) 0.18 ms
@@ -183,21 +267,42 @@ __global__ void __launch_bounds__(kTThreads, 1)
   }
   __syncthreads();
   int eb[2];
-  const bool finite = fm[0] < 0x7FF && fm[1] < 0x7FF;
   for (int s = 0; s < 2; ++s) {
     float q = 0.f;
     for (int w = 0; w < kTWarps; ++w) q += s_sum[s][w];
     eb[s] = norm_exponent((int)fm[s], q);
+  }
+  // (the sweep sent every vector that is not finite to FP64)
+  bool apart = false;
+  int most = 0;
+  for (int kv = lane; kv < nv; kv += 32) {
+    const int p = a.scale[v0 + kv], c = a.scale[a.nvec + v0 + kv];
+    apart = apart || p < 0 || c < 0;
+    most = max(most, p + c);
+  }
+  most = __reduce_max_sync(0xFFFFFFFFu, most);
+  apart = __any_sync(0xFFFFFFFFu, apart) || most + kApart < eb[0] + eb[1];
+  for (int s = 0; s < 2 && !apart; ++s) {
     double2* raw = reinterpret_cast<double2*>(cell + (size_t)s * a.KV * a.d);
     int4* c = cell + (size_t)s * a.KV * a.d;
-    if (finite)
 #pragma unroll 4
-      for (int i = tid; i < n; i += kTThreads) c[i] = split_amp(raw[i], eb[s]);
+    for (int i = tid; i < n; i += kTThreads) c[i] = split_amp(raw[i], eb[s]);
   }
   __syncthreads();
   const int4* psi = cell;
   const int4* g = cell + (size_t)a.KV * a.d;
-  if (finite)
+  if (apart) {
+    for (int u = warp; u < a.npass * kTUnits; u += kTWarps) {
+      const int ip = u / kTUnits, q = u - ip * kTUnits;
+      const TPassDev pd = a.tpass[ip];
+      const double2* p = reinterpret_cast<const double2*>(psi);
+      const double2* c = reinterpret_cast<const double2*>(g);
+      if (pd.keep & 0x8421u)
+        unit64<true>(a, pd, q, nv, p, c, lane, tsm + ip * 64);
+      else
+        unit64<false>(a, pd, q, nv, p, c, lane, tsm + ip * 64);
+    }
+  } else {
     for (int u = warp; u < a.npass * kTUnits; u += kTWarps) {
       const int ip = u / kTUnits, q = u - ip * kTUnits;
       const TPassDev pd = a.tpass[ip];
@@ -233,6 +338,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
         atomicAdd(tsm + (ip * 32 + lane) * 2 + 1, (unsigned long long)v[1]);
       }
     }
+  }
   __syncthreads();
   for (int i = tid; i < a.npass * 32; i += kTThreads) {
     const TPassDev pd = a.tpass[i >> 5];
@@ -240,8 +346,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
     if (!(pd.keep & (1u << slot))) continue;
     // hh 2^52 + cr 2^26 in units of 2^(E_psi + E_g - 112)
     const double s = (double)(long long)tsm[2 * i] + ldexp((double)(long long)tsm[2 * i + 1], -26);
-    const double x = finite ? scalbn(s, eb[0] + eb[1] - 2 * 1023 - 60)
-                            : __longlong_as_double(0x7FF8000000000000ll);
+    const double x = apart ? __longlong_as_double((long long)tsm[2 * i])
+                           : scalbn(s, eb[0] + eb[1] - 2 * 1023 - 60);
     const int p = pd.q[slot >> 2], q = pd.q[slot & 3];
     atomicAdd(a.T + 2 * (p * a.norb + q) + (i & 1), x);
   }
@@ -259,7 +365,7 @@ bool trans_fx_supported(const Ctx* ctx, const Space* sthis) {
 }
 
 void launch_trans_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, const void* psi,
-                     const void* g, double* T, cudaStream_t st) {
+                     const void* g, const int* scale, double* T, cudaStream_t st) {
   const Space* sthis = dir == 0 ? sa : sb;
   const Space* sother = dir == 0 ? sb : sa;
   fx::TransArgs a{};
@@ -273,6 +379,7 @@ void launch_trans_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, const 
   a.norb = sthis->norb;
   a.tpass = sthis->tpass;
   a.trec = sthis->trec;
+  a.scale = scale;
   a.T = T;
   // vectors per slab: the fewest waves of slabs, then the narrowest slab
   const size_t avail = (size_t)ctx->prop.sharedMemPerBlockOptin - 1024;

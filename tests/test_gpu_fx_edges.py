@@ -204,3 +204,39 @@ def test_phases_behind_a_rotation_of_wide_range(lib, ctx):
     J[0, 2, 9] = J[0, 9, 2] = np.inf
     got, ref, _ = _both(lib, ctx, run)
     assert np.isnan(ref).any() and (np.isnan(got) == np.isnan(ref)).all()
+
+
+@pytest.mark.parametrize("norb,nelec", [(8, (4, 4)), (10, (5, 4)), (12, (6, 5))])
+@pytest.mark.parametrize("swap", [False, True])
+def test_gradient_entries_between_blocks(lib, ctx, norb, nelec, swap):
+    """Generators that keep each half of the orbitals, a state and a cotangent
+    whose blocks (electrons in the upper half) step down by 1e-9, or one up
+    and one down: the entries of dK between the halves, 1e-9 of the others and
+    less, to TOL of the largest of them.  (Each is a sum over the amplitudes
+    that the excitation joins, where FP64 rounds at 2^-53 of these.)"""
+    g = inputs.rng(42600 + norb)
+    h = norb // 2
+    K = np.zeros((2, norb, norb), complex)
+    for k in K:
+        k[:h, :h] = inputs.random_antihermitian(h, 0.5, g)
+        k[h:, h:] = inputs.random_antihermitian(norb - h, 0.5, g)
+    Ja = np.array([inputs.random_symmetric(norb, 0.5, g) for _ in range(2)])
+    Jb = np.array([inputs.random_symmetric(norb, 0.5, g) for _ in range(2)])
+    la, lb = _levels(lib, ctx, norb, nelec, (1 << h) - 1)
+    level = (la[:, None] + lb[None, :]).astype(float)
+    v, cot = inputs.random_state(norb, nelec, g), inputs.random_state(norb, nelec, g)
+    v *= 1e-9 ** level
+    cot *= 1e-9 ** (level.max() - level if swap else level)
+
+    def run():
+        x, c = torch.from_numpy(v).cuda(), torch.from_numpy(cot).cuda()
+        lib.lucj_forward_(x, K, Ja, Jb, norb, nelec, ctx=ctx)
+        dK = lib.lucj_vjp_(x, c, K, Ja, Jb, norb, nelec, ctx=ctx)[0]
+        return dK, c.cpu().numpy()
+    got, ref, used = _both(lib, ctx, run)
+    assert any(k.startswith("trans_") for k in used), used
+    for block in (np.s_[:, :h, :h], np.s_[:, h:, h:], np.s_[:, :h, h:], np.s_[:, h:, :h]):
+        scale = np.max(np.abs(ref[0][block]))
+        assert scale > 0
+        assert np.max(np.abs(got[0][block] - ref[0][block])) <= TOL * scale, (block, scale)
+    _close_by_level(got[1], ref[1], la, lb)
