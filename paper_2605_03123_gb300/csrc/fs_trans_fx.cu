@@ -15,10 +15,13 @@ constexpr int kTThreads = 256;
 constexpr int kTWarps = kTThreads / 32;
 constexpr int kTUnits = 4;  // units per pass
 
+// Cells of a slab: what the sums below are bounded for (an SM holds 7200).
+constexpr int kMaxVec = 64, kMaxCells = 8191;
+
 // A slab's products are held relative to the product of its two norms.  Where
 // no vector of it comes within 2^-kApart of that (psi and g in different
 // vectors), or one of its vectors was rotated in FP64, the slab is summed in
-// FP64: the digits keep 2^-57 of the norms, FP64 2^-53 of the amplitudes that
+// FP64: the integers keep 2^-59 of the norms, FP64 2^-53 of the amplitudes that
 // meet.  (KV equal vectors are 2^-8 apart at most, for KV = 64.)
 constexpr int kApart = 10;
 
@@ -32,12 +35,12 @@ struct TransArgs {
   double* T;
 };
 
-// An amplitude as integers: each part X = hi 2^26 + lo, |X| <= 2^56 (the
-// slab's 2-norm is below 2^56), lo balanced.
+// An amplitude as integers: each part X = hi 2^27 + lo, |X| < 2^58 (the
+// slab's 2-norm is below 2^58 / 1.001), lo balanced.
 __device__ __forceinline__ int4 split_amp(double2 x, int eb) {
-  const long long a = from_double(x.x, eb + 6), b = from_double(x.y, eb + 6);
-  const int al = (int)((uint32_t)a << 6) >> 6, bl = (int)((uint32_t)b << 6) >> 6;
-  return make_int4((int)((a - al) >> 26), al, (int)((b - bl) >> 26), bl);
+  const long long a = from_double(x.x, eb + 4), b = from_double(x.y, eb + 4);
+  const int al = (int)((uint32_t)a << 5) >> 5, bl = (int)((uint32_t)b << 5) >> 5;
+  return make_int4((int)((a - al) >> 27), al, (int)((b - bl) >> 27), bl);
 }
 __host__ __device__ constexpr int popc4(int x) {
   return (x & 1) + ((x >> 1) & 1) + ((x >> 2) & 1) + ((x >> 3) & 1);
@@ -55,10 +58,14 @@ __host__ __device__ constexpr int sub_index(int M, int mask) {
 __host__ __device__ constexpr int sub_count(int M) { return M == 2 ? 6 : M == 4 ? 1 : 4; }
 
 // Sums of one warp unit: per local slot and part, the products of the high
-// halves and the cross products of high and low halves (the low-low ones are
-// below the last bit kept).  Neither can pass 2^63: by Cauchy-Schwarz the
-// first stays below 2^60, and the second below 2^62.5 for the at most 7100
-// amplitudes of a slab.
+// halves and the cross products of high and low halves.  The low-low ones are
+// left out: with low halves of either sign some 2^-59 of the norms' product, as
+// much as the rounding of X.  Neither sum can pass 2^63, by Cauchy-Schwarz with
+// a norm of 2^31 of the high and 2^26 sqrt(2 T) of the low halves of T amplitudes:
+// the first stays below 2^62, and the second, 2^58 sqrt(2 T), below 2^62.8 for a
+// lane's at most 3 (kMaxCells / 128 + kMaxVec) amplitudes a slot (a record holds
+// three of them at most), and below 2^62 for a slab's kMaxCells once every lane
+// has divided it by 8.
 struct Sums {
   long long hh[16][2], cr[16][2];
 };
@@ -322,7 +329,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
           v[4 * i + 2 * r] = t.hh[i][r];
-          v[4 * i + 2 * r + 1] = t.cr[i][r];
+          v[4 * i + 2 * r + 1] = (t.cr[i][r] + 4) >> 3;
         }
 #pragma unroll
       for (int s = 16; s > 0; s >>= 1) {
@@ -344,10 +351,10 @@ __global__ void __launch_bounds__(kTThreads, 1)
     const TPassDev pd = a.tpass[i >> 5];
     const int slot = (i & 31) >> 1;
     if (!(pd.keep & (1u << slot))) continue;
-    // hh 2^52 + cr 2^26 in units of 2^(E_psi + E_g - 112)
-    const double s = (double)(long long)tsm[2 * i] + ldexp((double)(long long)tsm[2 * i + 1], -26);
+    // hh 2^54 + cr 2^30 in units of 2^(E_psi + E_g - 116)
+    const double s = (double)(long long)tsm[2 * i] + ldexp((double)(long long)tsm[2 * i + 1], -24);
     const double x = apart ? __longlong_as_double((long long)tsm[2 * i])
-                           : scalbn(s, eb[0] + eb[1] - 2 * 1023 - 60);
+                           : scalbn(s, eb[0] + eb[1] - 2 * 1023 - 62);
     const int p = pd.q[slot >> 2], q = pd.q[slot & 3];
     atomicAdd(a.T + 2 * (p * a.norb + q) + (i & 1), x);
   }
@@ -360,7 +367,7 @@ static size_t trans_smem(const Space* sp, int KV, int npass) {
 }  // namespace fx
 
 bool trans_fx_supported(const Ctx* ctx, const Space* sthis) {
-  return sthis->npass > 0 &&
+  return sthis->npass > 0 && sthis->dim <= fx::kMaxCells &&
          fx::trans_smem(sthis, 1, sthis->npass) <= (size_t)ctx->prop.sharedMemPerBlockOptin - 1024;
 }
 
@@ -385,7 +392,9 @@ void launch_trans_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, const 
   const size_t avail = (size_t)ctx->prop.sharedMemPerBlockOptin - 1024;
   const int sms = ctx->prop.multiProcessorCount;
   double best = 0;
-  for (int kv = 1; kv <= 64 && fx::trans_smem(sthis, kv, a.npass) <= avail; ++kv) {
+  for (int kv = 1; kv <= fx::kMaxVec && (int64_t)kv * a.d <= fx::kMaxCells &&
+                   fx::trans_smem(sthis, kv, a.npass) <= avail;
+       ++kv) {
     const int slabs = (a.nvec + kv - 1) / kv;
     const double c = ((slabs + sms - 1) / sms) * (kv + 400.0 / a.d);
     if (kv == 1 || c < best) {
