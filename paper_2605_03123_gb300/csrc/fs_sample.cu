@@ -561,7 +561,7 @@ __global__ void __launch_bounds__(256)
   using A = Acc<R>;
   using T = typename A::T;
   __shared__ T srun[8][8][32];  // [warp][k][lane]: running sums of a lane's slice
-  __shared__ T sincl[8][32], sexcl[8][32];
+  __shared__ T stop[8][32], sexcl[8][32];
   __shared__ uint8_t smass[8][32];  // which of the slice's eight hold mass
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const T total = tc[ntiles - 1];
@@ -623,7 +623,23 @@ __global__ void __launch_bounds__(256)
       }
       T excl = A::shfl_up(incl, 1);
       if (lane == 0) excl = A::zero();
-      sincl[warp][lane] = incl;
+      // Sums that ascend, and rise at slices with mass only, show the first such
+      // slice past a target by themselves.  The scan adds in another order per
+      // lane, so that now and then they do not (a slice without mass ends above
+      // the one before it); then their running maximum over the slices with
+      // mass does (taken always, it cost 12 of 337 us for 1e6 shots from N = 15).
+      T top = incl;
+      const bool rises =
+          A::pos(own) ? A::ge(incl, excl) : !(A::gt(incl, excl) || A::gt(excl, incl));
+      if (__ballot_sync(0xffffffffu, rises) != 0xffffffffu) {
+        if (!A::pos(own)) top = A::zero();
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const T y = A::shfl_up(top, d);
+          if (lane >= d && A::gt(y, top)) top = y;
+        }
+      }
+      stop[warp][lane] = top;
       sexcl[warp][lane] = excl;
       has = __ballot_sync(0xffffffffu, A::pos(own));
       have = g;
@@ -632,12 +648,11 @@ __global__ void __launch_bounds__(256)
     if (lane < cnt) {
       T xg;
       unpack_acc(r.x, xg);
-      // the first slice that crosses the target: sums ascend over the slices
-      int f = 0;
+      int f = 0;  // the first slice with mass that crosses the target
 #pragma unroll
       for (int h = 16; h > 0; h >>= 1)
-        if (!A::gt(sincl[warp][f + h - 1], xg)) f += h;
-      const bool scan = A::gt(sincl[warp][f], xg) && ((has >> f) & 1u);
+        if (!A::gt(stop[warp][f + h - 1], xg)) f += h;
+      const bool scan = A::gt(stop[warp][f], xg);
       if (!scan) f = has ? 31 - __clz(has) : 0;  // the last slice that holds mass
       const unsigned mass = smass[warp][f];
       int pick = -1;

@@ -1,0 +1,101 @@
+"""Shots ordered by group (at least as many shots as groups of 256 amplitudes)
+against the same uniforms drawn one at a time, where the two could part: slices
+without mass inside a group, targets on the rounding of the prefix sums, and
+states that put all shots into a few groups."""
+
+import os
+
+import numpy as np
+import pytest
+
+from paper_2605_03123_gb300 import inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def lib():
+    assert torch.cuda.is_available(), "the GPU tests need a CUDA device"
+    from paper_2605_03123_gb300 import build, fsgpu
+    if not os.path.exists(build.lib_path()):
+        build.build()
+    fsgpu.load_library()
+    return fsgpu
+
+
+def _sums(p):
+    """FP64 sums of one group of 256 masses as the kernels form them: the
+    total (each of 32 lanes eight strided masses, then a butterfly), and the
+    inclusive shuffle scan over the 32 slices of eight neighbours."""
+    lane = np.zeros(32)
+    for k in range(8):
+        lane = lane + p[32 * k:32 * k + 32]
+    for m in (16, 8, 4, 2, 1):
+        lane = lane + lane[np.arange(32) ^ m]
+    own = np.zeros(32)
+    for k in range(8):
+        own = own + p[k::8]
+    incl = own.copy()
+    for d in (1, 2, 4, 8, 16):
+        y = incl.copy()
+        y[d:] = incl[:-d] + incl[d:]
+        incl = y
+    return lane[0], own, incl
+
+
+def _gap_uniforms(x):
+    """Uniforms whose target is the sum before an empty slice, where that
+    slice's own sum lies above it."""
+    total, own, incl = _sums(x * x)
+    out = []
+    for l in range(1, 31):
+        if own[l] == 0 and incl[l] > incl[l - 1] and (own[l + 1:] > 0).sum() > 1:
+            u = incl[l - 1] / total
+            for w in (u, np.nextafter(u, 0), np.nextafter(u, 1)):
+                if w * total == incl[l - 1]:
+                    out.append(w)
+                    break
+    return out
+
+
+def test_target_in_the_rounding_of_an_empty_slice(lib):
+    """The shuffle scan adds in another order per lane, so that a slice without
+    mass can end above the one before it: a target between the two belongs to
+    the next slice with mass, in both forms of the search."""
+    norb, nelec = 6, (3, 3)  # 400 amplitudes: two groups, the second empty
+    found = 0
+    for seed in range(40):
+        g = inputs.rng(1700 + seed)
+        x = np.zeros(400)
+        x[:256] = g.standard_normal(256) * np.repeat(g.random(32) < 0.6, 8)
+        us = _gap_uniforms(x[:256])
+        if not us:
+            continue
+        found += len(us)
+        v = torch.from_numpy(x.astype(np.complex128).reshape(20, 20)).cuda()
+        alone = torch.cat([lib.sample_state(v, norb, nelec, uniforms=np.array([u])) for u in us])
+        u2 = np.array(us + [0.5, 0.25])  # at least two shots: ordered by group
+        got = lib.sample_state(v, norb, nelec, uniforms=u2)[:len(us)]
+        assert torch.equal(got, alone), (seed, got, alone)
+    assert found > 10
+
+
+@pytest.mark.parametrize("dt", [torch.complex64, torch.complex128])
+@pytest.mark.parametrize("norb,nelec,shots", [(6, (3, 3), 300), (8, (4, 4), 3000), (12, (6, 5), 9000)])
+def test_states_with_empty_slices(lib, dt, norb, nelec, shots):
+    """Six in ten slices of eight amplitudes empty, single amplitudes too."""
+    g = inputs.rng(1750 + norb)
+    v = inputs.random_state(norb, nelec, g)
+    flat = v.reshape(-1)
+    flat[np.repeat(g.random((flat.size + 7) // 8) < 0.6, 8)[:flat.size]] = 0
+    flat[g.random(flat.size) < 0.2] = 0
+    x = torch.from_numpy(v).cuda().to(dt)
+    u = torch.from_numpy(g.random(shots)).cuda()
+    groups = (flat.size + 255) // 256
+    assert shots >= groups > 1
+    got = lib.sample_state(x, norb, nelec, uniforms=u)
+    few = groups - 1
+    alone = torch.cat([lib.sample_state(x, norb, nelec, uniforms=u[i:i + few])
+                       for i in range(0, shots, few)])
+    assert torch.equal(got, alone)
