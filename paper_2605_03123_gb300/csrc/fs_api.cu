@@ -40,6 +40,7 @@ void* scratch(Ctx* ctx, const std::string& name, size_t bytes) {
     s.bytes = 0;
     cudaError_t e = cudaMalloc(&s.ptr, bytes);
     if (e != cudaSuccess) {
+      (void)cudaGetLastError();  // reported here, not by the next launch
       set_error("scratch allocation of " + std::to_string(bytes) + " bytes failed: " +
                 cudaGetErrorString(e));
       throw Fail{FS_ERR_NOMEM};
@@ -47,6 +48,17 @@ void* scratch(Ctx* ctx, const std::string& name, size_t bytes) {
     s.bytes = bytes;
   }
   return s.ptr;
+}
+
+bool scratch_fits(const Ctx* ctx, const std::string& name, size_t bytes) {
+  const auto it = ctx->scratch.find(name);
+  return it != ctx->scratch.end() && it->second.bytes >= bytes;
+}
+
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) != cudaSuccess) (void)cudaGetLastError();
+  return s != cudaStreamCaptureStatusNone;
 }
 
 static std::vector<zd> load_cmat(const double* p, int n) {

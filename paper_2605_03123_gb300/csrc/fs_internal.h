@@ -300,6 +300,10 @@ struct ProfScope {  // brackets `kernels` kernel launches
 Space* get_space(Ctx* ctx, int norb, int nocc, cudaStream_t st);
 void free_space(Space* s);
 void* scratch(Ctx* ctx, const std::string& name, size_t bytes);
+// Whether that would allocate nothing; whether the stream is being captured
+// (then nothing can be allocated).
+bool scratch_fits(const Ctx* ctx, const std::string& name, size_t bytes);
+bool capturing(cudaStream_t st);
 
 // ------------------------------------------------------------- errors
 void set_error(const std::string& msg);
@@ -604,7 +608,11 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir,
                   void* st0, void* st1, int nst, int dtype,
                   const RotProgram& prog, const PhaseDev& ph, cudaStream_t st,
                   const RevArgs* rev = nullptr, const FxPlan* fx = nullptr);
-// forward: spins that the small-space sweep takes get no plan.
+// Window tables of the FP64 forward sweeps.
+void build_forward_tables_f64(Space* sp);
+// forward: spins that the small-space sweep takes get no plan.  Builds the tables
+// of every complex128 forward sweep of the two spaces, whatever the program:
+// which sweep a program takes must not decide whether a call allocates.
 FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const RotProgram& pa,
                   const RotProgram& pb, bool forward, cudaStream_t st);
 // That sweep of the program rp, on st0 and (unless null) st1, with the phase

@@ -830,11 +830,16 @@ static void sample_state_t(Ctx* ctx, const cx_t<R>* vec, int64_t n, const double
   // (fewer: as many groups to read as shots, and the ordering on top); 2^24
   // shots at a time bound its scratch to 0.5 GB, group counts to 32 bits.
   constexpr int64_t kOrdered = (int64_t)1 << 24;
-  if (shots >= ngroups && ngroups <= kOrdered) {
+  // A captured call whose scratch an earlier one has not allocated goes one by
+  // one.
+  const int64_t cap = std::min(shots, kOrdered), nblk = (ngroups + 1023) / 1024;
+  const size_t nc = (size_t)(ngroups + nblk) * 4, nr = 2 * (size_t)cap * sizeof(ShotRec);
+  if (shots >= ngroups && ngroups <= kOrdered &&
+      ((scratch_fits(ctx, "sample_count", nc) && scratch_fits(ctx, "sample_shots", nr)) ||
+       !capturing(st))) {
     ProfScope ps("sample_search", st, 6);
-    const int64_t cap = std::min(shots, kOrdered), nblk = (ngroups + 1023) / 1024;
-    uint32_t* count = (uint32_t*)scratch(ctx, "sample_count", (size_t)(ngroups + nblk) * 4);
-    ShotRec* rec = (ShotRec*)scratch(ctx, "sample_shots", 2 * (size_t)cap * sizeof(ShotRec));
+    uint32_t* count = (uint32_t*)scratch(ctx, "sample_count", nc);
+    ShotRec* rec = (ShotRec*)scratch(ctx, "sample_shots", nr);
     for (int64_t s0 = 0; s0 < shots; s0 += cap) {
       const int64_t c = std::min(cap, shots - s0);
       const unsigned grid = (unsigned)((c + 255) / 256);

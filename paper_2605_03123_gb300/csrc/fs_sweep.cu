@@ -321,6 +321,11 @@ static void set_window_geom(SweepGeom& g, Space* sp, int W) {
   g.offs_stride = (sp->nocc + 1) << W;
 }
 
+void build_forward_tables_f64(Space* sp) {
+  constexpr int W = window_width<double, 1>();
+  if (sp->norb >= W && sp->dim > 1 && sp->dim <= kMaxSweepDim) build_window_tables(sp, W);
+}
+
 // The packed tables of a slab of nk sets.
 static void set_packed_geom(SweepGeom& g, const Space* sp, int W, int nk) {
   const Space::Win& wt = sp->win[W];

@@ -1025,6 +1025,15 @@ FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const R
     return r;
   const RotProgram* rp[2] = {&pa, &pb};
   bool sect[2] = {fx_sector(ctx, sa, sb), fx_sector(ctx, sb, sa)};
+  unsigned char* img = nullptr;
+  for (int s = 0; s < 2; ++s) {
+    Space* sp = const_cast<Space*>(s ? sb : sa);
+    if (forward) build_forward_tables_f64(sp);
+    if (!sect[s]) continue;
+    fx::build_index(sp);
+    // (of the longest programs, of both spins)
+    img = (unsigned char*)scratch(ctx, "fx_images", (size_t)2 * fx::kMaxSteps * fx::kStepBytes);
+  }
   if (forward)
     for (int s = 0; s < 2; ++s)
       sect[s] = sect[s] && !pairs_supported(ctx, s ? sb : sa, s ? sa : sb, dtype, *rp[s]);
@@ -1037,8 +1046,6 @@ FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const R
   }
   const int n0 = ok[0] ? r.plan[0].nsteps : 0, n1 = ok[1] ? r.plan[1].nsteps : 0;
   if (n0 + n1 == 0) return r;
-  unsigned char* img =
-      (unsigned char*)scratch(ctx, "fx_images", (size_t)(n0 + n1) * fx::kStepBytes);
   r.plan[0].img = img;
   r.plan[1].img = img + (size_t)n0 * fx::kStepBytes;
   {
@@ -1074,7 +1081,6 @@ void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* 
                      cudaStream_t st, int* scale) {
   const Space* sthis = dir == 0 ? sa : sb;
   const Space* sother = dir == 0 ? sb : sa;
-  fx::build_index(const_cast<Space*>(sthis));
   fx::Args g{};
   g.st[0] = (double2*)st0;
   g.st[1] = (double2*)st1;
