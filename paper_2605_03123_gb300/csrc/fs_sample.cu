@@ -827,36 +827,47 @@ static void sample_state_t(Ctx* ctx, const cx_t<R>* vec, int64_t n, const double
     FS_CUDA(cudaGetLastError());
   }
   // Ordered by group where the groups get at least one shot each on average
-  // (fewer: as many groups to read as shots, and the ordering on top); 2^24
-  // shots at a time bound its scratch to 0.5 GB, group counts to 32 bits.
-  constexpr int64_t kOrdered = (int64_t)1 << 24;
-  // A captured call whose scratch an earlier one has not allocated goes one by
-  // one.
-  const int64_t cap = std::min(shots, kOrdered), nblk = (ngroups + 1023) / 1024;
-  const size_t nc = (size_t)(ngroups + nblk) * 4, nr = 2 * (size_t)cap * sizeof(ShotRec);
-  if (shots >= ngroups && ngroups <= kOrdered &&
-      ((scratch_fits(ctx, "sample_count", nc) && scratch_fits(ctx, "sample_shots", nr)) ||
-       !capturing(st))) {
-    ProfScope ps("sample_search", st, 6);
-    uint32_t* count = (uint32_t*)scratch(ctx, "sample_count", nc);
-    ShotRec* rec = (ShotRec*)scratch(ctx, "sample_shots", nr);
-    for (int64_t s0 = 0; s0 < shots; s0 += cap) {
-      const int64_t c = std::min(cap, shots - s0);
-      const unsigned grid = (unsigned)((c + 255) / 256);
-      FS_CUDA(cudaMemsetAsync(count, 0, (size_t)ngroups * 4, st));
-      k_shot_groups<R><<<grid, 256, 0, st>>>((int)ngroups, (int)ntiles, gc, tc, u + s0, c, count, rec);
-      FS_CUDA(cudaGetLastError());
-      k_count_prefix<<<(unsigned)nblk, 1024, 0, st>>>(count, count + ngroups, ngroups);
-      FS_CUDA(cudaGetLastError());
-      k_block_prefix<<<1, 1024, 0, st>>>(count + ngroups, nblk);
-      FS_CUDA(cudaGetLastError());
-      k_order<<<grid, 256, 0, st>>>(rec, c, count, count + ngroups, rec + cap);
-      FS_CUDA(cudaGetLastError());
-      k_pick<R><<<(unsigned)((c + 511) / 512), 256, 0, st>>>(vec, n, ntiles, tc, rec + cap, c,
-                                                           out + s0);
-      FS_CUDA(cudaGetLastError());
+  // (fewer: as many groups to read as shots, and the ordering on top), in parts
+  // of 2^21 shots or four a group: 64 MB of scratch, or a sixteenth of a
+  // complex64 state.  Without room for it, as in a captured call whose scratch
+  // no earlier one has allocated, one warp per shot.
+  constexpr int64_t kMaxGroups = (int64_t)1 << 24;  // group counts have 32 bits
+  if (shots >= ngroups && ngroups <= kMaxGroups) {
+    const int64_t most = std::max<int64_t>((int64_t)1 << 21, 4 * ngroups);
+    const int64_t parts = (shots + most - 1) / most, cap = (shots + parts - 1) / parts;
+    const int64_t nblk = (ngroups + 1023) / 1024;
+    const size_t nc = (size_t)(ngroups + nblk) * 4, nr = 2 * (size_t)cap * sizeof(ShotRec);
+    uint32_t* count = nullptr;
+    ShotRec* rec = nullptr;
+    if ((scratch_fits(ctx, "sample_count", nc) && scratch_fits(ctx, "sample_shots", nr)) ||
+        !capturing(st)) {
+      try {
+        count = (uint32_t*)scratch(ctx, "sample_count", nc);
+        rec = (ShotRec*)scratch(ctx, "sample_shots", nr);
+      } catch (const Fail& f) {
+        if (f.code != FS_ERR_NOMEM) throw;
+      }
     }
-    return;
+    if (rec) {
+      ProfScope ps("sample_search", st, (int)(6 * parts));
+      for (int64_t s0 = 0; s0 < shots; s0 += cap) {
+        const int64_t c = std::min(cap, shots - s0);
+        const unsigned grid = (unsigned)((c + 255) / 256);
+        FS_CUDA(cudaMemsetAsync(count, 0, (size_t)ngroups * 4, st));
+        k_shot_groups<R><<<grid, 256, 0, st>>>((int)ngroups, (int)ntiles, gc, tc, u + s0, c, count, rec);
+        FS_CUDA(cudaGetLastError());
+        k_count_prefix<<<(unsigned)nblk, 1024, 0, st>>>(count, count + ngroups, ngroups);
+        FS_CUDA(cudaGetLastError());
+        k_block_prefix<<<1, 1024, 0, st>>>(count + ngroups, nblk);
+        FS_CUDA(cudaGetLastError());
+        k_order<<<grid, 256, 0, st>>>(rec, c, count, count + ngroups, rec + cap);
+        FS_CUDA(cudaGetLastError());
+        k_pick<R><<<(unsigned)((c + 511) / 512), 256, 0, st>>>(vec, n, ntiles, tc, rec + cap, c,
+                                                             out + s0);
+        FS_CUDA(cudaGetLastError());
+      }
+      return;
+    }
   }
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((shots + 7) / 8, (int64_t)sms * 16));
   ProfScope ps("sample_search", st);

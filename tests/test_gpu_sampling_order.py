@@ -99,3 +99,52 @@ def test_states_with_empty_slices(lib, dt, norb, nelec, shots):
     alone = torch.cat([lib.sample_state(x, norb, nelec, uniforms=u[i:i + few])
                        for i in range(0, shots, few)])
     assert torch.equal(got, alone)
+
+
+def test_scratch_of_many_shots(lib):
+    """Ten million shots of a small state: ordered in parts whose scratch stays
+    below 80 MB (32 bytes a shot for 2^21 shots at a time, 64 MB, and a few
+    2 MB granules of the allocator), the same shots as in one part each."""
+    norb, nelec = 10, (5, 5)
+    shots = 10_000_000
+    g = inputs.rng(1790)
+    v = torch.from_numpy(inputs.random_state(norb, nelec, g)).cuda().to(torch.complex64)
+    u = torch.rand(shots, dtype=torch.float64, device="cuda")
+    ctx = lib.Context(0)
+    lib.sample_state(v, norb, nelec, uniforms=u[:1000], ctx=ctx)
+    out = torch.empty(shots, dtype=torch.int64, device="cuda")
+    del out  # stays in the caching allocator for the call
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    got = lib.sample_state(v, norb, nelec, uniforms=u, ctx=ctx)
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] < 80 << 20
+    for i in (0, 2 ** 21 - 1000, shots - 20000):
+        assert torch.equal(got[i:i + 20000], lib.sample_state(v, norb, nelec,
+                                                              uniforms=u[i:i + 20000], ctx=ctx))
+    ctx.close()
+
+
+def test_shots_without_room_to_order_them(lib):
+    """A call whose scratch cannot be had draws one shot per warp instead."""
+    norb, nelec = 10, (5, 5)
+    shots = 1_000_000  # 32 MB to order
+    g = inputs.rng(1791)
+    v = torch.from_numpy(inputs.random_state(norb, nelec, g)).cuda().to(torch.complex64)
+    u = torch.rand(shots, dtype=torch.float64, device="cuda")
+    ref = lib.sample_state(v, norb, nelec, uniforms=u)
+    ctx = lib.Context(0)
+    lib.sample_state(v, norb, nelec, uniforms=u[:10], ctx=ctx)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    out = torch.empty(shots, dtype=torch.int64, device="cuda")
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (24 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        del out
+        got = lib.sample_state(v, norb, nelec, uniforms=u, ctx=ctx)
+        torch.cuda.synchronize()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert torch.equal(got, ref)
+    ctx.close()
