@@ -187,12 +187,16 @@ static void build_window_tables(Space* sp, int W) {
     std::vector<uint16_t> rows;
     std::vector<uint2> cls;
     window_rows_host(sp->nocc, W, orbits, off, offs, cls, rows);
-    // every width whose cells fit the 227 KB of a CTA, so that no later call
+    // every width whose cells fit a CTA's shared memory, so that no later call
     // allocates
     wt.pk_at.clear();
     std::vector<uint4> all, chunk;
     std::vector<int> alloff, coff;
-    const int nkmax = (int)std::min<int64_t>(kMaxKV, std::max<int64_t>(1, 232448 / (16 * sp->dim)));
+    int dev = 0, optin = 0;
+    FS_CUDA(cudaGetDevice(&dev));
+    FS_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    const int nkmax =
+        (int)std::min<int64_t>(kMaxKV, std::max<int64_t>(1, optin / (16 * sp->dim)));
     for (int nk = 1; nk <= nkmax; ++nk) {
       window_chunks_host(W, nk, cls, coff, chunk);
       wt.pk_at.push_back((int)all.size());
@@ -676,7 +680,9 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
   if (pair_slab && lg == 0) lg = 1;
   int KV = 1 << lg;
   g.tgrp = KV;
-  if (dtype == FS_C64 && CS == 1 && sthis->norb >= window_width<float, 1>() && sthis->dim > 1) {
+  const bool packed =
+      dtype == FS_C64 && CS == 1 && sthis->norb >= window_width<float, 1>() && sthis->dim > 1;
+  if (packed) {
     // packed slabs take any width (pairs of vectors when forward; reverse,
     // multiples of the power of two above, which stays the length of the FP32
     // sums: longer ones move the gradients by some 1.5e-7): the one with the
@@ -705,7 +711,7 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
   }
   g.nv = KV;
   const int nslabs = (g.nvec + KV - 1) / KV;
-  if (dtype == FS_C64 && CS == 1) {
+  if (packed) {  // (the other kernels advance by KV)
     const int p = packed_pitch(nst, KV);
     if (smem_for(1, p) + tsum * (KV / g.tgrp - 1) + kStaticSlack <= budget) KV = p;
   }
