@@ -258,8 +258,9 @@ static CMat cmat_of(const std::vector<zd>& U, int n) {
 }
 
 // Orbital rotation by the selected method.  FS_ROT_AUTO measures both
-// methods once per (sector, dtype) on a scratch copy of the state (the
-// first such call synchronizes the stream) and keeps the faster.
+// methods once per (sector, dtype, sweep engine) on a scratch copy of the state
+// (the first such call synchronizes the stream) and keeps the faster; a captured
+// call of a sector and engine without a choice takes the sweeps.
 static void rotate_any(Ctx* ctx, Space* sa, Space* sb, void* vec, int dtype,
                        const std::vector<zd>& Ua, const std::vector<zd>& Ub,
                        const RotProgram& pa, const RotProgram& pb, cudaStream_t st) {
@@ -269,10 +270,12 @@ static void rotate_any(Ctx* ctx, Space* sa, Space* sb, void* vec, int dtype,
     if (!minor_path_supported(sa, sb)) {
       path = FS_ROT_GIVENS;
     } else {
-      auto key = std::make_tuple(n, sa->nocc, sb->nocc, dtype);
+      auto key = std::make_tuple(n, sa->nocc, sb->nocc, dtype, ctx->sweep_engine);
       auto it = ctx->rot_choice.find(key);
       if (it != ctx->rot_choice.end()) {
         path = it->second;
+      } else if (capturing(st)) {
+        path = FS_ROT_GIVENS;
       } else {
         const size_t bytes = sa->dim * sb->dim * (dtype == FS_C64 ? 8 : 16);
         void* tv = scratch(ctx, "autotune_state", bytes);

@@ -244,8 +244,9 @@ struct ProfRec {
 
 struct Ctx {
   int device = 0;
-  // autotuned orbital-rotation method per (norb, n_alpha, n_beta, dtype)
-  std::map<std::tuple<int, int, int, int>, int> rot_choice;
+  // autotuned orbital-rotation method per (norb, n_alpha, n_beta, dtype, sweep
+  // engine)
+  std::map<std::tuple<int, int, int, int, int>, int> rot_choice;
   // autotuned slab width (log2 of vectors per CTA) of the batched sweeps per
   // (norb, electrons of the rotated and the other spin, dtype, states,
   // reverse, cross term, shared-memory budget in KB), and the timings behind

@@ -240,3 +240,23 @@ def test_gradient_entries_between_blocks(lib, ctx, norb, nelec, swap):
         assert scale > 0
         assert np.max(np.abs(got[0][block] - ref[0][block])) <= TOL * scale, (block, scale)
     _close_by_level(got[1], ref[1], la, lb)
+
+
+def test_rotation_method_is_measured_per_engine(lib):
+    """FS_ROT_AUTO times sweeps and minors once under each sweep engine: the
+    sweeps of another engine take another time."""
+    c = lib.Context(0)
+    norb, nelec = 9, (4, 5)
+    g = inputs.rng(42800)
+    U = inputs.haar_unitary(norb, g)
+    x = torch.from_numpy(inputs.random_state(norb, nelec, g)).cuda()
+    measured = []
+    for engine in (lib.FS_SWEEP_CUDA_CORE, lib.FS_SWEEP_AUTO, lib.FS_SWEEP_CUDA_CORE):
+        c.set_sweep_engine(engine)
+        c.profile_start()
+        lib.apply_orbital_rotation_(x, U, norb, nelec, ctx=c)
+        used = c.profile_stop()
+        measured.append(any(k.startswith("minor_") for k in used)
+                        and any(k.startswith("sweep_") for k in used))
+    c.close()
+    assert measured == [True, True, False]
