@@ -346,6 +346,21 @@ static int guarded(F&& f) {
   }
 }
 
+// Allows a kernel all the dynamic shared memory a CTA can have.  A launch may
+// not set what it needs itself: the attribute belongs to the kernel, and another
+// thread's launch of it (another context, another sector) may come in between.
+template <typename K>
+void allow_shared_memory(K* kern) {
+  cudaFuncAttributes a;
+  FS_CUDA(cudaFuncGetAttributes(&a, kern));
+  int dev = 0, optin = 0;
+  FS_CUDA(cudaGetDevice(&dev));
+  FS_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+  const int most = optin - (int)a.sharedSizeBytes;
+  if (a.maxDynamicSharedSizeBytes < most)
+    FS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+}
+
 // ------------------------------------------------------ kernel launchers
 // Small matrices travel to the kernels by value, as kernel parameters.
 struct Mat {

@@ -183,8 +183,7 @@ static void same_launch(cx_t<R>* F, int64_t fstride, const cx_t<R>* X, int64_t l
                         int64_t ncol, const Space* sp, int N, const R* V, const Mat& kmat,
                         cudaStream_t st) {
   const size_t smem = same_smem<R>(sp->ne);
-  FS_CUDA(cudaFuncSetAttribute(k_op_same<R, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem));
+  allow_shared_memory(k_op_same<R, L>);
   // four column tiles per CTA: the weights of a string (2000 scattered reads at
   // N = 12) cost as much as one tile's products
   const unsigned ty = (unsigned)std::max<int64_t>(1, std::min<int64_t>((ncol + 511) / 512, 65535));
@@ -399,8 +398,7 @@ static void molecular_hamiltonian_t(Ctx* ctx, Space* sa, Space* sb, const void* 
   const size_t mixed_smem = (size_t)lcap * NN * sizeof(R);
   FS_REQUIRE(same_smem<R>(nea) <= smax && same_smem<R>(neb) <= smax && mixed_smem <= smax, FS_ERR_UNSUPPORTED,
              "operator action: weights exceed shared memory");
-  FS_CUDA(cudaFuncSetAttribute(k_op_mixed<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)mixed_smem));
+  allow_shared_memory(k_op_mixed<R>);
   {
     ProfScope ps("op_weights", st);
     k_op_weights<R><<<(unsigned)std::min<size_t>((nw + 255) / 256, 8 * sms), 256, 0, st>>>(

@@ -912,8 +912,7 @@ void sample_slater(Ctx* ctx, const std::vector<zd>& Phi, int N, int n, const dou
     const int64_t nn = (int64_t)N * N;
     k_projector<<<(unsigned)((nn + 255) / 256), 256, 0, st>>>(K, P, N, n);
   }
-  FS_CUDA(cudaFuncSetAttribute(k_sample_slater, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem));
+  allow_shared_memory(k_sample_slater);
   ProfScope ps("slater_sample", st);
   k_sample_slater<<<(unsigned)grid, B, smem, st>>>(K, N, n, u, shots, out, words, Cg,
                                                    c_smem ? 1 : 0);

@@ -1154,8 +1154,7 @@ void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* 
   // more than half an SM's shared memory: the CTA owns all TMEM of its SM
   const size_t smem = std::max(fixed + (size_t)g.KV * ((size_t)g.d * 16 + tab),
                                (size_t)ctx->prop.sharedMemPerMultiprocessor / 2 + 1024);
-  FS_CUDA(cudaFuncSetAttribute(fx::k_sweep_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem));
+  allow_shared_memory(fx::k_sweep_fx);
   ProfScope ps(dir == 0 ? "sweep_alpha_fx" : "sweep_beta_fx", st);
   fx::k_sweep_fx<<<dim3((g.nvec + g.KV - 1) / g.KV, nst), fx::kCta, smem, st>>>(g, ph.X);
   FS_CUDA(cudaGetLastError());

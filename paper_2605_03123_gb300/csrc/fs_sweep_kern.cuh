@@ -1471,8 +1471,7 @@ template <typename R, int CS, int NST, bool VJP, int W, int NT, bool SPLIT, type
 void launch_sweep_t(const SweepGeom& g, const P& prog, const Mat& X,
                            int nslabs, size_t smem, cudaStream_t st) {
   auto kern = k_sweep<R, CS, NST, VJP, W, NT, SPLIT, TC, PK>;
-  FS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem));
+  allow_shared_memory(kern);
   static const char* names[2][2][2] = {  // [f64][reverse][beta]
       {{"sweep_alpha_f32", "sweep_beta_f32"}, {"sweep_vjp_alpha_f32", "sweep_vjp_beta_f32"}},
       {{"sweep_alpha_f64", "sweep_beta_f64"}, {"sweep_vjp_alpha_f64", "sweep_vjp_beta_f64"}}};
@@ -1508,12 +1507,8 @@ template <typename R, int NST, bool VJP, int W, int NT, bool SPLIT, bool PK = fa
 void launch_batch_t(const SweepJob* jobs, int njobs, int total, int* counter, size_t smem,
                            int grid, cudaStream_t st) {
   auto kern = k_sweep_batch<R, NST, VJP, W, NT, SPLIT, PK>;
-  if (!jobs) {  // attribute only (called before a stream capture); only ever
-                // raised, since several stages share one kernel
-    cudaFuncAttributes fa;
-    FS_CUDA(cudaFuncGetAttributes(&fa, kern));
-    if ((size_t)fa.maxDynamicSharedSizeBytes < smem)
-      FS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (!jobs) {  // attribute only (called before a stream capture)
+    allow_shared_memory(kern);
     return;
   }
   kern<<<grid, NT, smem, st>>>(jobs, njobs, total, counter);

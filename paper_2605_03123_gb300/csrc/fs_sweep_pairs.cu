@@ -161,8 +161,7 @@ void launch_sweep_pairs(Ctx*, const Space* sa, const Space* sb, int dir, void* v
     g.si[k] = rp.g[k].s.imag();
   }
   const size_t smem = pairs::smem_bytes(g);
-  FS_CUDA(cudaFuncSetAttribute(pairs::k_sweep_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem));
+  allow_shared_memory(pairs::k_sweep_pairs);
   const int nt = std::min(256, std::max(64, (4 * g.npp + 31) / 32 * 32));
   ProfScope ps(dir == 0 ? "sweep_alpha_pairs" : "sweep_beta_pairs", st);
   pairs::k_sweep_pairs<<<(unsigned)g.nvec, nt, smem, st>>>(g, ph.X);

@@ -403,8 +403,7 @@ void launch_trans_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, const 
     }
   }
   const size_t smem = fx::trans_smem(sthis, a.KV, a.npass);
-  FS_CUDA(cudaFuncSetAttribute(fx::k_trans_fx, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)smem));
+  allow_shared_memory(fx::k_trans_fx);
   ProfScope ps(dir == 0 ? "trans_alpha_fx" : "trans_beta_fx", st);
   fx::k_trans_fx<<<(a.nvec + a.KV - 1) / a.KV, fx::kTThreads, smem, st>>>(a);
   FS_CUDA(cudaGetLastError());
