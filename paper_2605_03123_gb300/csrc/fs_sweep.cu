@@ -689,8 +689,11 @@ void launch_sweep(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* st0
     // least modelled time.  A slab costs its vectors and a fixed part worth c0
     // of them; slabs run in waves of two per SM (forward slabs that fit half an
     // SM) or one, and a last wave of at most one per SM runs 0.6 as long.
-    // N = 12 (6,6), 924 vectors: 4 forward, 8 reverse (84 to 104 us a sweep;
-    // 2: 127 to 160, 4: 98 to 120).
+    // Measured, forward: N = 12 (6,6) 4 vectors 38 us (chosen), 2 50, 8 46;
+    // N = 13 (5,7) alpha 6 64 (chosen), 2 98, 8 80, beta 2 87 (chosen), 6 69;
+    // N = 16 (3,8) alpha 22 219 (chosen), 2 667, 8 325; N = 10 (5,5) 2 21
+    // (chosen), 16 27.  Reverse: N = 12 (6,6) 8 84 to 97 (chosen), 4 99 to 114,
+    // 2 127 to 150; N = 10 (5,5) 2 33 (chosen), 1 47, 8 59.
     const int unit = nst == 1 ? 2 : g.tgrp, slots = (two_per_sm ? 2 : 1) * ctx->prop.multiProcessorCount;
     const double c0 = 450.0 / g.d + 0.1;
     double best = -1;

@@ -1123,8 +1123,13 @@ void launch_sweep_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, void* 
   g.ea_this = (const double2*)(dir == 0 ? ph.ea_a : ph.ea_b);
   g.ea_other = (const double2*)(dir == 0 ? ph.ea_b : ph.ea_a);
   g.status = ctx->d_status;
-  // vectors per slab: the width with the least modelled time, a wave of
-  // slabs costing its tiles (class 3 the most) and its amplitudes
+  // vectors per slab: the width with the least modelled time, a wave of slabs
+  // costing its tiles (weights of the classes' accumulator columns, 48, 32 and
+  // 16, and what they do not share) and, worth a thousandth of a class 3 tile
+  // each, its amplitudes' load and store.  Measured, one spin: N = 12 (6,6) 7
+  // vectors 98 us (chosen), 4 147, 2 270, 10 125; N = 11 (6,5) 4 73 (chosen), 2
+  // 135, 8 77, 16 110; N = 13 (5,7) alpha 6 272 (chosen), 4 387, 7 321; N = 16
+  // (3,3) 4 114 (chosen), 2 187, 8 133, 16 214.
   const size_t tab = ph.has_x ? (size_t)g.nchunk * 256 * 16 : 0;
   int caps[2];
   fx::caps(sthis->norb, sthis->nocc, caps);

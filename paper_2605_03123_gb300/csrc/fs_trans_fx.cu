@@ -388,7 +388,11 @@ void launch_trans_fx(Ctx* ctx, const Space* sa, const Space* sb, int dir, const 
   a.trec = sthis->trec;
   a.scale = scale;
   a.T = T;
-  // vectors per slab: the fewest waves of slabs, then the narrowest slab
+  // vectors per slab: the least modelled time, a wave of slabs costing its
+  // vectors and what a slab costs by itself (its reductions and scale, worth 400
+  // strings).  Measured, one spin: N = 12 (6,6) 7 vectors 180 us (chosen), 4
+  // 219, 2 242, 6 296; N = 11 (6,5) 4 72 (chosen), 2 87, 1 127, 8 121; N = 9
+  // (4,5) 1 25 (chosen), 2 30, 8 76.
   const size_t avail = (size_t)ctx->prop.sharedMemPerBlockOptin - 1024;
   const int sms = ctx->prop.multiProcessorCount;
   double best = 0;
