@@ -386,8 +386,7 @@ __global__ void __launch_bounds__(256)
 }
 
 // ------------------------------------------- many shots per group
-// With at least as many shots as groups the shots are ordered by group first,
-// so that a group is read and summed once for all of them (one warp per shot
+// Many shots (see sample_state_t) are ordered by group first, so that a group is read and summed once for all of them (one warp per shot
 // reads 2 KB of the state for each: 1e6 shots from N = 15 (7,8), 162k groups,
 // 860 us; ordered, 225 us: locating 75, ordering 20, picking 130).  The decisions are those of k_sample_state: the
 // same sums in the same order, compared in the same way.
@@ -826,13 +825,24 @@ static void sample_state_t(Ctx* ctx, const cx_t<R>* vec, int64_t n, const double
     k_cdf_tiles<R><<<1, 1024, 0, st>>>(ts, ntiles, tc);
     FS_CUDA(cudaGetLastError());
   }
-  // Ordered by group where the groups get at least one shot each on average
-  // (fewer: as many groups to read as shots, and the ordering on top), in parts
-  // of 2^21 shots or four a group: 64 MB of scratch, or a sixteenth of a
+  // Ordered by group from a number of shots on that pays for the launches and
+  // the groups read by few shots.  Measured, one warp per shot against ordered:
+  //   complex64, 249 groups (N = 10): 20000 shots 50 against 62 us, 50000 71
+  //     against 69; 3336 (N = 12): 30000 59 against 77, 100000 114 against 69;
+  //     46011 (N = 14): 100000 137 against 151, 200000 222 against 140;
+  //     two groups, whose counters all shots meet at: 50000 54 against 64,
+  //     100000 87 against 85;
+  //   complex128 (FP64 sums): 20 groups: 3000 45 against 61, 10000 71 against
+  //     61; 3336: 10000 124 against 228, 30000 202 against 153; 46011: 50000 369
+  //     against 408, 100000 581 against 464.
+  // In parts of 2^21 shots or four a group: 64 MB of scratch, or a sixteenth of a
   // complex64 state.  Without room for it, as in a captured call whose scratch
   // no earlier one has allocated, one warp per shot.
   constexpr int64_t kMaxGroups = (int64_t)1 << 24;  // group counts have 32 bits
-  if (shots >= ngroups && ngroups <= kMaxGroups) {
+  const int64_t pays =
+      sizeof(R) == 4 ? (ngroups < 16 ? 100000 : 55000 + ngroups + ngroups / 4)
+                     : std::min<int64_t>(10000 + 7 * ngroups / 2, 32000 + 7 * ngroups / 10);
+  if (shots >= std::max(pays, ngroups) && ngroups <= kMaxGroups) {
     const int64_t most = std::max<int64_t>((int64_t)1 << 21, 4 * ngroups);
     const int64_t parts = (shots + most - 1) / most, cap = (shots + parts - 1) / parts;
     const int64_t nblk = (ngroups + 1023) / 1024;

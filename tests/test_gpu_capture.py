@@ -74,7 +74,7 @@ def test_more_shots_than_the_warm_call(lib, ctx, dt):
     norb, nelec = 9, (4, 5)
     g = inputs.rng(43100)
     v = torch.from_numpy(inputs.random_state(norb, nelec, g)).cuda().to(dt)
-    u = torch.from_numpy(g.random(20000)).cuda()
+    u = torch.from_numpy(g.random(200000)).cuda()
     lib.sample_state(v, norb, nelec, uniforms=u[:10], ctx=ctx)
     torch.cuda.synchronize()
     got = _captured(lambda: lib.sample_state(v, norb, nelec, uniforms=u, ctx=ctx))

@@ -1,7 +1,7 @@
-"""Shots ordered by group (at least as many shots as groups of 256 amplitudes)
-against the same uniforms drawn one at a time, where the two could part: slices
-without mass inside a group, targets on the rounding of the prefix sums, and
-states that put all shots into a few groups."""
+"""Shots ordered by group (calls of MANY shots) against the same uniforms drawn a
+FEW at a time, one warp each, where the two could part: slices without mass
+inside a group, targets on the rounding of the prefix sums, and states that put
+all shots into a few groups."""
 
 import os
 
@@ -12,6 +12,9 @@ from paper_2605_03123_gb300 import inputs
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
+
+# above and below the lines of both types for up to 3000 groups of 256 amplitudes
+MANY, FEW = 130_000, 9_000
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -74,16 +77,16 @@ def test_target_in_the_rounding_of_an_empty_slice(lib):
             continue
         found += len(us)
         v = torch.from_numpy(x.astype(np.complex128).reshape(20, 20)).cuda()
-        alone = torch.cat([lib.sample_state(v, norb, nelec, uniforms=np.array([u])) for u in us])
-        u2 = np.array(us + [0.5, 0.25])  # at least two shots: ordered by group
+        alone = lib.sample_state(v, norb, nelec, uniforms=np.array(us))
+        u2 = np.concatenate([us, g.random(MANY)])
         got = lib.sample_state(v, norb, nelec, uniforms=u2)[:len(us)]
         assert torch.equal(got, alone), (seed, got, alone)
     assert found > 10
 
 
 @pytest.mark.parametrize("dt", [torch.complex64, torch.complex128])
-@pytest.mark.parametrize("norb,nelec,shots", [(6, (3, 3), 300), (8, (4, 4), 3000), (12, (6, 5), 9000)])
-def test_states_with_empty_slices(lib, dt, norb, nelec, shots):
+@pytest.mark.parametrize("norb,nelec", [(6, (3, 3)), (8, (4, 4)), (12, (6, 5))])
+def test_states_with_empty_slices(lib, dt, norb, nelec):
     """Six in ten slices of eight amplitudes empty, single amplitudes too."""
     g = inputs.rng(1750 + norb)
     v = inputs.random_state(norb, nelec, g)
@@ -91,14 +94,47 @@ def test_states_with_empty_slices(lib, dt, norb, nelec, shots):
     flat[np.repeat(g.random((flat.size + 7) // 8) < 0.6, 8)[:flat.size]] = 0
     flat[g.random(flat.size) < 0.2] = 0
     x = torch.from_numpy(v).cuda().to(dt)
-    u = torch.from_numpy(g.random(shots)).cuda()
-    groups = (flat.size + 255) // 256
-    assert shots >= groups > 1
+    u = torch.from_numpy(g.random(MANY)).cuda()
     got = lib.sample_state(x, norb, nelec, uniforms=u)
-    few = groups - 1
-    alone = torch.cat([lib.sample_state(x, norb, nelec, uniforms=u[i:i + few])
-                       for i in range(0, shots, few)])
+    alone = torch.cat([lib.sample_state(x, norb, nelec, uniforms=u[i:i + FEW])
+                       for i in range(0, MANY, FEW)])
     assert torch.equal(got, alone)
+
+
+@pytest.mark.parametrize("dt", [torch.complex64, torch.complex128])
+def test_ends_and_unusable_states(lib, dt):
+    """The ends of the uniform's range, NaN, tails and groups without mass; a
+    state whose norm is no number."""
+    norb, nelec = 10, (5, 4)
+    g = inputs.rng(1780)
+    v = inputs.random_state(norb, nelec, g)
+    flat = v.reshape(-1)
+    flat[flat.size // 3:flat.size // 2] = 0
+    flat[-300:] = 0
+    x = torch.from_numpy(v).cuda().to(dt)
+    u = torch.from_numpy(np.concatenate([[0.0, 1.0, -1.0, np.nan, np.nextafter(1.0, 0.0)],
+                                         g.random(MANY)])).cuda()
+    got = lib.sample_state(x, norb, nelec, uniforms=u)
+    assert torch.equal(got[:FEW], lib.sample_state(x, norb, nelec, uniforms=u[:FEW]))
+    x.view(-1)[7] = float("inf")
+    assert (lib.sample_state(x, norb, nelec, uniforms=u) == -1).all()
+
+
+@pytest.mark.parametrize("dt,line", [(torch.complex64, 55000 + 69 + 17),
+                                     (torch.complex128, 10000 + 241)])
+def test_line_between_the_two_forms(lib, dt, line):
+    """Calls of one shot either side of the line, by their kernels' count."""
+    norb, nelec = 9, (4, 4)  # 63504 / 4 = 15876 amplitudes, 63 groups
+    ctx = lib.Context(0)
+    v = torch.from_numpy(inputs.random_state(norb, nelec, inputs.rng(1781))).cuda().to(dt)
+    u = torch.rand(120000, dtype=torch.float64, device="cuda")
+    used = []
+    for shots in (line - 200, line + 200):
+        ctx.profile_start()
+        lib.sample_state(v, norb, nelec, uniforms=u[:shots], ctx=ctx)
+        used.append(ctx.profile_stop()["sample_search"][2])
+    ctx.close()
+    assert used == [1, 6]
 
 
 def test_scratch_of_many_shots(lib):
