@@ -1018,6 +1018,23 @@ static bool fx_sector(const Ctx* ctx, const Space* sthis, const Space* sother) {
          (size_t)ctx->prop.sharedMemPerBlockOptin - fx::kStaticBytes;
 }
 
+// Whether the forward sweep of a program is faster in digits (engine AUTO).  On
+// few vectors both sweeps are chains of latencies.  Measured for one spin, up
+// to one vector an SM, the FP64 sweep takes some 18 us and 1.25 us a rotation up
+// to 300 strings, 1.65 at 924 (N = 12, n = 6), 3.4 at 3432; the digits 38 us
+// and 5 us a step at 120 strings, 8 to 11 from 300 on.  N = 12 (12,6): 134
+// against 95 us for a dense rotation (66 rotations, 6 steps), but 44 against 47
+// for one of six orbitals (15, 1), and 67 against 86 for a Givens gate between
+// the outer orbitals (21, 5).
+static bool fx_pays(Ctx* ctx, const Space* sthis, const Space* sother, const RotProgram& rp) {
+  const double d = (double)sthis->dim;
+  const int64_t sms = ctx->prop.multiProcessorCount;
+  const double waves = (double)((sother->dim + sms - 1) / sms);
+  const double steps = (double)window_schedule(ctx, rp, sthis->norb, tc::kW).size();
+  return (double)rp.g.size() * std::max(1.25, 1.0 + 7e-4 * d) * waves >=
+         20.0 + steps * std::min(2.5 + 0.02 * d, 8.2 + 7e-4 * d);
+}
+
 FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const RotProgram& pa,
                   const RotProgram& pb, bool forward, cudaStream_t st) {
   FxPair r;
@@ -1034,9 +1051,11 @@ FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const R
     // (of the longest programs, of both spins)
     img = (unsigned char*)scratch(ctx, "fx_images", (size_t)2 * fx::kMaxSteps * fx::kStepBytes);
   }
-  if (forward)
-    for (int s = 0; s < 2; ++s)
-      sect[s] = sect[s] && !pairs_supported(ctx, s ? sb : sa, s ? sa : sb, dtype, *rp[s]);
+  for (int s = 0; forward && s < 2; ++s) {
+    const Space *a = s ? sb : sa, *b = s ? sa : sb;
+    sect[s] = sect[s] && !pairs_supported(ctx, a, b, dtype, *rp[s]) &&
+              (ctx->sweep_engine != FS_SWEEP_AUTO || fx_pays(ctx, a, b, *rp[s]));
+  }
   const bool shared = &pa == &pb;  // one program for both spins
   bool ok[2] = {false, false};
   std::vector<std::array<int64_t, 72>> V[2];

@@ -260,3 +260,26 @@ def test_rotation_method_is_measured_per_engine(lib):
                         and any(k.startswith("sweep_") for k in used))
     c.close()
     assert measured == [True, True, False]
+
+
+@pytest.mark.parametrize("norb,nelec,gate,kernel", [
+    (12, (12, 6), "dense", "sweep_beta_fx"), (12, (12, 6), "givens", "sweep_beta_f64"),
+    (13, (0, 4), "block", "sweep_beta_f64"), (13, (2, 7), "block", "sweep_beta_fx"),
+    (14, (1, 4), "block", "sweep_beta_f64"), (14, (4, 4), "block", "sweep_beta_fx")])
+def test_small_programs_on_few_vectors_stay_in_fp64(lib, ctx, norb, nelec, gate, kernel):
+    """Where the digit sweep's images and steps take longer than the rotations."""
+    g = inputs.rng(42900 + norb)
+    U = inputs.haar_unitary(norb, g)
+    if gate == "givens":
+        c, s = np.cos(0.3), np.sin(0.3)
+        U = np.eye(norb)
+        U[np.ix_([0, norb - 1], [0, norb - 1])] = [[c, s], [-s, c]]
+    elif gate == "block":
+        h = norb // 2
+        U = np.eye(norb, dtype=complex)
+        U[:h, :h] = inputs.haar_unitary(h, g)
+    v = torch.from_numpy(inputs.random_state(norb, nelec, g)).cuda()
+    got, ref, used = _both(lib, ctx, lambda: lib.apply_orbital_rotation(
+        v, np.eye(norb), norb, nelec, U_b=U, ctx=ctx), "FS_SWEEP_AUTO")
+    assert kernel in used, used
+    assert float((got - ref).abs().max()) <= TOL
