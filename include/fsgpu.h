@@ -314,9 +314,10 @@ int fs_apply_quad_ham_evolution(fs_ctx *ctx, void *vec, int dtype, const double 
  * device states of the same sector and dtype; `vec` is read only, `out` is
  * overwritten.  The work runs in blocks whose intermediates (one amplitude
  * per single excitation of a string, n (N - n) + n of them) use at most
- * `workspace_bytes` of scratch (0: min(8 GiB, a quarter of free memory; a
- * single row or column of the state where that is more).  All of it runs in
- * the library's kernels, in the state's precision.
+ * `workspace_bytes` of scratch (0: 8 GiB or a quarter of free memory,
+ * whichever is less), or those of a single row or column of the state where
+ * these are more.  All of it runs in the library's kernels, in the state's
+ * precision.
  * N <= 32.  Asynchronous on `stream`. */
 int fs_apply_molecular_hamiltonian(fs_ctx *ctx, const void *vec, void *out, int dtype,
                                    const double *one_body, const double *two_body,
@@ -371,7 +372,10 @@ int fs_simulate_trotter_diag_coulomb(fs_ctx *ctx, void *vec, int dtype, const do
  * double-float pairs (about 48 significant bits) for FS_C64, so a uniform
  * within about 1e-13 * ||vec||^2 of a boundary may land on either side of
  * it.  Asynchronous on `stream`; the context's scratch holds the prefix
- * tables (8 bytes per 256 amplitudes). */
+ * tables (8 bytes per 256 amplitudes) and, after calls of many shots, at
+ * most 64 MB or 1/16 of the state to order them by groups of 256 amplitudes
+ * (without room for it, and in a captured call before any other has
+ * allocated it, a call draws its shots one by one). */
 int fs_sample_state(fs_ctx *ctx, const void *vec, int dtype, int norb, int n_alpha, int n_beta,
                     const double *uniforms, int64_t shots, int64_t *out, void *stream);
 
