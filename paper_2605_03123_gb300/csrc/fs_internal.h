@@ -315,6 +315,7 @@ struct Fail {
   do {                                                                         \
     cudaError_t e_ = (call);                                                   \
     if (e_ != cudaSuccess) {                                                   \
+      (void)cudaGetLastError(); /* reported here, not by the next launch */    \
       ::fs::set_error(std::string(#call) + ": " + cudaGetErrorString(e_));     \
       throw ::fs::Fail{FS_ERR_CUDA};                                           \
     }                                                                          \

@@ -903,13 +903,18 @@ static void build_index(Space* sp) {
     seg[a].cnt[5] = cnt;
   }
   while (idx.size() % 8) idx.push_back(0);
+  if (sp->fx_idx) FS_CUDA(cudaFree(sp->fx_idx));  // of an attempt without room for the rest
+  sp->fx_idx = nullptr;
   FS_CUDA(cudaMalloc(&sp->fx_idx, std::max<size_t>(idx.size(), 8) * sizeof(uint16_t)));
   FS_CUDA(cudaMemcpy(sp->fx_idx, idx.data(), idx.size() * sizeof(uint16_t),
                      cudaMemcpyHostToDevice));
   sp->fx_seg_h = seg;
   Seg* ds = nullptr;
   FS_CUDA(cudaMalloc(&ds, seg.size() * sizeof(Seg)));
-  FS_CUDA(cudaMemcpy(ds, seg.data(), seg.size() * sizeof(Seg), cudaMemcpyHostToDevice));
+  const cudaError_t e =
+      cudaMemcpy(ds, seg.data(), seg.size() * sizeof(Seg), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) cudaFree(ds);
+  FS_CUDA(e);
   sp->fx_seg = ds;
 }
 
@@ -1047,9 +1052,18 @@ FxPair fx_prepare(Ctx* ctx, const Space* sa, const Space* sb, int dtype, const R
     Space* sp = const_cast<Space*>(s ? sb : sa);
     if (forward) build_forward_tables_f64(sp);
     if (!sect[s]) continue;
-    fx::build_index(sp);
-    // (of the longest programs, of both spins)
-    img = (unsigned char*)scratch(ctx, "fx_images", (size_t)2 * fx::kMaxSteps * fx::kStepBytes);
+    // (images of the longest programs, of both spins)
+    constexpr size_t bytes = (size_t)2 * fx::kMaxSteps * fx::kStepBytes;
+    if (!(sp->fx_seg && scratch_fits(ctx, "fx_images", bytes)) && capturing(st)) {
+      sect[s] = false;
+      continue;
+    }
+    try {
+      fx::build_index(sp);
+      img = (unsigned char*)scratch(ctx, "fx_images", bytes);
+    } catch (const Fail&) {  // no room: the FP64 sweep needs neither
+      sect[s] = false;
+    }
   }
   for (int s = 0; forward && s < 2; ++s) {
     const Space *a = s ? sb : sa, *b = s ? sa : sb;

@@ -79,3 +79,18 @@ def test_more_shots_than_the_warm_call(lib, ctx, dt):
     torch.cuda.synchronize()
     got = _captured(lambda: lib.sample_state(v, norb, nelec, uniforms=u, ctx=ctx))
     assert torch.equal(got, lib.sample_state(v, norb, nelec, uniforms=u, ctx=ctx))
+
+
+def test_digit_sweep_of_a_space_known_to_fp64_only(lib, ctx):
+    """A captured call under FS_SWEEP_AUTO after warm ones under the FP64 engine."""
+    norb, nelec = 12, (6, 5)
+    g = inputs.rng(43200)
+    U = inputs.haar_unitary(norb, g)
+    v = torch.from_numpy(inputs.random_state(norb, nelec, g)).cuda()
+    ctx.set_sweep_engine(lib.FS_SWEEP_CUDA_CORE)
+    ref = lib.apply_orbital_rotation(v, U, norb, nelec, ctx=ctx)
+    ctx.set_sweep_engine(lib.FS_SWEEP_AUTO)
+    x = v.clone()
+    torch.cuda.synchronize()
+    _captured(lambda: lib.apply_orbital_rotation_(x, U, norb, nelec, ctx=ctx))
+    assert torch.equal(x, ref)

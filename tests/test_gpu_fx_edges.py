@@ -283,3 +283,33 @@ def test_small_programs_on_few_vectors_stay_in_fp64(lib, ctx, norb, nelec, gate,
         v, np.eye(norb), norb, nelec, U_b=U, ctx=ctx), "FS_SWEEP_AUTO")
     assert kernel in used, used
     assert float((got - ref).abs().max()) <= TOL
+
+
+def test_without_room_for_the_images(lib, ctx):
+    """A call whose images cannot be allocated rotates in FP64."""
+    norb, nelec = 12, (6, 6)
+    g = inputs.rng(43000)
+    U = inputs.haar_unitary(norb, g)
+    v = torch.from_numpy(inputs.random_state(norb, nelec, g)).cuda()
+    x = v.clone()
+    ctx.set_sweep_engine(lib.FS_SWEEP_CUDA_CORE)
+    ref = lib.apply_orbital_rotation(v, U, norb, nelec, ctx=ctx)
+    ctx.set_sweep_engine(lib.FS_SWEEP_AUTO)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = []
+    try:
+        for left in (256, 32, 4):  # MB; the images take 8.8
+            free = torch.cuda.mem_get_info()[0] - (left << 20)
+            if free > 0:
+                hold.append(torch.empty(free, dtype=torch.uint8, device="cuda"))
+        ctx.profile_start()
+        lib.apply_orbital_rotation_(x, U, norb, nelec, ctx=ctx)
+        used = ctx.profile_stop()
+    finally:
+        hold.clear()
+        torch.cuda.empty_cache()
+    assert not any(k.endswith("_fx") for k in used), used
+    assert torch.equal(x, ref)
+    lib.apply_orbital_rotation_(x, U, norb, nelec, ctx=ctx)  # with room again
+    assert ctx.sync_status() == 0
