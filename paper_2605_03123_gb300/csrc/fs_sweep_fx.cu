@@ -307,7 +307,7 @@ __device__ __forceinline__ void scatter(longlong2* slab, const Item& it, int h,
 // ansatz states near a determinant hold (12 orbitals, generators of 0.1: the last
 // sixteenth of a vector at 2^-15 to 2^-20), whose sweeps would take 5 to 8 times
 // as long.
-//   A vector that starts with zeros is judged by its result under both, since
+//   A vector that starts with zeros is decided by its result under both, since
 // what comes into them may be small (a determinant under a weak rotation); under
 // a program with a rotation weaker than 2^-kWeakBits, where amplitudes could
 // vanish altogether in between, it goes to FP64.
@@ -480,13 +480,13 @@ __global__ void __launch_bounds__(kCta, 1)
   tc::fence_after();
   // bits per vector, the same in all threads: the vectors of a wide range as
   // counted, of zeros throughout, and (the first, before any rotation) those
-  // that go to FP64 at once and those that are judged by their result
+  // that go to FP64 at once and those that their result decides on
   const uint32_t small_bits = g.joined ? kSmallBits : kApartBits;
   auto wide_range = [&](const uint32_t (&count)[kMaxVec], uint32_t tiny) {
     return tiny | __ballot_sync(0xFFFFFFFFu,
                                 lane < nv && (count[lane] & 0xFFFFu) * 16 > (uint32_t)d);
   };
-  auto judge = [&](uint32_t& zero, uint32_t& later) {
+  auto decide = [&](uint32_t& zero, uint32_t& later) {
     const uint32_t nz = lane < nv ? s_range.in[lane] >> 16 : 0;
     const bool fin = lane < nv && s_eb[lane] >= 0;
     zero = __ballot_sync(0xFFFFFFFFu, fin && nz == 0);
@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(kCta, 1)
     }
     __syncthreads();  // the vectors are loaded
     uint32_t zero, later;
-    const bool skip = (judge(zero, later) | zero) == all;
+    const bool skip = (decide(zero, later) | zero) == all;
     if (lane == 0 && skip) {  // no tiles: the copies have to land all the same
       if (!tc::mbar_wait(bar_first, 0)) timeout(g.status);
       if (!tc::mbar_wait(bar_rest, 0)) timeout(g.status);
@@ -662,7 +662,7 @@ __global__ void __launch_bounds__(kCta, 1)
   uint32_t ph_mma = 0;
   __syncthreads();  // with the issuing warp
   uint32_t zero, later;
-  uint32_t wide = judge(zero, later);
+  uint32_t wide = decide(zero, later);
   const bool skip = (wide | zero) == all;
   if (skip) {  // the tables below go where the copies land
     if (!tc::mbar_wait(bar_first, 0)) timeout(g.status);
@@ -761,7 +761,7 @@ __global__ void __launch_bounds__(kCta, 1)
     tc::fence_after();
     tc::tmem_dealloc(s_tmem, 512);
   }
-  // ---- the range of the vectors that are judged by it now
+  // ---- the range now of the vectors that it decides on
   if (later) {
     for (int kv = 0; kv < nv; ++kv) {
       if (!((later >> kv) & 1)) continue;
